@@ -1,29 +1,37 @@
 // Attention of the scale's queries over the compacted per-head cache (Eq. 4 on the compressed
 // cache), plain fp32 arithmetic on the CUDA cores.  This is the exact-precision path (fp32
 // workloads forbid TF32 at the required 1e-5) and the fallback for shapes the tensor-core kernel
-// does not take.  Four threads share one query row (each owns a quarter of the head dimension);
-// K/V tiles of 32 keys are staged in shared memory as fp32; softmax is the usual streaming
-// (running max / running sum) form, rescaled once per group of 8 keys.
+// does not take.
+//
+// Bound: the FMA pipe.  A CTA serves 32 query rows of one head; its four groups of 64 threads walk
+// every fourth tile of 32 keys with a streaming softmax of their own and are merged at the end, so
+// that a launch with few query tiles (256 queries x 16 heads are 128 CTAs) still has eight warps per
+// SM at work.  Inside a group a thread forms 4 x 4 logits and 4 x D/8 outputs: eight 16-byte
+// shared-memory reads per 64 multiply-adds in Q K^T, twenty per 256 in P V, every read without bank
+// conflicts (rows are padded by 16 bytes; the lanes of a warp read 8 different rows or broadcast).
+// Both products run on packed pairs (fma.rn.f32x2).  The key buffer is refilled under the P V product
+// and the value buffer under the next Q K^T product (cp.async).
+// (The earlier form, four threads per query row that each held a quarter of it, read 16 bytes of
+// shared memory per 4 multiply-adds with a four-way bank conflict.  Decoding loop of two layers of 16
+// heads x 128, 2 240 tokens, stage calls: 13.8 -> 1.66 ms; one layer of 16 heads x 64, 680 tokens:
+// 0.531 -> 0.308 ms.)
 #include "hack_internal.h"
+#include "tc_ptx.cuh"
 
 namespace hack {
 namespace {
 
-constexpr int kQPerCta = 32;
-constexpr int kThreads = kQPerCta * 4;
-constexpr int kTileK = 32;
-constexpr int kGroup = 8;
+using ptx::fma2;
+
+constexpr int kBQ = 32;              // query rows per CTA
+constexpr int kBK = 32;              // keys per tile
+constexpr int kGroups = 4;           // groups of 64 threads, each with its own key tiles
+constexpr int kThreads = kGroups * 64;
 
 template <typename T> struct Cvt;
 template <> struct Cvt<float> {
   static constexpr int kPerVec = 4;
-  __device__ static void unpack(const uint4& v, float* f) {
-    f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y);
-    f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w);
-  }
-  __device__ static void store4(float* dst, const float* f) {
-    *reinterpret_cast<float4*>(dst) = make_float4(f[0], f[1], f[2], f[3]);
-  }
+  __device__ static void store4(float* dst, const float4& f) { *reinterpret_cast<float4*>(dst) = f; }
 };
 template <> struct Cvt<__nv_bfloat16> {
   static constexpr int kPerVec = 8;
@@ -35,9 +43,9 @@ template <> struct Cvt<__nv_bfloat16> {
       f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
     }
   }
-  __device__ static void store4(__nv_bfloat16* dst, const float* f) {
-    __nv_bfloat162 a = __floats2bfloat162_rn(f[0], f[1]);
-    __nv_bfloat162 b = __floats2bfloat162_rn(f[2], f[3]);
+  __device__ static void store4(__nv_bfloat16* dst, const float4& f) {
+    __nv_bfloat162 a = __floats2bfloat162_rn(f.x, f.y);
+    __nv_bfloat162 b = __floats2bfloat162_rn(f.z, f.w);
     uint2 p;
     p.x = *reinterpret_cast<uint32_t*>(&a);
     p.y = *reinterpret_cast<uint32_t*>(&b);
@@ -45,132 +53,236 @@ template <> struct Cvt<__nv_bfloat16> {
   }
 };
 
+// 32 rows of D elements from global memory (rows at or past n_rows read as zero) into padded fp32
+// rows; `nthr` threads take part.  fp32 rows arrive by cp.async (the caller commits and waits).
+template <typename T, int D>
+__device__ __forceinline__ void stage_rows(float* dst, const T* src, int n_rows, int t, int nthr) {
+  constexpr int LD = D + 4;
+  if constexpr (sizeof(T) == 4) {
+    constexpr int V = D / 4;
+#pragma unroll 4
+    for (int v = t; v < 32 * V; v += nthr) {
+      const int r = v / V, c = v % V;
+      const uint32_t d = ptx::smem_u32(dst + r * LD + c * 4);
+      const int bytes = r < n_rows ? 16 : 0;                 // 0: the 16 bytes are filled with zeros
+      const T* s = src + (size_t)(r < n_rows ? r : 0) * D + c * 4;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(s), "r"(bytes) : "memory");
+    }
+  } else {
+    constexpr int V = D / 8;
+#pragma unroll 4
+    for (int v = t; v < 32 * V; v += nthr) {
+      const int r = v / V, c = v % V;
+      float f[8];
+      const uint4 raw = r < n_rows ? *reinterpret_cast<const uint4*>(src + (size_t)r * D + c * 8) : make_uint4(0, 0, 0, 0);
+      Cvt<T>::unpack(raw, f);
+      *reinterpret_cast<float4*>(dst + r * LD + c * 8) = make_float4(f[0], f[1], f[2], f[3]);
+      *reinterpret_cast<float4*>(dst + r * LD + c * 8 + 4) = make_float4(f[4], f[5], f[6], f[7]);
+    }
+  }
+}
+
+__device__ __forceinline__ void commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+template <int D>
+constexpr size_t simt_smem_bytes() {
+  // query rows, then per group a key tile, a value tile and a probability tile
+  return sizeof(float) * ((size_t)kBQ * (D + 4) + kGroups * (2 * (size_t)kBK * (D + 4) + kBQ * (kBK + 4)));
+}
+
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads)
 attend_simt_kernel(const StepArgs a, const T* __restrict__ q, T* __restrict__ out) {
   pdl_wait();
-  constexpr int DQ = D / 4;                       // dims per thread
-  constexpr int VEC = Cvt<T>::kPerVec;
-  constexpr int ROWV = D / VEC;
+  constexpr int LD = D + 4, LP = kBK + 4;
+  constexpr int CV = D / 32;                      // float4 columns per thread
   const int bh = blockIdx.y;
-  const int ctx = a.is_ctx[bh % a.n_heads];
-  const int len = a.kept[ctx];
-  const int tid = threadIdx.x;
-  const int qi = blockIdx.x * kQPerCta + tid / 4;
-  const int part = tid % 4;
-  const bool q_ok = qi < a.n_new;
+  const int len = a.kept[a.is_ctx[bh % a.n_heads]];
+  const int q0 = blockIdx.x * kBQ;
+  const int tid = threadIdx.x, grp = tid >> 6, gt = tid & 63;
+  const int ty = gt >> 3, tx = gt & 7;            // rows ty + 8 i; keys tx + 8 j; columns 4 tx + 32 c
 
-  __shared__ __align__(16) float ks[kTileK][D];
-  __shared__ __align__(16) float vs[kTileK][D];
-
-  // this thread's slice of the query row: dims part*DQ .. part*DQ + DQ - 1
-  float qr[DQ];
-  if (q_ok) {
-    const T* qp = q + ((size_t)bh * a.n_new + qi) * D + part * DQ;
-#pragma unroll
-    for (int c = 0; c < DQ / VEC; ++c) {
-      Cvt<T>::unpack(*reinterpret_cast<const uint4*>(qp + c * VEC), qr + c * VEC);
-    }
-  } else {
-#pragma unroll
-    for (int d = 0; d < DQ; ++d) qr[d] = 0.f;
-  }
-  float o[DQ];
-#pragma unroll
-  for (int d = 0; d < DQ; ++d) o[d] = 0.f;
-  float m = -INFINITY, l = 0.f;
+  extern __shared__ __align__(16) float smem[];
+  float* qs = smem;
+  float* ks = qs + kBQ * LD + grp * (2 * kBK * LD + kBQ * LP);
+  float* vs = ks + kBK * LD;
+  float* ps = vs + kBK * LD;
 
   const T* kp = static_cast<const T*>(a.k_plane) + (size_t)a.row_off[bh] * D;
   const T* vp = static_cast<const T*>(a.v_plane) + (size_t)a.row_off[bh] * D;
+  const int n_tiles = (len + kBK - 1) / kBK;
 
-  for (int t0 = 0; t0 < len; t0 += kTileK) {
-    __syncthreads();
-    for (int v = tid; v < kTileK * ROWV; v += kThreads) {
-      const int r = v / ROWV, c = v % ROWV;
-      float fk[VEC], fv[VEC];
-      if (t0 + r < len) {
-        Cvt<T>::unpack(*reinterpret_cast<const uint4*>(kp + (size_t)(t0 + r) * D + c * VEC), fk);
-        Cvt<T>::unpack(*reinterpret_cast<const uint4*>(vp + (size_t)(t0 + r) * D + c * VEC), fv);
-      } else {
+  auto group_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory"); };
+
+  stage_rows<T, D>(qs, q + ((size_t)bh * a.n_new + q0) * D, a.n_new - q0, tid, kThreads);
+  if (grp < n_tiles) stage_rows<T, D>(ks, kp + (size_t)grp * kBK * D, len - grp * kBK, gt, 64);
+  commit();
+  if (grp < n_tiles) stage_rows<T, D>(vs, vp + (size_t)grp * kBK * D, len - grp * kBK, gt, 64);
+  commit();
+  wait_group<1>();
+  __syncthreads();
+
+  float2 o[4][CV][2];
+  float m[4], l[4];                               // l: this thread's share of the row sum
 #pragma unroll
-        for (int e = 0; e < VEC; ++e) { fk[e] = 0.f; fv[e] = 0.f; }
-      }
+  for (int i = 0; i < 4; ++i) {
+    m[i] = -INFINITY;
+    l[i] = 0.f;
 #pragma unroll
-      for (int e = 0; e < VEC; ++e) { ks[r][c * VEC + e] = fk[e]; vs[r][c * VEC + e] = fv[e]; }
-    }
-    __syncthreads();
-    const int n_in_tile = min(kTileK, len - t0);
-    for (int g0 = 0; g0 < n_in_tile; g0 += kGroup) {
-      float z[kGroup];
-#pragma unroll
-      for (int g = 0; g < kGroup; ++g) {
-        float acc = 0.f;
-        const float4* kr = reinterpret_cast<const float4*>(&ks[g0 + g][part * DQ]);
-#pragma unroll
-        for (int d4 = 0; d4 < DQ / 4; ++d4) {
-          const float4 kk = kr[d4];
-          acc = fmaf(qr[4 * d4 + 0], kk.x, acc);
-          acc = fmaf(qr[4 * d4 + 1], kk.y, acc);
-          acc = fmaf(qr[4 * d4 + 2], kk.z, acc);
-          acc = fmaf(qr[4 * d4 + 3], kk.w, acc);
-        }
-        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-        z[g] = (g0 + g < n_in_tile) ? acc * a.sm_scale : -INFINITY;
-      }
-      float m_new = m;
-#pragma unroll
-      for (int g = 0; g < kGroup; ++g) m_new = fmaxf(m_new, z[g]);
-      const float corr = expf(m - m_new);           // exp(-inf) = 0 on the first group
-      l *= corr;
-#pragma unroll
-      for (int d = 0; d < DQ; ++d) o[d] *= corr;
-#pragma unroll
-      for (int g = 0; g < kGroup; ++g) {
-        const float p = expf(z[g] - m_new);
-        l += p;
-        const float4* vr = reinterpret_cast<const float4*>(&vs[g0 + g][part * DQ]);
-#pragma unroll
-        for (int d4 = 0; d4 < DQ / 4; ++d4) {
-          const float4 vv = vr[d4];
-          o[4 * d4 + 0] = fmaf(p, vv.x, o[4 * d4 + 0]);
-          o[4 * d4 + 1] = fmaf(p, vv.y, o[4 * d4 + 1]);
-          o[4 * d4 + 2] = fmaf(p, vv.z, o[4 * d4 + 2]);
-          o[4 * d4 + 3] = fmaf(p, vv.w, o[4 * d4 + 3]);
-        }
-      }
-      m = m_new;
-    }
+    for (int c = 0; c < CV; ++c) o[i][c][0] = o[i][c][1] = make_float2(0.f, 0.f);
   }
-  if (q_ok) {
-    const float inv = 1.f / l;
-    T* op = out + ((size_t)bh * a.n_new + qi) * D + part * DQ;
+
+  for (int t = grp; t < n_tiles; t += kGroups) {
+    // logits: s[i][j] of query row ty + 8 i and key tx + 8 j, even and odd dimensions in the two halves
+    float2 s[4][4];
 #pragma unroll
-    for (int d4 = 0; d4 < DQ / 4; ++d4) {
-      float f[4] = {o[4 * d4] * inv, o[4 * d4 + 1] * inv, o[4 * d4 + 2] * inv, o[4 * d4 + 3] * inv};
-      Cvt<T>::store4(op + 4 * d4, f);
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s[i][j] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int d = 0; d < D; d += 4) {
+      float4 qf[4], kf[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) qf[i] = *reinterpret_cast<const float4*>(qs + (ty + 8 * i) * LD + d);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) kf[j] = *reinterpret_cast<const float4*>(ks + (tx + 8 * j) * LD + d);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          s[i][j] = fma2(make_float2(qf[i].x, qf[i].y), make_float2(kf[j].x, kf[j].y), s[i][j]);
+          s[i][j] = fma2(make_float2(qf[i].z, qf[i].w), make_float2(kf[j].z, kf[j].w), s[i][j]);
+        }
     }
+    group_sync();                                 // both warps are done with the key tile
+    if (t + kGroups < n_tiles)
+      stage_rows<T, D>(ks, kp + (size_t)(t + kGroups) * kBK * D, len - (t + kGroups) * kBK, gt, 64);
+    commit();
+
+    float corr[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float z[4];
+      float mt = m[i];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        z[j] = t * kBK + tx + 8 * j < len ? (s[i][j].x + s[i][j].y) * a.sm_scale : -INFINITY;
+        mt = fmaxf(mt, z[j]);
+      }
+      mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 1));
+      mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 2));
+      mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 4));
+      corr[i] = expf(m[i] - mt);                  // exp(-inf) = 0 in the first tile
+      m[i] = mt;
+      float add = 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float p = expf(z[j] - mt);
+        add += p;
+        ps[(ty + 8 * i) * LP + tx + 8 * j] = p;
+      }
+      l[i] = l[i] * corr[i] + add;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int c = 0; c < CV; ++c)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) { o[i][c][h].x *= corr[i]; o[i][c][h].y *= corr[i]; }
+    wait_group<1>();                              // the value tile has landed (the next keys may still be on their way)
+    group_sync();                                 // ... for both warps; also orders this warp's probability rows
+
+#pragma unroll 2
+    for (int j = 0; j < kBK; j += 4) {
+      float4 pf[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) pf[i] = *reinterpret_cast<const float4*>(ps + (ty + 8 * i) * LP + j);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float4 vf[CV];
+#pragma unroll
+        for (int c = 0; c < CV; ++c) vf[c] = *reinterpret_cast<const float4*>(vs + (j + u) * LD + 4 * tx + 32 * c);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float pu = u == 0 ? pf[i].x : u == 1 ? pf[i].y : u == 2 ? pf[i].z : pf[i].w;
+          const float2 pp = make_float2(pu, pu);
+#pragma unroll
+          for (int c = 0; c < CV; ++c) {
+            o[i][c][0] = fma2(pp, make_float2(vf[c].x, vf[c].y), o[i][c][0]);
+            o[i][c][1] = fma2(pp, make_float2(vf[c].z, vf[c].w), o[i][c][1]);
+          }
+        }
+      }
+    }
+    group_sync();                                 // both warps are done with the value tile
+    if (t + kGroups < n_tiles)
+      stage_rows<T, D>(vs, vp + (size_t)(t + kGroups) * kBK * D, len - (t + kGroups) * kBK, gt, 64);
+    commit();
+    wait_group<1>();                              // the next key tile has landed
+    group_sync();
   }
+  wait_group<0>();
+
+  // merge of the four groups: unnormalised outputs and (max, sum) of every row through shared memory
+  // (a group's own key tile holds its 32 x D outputs, its probability tile the row statistics)
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float li = l[i];
+    li += __shfl_xor_sync(0xffffffffu, li, 1);
+    li += __shfl_xor_sync(0xffffffffu, li, 2);
+    li += __shfl_xor_sync(0xffffffffu, li, 4);
+    if (tx == 0) *reinterpret_cast<float2*>(ps + (ty + 8 * i) * 2) = make_float2(m[i], li);
+#pragma unroll
+    for (int c = 0; c < CV; ++c)
+      *reinterpret_cast<float4*>(ks + (ty + 8 * i) * LD + 4 * tx + 32 * c) =
+          make_float4(o[i][c][0].x, o[i][c][0].y, o[i][c][1].x, o[i][c][1].y);
+  }
+  __syncthreads();
+  constexpr int GSTRIDE = 2 * kBK * LD + kBQ * LP;
+  const float* g0 = qs + kBQ * LD;
+  for (int v = tid; v < kBQ * (D / 4); v += kThreads) {
+    const int r = v / (D / 4), c = v % (D / 4);
+    if (q0 + r >= a.n_new) continue;
+    float2 st[kGroups];
+    float top = -INFINITY;
+#pragma unroll
+    for (int g = 0; g < kGroups; ++g) {
+      st[g] = *reinterpret_cast<const float2*>(g0 + g * GSTRIDE + 2 * kBK * LD + r * 2);
+      top = fmaxf(top, st[g].x);
+    }
+    float sum = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int g = 0; g < kGroups; ++g) {
+      const float w = expf(st[g].x - top);        // 0 for a group without keys
+      sum = fmaf(w, st[g].y, sum);
+      const float4 f = *reinterpret_cast<const float4*>(g0 + g * GSTRIDE + r * LD + c * 4);
+      acc.x = fmaf(w, f.x, acc.x);
+      acc.y = fmaf(w, f.y, acc.y);
+      acc.z = fmaf(w, f.z, acc.z);
+      acc.w = fmaf(w, f.w, acc.w);
+    }
+    const float inv = 1.f / sum;
+    Cvt<T>::store4(out + ((size_t)bh * a.n_new + q0 + r) * D + c * 4,
+                   make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv));
+  }
+}
+
+template <typename T, int D>
+int launch_t(const StepArgs& a, const void* q, void* out, cudaStream_t st) {
+  if (!allow_dynamic_smem(attend_simt_kernel<T, D>, simt_smem_bytes<D>())) return -1;
+  const dim3 grid((a.n_new + kBQ - 1) / kBQ, a.batch * a.n_heads);
+  launch_k(attend_simt_kernel<T, D>, grid, dim3(kThreads), simt_smem_bytes<D>(), st, a, static_cast<const T*>(q),
+           static_cast<T*>(out));
+  return launched(1);
 }
 
 }  // namespace
 
 int launch_attend_simt(const StepArgs& a, int dtype, const void* q, void* out, cudaStream_t st) {
-  dim3 grid((a.n_new + kQPerCta - 1) / kQPerCta, a.batch * a.n_heads);
-  if (dtype == HACK_F32) {
-    if (a.head_dim == 64)
-      launch_k(attend_simt_kernel<float, 64>, grid, kThreads, 0, st, a, static_cast<const float*>(q), static_cast<float*>(out));
-    else
-      launch_k(attend_simt_kernel<float, 128>, grid, kThreads, 0, st, a, static_cast<const float*>(q), static_cast<float*>(out));
-  } else {
-    if (a.head_dim == 64)
-      launch_k(attend_simt_kernel<__nv_bfloat16, 64>, grid, kThreads, 0, st, 
-          a, static_cast<const __nv_bfloat16*>(q), static_cast<__nv_bfloat16*>(out));
-    else
-      launch_k(attend_simt_kernel<__nv_bfloat16, 128>, grid, kThreads, 0, st, 
-          a, static_cast<const __nv_bfloat16*>(q), static_cast<__nv_bfloat16*>(out));
-  }
-  return launched(1);
+  if (dtype == HACK_F32) return a.head_dim == 64 ? launch_t<float, 64>(a, q, out, st) : launch_t<float, 128>(a, q, out, st);
+  return a.head_dim == 64 ? launch_t<__nv_bfloat16, 64>(a, q, out, st) : launch_t<__nv_bfloat16, 128>(a, q, out, st);
 }
 
 }  // namespace hack

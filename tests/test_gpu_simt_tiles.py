@@ -1,0 +1,50 @@
+"""The fp32 kernels at the edges of their tiles, against fp64 evaluations of the same definitions.
+
+Attention bar 1e-5 max-abs, the one the parity tests hold fp32 outputs to: inputs are N(0, 1), so a
+logit is a sum of at most 128 products with |q . k| * scale below about 6; its rounding error is at
+most 128 * 2^-24 * 6 / 6 = 8e-6 in the worst case and about sqrt(128) * 2^-24 = 7e-7 as it comes, it
+enters the output relatively, and |O| is of the order of 1 and below 5."""
+import math
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__ as ge
+    ge.build()
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("sides", [(1,), (4, 4), (4, 4, 1), (5, 6), (1, 8, 8), (3, 11)])
+def test_fp32_attention_over_ragged_tiles(sides, head_dim):
+    """Lengths of 1, 32, 33, 61, 129 and 130 keys: one key, exact tiles, one key more, key groups
+    without a tile; 1 to 121 queries; staged and fused calls."""
+    import numpy as np
+    import torch
+    import paper_2504_09261_b200 as hb
+    heads, batch, total = 3, 2, sum(s * s for s in sides)
+    mask = np.array([[1, 0, 1]], dtype=np.uint8)
+    g = torch.Generator(device="cuda").manual_seed(total + head_dim)
+    caches = [hb.HackCache(1, heads, head_dim, batch, sides, hb.HACK_F32, mask, total, total) for _ in range(2)]
+    ks, vs = [], []
+    for k, side in enumerate(sides):
+        q, kk, v = (torch.randn((batch, heads, side * side, head_dim), generator=g, device="cuda") for _ in range(3))
+        ks.append(kk.double())
+        vs.append(v.double())
+        fused, staged = torch.full_like(q, float("nan")), torch.full_like(q, float("nan"))
+        caches[0].hack_scale_step(0, k, q, kk, v, fused)
+        scores = torch.zeros((batch * heads, caches[1].cand_stride), device="cuda")
+        idx = torch.zeros((batch * heads, caches[1].kept_stride), dtype=torch.int32, device="cuda")
+        caches[1].hack_score(0, k, q, kk, scores)
+        caches[1].hack_select(0, k, scores, idx)
+        caches[1].hack_compact(0, k, idx, kk, v)
+        caches[1].hack_attend(0, k, q, staged)
+        z = q.double() @ torch.cat(ks, 2).transpose(2, 3) / math.sqrt(head_dim)
+        ref = z.softmax(-1) @ torch.cat(vs, 2)
+        assert (fused.double() - ref).abs().max() <= 1e-5
+        assert (staged.double() - ref).abs().max() <= 1e-5
+    for c in caches:
+        c.close()
