@@ -42,7 +42,7 @@ score_logits_kernel(const StepArgs a, const T* __restrict__ q, const T* __restri
       smem_raw, j0, cand, a.n_obs_rows, a.sm_scale,
       [&](int i) { return q + ((size_t)bh * a.n_new + obs_row(a, i)) * D; },     // floor(m * N_k / n) under the uniform rule
       [&](int j) { return cand_row(a, kp, k_new, bh, stored, j); },
-      [&](int i, int j) -> float& { return logits[((size_t)bh * kMaxObs + i) * a.cand_stride + j]; },
+      [&](int i, int j) { return logits + ((size_t)bh * kMaxObs + i) * a.cand_stride + j; },
       [&](int i) { return partials + (((size_t)bh * max_chunks + chunk) * kMaxObs + i) * 2; });
 }
 

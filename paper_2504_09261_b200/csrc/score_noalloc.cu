@@ -47,6 +47,7 @@ template <typename T, int D>
 __global__ void __launch_bounds__(kChunk)
 noalloc_logits_kernel(const DenseArgs a, const T* __restrict__ q, const T* __restrict__ k_cand,
                       float* __restrict__ logits, float* __restrict__ partials) {
+  pdl_wait();
   const int row = blockIdx.y;
   const int chunk = blockIdx.x;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -54,13 +55,14 @@ noalloc_logits_kernel(const DenseArgs a, const T* __restrict__ q, const T* __res
       smem_raw, chunk * kChunk, a.n_cand, a.n_obs_rows, a.sm_scale,
       [&](int i) { return q + ((size_t)row * a.n_queries + (int)(((long long)i * a.n_queries) / a.n_obs_rows)) * D; },
       [&](int j) { return k_cand + ((size_t)row * a.n_cand + j) * D; },
-      [&](int i, int j) -> float& { return logits[((size_t)row * kMaxObs + i) * a.n_cand + j]; },
+      [&](int i, int j) { return logits + ((size_t)row * kMaxObs + i) * a.n_cand + j; },
       [&](int i) { return partials + (((size_t)row * a.chunks_per_row + chunk) * kMaxObs + i) * 2; });
 }
 
 __global__ void __launch_bounds__(256)
 noalloc_reduce_kernel(const DenseArgs a, const float* __restrict__ logits,
                       const float* __restrict__ partials, float* __restrict__ scores, int score_stride) {
+  pdl_wait();
   const int row = blockIdx.y;
   __shared__ float row_m[kMaxObs], row_inv_l[kMaxObs];
   float s;
@@ -83,10 +85,10 @@ cudaError_t run(const DenseArgs& a, int n_rows, const void* q, const void* k, fl
   if (!allow_dynamic_smem(noalloc_logits_kernel<T, D>, smem)) return cudaErrorInvalidValue;
   float* logits = scratch;
   float* partials = scratch + kLogitFloats;
-  noalloc_logits_kernel<T, D><<<dim3(a.chunks_per_row, n_rows), kChunk, smem, st>>>(
-      a, static_cast<const T*>(q), static_cast<const T*>(k), logits, partials);
-  noalloc_reduce_kernel<<<dim3((a.n_cand + 255) / 256, n_rows), 256, 0, st>>>(a, logits, partials, scores,
-                                                                               score_stride);
+  launch_k(noalloc_logits_kernel<T, D>, dim3(a.chunks_per_row, n_rows), dim3(kChunk), smem, st, a,
+           static_cast<const T*>(q), static_cast<const T*>(k), logits, partials);
+  launch_k(noalloc_reduce_kernel, dim3((a.n_cand + 255) / 256, n_rows), dim3(256), 0, st, a, logits, partials, scores,
+           score_stride);
   return cudaGetLastError();
 }
 

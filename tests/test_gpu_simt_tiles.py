@@ -48,3 +48,27 @@ def test_fp32_attention_over_ragged_tiles(sides, head_dim):
         assert (staged.double() - ref).abs().max() <= 1e-5
     for c in caches:
         c.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("n_cand,n_obs,head_dim", [(1, 1, 64), (127, 8, 128), (128, 31, 64), (129, 32, 128), (1153, 32, 64)])
+def test_dense_scores_over_ragged_chunks(n_cand, n_obs, head_dim, dtype):
+    """Chunks of 128 keys cut short, filled and exceeded by one; more chunks than the eight threads
+    that merge a row's statistics; observation rows that leave warps idle.  Bar as in the parity
+    tests of the scores: 1e-4 relative + 1e-7 (fp32 sums of at most 1153 terms)."""
+    import torch
+    import paper_2504_09261_b200 as hb
+    rows, n_q = 3, 50
+    g = torch.Generator(device="cuda").manual_seed(n_cand)
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    q = torch.randn((rows, n_q, head_dim), generator=g, device="cuda").to(dt)
+    k = torch.randn((rows, n_cand, head_dim), generator=g, device="cuda").to(dt)
+    scores = torch.full((rows, n_cand + 3), -1.0, device="cuda")
+    hb.hack_score_noalloc(q, k, scores, rows, n_q, n_cand, n_cand + 3, head_dim,
+                          hb.HACK_F32 if dtype == "f32" else hb.HACK_BF16, n_obs)
+    obs = [m * n_q // n_obs for m in range(n_obs)]
+    z = torch.einsum("rnd,rcd->rnc", q[:, obs].double(), k.double()) / math.sqrt(head_dim)
+    ref = z.softmax(-1).sum(1)
+    got = scores[:, :n_cand].double()
+    assert bool(((got - ref).abs() <= 1e-4 * torch.maximum(got.abs(), ref.abs()) + 1e-7).all())
+    assert bool((scores[:, n_cand:] == -1.0).all())
