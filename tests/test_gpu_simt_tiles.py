@@ -28,7 +28,8 @@ def test_fp32_attention_over_ragged_tiles(sides, head_dim):
     heads, batch, total = 3, 2, sum(s * s for s in sides)
     mask = np.array([[1, 0, 1]], dtype=np.uint8)
     g = torch.Generator(device="cuda").manual_seed(total + head_dim)
-    caches = [hb.HackCache(1, heads, head_dim, batch, sides, hb.HACK_F32, mask, total, total) for _ in range(2)]
+    caches = [hb.HackCache(1, heads, head_dim, batch, sides, hb.HACK_F32, mask, total, total,
+                            n_init_scales=1) for _ in range(2)]
     ks, vs = [], []
     for k, side in enumerate(sides):
         q, kk, v = (torch.randn((batch, heads, side * side, head_dim), generator=g, device="cuda") for _ in range(3))
