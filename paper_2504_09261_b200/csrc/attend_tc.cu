@@ -40,12 +40,16 @@
 // (Tried and dropped: logits in two buffers of 64 keys per tile.  The 128 x 64 x 16 MMA re-reads the
 // whole Q operand from shared memory for half the keys and takes nearly as long as the
 // 128 x 128 x 16 one: the last-scale launch of the 10 521-token workload went from 0.233 to 0.301 ms.)
-// The keys and values of a head come in two segments: len_a rows of the head's cache, then len_b
-// rows of the new scale taken straight from the caller's K/V tensors (second pair of tensor maps).
+// The keys and values of a head come in two segments: len_b rows of the new scale taken straight from
+// the caller's K/V tensors (second pair of tensor maps), then len_a rows of the head's cache.
 // Heads that keep the whole new scale (steps without eviction; structural heads, whose latest scale
 // is protected, Eq. 11) are served that way before the new rows are in the cache: the append
 // (Eq. 3) is done by warp 3 of the same CTAs with bulk copies through a small staging buffer, each
 // CTA of a head taking a slice of the rows; nothing in this launch reads the rows they write.
+// Behind the step's compression launch each head waits (griddepcontrol.wait) only for what that
+// launch gives it: heads of a type the step does not compress for nothing, heads that keep the whole
+// new scale for their stored survivors, which come last, and only evicting contextual heads for
+// everything.  Their CTAs lead the grid and start on the SMs the compression leaves free.
 // A tile's output rows leave through the shared memory of its query tile (free once the last Q K^T
 // product has read it) and one tiled store per 64 columns; the store's 3-D tensor map of the output
 // clips the rows behind a head's last query.
@@ -74,10 +78,13 @@ constexpr uint32_t kCopyChunk = 16384;             // bytes per bulk copy of the
 constexpr float kRescaleThreshold = 32.0f;   // log2 units: p <= 2^32, far inside the bf16 / fp32 range
 
 struct TcParams {
-  int n_heads, n_new, n_pairs;           // n_pairs: CTAs per head
-  int tiles_per_cta;                     // 2, or 1 when the grid would not fill the GPU otherwise
-  int len_a[2], len_b[2];                // per head type: rows read from the cache, then from the caller's K/V
+  int n_new;
+  int first_type, first_heads;           // the head type at the front of head_order and its heads
+  int first_ctas;                        // its CTAs; the other type's follow
+  int n_pairs[2], tiles_per_cta[2];      // per head type: CTAs per head, query tiles per CTA (2, or 1)
+  int len_a[2], len_b[2];                // per head type: rows read from the cache, rows read from the caller's K/V
   int append_new;                        // heads with len_b > 0 also store those rows behind their len_a cache rows
+  int dep[2];                            // per head type: what lies behind the dependency wait (kDep*)
   int q_before_wait;                     // the queries may be read ahead of the dependency wait
   int pos_base;                          // global position of the new scale's first token
   int head_dim_pieces;                   // 16-byte pieces per row
@@ -89,13 +96,17 @@ struct TcParams {
   const uint4* k_new;                    // the caller's K/V (append only)
   const uint4* v_new;
   float scale_log2;                      // sm_scale * log2(e)
-  const uint8_t* is_ctx;
   const int32_t* row_off;
-  const int32_t* head_order;             // longest heads first
+  const int32_t* head_order;             // the heads of first_type, then the others
   __nv_bfloat16* out;
   float* row_stats;                      // optional [b*H, N_k, 2]: reference maximum and sum of every softmax row
   int* status;
 };
+
+// What a head has to wait for when the launch ahead in the stream may still be running.
+constexpr int kDepNothing = 0;           // nothing that launch touches: it compresses the other head type only
+constexpr int kDepCache = 1;             // the cache rows (and the place of the append); the new rows are the caller's
+constexpr int kDepAll = 2;
 
 struct Bars {
   uint64_t q_full[2];
@@ -147,23 +158,28 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   Bars* bars = reinterpret_cast<Bars*>(sm + (2 + kKStages + kVStages) * TILE_BYTES + 2 * kCopyChunk);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int bh = p.head_order[blockIdx.x / p.n_pairs];
-  const int pair = blockIdx.x % p.n_pairs;
-  const int type = p.is_ctx[bh % p.n_heads];
+  // CTAs of the first head type, then those of the other one
+  const bool second = (int)blockIdx.x >= p.first_ctas;
+  const int type = second ? 1 - p.first_type : p.first_type;
+  const int cta = second ? blockIdx.x - p.first_ctas : blockIdx.x;
+  const int n_pairs = p.n_pairs[type];
+  const int bh = p.head_order[(second ? p.first_heads : 0) + cta / n_pairs];
+  const int pair = cta % n_pairs;
+  const int dep = p.dep[type];
   const int len_a = p.len_a[type], len_b = p.len_b[type];
-  const int nblk_a = (len_a + kBN - 1) / kBN;
-  const int nblk = nblk_a + (len_b + kBN - 1) / kBN;      // >= 1: a head never attends over nothing
-  const int q0 = pair * p.tiles_per_cta * kBM;
-  const int ntile = (p.tiles_per_cta == 2 && q0 + kBM < p.n_new) ? 2 : 1;
+  const int nblk_b = (len_b + kBN - 1) / kBN;             // the caller's rows come first: they may not have to wait
+  const int nblk = nblk_b + (len_a + kBN - 1) / kBN;      // >= 1: a head never attends over nothing
+  const int q0 = pair * p.tiles_per_cta[type] * kBM;
+  const int ntile = (p.tiles_per_cta[type] == 2 && q0 + kBM < p.n_new) ? 2 : 1;
 
   const int qrow = bh * p.n_new + q0;
   const int krow = p.row_off[bh];
   const int nrow = bh * p.n_new;
   const long long wlim = p.wait_cycles;
   // K / V tile j of this head: which tensor it comes from and its first row there
-  auto k_src = [&](int j) { return j < nblk_a ? &tm_k : &tm_kn; };
-  auto v_src = [&](int j) { return j < nblk_a ? &tm_v : &tm_vn; };
-  auto tile_row = [&](int j) { return j < nblk_a ? krow + j * kBN : nrow + (j - nblk_a) * kBN; };
+  auto k_src = [&](int j) { return j < nblk_b ? &tm_kn : &tm_k; };
+  auto v_src = [&](int j) { return j < nblk_b ? &tm_vn : &tm_v; };
+  auto tile_row = [&](int j) { return j < nblk_b ? nrow + j * kBN : krow + (j - nblk_b) * kBN; };
   if (warp == kProducerWarp && lane == 0) {
     for (int t = 0; t < 2; ++t) {
       mbar_init(smem_u32(&bars->q_full[t]), 1);
@@ -192,10 +208,10 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       prefetch_tensormap(&tm_kn);
       prefetch_tensormap(&tm_vn);
     }
-    // The queries are the caller's input.  When the kernel ahead of this one in the stream is the
-    // step's own compression launch, whatever produced them had completed before that launch passed
-    // its dependency wait, hence before any CTA of this launch started: they are loaded ahead of the
-    // wait, under the compression's last CTAs.
+    // The queries, like the new rows, are the caller's input.  When the kernel ahead of this one in
+    // the stream is the step's own compression launch, whatever produced them had completed before
+    // that launch passed its own dependency wait, hence before any CTA of this launch started: they
+    // are loaded ahead of the wait.
     auto load_queries = [&]() {
       for (int t = 0; t < ntile; ++t) {
         const uint32_t bar = smem_u32(&bars->q_full[t]);
@@ -205,7 +221,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       }
     };
     if (p.q_before_wait) load_queries();
-    pdl_wait();
+    if (dep == kDepAll || (dep == kDepCache && nblk_b == 0)) pdl_grid_wait();
+    pdl_launch_dependents();
     if (!p.q_before_wait) load_queries();
     mbar_expect_tx(smem_u32(&bars->k_full[0]), TILE_BYTES);
     for (int c = 0; c < SUB; ++c) tma_load_2d(k_sm + c * SUB_BYTES, k_src(0), c * 64, tile_row(0), smem_u32(&bars->k_full[0]));
@@ -220,7 +237,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&bars->tmem_base);
-  pdl_wait();     // everything above overlaps the tail of the previous kernel
+  // Everything above overlaps the tail of the previous kernel.  What waits for that kernel is the
+  // producer (and so everything behind the tiles it loads) and the append.
 
   if (warp == kPvWarp) {
     // ------------------------------------------------------------------ issuer of the P V products
@@ -258,7 +276,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       // contiguous run in the caller's tensor and in the cache plane; the CTAs of the head share
       // them, and one thread moves this CTA's slice with bulk copies through two staging halves
       // (global -> shared -> global), so the append costs no registers and no issue slots.
-      const int per_cta = (len_b + p.n_pairs - 1) / p.n_pairs;
+      if (dep != kDepNothing) pdl_grid_wait();
+      const int per_cta = (len_b + n_pairs - 1) / n_pairs;
       const int r0 = pair * per_cta, r1 = min(len_b, r0 + per_cta);
       for (int r = r0 + lane; r < r1; r += 32) p.pos_plane[krow + len_a + r] = p.pos_base + r;
       if (lane == 0 && r1 > r0) {
@@ -294,6 +313,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       int k_issued = 1, v_issued = 1;               // Q and tile 0 of K and V are already on their way
       bool ok = true;
       for (int j = 1; j < nblk && ok; ++j) {
+        if (dep == kDepCache && j == nblk_b) pdl_grid_wait();   // the head's stored survivors are in place
         {
           const int s = j % kKStages;
           ok = wait_bar(&bars->k_empty[s], ((j / kKStages) & 1) ^ 1, bars, p.status, 1, wlim);
@@ -404,7 +424,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bars->s_free));
         // live keys of this tile: fewer than 128 only in the last tile of either segment
-        const int valid = j < nblk_a ? len_a - j * kBN : len_b - (j - nblk_a) * kBN;
+        const int valid = j < nblk_b ? len_b - j * kBN : len_a - (j - nblk_b) * kBN;
         if (valid < kBN) {
 #pragma unroll
           for (int i = 0; i < kBN; ++i)
@@ -546,6 +566,9 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
+  // The launch behind this one relies on everything ahead of it being complete once this grid is, so
+  // one CTA does not leave before the launch ahead has completed, whatever its heads depend on.
+  if (blockIdx.x == gridDim.x - 1 && tid == 0) pdl_grid_wait();
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -600,9 +623,8 @@ bool make_out_map(CUtensorMap* out_map, const void* base, int heads, int n_new, 
 }
 }  // namespace
 
-int launch_attend_tc(const StepArgs& a, const void* k_map, const void* v_map, const int32_t* head_order,
-                     const void* q, void* out, float* row_stats, const void* k_new, const void* v_new,
-                     int n_heads_served, bool shares_gpu, cudaStream_t st, bool follows_compression) {
+int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_stats, const void* k_new,
+                     const void* v_new, cudaStream_t st, int compression_ctas) {
   CUtensorMap tm_q;
   if (!make_rows_map(&tm_q, q, (uint64_t)a.batch * a.n_heads * a.n_new, a.head_dim)) {
     set_error("attention: cuTensorMapEncodeTiled failed for the queries");
@@ -614,17 +636,9 @@ int launch_attend_tc(const StepArgs& a, const void* k_map, const void* v_map, co
     return -1;
   }
   TcParams p;
-  p.n_heads = a.n_heads;
   p.n_new = a.n_new;
-  const int n_tiles = (a.n_new + kBM - 1) / kBM;
-  // n_heads_served < all heads: only the first heads of head_order (those of one type) are served
-  const int heads = n_heads_served > 0 ? n_heads_served : a.batch * a.n_heads;
-  // one query tile per CTA while that still fits one wave: twice the CTAs, no idle SMs; a launch
-  // that shares the GPU with the other head type's compression keeps two
-  p.tiles_per_cta = (!shares_gpu && n_tiles * heads <= sm_count()) ? 1 : 2;
-  p.n_pairs = (n_tiles + p.tiles_per_cta - 1) / p.tiles_per_cta;
-  const CUtensorMap& tk = *static_cast<const CUtensorMap*>(k_map);
-  const CUtensorMap& tv = *static_cast<const CUtensorMap*>(v_map);
+  const CUtensorMap& tk = *static_cast<const CUtensorMap*>(a.k_map);
+  const CUtensorMap& tv = *static_cast<const CUtensorMap*>(a.v_map);
   CUtensorMap tm_kn = tk, tm_vn = tv;       // placeholders unless a head type reads the caller's rows
   p.append_new = 0;
   for (int t = 0; t < 2; ++t) {
@@ -640,7 +654,26 @@ int launch_attend_tc(const StepArgs& a, const void* k_map, const void* v_map, co
       return -1;
     }
   }
-  p.q_before_wait = follows_compression ? 1 : 0;
+  // Behind the step's compression launch a head type that the step does not compress waits for
+  // nothing, one that keeps the whole new scale waits only for its stored survivors.  The type that
+  // waits least goes first (its CTAs start on the SMs the compression leaves free), then the longer one.
+  for (int t = 0; t < 2; ++t)
+    p.dep[t] = compression_ctas == 0 ? kDepAll : !a.trig[t] ? kDepNothing : p.len_b[t] > 0 ? kDepCache : kDepAll;
+  p.q_before_wait = compression_ctas > 0;
+  p.first_type = p.dep[0] != p.dep[1] ? (p.dep[1] < p.dep[0]) : (a.kept[1] > a.kept[0]);
+  p.first_heads = a.heads_of[p.first_type];
+  // One query tile per CTA while that still fits one wave (twice the CTAs, no idle SMs), else two.  A
+  // type that does not wait for the compression has the SMs that launch does not hold.
+  const int n_tiles = (a.n_new + kBM - 1) / kBM;
+  const bool apart = p.dep[p.first_type] == kDepNothing && p.dep[1 - p.first_type] != kDepNothing;   // one type runs after the other
+  for (int t = 0; t < 2; ++t) {
+    const int heads = apart ? a.heads_of[t] : a.heads_of[0] + a.heads_of[1];
+    const int sms = sm_count() - (p.dep[t] == kDepNothing ? compression_ctas : 0);
+    p.tiles_per_cta[t] = n_tiles * heads <= sms ? 1 : 2;
+    p.n_pairs[t] = (n_tiles + p.tiles_per_cta[t] - 1) / p.tiles_per_cta[t];
+  }
+  p.first_ctas = p.n_pairs[p.first_type] * p.first_heads;
+  const int grid = p.first_ctas + p.n_pairs[1 - p.first_type] * a.heads_of[1 - p.first_type];
   p.pos_base = a.pos_base;
   p.head_dim_pieces = a.head_dim * 2 / 16;
   p.cap[0] = a.cap[0];
@@ -652,13 +685,11 @@ int launch_attend_tc(const StepArgs& a, const void* k_map, const void* v_map, co
   p.k_new = static_cast<const uint4*>(k_new);
   p.v_new = static_cast<const uint4*>(v_new);
   p.scale_log2 = a.sm_scale * 1.4426950408889634f;
-  p.is_ctx = a.is_ctx;
   p.row_off = a.row_off;
-  p.head_order = head_order;
+  p.head_order = a.head_order + (size_t)p.first_type * a.batch * a.n_heads;
   p.out = static_cast<__nv_bfloat16*>(out);
   p.row_stats = row_stats;
   p.status = a.status;
-  const int grid = p.n_pairs * heads;
   if (a.head_dim == 128) {
     if (!allow_dynamic_smem(attend_tc_kernel<128>, tc_smem_bytes<128>())) return -1;
     launch_k(attend_tc_kernel<128>, grid, kThreadsTc, tc_smem_bytes<128>(), st, tm_q, tk, tv, tm_kn, tm_vn, tm_o, p);

@@ -78,7 +78,6 @@ struct CkParams {
   int stage_rows;             // rows (K and V) a CTA stages in shared memory per round of the compaction
   int score_only;             // stop after the scores
   float* scores;              // [b*H, cand_stride] or nullptr
-  int32_t* idx;               // [b*H, kept_stride]
   const uint4* k_new;         // caller's K/V of this scale (compaction of heads whose new rows compete)
   const uint4* v_new;
 };
@@ -872,40 +871,37 @@ int launch_t(const StepArgs& a, const CUtensorMap& tm_cache, const CUtensorMap& 
   cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = ck_config<D>(a, p, attr, st);
   cudaLaunchKernelEx(&cfg, compress_cluster_kernel<D>, tm_cache, tm_new, a, static_cast<const __nv_bfloat16*>(q), p);
-  return launched(1);
+  return launched(n_clusters * cl);
 }
 
 }  // namespace
 
-// Scores only (scores != nullptr, idx == nullptr) or the whole compression of the step (idx != nullptr).
-// Returns 1 (one launch), -1 on a launch error, or 0 when this step is outside what the kernel holds
+// Scores only (scores != nullptr) or the whole compression of the step.  Returns the working CTAs of
+// its one launch, -1 on a launch error, or 0 when this step is outside what the kernel holds
 // (candidate lists beyond 8 x 21 chunks per head, the every-query scoring rounds): the caller then
-// takes the separate scoring, selection and compaction launches.  reserved_sms: CTAs of a launch
-// that is enqueued to run beside this one (0 if none).
+// takes the separate scoring, selection and compaction launches.  reserved_sms: CTAs of the launch
+// behind this one that can run beside it (0 if none).
 int launch_compress_cluster(const StepArgs& a, const void* q, const void* k_new, const void* v_new, float* scores,
-                            int32_t* idx, cudaStream_t st, int reserved_sms) {
+                            cudaStream_t st, int reserved_sms) {
   if (!a.k_map || a.obs_full || a.score_accumulate) return 0;
-  int max_chunks = 0, types = 0;
+  int max_chunks = 0;
   const int n_new_chunks = (a.n_new + kCkChunk - 1) / kCkChunk;
   for (int t = 0; t < 2; ++t)
     if (a.trig[t]) {
       max_chunks = std::max(max_chunks, (a.stored[t] + kCkChunk - 1) / kCkChunk + n_new_chunks);
-      ++types;
     }
-  if (types == 0) return 0;
+  if (max_chunks == 0) return 0;
   int cl = 1;
   while (cl <= kMaxCluster && (max_chunks + cl - 1) / cl > kMaxCpc) cl *= 2;
   if (cl > kMaxCluster) return 0;
   CkParams p{};
   p.cluster = cl;
-  p.score_only = idx == nullptr;
+  p.score_only = scores != nullptr;
   p.scores = scores;
-  p.idx = idx;
   p.k_new = static_cast<const uint4*>(k_new);
   p.v_new = static_cast<const uint4*>(v_new);
-  // clusters that do work: the heads of the triggered types (the split between the types is not
-  // known here; half of the heads each is the usual case)
-  const int n_clusters = std::max(1, a.batch * a.n_heads * types / 2);
+  // clusters that do work: the heads of the triggered types
+  const int n_clusters = std::max(1, a.heads_of[0] * a.trig[0] + a.heads_of[1] * a.trig[1]);
   CUtensorMap tm_new;
   if (!make_rows_map(&tm_new, k_new, (uint64_t)a.batch * a.n_heads * a.n_new, a.head_dim)) {
     set_error("compression: cuTensorMapEncodeTiled failed for the new scale's keys");

@@ -54,7 +54,7 @@ bool attend_tc_serves(const StepArgs& a, int dtype) {
 
 int launch_attend(const StepArgs& a, int dtype, const void* q, void* out, cudaStream_t st) {
   if (attend_tc_serves(a, dtype))
-    return launch_attend_tc(a, a.k_map, a.v_map, a.head_order, q, out, nullptr, nullptr, nullptr, 0, false, st);
+    return launch_attend_tc(a, q, out, nullptr, nullptr, nullptr, st, 0);
   return launch_attend_simt(a, dtype, q, out, st);
 }
 
@@ -121,10 +121,6 @@ struct hack_cache {
   size_t reserved_bytes = 0, peak_bytes = 0;
   uint64_t launches = 0;
   long long wait_cycles = hack::kDefaultWaitCycles;   // limit of the kernels' bounded waits
-  // fused step with one head type compressing: the attention of the other type runs beside the
-  // compression on this stream, forked from and joined to the caller's stream by the two events
-  cudaStream_t side_stream = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool poisoned = false;                        // a launch failed after part of a step had been enqueued
   // optional per-stage device timing (score, select, compact, attend)
   bool timing = false;
@@ -193,6 +189,8 @@ hack::StepArgs make_args(const hack_cache* c, int layer, int scale, const hack_s
   a.kept[0] = p.kept_s;     a.kept[1] = p.kept_c;
   a.cap[0] = c->cap[0];     a.cap[1] = c->cap[1];
   a.trig[0] = p.triggered_s; a.trig[1] = p.triggered_c;
+  a.heads_of[1] = c->cfg.batch * c->n_ctx_heads[layer];
+  a.heads_of[0] = c->cfg.batch * c->cfg.n_heads - a.heads_of[1];
   a.n_obs_rows = p.n_obs_rows;
   // the query subset of Eq. 9: uniform spacing, or one of the ablation's alternatives
   a.obs_first = c->cfg.obs_sampler == HACK_OBS_RECENT ? p.n_new - p.n_obs_rows : 0;
@@ -218,7 +216,7 @@ hack::StepArgs make_args(const hack_cache* c, int layer, int scale, const hack_s
     a.k_map = &c->k_maps[layer];
     a.v_map = &c->v_maps[layer];
     const int bh = c->cfg.batch * c->cfg.n_heads;
-    a.head_order = c->head_order + ((size_t)layer * 2 + (p.kept_c > p.kept_s ? 1 : 0)) * bh;
+    a.head_order = c->head_order + (size_t)layer * 2 * bh;
   }
   return a;
 }
@@ -521,11 +519,6 @@ hack_status_t hack_init_cache(const hack_config_t* cfg, hack_cache_t** out) {
     HACK_TRY(cudaMemset(c->obs_rows, 0, (size_t)cfg->n_scales * hack::kMaxObs * sizeof(int32_t)));
     c->obs_rows_set.assign(cfg->n_scales, 0);
   }
-  if (cfg->dtype == HACK_BF16) {
-    HACK_TRY(cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking));
-    HACK_TRY(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
-    HACK_TRY(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
-  }
   HACK_TRY(cudaMalloc(&c->status, sizeof(int)));
   HACK_TRY(cudaMemset(c->status, 0, sizeof(int)));
   HACK_TRY(cudaDeviceSynchronize());
@@ -559,9 +552,6 @@ hack_status_t hack_free_cache(hack_cache_t* c) {
     if (c->ev_step[sl]) cudaEventDestroy(c->ev_step[sl]);
     if (c->ev_out[sl]) cudaEventDestroy(c->ev_out[sl]);
   }
-  if (c->side_stream) cudaStreamDestroy(c->side_stream);
-  if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-  if (c->ev_join) cudaEventDestroy(c->ev_join);
   if (c->h2d_stream) cudaStreamDestroy(c->h2d_stream);
   if (c->d2h_stream) cudaStreamDestroy(c->d2h_stream);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
@@ -625,7 +615,8 @@ hack_status_t hack_score(hack_cache_t* c, int32_t layer, int32_t scale, const vo
   const hack::StepArgs a = make_args(c, layer, scale, p);
   StageScope ts(c, (cudaStream_t)stream, 0);
   int n = c->cfg.dtype == HACK_BF16
-              ? hack::launch_compress_cluster(a, q, k_new, nullptr, scores, nullptr, (cudaStream_t)stream) : 0;
+              ? hack::launch_compress_cluster(a, q, k_new, nullptr, scores, (cudaStream_t)stream) : 0;
+  if (n > 0) n = 1;                  // one launch
   if (n == 0) n = hack::launch_score(a, c->cfg.dtype, q, k_new, scores, c->scratch, (cudaStream_t)stream);
   if (n < 0) return HACK_ERR_CUDA;   // text recorded by the launcher
   ts.done(n);
@@ -688,12 +679,17 @@ hack_status_t hack_compact(hack_cache_t* c, int32_t layer, int32_t scale, const 
   return HACK_OK;
 }
 
-// k_new / v_new / seg_new: fused step only; head types flagged in seg_new have their new rows read
-// from the caller's tensors and appended by the attention kernel itself.
+// fused: the arguments of a fused step whose tensor-core attention reads the new rows of the head types
+// flagged in seg_new from the caller's tensors and appends them itself (compression_ctas: CTAs of the
+// step's compression launch, 0 if there is none).
+struct FusedAttend {
+  const void* k_new;
+  const void* v_new;
+  const hack::StepArgs* args;
+  int compression_ctas;
+};
 static hack_status_t attend_impl(hack_cache* c, int layer, int scale, const void* q, void* out, float* sigma,
-                                 cudaStream_t st, const void* k_new = nullptr, const void* v_new = nullptr,
-                                 const int* seg_new = nullptr, int only_type = -1, bool finish = true,
-                                 bool shares_gpu = false, bool follows_compression = false) {
+                                 cudaStream_t st, const FusedAttend* fused = nullptr) {
   // lengths are already those after compaction
   LayerState& ls = c->layers[layer];
   hack_step_info_t p{};
@@ -701,40 +697,28 @@ static hack_status_t attend_impl(hack_cache* c, int layer, int scale, const void
   p.kept_s = ls.len[0];
   p.kept_c = ls.len[1];
   p.n_obs_rows = std::min(c->cfg.n_obs, p.n_new);
-  hack::StepArgs a = make_args(c, layer, scale, p);
-  if (seg_new) { a.seg_new[0] = seg_new[0]; a.seg_new[1] = seg_new[1]; }
+  const hack::StepArgs a = fused ? *fused->args : make_args(c, layer, scale, p);
   StageScope ts(c, st, 3);
   int n;
   if (sigma) {
     // Eq. 6 needs the statistics of every softmax row; the tensor-core attention kernel leaves them
     if (!hack::attend_tc_serves(a, c->cfg.dtype))
       return fail(HACK_ERR_UNSUPPORTED, "hack_attend_variance needs a bf16 cache and a scale of at least 32 tokens (128 query rows over all heads)");
-    n = hack::launch_attend_tc(a, a.k_map, a.v_map, a.head_order, q, out, c->attn_row_stats, nullptr, nullptr, 0, false, st);
+    n = hack::launch_attend_tc(a, q, out, c->attn_row_stats, nullptr, nullptr, st, 0);
     if (n >= 0) {
       const int m = hack::launch_attention_variance(a, q, c->attn_row_stats, c->attn_block_var, c->var_blocks, sigma, st);
       n = m < 0 ? m : n + m;
     }
-  } else if (seg_new) {
-    int served = 0;
-    if (only_type >= 0) {
-      // the heads of one type: they lead the head order that puts that type first
-      const int bh = c->cfg.batch * c->cfg.n_heads;
-      const int n_ctx = c->cfg.batch * c->n_ctx_heads[layer];
-      served = only_type == 1 ? n_ctx : bh - n_ctx;
-      a.head_order = c->head_order + ((size_t)layer * 2 + only_type) * bh;
-    }
-    n = hack::launch_attend_tc(a, a.k_map, a.v_map, a.head_order, q, out, nullptr, k_new, v_new, served, shares_gpu, st,
-                               follows_compression);
+  } else if (fused) {
+    n = hack::launch_attend_tc(a, q, out, nullptr, fused->k_new, fused->v_new, st, fused->compression_ctas);
   } else {
     n = hack::launch_attend(a, c->cfg.dtype, q, out, st);
   }
   if (n < 0) return HACK_ERR_CUDA;   // text recorded by the launcher
   ts.done(n);
   c->launches += n;
-  if (finish) {
-    ls.phase = 0;
-    ls.next_scale = scale + 1;
-  }
+  ls.phase = 0;
+  ls.next_scale = scale + 1;
   return HACK_OK;
 }
 
@@ -795,13 +779,10 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
   // new rows as well (Eq. 10) and are compacted first.  The final-scale merge keeps the separate
   // compaction it is wrapped around.
   const bool merge_step = c->cfg.merge_last && scale == c->cfg.n_scales - 1 && p.triggered_c;
-  int seg_new[2] = {0, 0};
   const bool fused_append = hack::attend_tc_serves(a, c->cfg.dtype) && !merge_step;
   if (fused_append) {
-    seg_new[0] = !p.triggered_s || a.protect_new;
-    seg_new[1] = !p.triggered_c;
-    a.seg_new[0] = seg_new[0];
-    a.seg_new[1] = seg_new[1];
+    a.seg_new[0] = !p.triggered_s || a.protect_new;
+    a.seg_new[1] = !p.triggered_c;
   }
   if (!any && p.n_new <= hack::kSmallQueries) {
     // nothing is evicted and the scale is small: one launch appends and attends
@@ -815,45 +796,21 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
     ls.next_scale = scale + 1;
     return HACK_OK;
   }
-  bool compressed = false;
-  // One head type compresses, the other only appends: the attention of the appending heads does
-  // not depend on the compression, so it is enqueued on the cache's side stream, forked here (before
-  // the compression launch) and joined at the end of the step.  Every (batch, head) is independent,
-  // the two launches touch disjoint heads.
-  const int n_ctx_bh = c->cfg.batch * c->n_ctx_heads[layer];
-  const int n_heads_of[2] = {c->cfg.batch * c->cfg.n_heads - n_ctx_bh, n_ctx_bh};
-  const int trig_type = p.triggered_c ? 1 : 0;
-  const bool can_fork = any && fused_append && p.triggered_c != p.triggered_s && !c->timing && c->side_stream &&
-                        n_heads_of[0] > 0 && n_heads_of[1] > 0;
-  if (can_fork) {
-    HACK_CUDA(cudaEventRecord(c->ev_fork, st));
-    HACK_CUDA(cudaStreamWaitEvent(c->side_stream, c->ev_fork, 0));
-  }
+  int compression_ctas = 0;
   if (any && fused_append) {
-    // score, select and compact in one cluster launch per head (counted with the scoring stage)
+    // score, select and compact in one cluster launch per head (counted with the scoring stage).  The
+    // attention launch behind it starts the heads that do not depend on it (a head type that evicts
+    // nothing, two query tiles per CTA) on the SMs it leaves free.
     StageScope ts(c, st, 0);
-    // the appending heads' attention (two query tiles per CTA) runs beside this launch
-    const int beside = can_fork ? n_heads_of[1 - trig_type] * ((p.n_new + 255) / 256) : 0;
-    if ((r = hack::launch_compress_cluster(a, q, k, v, nullptr, c->idx, st, beside)) < 0) return HACK_ERR_CUDA;
-    ts.done(r);
-    n += r;
-    compressed = r > 0;
+    int beside = 0;
+    for (int t = 0; t < 2; ++t)
+      if (!a.trig[t]) beside = a.heads_of[t] * ((p.n_new + 255) / 256);
+    if ((r = hack::launch_compress_cluster(a, q, k, v, nullptr, st, beside)) < 0) return HACK_ERR_CUDA;
+    compression_ctas = r;
+    ts.done(r > 0);
+    n += r > 0;
   }
-  if (can_fork) {
-    if (compressed) {
-      c->launches += n;
-      advance_after_compact(c, layer, p);
-      s = attend_impl(c, layer, scale, q, out, nullptr, c->side_stream, k, v, seg_new, 1 - trig_type, false, true);
-      if (s == HACK_OK) s = attend_impl(c, layer, scale, q, out, nullptr, st, k, v, seg_new, trig_type, true, false, true);
-    }
-    // the side stream always comes back to the caller's stream (it may be part of a capture)
-    cudaEventRecord(c->ev_join, c->side_stream);
-    cudaStreamWaitEvent(st, c->ev_join, 0);
-    if (compressed) {
-      if (s == HACK_ERR_CUDA) c->poisoned = true;
-      return s;
-    }
-  }
+  const bool compressed = compression_ctas > 0;
   if (any && !compressed) {
     {
       StageScope ts(c, st, 0);
@@ -876,8 +833,8 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
   }
   c->launches += n;
   advance_after_compact(c, layer, p);
-  s = attend_impl(c, layer, scale, q, out, nullptr, st, k, v, fused_append ? seg_new : nullptr, -1, true, false,
-                  fused_append && compressed);
+  const FusedAttend fused = {k, v, &a, compression_ctas};
+  s = attend_impl(c, layer, scale, q, out, nullptr, st, fused_append ? &fused : nullptr);
   if (s == HACK_ERR_CUDA) c->poisoned = true;     // compacted, attention not enqueued
   return s;
 }

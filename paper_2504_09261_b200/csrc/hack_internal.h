@@ -25,6 +25,7 @@ struct StepArgs {
   int kept[2];          // length after the step
   int cap[2];           // rows a head of this type owns in the planes (checked builds compare against it)
   int trig[2];          // compression triggered for this type
+  int heads_of[2];      // (batch, head) pairs of this type in the layer
   int seg_new[2];       // tensor-core attention reads this type's new rows from the caller's K/V and
                         // appends them itself (the type keeps the whole new scale in this step)
   long long wait_cycles;   // limit of every bounded device-side wait of the step's kernels
@@ -48,7 +49,7 @@ struct StepArgs {
   // tensor-core attention only (host pointers to 128-byte tensor maps of this layer's planes)
   const void* k_map;
   const void* v_map;
-  const int32_t* head_order;   // device, [batch*n_heads], heads with the longer cache first
+  const int32_t* head_order;   // device, [2][batch*n_heads]: structural heads first, contextual heads first
 };
 
 struct Scratch {
@@ -83,11 +84,12 @@ int launch_score_tc(const StepArgs& a, const void* q, const void* k_new, float* 
                     cudaStream_t st);
 int launch_select(const StepArgs& a, const float* scores, int32_t* idx, int32_t* kept_out,
                   cudaStream_t st);
-// bf16 caches: scores only (idx == nullptr) or scoring, selection and in-place compaction of the step
-// in one launch of one thread-block cluster per head.  1: launched; 0: the step is outside what the
-// kernel holds, take the separate launches; -1: launch error.
+// bf16 caches: scores only (scores != nullptr) or scoring, selection and in-place compaction of the step
+// in one launch of one thread-block cluster per head.  Its CTAs if launched; 0: the step is outside what
+// the kernel holds, take the separate launches; -1: launch error.  reserved_sms: SMs that CTAs of the
+// launch behind this one can use at the same time.
 int launch_compress_cluster(const StepArgs& a, const void* q, const void* k_new, const void* v_new, float* scores,
-                            int32_t* idx, cudaStream_t st, int reserved_sms = 0);
+                            cudaStream_t st, int reserved_sms = 0);
 // idx == nullptr: every head appends (keeps all candidates).  idx_all != 0: idx rows are valid for
 // heads that are not triggered as well (identity lists written by launch_select).
 int launch_compact(const StepArgs& a, int dtype, const int32_t* idx, int idx_all, const void* k_new,
@@ -98,15 +100,12 @@ int launch_attend_simt(const StepArgs& a, int dtype, const void* q, void* out, c
 // row_stats (optional, device [b*H, N_k, 2]): per query row the reference maximum m (raw logit
 // units; within the lazy-rescaling margin of the true maximum) and l = sum_j exp2(c (z_j - m)).
 // k_new / v_new (optional): the caller's K/V of this scale; head types with a.seg_new set then attend
-// over [kept - N_k cache rows ; the N_k new rows read from k_new / v_new] and the kernel appends
-// those rows to the cache, so no append or copy launch precedes it for them.  n_heads_served: 0 for
-// every head, else only the first n_heads_served heads of head_order are served (the heads of one type);
-// shares_gpu: another kernel of the step runs beside this launch.  follows_compression: the launch ahead
-// of this one in the stream is the step's compression launch (the queries, which no kernel of the step
-// writes, may then be read before the dependency wait).
-int launch_attend_tc(const StepArgs& a, const void* k_map, const void* v_map, const int32_t* head_order,
-                     const void* q, void* out, float* row_stats, const void* k_new, const void* v_new,
-                     int n_heads_served, bool shares_gpu, cudaStream_t st, bool follows_compression = false);
+// over [the N_k new rows read from k_new / v_new ; kept - N_k cache rows] and the kernel appends
+// those rows to the cache, so no append or copy launch precedes it for them.  compression_ctas: CTAs
+// of the step's compression launch when that is the launch ahead of this one in the stream (heads that
+// do not depend on it then start beside it), 0 if it is not.
+int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_stats, const void* k_new,
+                     const void* v_new, cudaStream_t st, int compression_ctas);
 constexpr long long kDefaultWaitCycles = 2000000000ll;   // about one second: no wait is legitimately longer
 // Attention variance per (batch, head) over the compacted cache (Eq. 6) from the row statistics of
 // launch_attend_tc; block_var: device scratch [b*H, max_blocks]; sigma: device [b*H].  bf16 only.
@@ -166,9 +165,11 @@ __device__ __forceinline__ bool dbg_ok(bool, int*, int) { return true; }
 __device__ __forceinline__ int obs_row(const StepArgs& a, int i) {
   return a.obs_rows ? a.obs_rows[i] : a.obs_first + (int)(((long long)i * a.obs_span) / a.n_obs_rows);
 }
+__device__ __forceinline__ void pdl_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_grid_wait();
+  pdl_launch_dependents();
 }
 #endif
 
