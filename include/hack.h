@@ -197,10 +197,9 @@ HACK_API hack_status_t hack_classify_heads(const double* sigma, int32_t n_layers
  * candidate count does not exceed their budget skip scoring and selection and keep everything
  * (section "KV Cache Compression for VAR": compress whenever the length exceeds the budget).
  * bf16 caches: at most two launches (one cluster launch that scores, selects and compacts, one
- * attention launch that also appends the rows of heads which keep the whole new scale).  When one
- * head type compresses and the other only appends, the appending heads' attention is enqueued on a
- * stream of the cache's own, forked from `stream` at the start of the call and joined to it before
- * the call returns, so `stream` still orders everything (also inside a stream capture). */
+ * attention launch that also appends the rows of heads which keep the whole new scale).  The
+ * attention of heads that do not depend on the compression runs beside it; `stream` orders everything
+ * (also inside a stream capture). */
 HACK_API hack_status_t hack_scale_step(hack_cache_t* cache, int32_t layer, int32_t scale, const void* q,
                               const void* k, const void* v, void* out, void* stream);
 

@@ -623,6 +623,12 @@ bool make_out_map(CUtensorMap* out_map, const void* base, int heads, int n_new, 
 }
 }  // namespace
 
+float attend_tc_sm_us(const StepArgs& a, int type) {
+  // 4.5 us around the steps of a CTA; a step of 128 keys is bound by the exponentials at head_dim 64
+  const float step_us = a.head_dim == 128 ? 1.6f : 1.2f;
+  return (float)a.heads_of[type] * ((a.n_new + 2 * kBM - 1) / (2 * kBM)) * (4.5f + step_us * ((a.kept[type] + kBN - 1) / kBN));
+}
+
 int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_stats, const void* k_new,
                      const void* v_new, cudaStream_t st, int compression_ctas) {
   CUtensorMap tm_q;

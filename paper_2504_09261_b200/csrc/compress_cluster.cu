@@ -9,31 +9,39 @@
 //
 //   1. scores, pass 1: each CTA streams its chunks through a TMA ring and forms their logits
 //      against the (at most 32) observation rows with tcgen05.mma, as score_tc.cu does, but every
-//      chunk keeps its own accumulator [128 lanes x 32 columns] in tensor memory (chunks past the
-//      15th go through one bounce accumulator into shared memory).  Consumer thread r owns key r
-//      of a chunk and keeps the running (max, sum-exp) of the 32 softmax rows.
+//      chunk keeps its own accumulator [128 lanes x 32 columns] in tensor memory (the ones that do not
+//      fit take turns on two bounce accumulators and go to shared memory if they are read again).
+//      Thread r of a consumer set owns key r of a chunk and keeps (reference maximum, sum-exp) of half
+//      of the softmax rows; the 32 keys of a warp are merged by exchanging halves between lanes.
 //   2. the CTAs publish their row statistics in shared memory; after a cluster barrier every CTA
 //      merges all of them, in rank order, through distributed shared memory.
 //   3. scores, pass 2: the logits are read back from tensor / shared memory (no second key
 //      load, no second MMA) and s_j = sum_i exp(z_ij - m_i) / l_i becomes an order-preserving
-//      32-bit key in shared memory (protected candidates of structural heads carry the top key).
+//      32-bit key in shared memory (protected candidates of structural heads carry the top key).  The new
+//      scale of a head that keeps it whole ends with pass 1: it is neither ranked nor listed.
 //   4. exact radix select over the cluster: digits of 12, 12 and 8 bits; every CTA builds the
-//      histogram of its own keys (the first one while it forms them), the histograms are added
-//      through distributed shared memory after a cluster barrier, and every CTA locates the same
-//      digit.  The select stops once all entries left in the located bin survive.  Ties at the
-//      threshold go to the lowest candidate indices.
-//   5. the CTAs exchange their counts of kept entries, which gives every CTA its offset in the
-//      head's ascending index list; every entry goes straight into the shared memory of the CTA
-//      that will move it (the list never touches global memory).
+//      histogram of its own keys (the first one while it forms them) and publishes it in groups of 16
+//      bins; after a cluster barrier a thread adds one group over the cluster (4 bytes per CTA instead
+//      of 32), and one warp reads the bins of the group that holds the wanted rank, which also gives
+//      every CTA's counts and so its offset in the head's index list.  The select stops once all
+//      entries left in the located bin survive.  Ties at the threshold go to the lowest indices.
+//   5. ascending index list by ballot counts; every entry goes straight into the shared memory of the
+//      CTA that will move it (the list never touches global memory).
 //   6. compaction in rounds: entry o of the list becomes row o of the head.  In a round every CTA
 //      takes a run of consecutive entries out of memory (a stored survivor comes from the head's
-//      own rows, at or behind its destination; a surviving new row from the caller's K/V), most of
-//      them into shared memory, the rest into registers, the cluster meets, and the run goes out
-//      (bulk stores for the shared-memory part).  The destinations of a round lie at or before
-//      its own cache sources and before those of every later round: in place.
+//      own rows, at or behind its destination; a surviving new row from the caller's K/V) into shared
+//      memory, the cluster meets, and the run goes out with bulk stores.  The destinations of a round
+//      lie at or before its own cache sources and before those of every later round: in place.
 //   7. heads that keep the whole new scale stop behind their stored survivors; the attention
 //      launch reads their new rows from the caller's tensors and appends them itself.
 //
+// What bounds it is the chain of dependent round trips once the keys have arrived: a head of two chunks
+// (head_dim 64, one CTA) takes 8.4 us, one of 50 chunks (head_dim 128, four CTAs) 35 us, of which 13 are
+// the key stream.  (With the rows' statistics folded through shared memory, 16 histogram bins per thread
+// and CTA read through distributed shared memory, and an exchange of counts behind the select: 13.2
+// and 44 us; 7 us per digit where that traffic met the attention of the other heads.)  One CTA per
+// head where the GPU is full of heads, two CTAs per SM where there are more heads than SMs: 256 heads of
+// 680 candidates 51 -> 40 us per step, attention included.
 // In score-only mode the kernel stops after step 3 and writes the fp32 scores (hack_score).
 // Every mbarrier wait is bounded; a CTA whose wait gives up raises the status word, and the
 // cluster agrees at the first exchange to skip the rest, so that every CTA still reaches every
@@ -52,11 +60,15 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kCkThreads = 256;
+constexpr int kWorkers = 256;              // warps 0-7: two sets of four, one warp per TMEM lane quadrant
+constexpr int kCkThreads = kWorkers + 32;  // and one issuing warp (a consumer that also issues slowed the key stream by a fifth)
+constexpr int kCkWarps = kCkThreads / 32;
+constexpr int kIssueWarp = kWorkers / 32;
 constexpr int kCkChunk = 128;
-constexpr int kTmemChunks = 16;            // accumulators of 32 columns in 512 columns of tensor memory
-constexpr int kMaxOver = 6;                // chunks per CTA whose logits live in shared memory
-constexpr int kMaxCpc = kTmemChunks - 1 + kMaxOver;      // 21 chunks = 2688 keys per CTA
+constexpr int kHalfObs = kMaxObs / 2;      // observation rows a consumer set takes in pass 1
+constexpr int kMaxSlots = 16;              // accumulators of 32 columns in 512 columns of tensor memory
+constexpr int kMaxOver = 7;                // chunks per CTA whose logits live in shared memory
+constexpr int kMaxCpc = 40;                // chunks per CTA
 constexpr int kMaxCluster = 8;
 constexpr uint32_t kCkDrainSpins = 1u << 22;
 constexpr int kMaxStages = 4;              // key tiles in flight per CTA (deeper rings measured no faster)
@@ -64,15 +76,19 @@ constexpr int kHistBins = 4096;            // bins of a 12-bit digit of the radi
 constexpr int kHistWords = kHistBins / 2;  // 16-bit counters, two per word
 constexpr int kMaxStageRows = 512;         // rows (K and V) in a CTA's staging buffers of the compaction
 constexpr int kMoveBuffers = 3;            // staging buffers of the compaction: loads run two rounds ahead of the stores
-constexpr size_t kSmemBudget = 227 * 1024; // dynamic shared memory a CTA may ask for
-static_assert(kHistBins == 16 * kCkThreads, "a thread sums 16 bins of the cluster's histograms");
+constexpr size_t kSmemBudget = 227 * 1024; // dynamic shared memory a CTA may ask for ...
+constexpr size_t kSmemShared = 112 * 1024; // ... and half an SM's, for two CTAs per SM
+constexpr float kLazyMax = 16.0f;          // log2 units a logit may exceed a thread's reference maximum
+static_assert(kHistBins == 16 * kWorkers, "a worker sums 16 bins of a histogram");
 static_assert(kMaxCpc * kCkChunk < 65536, "16-bit counters per CTA");
 
 struct CkParams {
   int cluster;                // CTAs per head
-  int cpc_max;                // most chunks any CTA of this launch holds (sizes shared / tensor memory)
+  int p_max;                  // most chunks of any CTA whose logits are read twice (sizes shared memory)
+  int cpc_max;                // most chunks of any CTA
+  int slots;                  // accumulators in tensor memory
+  int direct;                 // chunks with an accumulator of their own; the others share the last two
   int n_over;                 // chunks of shared-memory logits reserved per CTA
-  int tmem_cols;              // power of two >= 32
   int stages;                 // key tiles in the TMA ring (2 .. kMaxStages)
   int region_bytes;           // front region of shared memory: ring, observation rows, overflow logits; later the row staging
   int stage_rows;             // rows (K and V) a CTA stages in shared memory per round of the compaction
@@ -85,19 +101,18 @@ struct CkParams {
 struct CkShared {
   uint64_t full[kMaxStages], empty[kMaxStages];
   uint64_t acc_full[kMaxCpc];
-  uint64_t acc_free;
+  uint64_t acc_free[2];
   uint64_t drain;
   uint32_t tmem_base;
   int abort_flag;
-  int pub_abort;                         // read by the other CTAs of the cluster
-  float pub_stats[kMaxObs][2];           // this CTA's (max, sum-exp) per observation row
-  int pub_counts[4];                     // kept above the threshold, equal to it; the same among stored candidates
-  int cnt_all[kMaxCluster][4];           // the counts of every CTA of the cluster
-  float row_m[kMaxObs], row_inv_l[kMaxObs];
-  int warp_sums[kCkThreads / 32 + 1];
-  int digit_of[2][2];                    // the located digit, the rank left inside its bin, the bin's count
-  int sh_abort;
-  int cnt_old[2];
+  int pub_abort;                              // read by the other CTAs of the cluster
+  int digit, need_in_bin, bin_count;          // the located digit, the rank left inside its bin, the bin's count
+  int cnt_gt[kMaxCluster], cnt_eq[kMaxCluster];   // per CTA: keys above the threshold, keys in the located bin
+  int warp_sums[2][kCkWarps + 3];
+  float2 pub_stats[4][kMaxObs];               // per lane quadrant (max, sum-exp) of every observation row; read by the cluster
+  float2 part[4][kMaxObs];                    // the same merged over the CTAs of the cluster
+  float4 row_stat[kMaxObs / 2];               // (max, 1 / sum) of the whole head, two rows a piece
+  uint32_t coarse[2][kWorkers];               // per 16 bins: their count << 16 | the count of all bins above them; read by the cluster
 };
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -105,14 +120,16 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+// Barrier of the cluster; for a cluster of one CTA the block's own (0.1 us instead of 0.7).
+__device__ __forceinline__ void cluster_sync(int cl) {
+  if (cl == 1) __syncthreads();
+  else asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // Execution barrier of the cluster without memory ordering: for a point that only has to come after
 // every CTA's loads have landed (nothing written before it is read by another CTA after it).
-__device__ __forceinline__ void cluster_sync_relaxed() {
+__device__ __forceinline__ void cluster_sync_relaxed(int cl) {
   __syncthreads();
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+  if (cl > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 // Address of the same shared-memory object in the CTA of rank `rank`.
 __device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
@@ -125,15 +142,9 @@ __device__ __forceinline__ int ld_peer_i32(uint32_t addr) {
   asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
   return v;
 }
-__device__ __forceinline__ float ld_peer_f32(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint4 ld_peer_v4(uint32_t addr) {
-  uint4 v;
-  asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+__device__ __forceinline__ float2 ld_peer_f2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
   return v;
 }
 __device__ __forceinline__ void st_peer_i32(uint32_t addr, int v) {
@@ -168,8 +179,6 @@ __device__ __forceinline__ bool ck_wait(uint64_t* bar, uint32_t parity, CkShared
   return false;
 }
 
-__device__ __forceinline__ void ck_consumer_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-
 // Order-preserving map from fp32 bits to unsigned (larger float -> larger key).
 __device__ __forceinline__ uint32_t ck_orderable(float f) {
   const uint32_t u = __float_as_uint(f);
@@ -184,38 +193,43 @@ __device__ __forceinline__ void hist_add(uint32_t* hist, bool in, uint32_t digit
     atomicAdd(&hist[digit >> 1], (uint32_t)__popc(peers) << (16 * (digit & 1)));
 }
 
-// Exclusive prefix sum of one value per thread over the CTA's kCkThreads threads, and the total.
-__device__ __forceinline__ int ck_block_scan(int v, int* warp_sums, int& total) {
-  constexpr int NW = kCkThreads / 32;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// (max, sum-exp) of two disjoint sets of keys; a set without keys is (-inf, 0).
+__device__ __forceinline__ float2 merge_stats(float2 x, float2 y) {
+  const float m = fmaxf(x.x, y.x);
+  const float lx = x.y == 0.f ? 0.f : x.y * ex2(x.x - m), ly = y.y == 0.f ? 0.f : y.y * ex2(y.x - m);
+  return make_float2(m, lx + ly);
+}
+
+// Sum over the CTA's warps of one value per warp: what the warps before this one hold, and the total.
+// `sums` is free again after the next block barrier.
+__device__ __forceinline__ int ck_warp_prefix(int v, int* sums, int& total) {
+  const int warp = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) sums[warp] = v;
+  __syncthreads();
+  int before = 0;
+  total = 0;
+#pragma unroll
+  for (int w = 0; w < kCkWarps; ++w) {
+    const int x = sums[w];
+    if (w < warp) before += x;
+    total += x;
+  }
+  return before;
+}
+// Exclusive prefix sum of one value per thread over the CTA, and the total.
+__device__ __forceinline__ int ck_block_scan(int v, int* sums, int& total) {
+  const int lane = threadIdx.x & 31;
   int incl = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int n = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += n;
   }
-  if (lane == 31) warp_sums[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    const int w = lane < NW ? warp_sums[lane] : 0;
-    int wi = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int n = __shfl_up_sync(0xffffffffu, wi, o);
-      if (lane >= o) wi += n;
-    }
-    if (lane < NW) warp_sums[lane] = wi - w;
-    if (lane == 31) warp_sums[NW] = wi;
-  }
-  __syncthreads();
-  const int res = warp_sums[warp] + incl - v;
-  total = warp_sums[NW];
-  __syncthreads();
-  return res;
+  return ck_warp_prefix(__shfl_sync(0xffffffffu, incl, 31), sums, total) + incl - v;
 }
 
 template <int D>
-__global__ void __launch_bounds__(kCkThreads, 1)
+__global__ void __launch_bounds__(kCkThreads, 2)
 compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __grid_constant__ CUtensorMap tm_new,
                         const StepArgs a, const __nv_bfloat16* __restrict__ q, const CkParams p) {
   constexpr int SUB = D / 64;
@@ -223,27 +237,32 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   constexpr uint32_t Q_SUB_BYTES = kMaxObs * 128;
   constexpr uint32_t K_BYTES = SUB * K_SUB_BYTES;
   constexpr int PIECES = D * 2 / 16;                      // 16-byte pieces per row
-  static_assert(2 * K_BYTES >= 2 * kMaxObs * kCkChunk * sizeof(float), "two ring stages hold the fold");
+  static_assert(2 * K_BYTES >= 2 * kHistWords * sizeof(uint32_t), "two ring stages hold the histograms");
   const int STAGES = p.stages;
   const uint32_t RING_BYTES = (uint32_t)STAGES * K_BYTES;
 
-  // Nothing that another kernel writes is touched before pdl_wait() below: the head-type table is
-  // written when the cache is created, the step's lengths travel in the arguments.
+  // Nothing that another kernel writes is touched before the dependency wait below: the head-type
+  // table is written when the cache is created, the step's lengths travel in the arguments.
   const int bh = blockIdx.y;
   const int ctx = a.is_ctx[bh % a.n_heads];
   if (!a.trig[ctx]) {                                     // the whole cluster leaves together
     pdl_wait();
     return;
   }
-  const int rank = (int)cluster_rank();
   const int CL = p.cluster;
-  const int stored = a.stored[ctx], n_new = a.n_new, n_keep = a.kept[ctx];
-  const int n_sc = (stored + kCkChunk - 1) / kCkChunk;
-  const int n_chunks = n_sc + (n_new + kCkChunk - 1) / kCkChunk;
-  const int cpc = (n_chunks + CL - 1) / CL;               // <= p.cpc_max
-  const int c_begin = rank * cpc;
-  const int n_run = max(0, min(cpc, n_chunks - c_begin));
-  const int n_persist = p.cpc_max <= kTmemChunks ? kTmemChunks : kTmemChunks - 1;   // chunks with an accumulator of their own
+  const int rank = CL > 1 ? (int)cluster_rank() : 0;
+  const int stored = a.stored[ctx], n_new = a.n_new;
+  // A structural head that keeps the whole new scale ranks its stored candidates only: the new keys
+  // enter the softmax denominators and are then done with.
+  const bool drop_new = ctx == 0 && a.protect_new && !p.scores;
+  const int n_rows = drop_new ? a.kept[ctx] - n_new : a.kept[ctx];   // survivors this kernel lists and moves
+  const int n_sc = (stored + kCkChunk - 1) / kCkChunk, n_nc = (n_new + kCkChunk - 1) / kCkChunk;
+  // This CTA's chunks: first a consecutive run of ranked candidates, then (drop_new) of the others.
+  const int n_ranked = drop_new ? n_sc : n_sc + n_nc;
+  const int cpr = (n_ranked + CL - 1) / CL, cpt = drop_new ? (n_nc + CL - 1) / CL : 0;
+  const int c_begin = rank * cpr, t_begin = rank * cpt;
+  const int n_p = max(0, min(cpr, n_ranked - c_begin));
+  const int n_run = n_p + (drop_new ? max(0, min(cpt, n_nc - t_begin)) : 0);      // <= p.cpc_max
   const float zscale = a.sm_scale * 1.4426950408889634f;  // logits in log2 units
   const long long wlim = a.wait_cycles;
 
@@ -255,88 +274,118 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   const uint32_t q_sm = base + RING_BYTES;
   float* over = reinterpret_cast<float*>(sm + RING_BYTES + SUB * Q_SUB_BYTES);            // [n_over][32][128]
   const int S_ROWS = p.stage_rows;                          // rows a CTA holds in its staging buffers
-  uint32_t* keys = reinterpret_cast<uint32_t*>(sm + p.region_bytes);                            // [cpc_max * 128]
-  int32_t* pos_stage = reinterpret_cast<int32_t*>(keys + (size_t)p.cpc_max * kCkChunk);        // [S_ROWS]
-  int32_t* src_all = pos_stage + S_ROWS;                    // [cpc_max * 128 + S_ROWS]: this CTA's list entries of every round
-  CkShared* sh = reinterpret_cast<CkShared*>(src_all + (size_t)p.cpc_max * kCkChunk + S_ROWS);
-  float* fold_m = reinterpret_cast<float*>(sm);           // [32][128], reuses the ring
-  float* fold_l = fold_m + kMaxObs * kCkChunk;
-  uint32_t* hist32 = reinterpret_cast<uint32_t*>(sm);     // [2][kHistWords], reuses the ring after the fold
+  uint32_t* keys = reinterpret_cast<uint32_t*>(sm + p.region_bytes);                            // [p_max * 128]
+  int32_t* pos_stage = reinterpret_cast<int32_t*>(keys + (size_t)p.p_max * kCkChunk);          // [S_ROWS]
+  int32_t* src_all = pos_stage + S_ROWS;                    // [p_max * 128 + S_ROWS]: this CTA's list entries of every round
+  CkShared* sh = reinterpret_cast<CkShared*>(src_all + (size_t)p.p_max * kCkChunk + S_ROWS);
+  uint32_t* hist32 = reinterpret_cast<uint32_t*>(sm);     // [2][kHistWords], reuses the ring once it is idle
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+  // chunk behind local index i: does it come from the cache, and its index in its part of the list
+  auto chunk_part = [&](int i, bool& from_cache) -> int {
+    const int chunk = i < n_p ? c_begin + i : n_sc + t_begin + (i - n_p);
+    from_cache = chunk < n_sc;
+    return from_cache ? chunk : chunk - n_sc;
+  };
   // candidate behind slot (local chunk i, key r): is it a live entry, and its candidate index
   auto slot_info = [&](int slot, int& j) -> bool {
-    const int i = slot >> 7, r = slot & 127;
-    if (i >= n_run) return false;
-    const int chunk = c_begin + i;
-    const bool from_cache = chunk < n_sc;
-    const int part_row = (from_cache ? chunk : chunk - n_sc) * kCkChunk + r;
+    bool from_cache;
+    const int part_row = chunk_part(slot >> 7, from_cache) * kCkChunk + (slot & 127);
     j = (from_cache ? 0 : stored) + part_row;
     return part_row < (from_cache ? stored : n_new);
   };
 
-  if (tid == 0) {
+  int issued = 0;                                           // issuing thread: key tiles on their way
+  auto load_tile = [&](int i) {
+    bool from_cache;
+    const int part = chunk_part(i, from_cache);
+    const CUtensorMap* tm = from_cache ? &tm_cache : &tm_new;
+    const int row = (from_cache ? a.row_off[bh] : bh * n_new) + part * kCkChunk;
+    const int s = i % STAGES;
+    const uint32_t bar = smem_u32(&sh->full[s]);
+    mbar_expect_tx(bar, K_BYTES);
+#pragma unroll
+    for (int c = 0; c < SUB; ++c) tma_load_2d(k_sm + s * K_BYTES + c * K_SUB_BYTES, tm, c * 64, row, bar);
+    ++issued;
+  };
+  if (warp == kIssueWarp && lane == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(smem_u32(&sh->full[s]), 1); mbar_init(smem_u32(&sh->empty[s]), 1); }
-    for (int i = 0; i < kMaxCpc; ++i) mbar_init(smem_u32(&sh->acc_full[i]), 1);
-    mbar_init(smem_u32(&sh->acc_free), kCkChunk);
+    for (int i = 0; i < n_run; ++i) mbar_init(smem_u32(&sh->acc_full[i]), 1);
+    mbar_init(smem_u32(&sh->acc_free[0]), kWorkers);
+    mbar_init(smem_u32(&sh->acc_free[1]), kWorkers);
     mbar_init(smem_u32(&sh->drain), 1);
     sh->abort_flag = 0;
-    sh->cnt_old[0] = 0;
-    sh->cnt_old[1] = 0;
     fence_barrier_init();
     fence_proxy_async();
-  }
-  if (warp == 1) {
-    tmem_alloc(smem_u32(&sh->tmem_base), p.tmem_cols);
-    tmem_relinquish();
-  }
-  if (warp == 0 && lane == 0) {
     prefetch_tensormap(&tm_cache);
     prefetch_tensormap(&tm_new);
   }
-  pdl_wait();     // everything above overlaps the tail of the previous kernel
-  // observation rows into the swizzled B tile; unused rows are zero
-  for (int v = tid; v < kMaxObs * (D / 8); v += kCkThreads) {
-    const int i = v / (D / 8), c = v % (D / 8);
-    uint4 val = make_uint4(0, 0, 0, 0);
-    if (i < a.n_obs_rows) {
-      const int row = obs_row(a, i);
-      val = *reinterpret_cast<const uint4*>(q + ((size_t)bh * n_new + row) * D + c * 8);
-    }
-    const uint32_t off = (c / 8) * Q_SUB_BYTES + i * 128 + (((c % 8) ^ (i & 7)) << 4);
-    *reinterpret_cast<uint4*>(sm + RING_BYTES + off) = val;
+  if (warp == 0) {
+    tmem_alloc(smem_u32(&sh->tmem_base), kMaxObs * p.slots);
+    tmem_relinquish();
   }
-  fence_proxy_async();
+  pdl_grid_wait();     // everything above overlaps the tail of the previous kernel
+  // the next launch may start once every CTA holds its tensor memory
+  if (warp == 0) pdl_launch_dependents();
+  if (warp == kIssueWarp) {
+    // the first key tiles are on their way while the other warps fetch the observation rows
+    if (lane == 0)
+      for (int i = 0; i < min(STAGES, n_run); ++i) load_tile(i);
+    __syncwarp();
+  } else {
+    // observation rows into the swizzled B tile; unused rows are zero
+    for (int v = tid; v < kMaxObs * (D / 8); v += kWorkers) {
+      const int i = v / (D / 8), c = v % (D / 8);
+      uint4 val = make_uint4(0, 0, 0, 0);
+      if (i < a.n_obs_rows)
+        val = *reinterpret_cast<const uint4*>(q + ((size_t)bh * n_new + obs_row(a, i)) * D + c * 8);
+      const uint32_t off = (c / 8) * Q_SUB_BYTES + i * 128 + (((c % 8) ^ (i & 7)) << 4);
+      *reinterpret_cast<uint4*>(sm + RING_BYTES + off) = val;
+    }
+    fence_proxy_async();
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&sh->tmem_base);
 
   // ------------------------------------------------------------------ 1. scores, pass 1
-  const int quad = warp & 3;                                // TMEM lane quadrant a consumer warp may read
-  const int key_row = quad * 32 + lane;
-  const uint32_t t_lane = tmem + (static_cast<uint32_t>(quad * 32) << 16);
-  if (warp == 0) {
+  const int set = warp >> 2;
+  const int key_row = (warp & 3) * 32 + lane;
+  const uint32_t t_lane = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+  // Chunks past the `direct` ones take turns on the last two accumulators.
+  auto acc_slot = [&](int i) { return i < p.direct ? i : p.slots - 2 + ((i - p.direct) & 1); };
+  if (warp == kIssueWarp) {
     if (lane == 0) {
-      int issued = 0;
+      constexpr uint32_t IDESC = idesc_bf16_f32(kCkChunk, kMaxObs, 0);
+      const uint64_t q_desc = smem_desc_sw128(q_sm, 16, 1024);
       bool ok = true;
-      for (int i = 0; i < n_run; ++i) {
+      for (int i = 0; i < n_run && ok; ++i) {
         const int s = i % STAGES;
-        ok = ck_wait(&sh->empty[s], ((i / STAGES) & 1) ^ 1, sh, a.status, 51, wlim);
+        ok = ck_wait(&sh->full[s], (i / STAGES) & 1, sh, a.status, 52, wlim);
+        // a shared accumulator is free again once all consumers have read the chunk before
+        if (ok && i >= p.direct)
+          ok = ck_wait(&sh->acc_free[(i - p.direct) & 1], (((i - p.direct) >> 1) & 1) ^ 1, sh, a.status, 53, wlim);
         if (!ok) break;
-        const int chunk = c_begin + i;
-        const bool from_cache = chunk < n_sc;
-        const CUtensorMap* tm = from_cache ? &tm_cache : &tm_new;
-        const int row = from_cache ? a.row_off[bh] + chunk * kCkChunk : bh * n_new + (chunk - n_sc) * kCkChunk;
-        const uint32_t bar = smem_u32(&sh->full[s]);
-        mbar_expect_tx(bar, K_BYTES);
-#pragma unroll
-        for (int c = 0; c < SUB; ++c) tma_load_2d(k_sm + s * K_BYTES + c * K_SUB_BYTES, tm, c * 64, row, bar);
-        ++issued;
+        tc_fence_after();
+        const uint64_t k_desc = smem_desc_sw128(k_sm + s * K_BYTES, 16, 1024);
+        const uint32_t acc = tmem + acc_slot(i) * kMaxObs;
+        if constexpr (D == 128) mma_ss_chain8_b32rows(acc, k_desc, q_desc, IDESC, 0);
+        else mma_ss_chain4(acc, k_desc, q_desc, IDESC, 0);
+        mma_commit(smem_u32(&sh->empty[s]));
+        mma_commit(smem_u32(&sh->acc_full[i]));
+        // the tile of the product before this one is free: refill its stage
+        const int f = i - 1 + STAGES;
+        if (i > 0 && f < n_run) {
+          ok = ck_wait(&sh->empty[f % STAGES], (f / STAGES - 1) & 1, sh, a.status, 51, wlim);
+          if (ok) load_tile(f);
+        }
       }
       if (!ok) {
-        // give the copies already in flight a bounded chance to land before the ring is reused
+        // what is in flight gets a bounded chance to finish before the ring is reused
+        mma_commit(smem_u32(&sh->drain));
+        for (uint32_t it = 0; it < kCkDrainSpins && !mbar_try_wait(smem_u32(&sh->drain), 0); ++it) {}
         for (int i = max(0, issued - STAGES); i < issued; ++i) {
           const uint32_t bar = smem_u32(&sh->full[i % STAGES]);
           for (uint32_t it = 0; it < kCkDrainSpins && !mbar_try_wait(bar, (i / STAGES) & 1); ++it) {}
@@ -344,162 +393,138 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
       }
     }
     __syncwarp();
-  } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t IDESC = idesc_bf16_f32(kCkChunk, kMaxObs, 0);
-      const uint64_t q_desc = smem_desc_sw128(q_sm, 16, 1024);
-      bool ok = true;
-      for (int i = 0; i < n_run && ok; ++i) {
-        const int s = i % STAGES;
-        const int slot = i < n_persist ? i : kTmemChunks - 1;
-        ok = ck_wait(&sh->full[s], (i / STAGES) & 1, sh, a.status, 52, wlim);
-        // the bounce accumulator is free again once all 128 consumers have read its previous chunk
-        if (ok && i >= n_persist) ok = ck_wait(&sh->acc_free, ((i - n_persist) & 1) ^ 1, sh, a.status, 53, wlim);
-        if (!ok) break;
-        tc_fence_after();
-        const uint64_t k_desc = smem_desc_sw128(k_sm + s * K_BYTES, 16, 1024);
-        if constexpr (D == 128) mma_ss_chain8_b32rows(tmem + slot * kMaxObs, k_desc, q_desc, IDESC, 0);
-        else mma_ss_chain4(tmem + slot * kMaxObs, k_desc, q_desc, IDESC, 0);
-        mma_commit(smem_u32(&sh->empty[s]));
-        mma_commit(smem_u32(&sh->acc_full[i]));
-      }
-      if (!ok) {
-        mma_commit(smem_u32(&sh->drain));
-        for (uint32_t it = 0; it < kCkDrainSpins && !mbar_try_wait(smem_u32(&sh->drain), 0); ++it) {}
-      }
-    }
-    __syncwarp();
-  } else if (warp < 6) {
-    const int w = warp - 2;
-    const int ct = tid - 64;                                  // 0..127
-    float rm[kMaxObs], rl[kMaxObs];
+  } else {
+    // Thread r of a set owns key r of every chunk and keeps (reference maximum, sum-exp) of the set's 16
+    // rows (all 32 in one thread would not leave registers for two CTAs per SM).  The reference starts
+    // at the thread's first logit and is raised only when a logit exceeds it by 2^kLazyMax, so that an
+    // entry usually costs one exponential.
+    float rm[kHalfObs], rl[kHalfObs];
 #pragma unroll
-    for (int i = 0; i < kMaxObs; ++i) { rm[i] = -INFINITY; rl[i] = 0.f; }
-    bool ok = true;
+    for (int i = 0; i < kHalfObs; ++i) { rm[i] = -INFINITY; rl[i] = 0.f; }
+    bool ok = true, first = true;
     for (int i = 0; i < n_run; ++i) {
       ok = __all_sync(0xffffffffu, ck_wait(&sh->acc_full[i], 0, sh, a.status, 54, wlim));
       if (!ok) break;
       tc_fence_after();
-      uint32_t acc[kMaxObs];
-      tmem_ld32(t_lane + (i < n_persist ? i : kTmemChunks - 1) * kMaxObs, acc);
+      uint32_t acc[kHalfObs];
+      tmem_ld16(t_lane + acc_slot(i) * kMaxObs + set * kHalfObs, acc);
       tmem_wait_ld();
-      if (i >= n_persist) {
-        float* dst = over + (size_t)(i - n_persist) * kMaxObs * kCkChunk + key_row;
-#pragma unroll
-        for (int r = 0; r < kMaxObs; ++r) dst[r * kCkChunk] = __uint_as_float(acc[r]);
+      if (i >= p.direct) {
         tc_fence_before();
-        mbar_arrive(smem_u32(&sh->acc_free));
+        mbar_arrive(smem_u32(&sh->acc_free[(i - p.direct) & 1]));
+        if (i < n_p) {
+          float* dst = over + ((size_t)(i - p.direct) * kMaxObs + set * kHalfObs) * kCkChunk + key_row;
+#pragma unroll
+          for (int r = 0; r < kHalfObs; ++r) dst[r * kCkChunk] = __uint_as_float(acc[r]);
+        }
       }
       int j;
       if (slot_info(i * kCkChunk + key_row, j)) {
+        if (first) {
+          first = false;
 #pragma unroll
-        for (int r = 0; r < kMaxObs; ++r) {
-          const float z = __uint_as_float(acc[r]) * zscale;
-          const float mn = fmaxf(rm[r], z);
-          rl[r] = rl[r] * ex2(rm[r] - mn) + ex2(z - mn);
-          rm[r] = mn;
+          for (int r = 0; r < kHalfObs; ++r) { rm[r] = __uint_as_float(acc[r]) * zscale; rl[r] = 1.f; }
+        } else {
+          float d[kHalfObs], top = -INFINITY;
+#pragma unroll
+          for (int r = 0; r < kHalfObs; ++r) {
+            d[r] = fmaf(__uint_as_float(acc[r]), zscale, -rm[r]);
+            top = fmaxf(top, d[r]);
+          }
+          if (top > kLazyMax) {
+#pragma unroll
+            for (int r = 0; r < kHalfObs; ++r) {
+              const float z = __uint_as_float(acc[r]) * zscale;
+              const float mn = fmaxf(rm[r], z);
+              rl[r] = rl[r] * ex2(rm[r] - mn) + ex2(z - mn);
+              rm[r] = mn;
+            }
+          } else {
+#pragma unroll
+            for (int r = 0; r < kHalfObs; ++r) rl[r] += ex2(d[r]);
+          }
         }
       }
     }
-    // the consumers meet on their named barrier below, so they agree first on whether all of them got through
-    uint32_t all_ok;
-    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.and.pred p, 1, 128, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(all_ok) : "r"((uint32_t)ok) : "memory");
-    if (all_ok) {
-      // every accumulator has been read, so every MMA and every key load is complete: the ring is free
+    if (ok) {
+      // merge over the warp's 32 keys: in every step a lane hands half of its rows to its partner, so
+      // that lanes r and r + 16 end up with row r of the set; then those two are merged
 #pragma unroll
-      for (int r = 0; r < kMaxObs; ++r) { fold_m[r * kCkChunk + ct] = rm[r]; fold_l[r * kCkChunk + ct] = rl[r]; }
-      ck_consumer_sync();
-      for (int r = w; r < kMaxObs; r += 4) {
-        float m4[4], l4[4];
-        float m = -INFINITY;
+      for (int o = kHalfObs / 2; o > 0; o >>= 1) {
+        const bool hi = lane & o;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          m4[u] = fold_m[r * kCkChunk + u * 32 + lane];
-          l4[u] = fold_l[r * kCkChunk + u * 32 + lane];
-          m = fmaxf(m, m4[u]);
+        for (int r = 0; r < o; ++r) {
+          const float2 keep = hi ? make_float2(rm[r + o], rl[r + o]) : make_float2(rm[r], rl[r]);
+          const float2 give = hi ? make_float2(rm[r], rl[r]) : make_float2(rm[r + o], rl[r + o]);
+          const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, give.x, o), __shfl_xor_sync(0xffffffffu, give.y, o));
+          const float2 m = merge_stats(keep, got);
+          rm[r] = m.x;
+          rl[r] = m.y;
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        float l = 0.f;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) l += l4[u] == 0.f ? 0.f : l4[u] * ex2(m4[u] - m);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-        if (lane == 0) { sh->pub_stats[r][0] = m; sh->pub_stats[r][1] = l; }
       }
+      const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, rm[0], 16), __shfl_xor_sync(0xffffffffu, rl[0], 16));
+      if (lane < kHalfObs) sh->pub_stats[warp & 3][set * kHalfObs + lane] = merge_stats(make_float2(rm[0], rl[0]), got);
     }
   }
   __syncthreads();
   if (tid == 0) sh->pub_abort = *reinterpret_cast<volatile int*>(&sh->abort_flag);
   // the ring is idle from here on; its first 16 KB become the two histograms of the radix select
-  {
+  if (tid < kWorkers) {
     uint4* z = reinterpret_cast<uint4*>(hist32 + 8 * tid);
     z[0] = z[1] = make_uint4(0, 0, 0, 0);
     z[kHistWords / 4] = z[kHistWords / 4 + 1] = make_uint4(0, 0, 0, 0);
   }
 
   // ------------------------------------------------------------------ 2. row statistics of the whole head
-  cluster_sync();
-  if (tid < kMaxObs) {
-    float mr[kMaxCluster], lr[kMaxCluster];
+  cluster_sync(CL);
+  if (tid < 4 * kMaxObs) {
+    float2 got[kMaxCluster];
 #pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r) {                 // all loads in flight at once
-      mr[r] = lr[r] = 0.f;
-      if (r < CL) {
-        mr[r] = ld_peer_f32(peer_addr(&sh->pub_stats[tid][0], r));
-        lr[r] = ld_peer_f32(peer_addr(&sh->pub_stats[tid][1], r));
-      }
-    }
-    float m = -INFINITY;
+    for (int r = 0; r < kMaxCluster; ++r)                   // all loads in flight at once
+      if (r < CL) got[r] = ld_peer_f2(peer_addr(&sh->pub_stats[warp][lane], r));
+    float2 st = got[0];
 #pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r)
-      if (r < CL) m = fmaxf(m, mr[r]);
-    float l = 0.f;
-#pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r)
-      if (r < CL) l += lr[r] == 0.f ? 0.f : lr[r] * ex2(mr[r] - m);
-    // rows past n_obs_rows are padding: weight 0, finite reference
-    sh->row_m[tid] = tid < a.n_obs_rows ? m : 0.f;
-    sh->row_inv_l[tid] = tid < a.n_obs_rows ? 1.f / l : 0.f;
+    for (int r = 1; r < kMaxCluster; ++r)
+      if (r < CL) st = merge_stats(st, got[r]);
+    sh->part[warp][lane] = st;
   }
-  if (tid == 32) {
-    int any = 0;
-    for (int r = 0; r < CL; ++r) any |= ld_peer_i32(peer_addr(&sh->pub_abort, r));
-    sh->sh_abort = any;
+  bool any_abort = false;
+  if (lane < CL) any_abort = ld_peer_i32(peer_addr(&sh->pub_abort, lane)) != 0;
+  const bool aborted = __any_sync(0xffffffffu, any_abort);  // the same in every CTA of the cluster
+  __syncthreads();
+  if (warp == 0) {
+    float2 st = sh->part[0][lane];
+#pragma unroll
+    for (int w = 1; w < 4; ++w) st = merge_stats(st, sh->part[w][lane]);
+    // rows past n_obs_rows are padding: weight 0, finite reference
+    reinterpret_cast<float2*>(sh->row_stat)[lane] = lane < a.n_obs_rows ? make_float2(st.x, 1.f / st.y) : make_float2(0.f, 0.f);
   }
   __syncthreads();
-  const bool aborted = sh->sh_abort != 0;                   // the same value in every CTA of the cluster
+  const bool select = !aborted && !p.score_only && n_rows > 0;
 
   // ------------------------------------------------------------------ 3. scores, pass 2
-  if (!aborted) {
-    // all eight warps: warps 2-5 take the even chunks, warps 6, 7, 0, 1 (the same four lane quadrants)
-    // the odd ones; a key's 32 terms are added in the same order by either set
-    float rm[kMaxObs], rl[kMaxObs];
-#pragma unroll
-    for (int i = 0; i < kMaxObs; ++i) { rm[i] = sh->row_m[i]; rl[i] = sh->row_inv_l[i]; }
+  if (!aborted && tid < kWorkers) {
     const bool structural = ctx == 0;
-    for (int i = (warp >= 2 && warp < 6) ? 0 : 1; i < n_run; i += 2) {
-      // a chunk of protected candidates only (the new scale of a structural head) is kept whatever
-      // its scores are; they are formed only when the caller wants them
-      if (!p.scores && structural && a.protect_new && c_begin + i >= n_sc) {
-        int j;
-        keys[i * kCkChunk + key_row] = 0xffffffffu;
-        hist_add(hist32, slot_info(i * kCkChunk + key_row, j), kHistBins - 1);
-        continue;
-      }
-      uint32_t acc[kMaxObs];
-      if (i < n_persist) {
-        tmem_ld32(t_lane + i * kMaxObs, acc);
-        tmem_wait_ld();
-      } else {
-        const float* src = over + (size_t)(i - n_persist) * kMaxObs * kCkChunk + key_row;
-#pragma unroll
-        for (int r = 0; r < kMaxObs; ++r) acc[r] = __float_as_uint(src[r * kCkChunk]);
-      }
+    for (int i = set; i < n_p; i += 2) {                    // a set takes every other chunk here
       float s = 0.f;
 #pragma unroll
-      for (int r = 0; r < kMaxObs; ++r) s = fmaf(ex2(fmaf(__uint_as_float(acc[r]), zscale, -rm[r])), rl[r], s);
+      for (int h = 0; h < 2; ++h) {
+        uint32_t acc[kHalfObs];
+        if (i < p.direct) {
+          tmem_ld16(t_lane + i * kMaxObs + h * kHalfObs, acc);
+          tmem_wait_ld();
+        } else {
+          const float* src = over + ((size_t)(i - p.direct) * kMaxObs + h * kHalfObs) * kCkChunk + key_row;
+#pragma unroll
+          for (int r = 0; r < kHalfObs; ++r) acc[r] = __float_as_uint(src[r * kCkChunk]);
+        }
+#pragma unroll
+        for (int r = 0; r < kHalfObs; r += 2) {
+          const float4 st = sh->row_stat[(h * kHalfObs + r) / 2];
+          s = fmaf(ex2(fmaf(__uint_as_float(acc[r]), zscale, -st.x)), st.y, s);
+          s = fmaf(ex2(fmaf(__uint_as_float(acc[r + 1]), zscale, -st.z)), st.w, s);
+        }
+      }
       int j = 0;
       const bool live = slot_info(i * kCkChunk + key_row, j);
       uint32_t key = 0;
@@ -519,155 +544,178 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   tc_fence_before();
   __syncthreads();
 
-  if (!aborted && !p.score_only) {
+  if (select) {
     // ---------------------------------------------------------------- 4. radix select over the cluster
     // Digits of 12, 12 and 8 bits.  The local histogram of the first digit was filled while the keys
     // were formed; the select stops as soon as every entry left in the located bin survives, which
-    // with 24 bits fixed is the usual case.
-    const int n_slots = cpc * kCkChunk;
+    // with 24 bits fixed is the usual case.  Before the cluster meets, every CTA adds its bins in groups
+    // of 16 and forms the counts above each group; afterwards worker t adds the CL words of group t, the
+    // one warp whose groups hold the wanted rank reads that group's bins, and it learns on the
+    // way how many keys each CTA holds above the located bin and in it.
+    const int n_slots = n_p * kCkChunk;
     uint32_t prefix = 0, mask = 0;
-    int need = n_keep;
+    int need = n_rows;
+    if (tid < CL) sh->cnt_gt[tid] = 0;
 #pragma unroll 1
     for (int pass = 0; pass < 3; ++pass) {
       const int shift = pass == 0 ? 20 : (pass == 1 ? 8 : 0);
       const uint32_t dmask = pass == 2 ? 255u : 4095u;
       uint32_t* hist = hist32 + (pass & 1) * kHistWords;
       if (pass > 0) {
-        for (int s0 = 0; s0 < n_slots; s0 += kCkThreads) {
-          const int slot = s0 + tid;
+        for (int slot = tid; slot < n_slots; slot += kCkThreads) {
           int j;
-          const bool live = slot < n_slots && slot_info(slot, j);
-          const uint32_t k = live ? keys[slot] : 0u;
-          const bool in = live && ((k & mask) == prefix);
-          hist_add(hist, in, (k >> shift) & dmask);
+          const uint32_t k = keys[slot];
+          // few entries are left and they differ: plain additions
+          if ((k & mask) == prefix && slot_info(slot, j)) {
+            const uint32_t digit = (k >> shift) & dmask;
+            atomicAdd(&hist[digit >> 1], 1u << (16 * (digit & 1)));
+          }
         }
-      }
-      cluster_sync();                                         // (orders the CTA's own threads as well)
-      // thread t owns bins [16 t, 16 t + 16): two 16-bit counters per word
-      int c[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) c[i] = 0;
-      {
-        uint4 part[kMaxCluster][2];
-#pragma unroll
-        for (int r = 0; r < kMaxCluster; ++r)                 // all loads in flight at once
-          if (r < CL && (pass < 2 || tid < 16)) {               // the 8-bit digit fills 256 bins only
-            const uint32_t addr = peer_addr(hist + 8 * tid, r);
-            part[r][0] = ld_peer_v4(addr);
-            part[r][1] = ld_peer_v4(addr + 16);
-          } else {
-            part[r][0] = part[r][1] = make_uint4(0, 0, 0, 0);
-          }
-#pragma unroll
-        for (int r = 0; r < kMaxCluster; ++r)
-          if (r < CL) {
-            const uint32_t w[8] = {part[r][0].x, part[r][0].y, part[r][0].z, part[r][0].w,
-                                   part[r][1].x, part[r][1].y, part[r][1].z, part[r][1].w};
-#pragma unroll
-            for (int i = 0; i < 8; ++i) { c[2 * i] += (int)(w[i] & 0xffffu); c[2 * i + 1] += (int)(w[i] >> 16); }
-          }
-      }
-      // the other buffer is free: every CTA read it before it arrived at the barrier above
-      {
-        uint4* z = reinterpret_cast<uint4*>(hist32 + ((pass & 1) ^ 1) * kHistWords + 8 * tid);
-        z[0] = make_uint4(0, 0, 0, 0);
-        z[1] = make_uint4(0, 0, 0, 0);
+        __syncthreads();
       }
       int mine = 0;
-#pragma unroll
-      for (int i = 0; i < 16; ++i) mine += c[i];
+      if (tid < kWorkers) {
+        const uint4 h0 = *reinterpret_cast<const uint4*>(hist + 8 * tid), h1 = *reinterpret_cast<const uint4*>(hist + 8 * tid + 4);
+        const uint32_t w = (h0.x + h0.y + h0.z + h0.w) + (h1.x + h1.y + h1.z + h1.w);   // two 16-bit sums: a CTA holds fewer than 65 536 keys
+        mine = (int)((w & 0xffffu) + (w >> 16));
+      }
       int total;
-      const int below = ck_block_scan(mine, sh->warp_sums, total);
-      const int above = total - below - mine;                 // entries in the bins of the threads behind this one
-      if (above < need && need <= above + mine) {
-        int cum = above;
+      const int below = ck_block_scan(mine, sh->warp_sums[pass & 1], total);
+      if (tid < kWorkers) sh->coarse[pass & 1][tid] = (uint32_t)mine << 16 | (uint32_t)(total - below - mine);
+      cluster_sync(CL);                                       // (orders the CTA's own threads as well)
+      if (tid < kWorkers) {
+        uint32_t g[kMaxCluster];
 #pragma unroll
-        for (int i = 15; i >= 0; --i) {
-          if (cum < need && need <= cum + c[i]) {
-            sh->digit_of[0][0] = 16 * tid + i;
-            sh->digit_of[0][1] = need - cum;
-            sh->digit_of[1][0] = c[i];
+        for (int r = 0; r < kMaxCluster; ++r) {               // all loads in flight at once
+          g[r] = 0;
+          if (r < CL) g[r] = (uint32_t)ld_peer_i32(peer_addr(&sh->coarse[pass & 1][tid], r));
+        }
+        int above = 0, group = 0;
+#pragma unroll
+        for (int r = 0; r < kMaxCluster; ++r) { above += (int)(g[r] & 0xffffu); group += (int)(g[r] >> 16); }
+        // exactly one group holds the wanted rank; its warp reads the group's bins, lane (r, u) word u of CTA r
+        const uint32_t winner = __ballot_sync(0xffffffffu, above < need && need <= above + group);
+        if (winner) {
+          const int src = __ffs(winner) - 1;
+          const int grp = (tid & ~31) + src;
+          above = __shfl_sync(0xffffffffu, above, src);
+          uint32_t lo[2] = {0, 0};                            // word lane & 7 of the CTAs lane >> 3 and 4 + (lane >> 3)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if ((lane >> 3) + 4 * h < CL)
+              lo[h] = (uint32_t)ld_peer_i32(peer_addr(hist + 8 * grp + (lane & 7), (lane >> 3) + 4 * h));
+          // bins 2 u and 2 u + 1 over the CTAs, each in a word of its own
+          int c0 = (int)(lo[0] & 0xffffu) + (int)(lo[1] & 0xffffu), c1 = (int)(lo[0] >> 16) + (int)(lo[1] >> 16);
+#pragma unroll
+          for (int o = 8; o <= 16; o <<= 1) {
+            c0 += __shfl_xor_sync(0xffffffffu, c0, o);
+            c1 += __shfl_xor_sync(0xffffffffu, c1, o);
           }
-          cum += c[i];
+          // entries in the words above this lane's (u = lane & 7), by a suffix sum over 8 lanes
+          int suf = c0 + c1;
+#pragma unroll
+          for (int o = 1; o < 8; o <<= 1) {
+            const int n = __shfl_down_sync(0xffffffffu, suf, o, 8);
+            if ((lane & 7) + o < 8) suf += n;
+          }
+          const int over1 = above + suf - c0 - c1, over0 = over1 + c1;
+          const bool hit1 = over1 < need && need <= over1 + c1, hit0 = over0 < need && need <= over0 + c0;
+          const int u = (__ffs(__ballot_sync(0xffffffffu, hit0 || hit1)) - 1) & 7;
+          const bool odd = __shfl_sync(0xffffffffu, (int)hit1, u);
+          if (lane == u) {
+            sh->digit = 16 * grp + 2 * u + (odd ? 1 : 0);
+            sh->need_in_bin = need - (odd ? over1 : over0);
+            sh->bin_count = odd ? c1 : c0;
+          }
+          // per CTA: entries of this group above the located bin, and in it
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int w = lane & 7, b0 = (int)(lo[h] & 0xffffu), b1 = (int)(lo[h] >> 16);
+            int gt = w > u ? b0 + b1 : (w == u && !odd) ? b1 : 0;
+            int eq = w == u ? (odd ? b1 : b0) : 0;
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+              gt += __shfl_xor_sync(0xffffffffu, gt, o);
+              eq += __shfl_xor_sync(0xffffffffu, eq, o);
+            }
+            const int r = (lane >> 3) + 4 * h;
+            if (w == 0 && r < CL) {
+              sh->cnt_gt[r] += gt;
+              sh->cnt_eq[r] = eq;
+            }
+          }
+          __syncwarp();
+          if (lane == src) {
+#pragma unroll
+            for (int r = 0; r < kMaxCluster; ++r)
+              if (r < CL) sh->cnt_gt[r] += (int)(g[r] & 0xffffu);
+          }
         }
       }
+      // the first histogram is free: every CTA read it before it arrived at the barrier above
+      if (pass == 1 && tid < kWorkers) {
+        uint4* z = reinterpret_cast<uint4*>(hist32 + 8 * tid);
+        z[0] = z[1] = make_uint4(0, 0, 0, 0);
+      }
       __syncthreads();
-      prefix |= (uint32_t)sh->digit_of[0][0] << shift;
-      need = sh->digit_of[0][1];
+      prefix |= (uint32_t)sh->digit << shift;
+      need = sh->need_in_bin;
       mask |= dmask << shift;
-      if (need == sh->digit_of[1][0]) break;                  // the same in every CTA of the cluster
+      if (need == sh->bin_count) break;                       // the same in every CTA of the cluster
+      __syncthreads();                                        // before the next pass writes what was just read
     }
     // ---------------------------------------------------------------- 5. ascending index list
-    // prefix = the fixed digits of the n_keep-th largest key; of the entries that agree with it in
-    // those digits `need` survive (lowest indices; all of them when the select stopped early)
+    // prefix = the fixed digits of the n_rows-th largest key; of the entries that agree with it in
+    // those digits `need` survive (lowest indices; all of them when the select stopped early).  A warp
+    // takes a run of consecutive slots, 32 at a time: the survivors' places are ballot counts.
     const uint32_t thr = prefix;
-    const int per = (n_slots + kCkThreads - 1) / kCkThreads;  // thread t owns slots [t*per, t*per + per)
-    int gt = 0, eq = 0, gt_old = 0, eq_old = 0;
-    for (int e = 0; e < per; ++e) {
-      const int slot = tid * per + e;
-      int j;
-      if (slot < n_slots && slot_info(slot, j)) {
-        const uint32_t k = keys[slot] & mask;
-        gt += k > thr;
-        eq += k == thr;
-        if (j < stored) { gt_old += k > thr; eq_old += k == thr; }
-      }
-    }
-    if (gt_old) atomicAdd(&sh->cnt_old[0], gt_old);
-    if (eq_old) atomicAdd(&sh->cnt_old[1], eq_old);
-    int total;
-    const int packed = ck_block_scan(gt | (eq << 16), sh->warp_sums, total);
-    if (tid == 0) {
-      sh->pub_counts[0] = total & 0xffff;
-      sh->pub_counts[1] = total >> 16;
-      sh->pub_counts[2] = sh->cnt_old[0];
-      sh->pub_counts[3] = sh->cnt_old[1];
-    }
-    cluster_sync();
-    int gt_before = packed & 0xffff, eq_before = packed >> 16;
-    int gt_old_all = 0, eq_old_all = 0;
-    // one remote load per count, then every thread reads the CTA's own copy
-    if (tid < 4 * CL) sh->cnt_all[tid >> 2][tid & 3] = ld_peer_i32(peer_addr(&sh->pub_counts[tid & 3], tid >> 2));
-    __syncthreads();
+    int gt_before = 0, eq_before = 0;
 #pragma unroll
     for (int r = 0; r < kMaxCluster; ++r)
-      if (r < CL) {
-        if (r < rank) { gt_before += sh->cnt_all[r][0]; eq_before += sh->cnt_all[r][1]; }
-        gt_old_all += sh->cnt_all[r][2];
-        eq_old_all += sh->cnt_all[r][3];
-      }
-    const int n_old = gt_old_all + min(eq_old_all, need);     // survivors that were already stored
+      if (r < rank) { gt_before += sh->cnt_gt[r]; eq_before += sh->cnt_eq[r]; }
+    const int n_groups = n_slots / 32, per = (n_groups + kCkWarps - 1) / kCkWarps;
+    const int g_begin = min(n_groups, warp * per), g_end = min(n_groups, g_begin + per);
+    int gt = 0, eq = 0;
+    for (int g = g_begin; g < g_end; ++g) {
+      const int slot = g * 32 + lane;
+      int j;
+      const bool live = slot_info(slot, j);
+      const uint32_t k = keys[slot] & mask;
+      gt += __popc(__ballot_sync(0xffffffffu, live && k > thr));
+      eq += __popc(__ballot_sync(0xffffffffu, live && k == thr));
+    }
+    int total;
+    const int packed = ck_warp_prefix(gt | (eq << 16), sh->warp_sums[0], total);
+    gt_before += packed & 0xffff;
+    eq_before += packed >> 16;
     // Entry o of the head's ascending list is candidate j.  Entry o becomes row o of the head, and
     // rows are compacted in rounds of CL * S consecutive entries, CTA `rk` of the cluster staging S
-    // of them: the entry goes straight into that CTA's shared memory.  Heads that keep the whole new
-    // scale need only their stored survivors (the attention launch appends the rest).
-    const bool attend_appends = a.seg_new[ctx] != 0;
-    const int n_rows = attend_appends ? n_old : n_keep;
+    // of them: the entry goes straight into that CTA's shared memory.
     // rounds: as few as the staging buffers (a third of the staging rows each) allow, of equal size
     const int s_cap = S_ROWS / kMoveBuffers;
     const int n_rounds = (n_rows + CL * s_cap - 1) / (CL * s_cap);
-    const int S = n_rounds > 0 ? (n_rows + CL * n_rounds - 1) / (CL * n_rounds) : 1, RS = CL * S;
-    auto deliver = [&](int o, int j) {
-      if (o < n_rows && dbg_ok(o >= 0 && o < n_keep, a.status, 9)) {
-        const int t = o / RS, w = o - t * RS, rk = w / S, lr = w - rk * S;
+    const int S = (n_rows + CL * n_rounds - 1) / (CL * n_rounds), RS = CL * S;
+    // o / S and o / RS by a multiplication: exact for o < 65 536 and divisors up to 65 536
+    const uint32_t inv_s = 0xffffffffu / (uint32_t)S + 1u, inv_rs = 0xffffffffu / (uint32_t)RS + 1u;
+    const uint32_t lower = (1u << lane) - 1u;
+    for (int g = g_begin; g < g_end; ++g) {
+      const int slot = g * 32 + lane;
+      int j;
+      const bool live = slot_info(slot, j);
+      const uint32_t k = keys[slot] & mask;
+      const bool is_gt = live && k > thr, is_eq = live && k == thr;
+      const uint32_t m_gt = __ballot_sync(0xffffffffu, is_gt), m_eq = __ballot_sync(0xffffffffu, is_eq);
+      const int eq_rank = eq_before + __popc(m_eq & lower);
+      const int o = gt_before + __popc(m_gt & lower) + min(eq_rank, need);
+      if ((is_gt || (is_eq && eq_rank < need)) && dbg_ok(o >= 0 && o < n_rows, a.status, 9)) {
+        const int t = RS == 1 ? o : (int)__umulhi((uint32_t)o, inv_rs), w = o - t * RS;
+        const int rk = S == 1 ? w : (int)__umulhi((uint32_t)w, inv_s), lr = w - rk * S;
         st_peer_i32(peer_addr(&src_all[t * S + lr], rk), j);
       }
-    };
-    for (int e = 0; e < per; ++e) {
-      const int slot = tid * per + e;
-      int j;
-      if (slot < n_slots && slot_info(slot, j)) {
-        const uint32_t k = keys[slot] & mask;
-        if (k > thr) {
-          deliver(gt_before + min(eq_before, need), j);
-          ++gt_before;
-        } else if (k == thr) {
-          if (eq_before < need) deliver(gt_before + eq_before, j);
-          ++eq_before;
-        }
-      }
+      gt_before += __popc(m_gt);
+      eq_before += __popc(m_eq);
     }
-    cluster_sync();                                           // every CTA holds its part of the list
+    cluster_sync(CL);                                         // every CTA holds its part of the list
 
     // ---------------------------------------------------------------- 6. and 7. compaction in rounds
     // A stored survivor moves forward (its source is a row of the head at or behind its
@@ -724,7 +772,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
     for (int t = 0; t < n_rounds; ++t) {
       cp_async_wait_group<1>();                               // the loads of round t (all but the latest group) have landed
       fence_proxy_async();                                    // the bulk stores below read what these threads wrote
-      cluster_sync_relaxed();                                 // every source of this round has been read
+      cluster_sync_relaxed(CL);                               // every source of this round has been read
       const bool moving = slice_moves(t);
       if (moving) {
         const int first = slice_first(t), rows = slice_rows(t);
@@ -750,11 +798,11 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
     }
     if (tid == 0) bulk_wait_read<0>();                        // shared memory is read out before the CTA leaves
   }
-  // no CTA leaves while another may still read its shared memory
-  cluster_sync();
-  if (warp == 1) {
+  // no CTA leaves while another may still read its shared memory (past the list nobody does)
+  if (!select) cluster_sync(CL);
+  if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem, p.tmem_cols);
+    tmem_dealloc(tmem, kMaxObs * p.slots);
   }
 }
 
@@ -764,28 +812,30 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
 template <int D>
 size_t ck_smem_bytes(const CkParams& p) {
   const size_t rows = (size_t)p.stage_rows;
-  return 1024 + (size_t)p.region_bytes + (size_t)p.cpc_max * kCkChunk * sizeof(uint32_t) +
-         (2 * rows + (size_t)p.cpc_max * kCkChunk) * sizeof(int32_t) + sizeof(CkShared) + 64;
+  return 1024 + (size_t)p.region_bytes + (size_t)p.p_max * kCkChunk * sizeof(uint32_t) +
+         (2 * rows + (size_t)p.p_max * kCkChunk) * sizeof(int32_t) + sizeof(CkShared) + 64;
 }
 
 // Ring depth and staging rows for this launch: as many key tiles in flight as the CTA has chunks
-// (more would never be used) and as shared memory holds; the front region then grows to what is
-// left of the budget, so that a round of the compaction stages as many rows as possible.
+// (more would never be used) and as the budget holds; the front region then grows to what is left
+// of the budget, so that a round of the compaction stages as many rows as possible.  False if the
+// budget does not hold the launch.
 template <int D>
-void ck_size(CkParams& p) {
+bool ck_size(CkParams& p, size_t budget) {
   const size_t k_bytes = (size_t)(D / 64) * kCkChunk * 128;
   const size_t row_bytes = 2 * (size_t)D * 2;                // a key row and a value row
   const size_t q_over = (size_t)(D / 64) * kMaxObs * 128 + (size_t)p.n_over * kMaxObs * kCkChunk * sizeof(float);
   p.stage_rows = kMaxStageRows;
   p.region_bytes = 0;
   const size_t other = ck_smem_bytes<D>(p);                   // everything but the front region
-  const size_t room = kSmemBudget > other ? kSmemBudget - other : 0;
+  const size_t room = budget > other ? budget - other : 0;
   const int fit = room > q_over ? (int)((room - q_over) / k_bytes) : 0;
   p.stages = std::max(2, std::min({fit, kMaxStages, std::max(p.cpc_max, 2)}));
   const size_t need = p.stages * k_bytes + q_over;
   const size_t region = std::max(need, std::min(room, (size_t)kMaxStageRows * row_bytes)) / 1024 * 1024;
   p.region_bytes = (int)std::max(region, (need + 1023) / 1024 * 1024);
   p.stage_rows = (int)std::min<size_t>(kMaxStageRows, p.region_bytes / row_bytes);
+  return ck_smem_bytes<D>(p) <= budget;
 }
 
 template <int D>
@@ -806,9 +856,12 @@ cudaLaunchConfig_t ck_config(const StepArgs& a, const CkParams& p, cudaLaunchAtt
   return cfg;
 }
 
-// Clusters of this shape the device runs at the same time (asked once per shape and device).
+// Clusters of this shape the device runs at the same time (asked once per shape and device).  The
+// occupancy queries count one CTA per SM for any kernel that allocates tensor memory, so the two that
+// a shape for two CTAs per SM is made for (shared memory, registers and columns) are counted here.
 template <int D>
-int ck_active_clusters(const StepArgs& a, const CkParams& p) {
+int ck_active_clusters(const StepArgs& a, const CkParams& p, int per_sm) {
+  if (p.cluster == 1) return per_sm * sm_count();
   struct Known { int dev, cluster; size_t smem; int n; };
   static std::mutex mu;
   static std::vector<Known> known;
@@ -817,7 +870,7 @@ int ck_active_clusters(const StepArgs& a, const CkParams& p) {
   const size_t smem = ck_smem_bytes<D>(p);
   std::lock_guard<std::mutex> lock(mu);
   for (const Known& k : known)
-    if (k.dev == dev && k.cluster == p.cluster && k.smem == smem) return k.n;
+    if (k.dev == dev && k.cluster == p.cluster && k.smem == smem) return per_sm * k.n;
   cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = ck_config<D>(a, p, attr, nullptr);
   cfg.numAttrs = 2;
@@ -827,51 +880,83 @@ int ck_active_clusters(const StepArgs& a, const CkParams& p) {
     n = 0;
   }
   known.push_back({dev, p.cluster, smem, n});
-  return n;
+  return per_sm * n;
+}
+
+// Chunks of the candidate lists of a launch, per head type: those whose logits are read twice, and those
+// that only enter the softmax denominators (the new scale of a head that keeps it whole).
+struct CkLists {
+  int ranked[2], once[2];
+};
+
+// Shape of a launch with `cl` CTAs per head and `per_sm` CTAs per SM.  Two CTAs per SM share its tensor
+// memory (256 columns each) and shared memory; a CTA that takes all 512 columns asks for more than half
+// of the shared memory, so that no second one can be placed beside it and wait for columns.
+template <int D>
+bool ck_shape(CkParams& p, const CkLists& n, int cl, int per_sm) {
+  p.cluster = cl;
+  p.p_max = 1;
+  p.cpc_max = 1;
+  for (int t = 0; t < 2; ++t) {
+    const int ranked = (n.ranked[t] + cl - 1) / cl, once = (n.once[t] + cl - 1) / cl;
+    p.p_max = std::max(p.p_max, ranked);
+    p.cpc_max = std::max(p.cpc_max, ranked + once);
+  }
+  const int most = per_sm == 2 ? kMaxSlots / 2 : kMaxSlots;
+  p.slots = 1;
+  while (p.slots < std::min(p.cpc_max, most)) p.slots *= 2;
+  p.direct = p.cpc_max <= p.slots ? p.slots : p.slots - 2;
+  p.n_over = std::max(0, p.p_max - p.direct);
+  if (p.cpc_max > kMaxCpc || p.n_over > (per_sm == 2 ? 2 : kMaxOver)) return false;
+  if (!ck_size<D>(p, per_sm == 2 ? kSmemShared : kSmemBudget)) return false;
+  return p.slots <= kMaxSlots / 2 || ck_smem_bytes<D>(p) > kSmemShared + 4096;
+}
+
+// Device time of one cluster in microseconds, fitted to clock stamps inside the kernel over launches of
+// 1 to 50 chunks per head: 8 us of dependent round trips, 2.5 more where they cross CTAs, and per chunk
+// of a CTA its key tile, its two read-outs and its share of the row moves.  CTAs that share an SM slow
+// each other down.
+template <int D>
+float ck_cluster_us(const CkLists& n, int cl, bool crowded) {
+  const float ranked_us = D == 128 ? 1.8f : 1.2f, once_us = D == 128 ? 1.0f : 0.6f;
+  float most = 0.f;
+  for (int t = 0; t < 2; ++t)
+    most = std::max(most, ranked_us * ((n.ranked[t] + cl - 1) / cl) + once_us * ((n.once[t] + cl - 1) / cl));
+  return (cl > 1 ? 10.5f : 8.f) + (crowded ? 1.6f : 1.f) * most;
 }
 
 template <int D>
 int launch_t(const StepArgs& a, const CUtensorMap& tm_cache, const CUtensorMap& tm_new, const void* q, CkParams p,
-             int max_chunks, int n_clusters, int reserved_sms, cudaStream_t st) {
+             const CkLists& lists, int n_clusters, float beside_us, float behind_us, cudaStream_t st) {
   // the opt-in is made once per (kernel, device), so it asks for the most any launch can need
   if (!allow_dynamic_smem(compress_cluster_kernel<D>, kSmemBudget)) return -1;
-  // CTAs per head: at least what holds the longest candidate list; more spread the key stream over
-  // more SMs, as long as every cluster of the launch still runs at the same time
-  auto shape = [&](int cl) {
-    p.cluster = cl;
-    p.cpc_max = (max_chunks + cl - 1) / cl;
-    p.n_over = p.cpc_max > kTmemChunks ? p.cpc_max - (kTmemChunks - 1) : 0;
-    int cols = 32;
-    while (cols < kMaxObs * std::min(p.cpc_max, kTmemChunks)) cols *= 2;
-    p.tmem_cols = cols;
-    ck_size<D>(p);
-  };
-  int cl = p.cluster;
-  shape(cl);
-  // a launch that runs beside another one leaves that one its SMs, if both fit the device at all
-  const int sms = sm_count();
-  const bool beside = reserved_sms > 0 && n_clusters * cl + reserved_sms <= sms;
-  while (cl < kMaxCluster && (max_chunks + 2 * cl - 1) / (2 * cl) >= 2) {
-    if (beside && n_clusters * 2 * cl + reserved_sms > sms) break;
-    shape(2 * cl);
-    if (ck_active_clusters<D>(a, p) < n_clusters) break;
-    cl *= 2;
-  }
-  // beside another launch the SMs left over need not hold a power of two per head
-  while (beside && cl < kMaxCluster && (max_chunks + cl) / (cl + 1) >= 2 && n_clusters * (cl + 1) + reserved_sms <= sms) {
-    shape(cl + 1);
-    if (ck_active_clusters<D>(a, p) < n_clusters) break;
-    ++cl;
-  }
-  shape(cl);
-  if (ck_smem_bytes<D>(p) > kSmemBudget) {
-    set_error("compression: shared memory plan beyond the limit");
-    return -1;
-  }
+  // CTAs per head and per SM: the step ends when this launch and the attention that needs it are done,
+  // and not before the SMs have done all the work there is (larger clusters finish sooner and keep
+  // more SMs from the attention that could run beside them).
+  const float sms = (float)sm_count();
+  float best = 0.f;
+  int best_cl = 0, best_per_sm = 0;
+  for (int per_sm = 1; per_sm <= 2; ++per_sm)
+    for (int cl = 1; cl <= kMaxCluster; ++cl) {
+      if (!ck_shape<D>(p, lists, cl, per_sm)) continue;
+      const int active = ck_active_clusters<D>(a, p, per_sm);
+      if (active < 1) continue;
+      const int waves = (n_clusters + active - 1) / active;
+      const float us = waves * ck_cluster_us<D>(lists, cl, per_sm == 2 && std::min(n_clusters, active) * cl > sms);
+      const float sm_us = n_clusters * cl * us / (waves * per_sm);
+      const float cost = std::max(us + behind_us / sms, (sm_us + beside_us + behind_us) / sms);
+      if (!best_cl || cost < best) {
+        best = cost;
+        best_cl = cl;
+        best_per_sm = per_sm;
+      }
+    }
+  if (!best_cl) return 0;
+  ck_shape<D>(p, lists, best_cl, best_per_sm);
   cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = ck_config<D>(a, p, attr, st);
   cudaLaunchKernelEx(&cfg, compress_cluster_kernel<D>, tm_cache, tm_new, a, static_cast<const __nv_bfloat16*>(q), p);
-  return launched(n_clusters * cl);
+  return launched(n_clusters * p.cluster);
 }
 
 }  // namespace
@@ -879,27 +964,24 @@ int launch_t(const StepArgs& a, const CUtensorMap& tm_cache, const CUtensorMap& 
 // Scores only (scores != nullptr) or the whole compression of the step.  Returns the working CTAs of
 // its one launch, -1 on a launch error, or 0 when this step is outside what the kernel holds
 // (candidate lists beyond 8 x 21 chunks per head, the every-query scoring rounds): the caller then
-// takes the separate scoring, selection and compaction launches.  reserved_sms: CTAs of the launch
-// behind this one that can run beside it (0 if none).
+// takes the separate scoring, selection and compaction launches.
 int launch_compress_cluster(const StepArgs& a, const void* q, const void* k_new, const void* v_new, float* scores,
-                            cudaStream_t st, int reserved_sms) {
+                            cudaStream_t st, float beside_us, float behind_us) {
   if (!a.k_map || a.obs_full || a.score_accumulate) return 0;
-  int max_chunks = 0;
-  const int n_new_chunks = (a.n_new + kCkChunk - 1) / kCkChunk;
-  for (int t = 0; t < 2; ++t)
-    if (a.trig[t]) {
-      max_chunks = std::max(max_chunks, (a.stored[t] + kCkChunk - 1) / kCkChunk + n_new_chunks);
-    }
-  if (max_chunks == 0) return 0;
-  int cl = 1;
-  while (cl <= kMaxCluster && (max_chunks + cl - 1) / cl > kMaxCpc) cl *= 2;
-  if (cl > kMaxCluster) return 0;
+  if (!a.trig[0] && !a.trig[1]) return 0;
   CkParams p{};
-  p.cluster = cl;
   p.score_only = scores != nullptr;
   p.scores = scores;
   p.k_new = static_cast<const uint4*>(k_new);
   p.v_new = static_cast<const uint4*>(v_new);
+  CkLists lists = {};
+  const int n_new_chunks = (a.n_new + kCkChunk - 1) / kCkChunk;
+  for (int t = 0; t < 2; ++t)
+    if (a.trig[t] && a.heads_of[t] > 0) {
+      const bool drop_new = t == 0 && a.protect_new && !scores;
+      lists.ranked[t] = (a.stored[t] + kCkChunk - 1) / kCkChunk + (drop_new ? 0 : n_new_chunks);
+      lists.once[t] = drop_new ? n_new_chunks : 0;
+    }
   // clusters that do work: the heads of the triggered types
   const int n_clusters = std::max(1, a.heads_of[0] * a.trig[0] + a.heads_of[1] * a.trig[1]);
   CUtensorMap tm_new;
@@ -908,8 +990,8 @@ int launch_compress_cluster(const StepArgs& a, const void* q, const void* k_new,
     return -1;
   }
   const CUtensorMap& tm_cache = *static_cast<const CUtensorMap*>(a.k_map);
-  return a.head_dim == 128 ? launch_t<128>(a, tm_cache, tm_new, q, p, max_chunks, n_clusters, reserved_sms, st)
-                           : launch_t<64>(a, tm_cache, tm_new, q, p, max_chunks, n_clusters, reserved_sms, st);
+  return a.head_dim == 128 ? launch_t<128>(a, tm_cache, tm_new, q, p, lists, n_clusters, beside_us, behind_us, st)
+                           : launch_t<64>(a, tm_cache, tm_new, q, p, lists, n_clusters, beside_us, behind_us, st);
 }
 
 }  // namespace hack

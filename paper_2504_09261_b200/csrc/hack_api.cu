@@ -800,12 +800,11 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
   if (any && fused_append) {
     // score, select and compact in one cluster launch per head (counted with the scoring stage).  The
     // attention launch behind it starts the heads that do not depend on it (a head type that evicts
-    // nothing, two query tiles per CTA) on the SMs it leaves free.
+    // nothing) on the SMs it leaves free.
     StageScope ts(c, st, 0);
-    int beside = 0;
-    for (int t = 0; t < 2; ++t)
-      if (!a.trig[t]) beside = a.heads_of[t] * ((p.n_new + 255) / 256);
-    if ((r = hack::launch_compress_cluster(a, q, k, v, nullptr, st, beside)) < 0) return HACK_ERR_CUDA;
+    float beside_us = 0.f, behind_us = 0.f;
+    for (int t = 0; t < 2; ++t) (a.trig[t] ? behind_us : beside_us) += hack::attend_tc_sm_us(a, t);
+    if ((r = hack::launch_compress_cluster(a, q, k, v, nullptr, st, beside_us, behind_us)) < 0) return HACK_ERR_CUDA;
     compression_ctas = r;
     ts.done(r > 0);
     n += r > 0;

@@ -86,10 +86,10 @@ int launch_select(const StepArgs& a, const float* scores, int32_t* idx, int32_t*
                   cudaStream_t st);
 // bf16 caches: scores only (scores != nullptr) or scoring, selection and in-place compaction of the step
 // in one launch of one thread-block cluster per head.  Its CTAs if launched; 0: the step is outside what
-// the kernel holds, take the separate launches; -1: launch error.  reserved_sms: SMs that CTAs of the
-// launch behind this one can use at the same time.
+// the kernel holds, take the separate launches; -1: launch error.  beside_us, behind_us: SM-microseconds
+// of the attention launch behind this one that can run beside it, and that need its result.
 int launch_compress_cluster(const StepArgs& a, const void* q, const void* k_new, const void* v_new, float* scores,
-                            cudaStream_t st, int reserved_sms = 0);
+                            cudaStream_t st, float beside_us = 0.f, float behind_us = 0.f);
 // idx == nullptr: every head appends (keeps all candidates).  idx_all != 0: idx rows are valid for
 // heads that are not triggered as well (identity lists written by launch_select).
 int launch_compact(const StepArgs& a, int dtype, const int32_t* idx, int idx_all, const void* k_new,
@@ -106,6 +106,8 @@ int launch_attend_simt(const StepArgs& a, int dtype, const void* q, void* out, c
 // do not depend on it then start beside it), 0 if it is not.
 int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_stats, const void* k_new,
                      const void* v_new, cudaStream_t st, int compression_ctas);
+// Rough SM-microseconds of the tensor-core attention of one head type (two query tiles per CTA).
+float attend_tc_sm_us(const StepArgs& a, int type);
 constexpr long long kDefaultWaitCycles = 2000000000ll;   // about one second: no wait is legitimately longer
 // Attention variance per (batch, head) over the compacted cache (Eq. 6) from the row statistics of
 // launch_attend_tc; block_var: device scratch [b*H, max_blocks]; sigma: device [b*H].  bf16 only.
