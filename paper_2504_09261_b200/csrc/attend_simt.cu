@@ -1,7 +1,6 @@
 // Attention of the scale's queries over the compacted per-head cache (Eq. 4 on the compressed
-// cache), plain fp32 arithmetic on the CUDA cores.  This is the exact-precision path (fp32
-// workloads forbid TF32 at the required 1e-5) and the fallback for shapes the tensor-core kernel
-// does not take.
+// cache) of fp32 caches, plain fp32 arithmetic on the CUDA cores: the exact-precision path (fp32
+// workloads forbid TF32 at the required 1e-5).
 //
 // Bound: the FMA pipe.  A CTA serves 32 query rows of one head; its four groups of 64 threads walk
 // every fourth tile of 32 keys with a streaming softmax of their own and are merged at the end, so
@@ -28,57 +27,17 @@ constexpr int kBK = 32;              // keys per tile
 constexpr int kGroups = 4;           // groups of 64 threads, each with its own key tiles
 constexpr int kThreads = kGroups * 64;
 
-template <typename T> struct Cvt;
-template <> struct Cvt<float> {
-  static constexpr int kPerVec = 4;
-  __device__ static void store4(float* dst, const float4& f) { *reinterpret_cast<float4*>(dst) = f; }
-};
-template <> struct Cvt<__nv_bfloat16> {
-  static constexpr int kPerVec = 8;
-  __device__ static void unpack(const uint4& v, float* f) {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      f[2 * i] = __uint_as_float(w[i] << 16);
-      f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-    }
-  }
-  __device__ static void store4(__nv_bfloat16* dst, const float4& f) {
-    __nv_bfloat162 a = __floats2bfloat162_rn(f.x, f.y);
-    __nv_bfloat162 b = __floats2bfloat162_rn(f.z, f.w);
-    uint2 p;
-    p.x = *reinterpret_cast<uint32_t*>(&a);
-    p.y = *reinterpret_cast<uint32_t*>(&b);
-    *reinterpret_cast<uint2*>(dst) = p;
-  }
-};
-
-// 32 rows of D elements from global memory (rows at or past n_rows read as zero) into padded fp32
-// rows; `nthr` threads take part.  fp32 rows arrive by cp.async (the caller commits and waits).
-template <typename T, int D>
-__device__ __forceinline__ void stage_rows(float* dst, const T* src, int n_rows, int t, int nthr) {
-  constexpr int LD = D + 4;
-  if constexpr (sizeof(T) == 4) {
-    constexpr int V = D / 4;
+// 32 rows of D floats from global memory (rows at or past n_rows read as zero) into padded rows by
+// cp.async (the caller commits and waits); `nthr` threads take part.
+template <int D>
+__device__ __forceinline__ void stage_rows(float* dst, const float* src, int n_rows, int t, int nthr) {
+  constexpr int LD = D + 4, V = D / 4;
 #pragma unroll 4
-    for (int v = t; v < 32 * V; v += nthr) {
-      const int r = v / V, c = v % V;
-      const uint32_t d = ptx::smem_u32(dst + r * LD + c * 4);
-      const int bytes = r < n_rows ? 16 : 0;                 // 0: the 16 bytes are filled with zeros
-      const T* s = src + (size_t)(r < n_rows ? r : 0) * D + c * 4;
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(s), "r"(bytes) : "memory");
-    }
-  } else {
-    constexpr int V = D / 8;
-#pragma unroll 4
-    for (int v = t; v < 32 * V; v += nthr) {
-      const int r = v / V, c = v % V;
-      float f[8];
-      const uint4 raw = r < n_rows ? *reinterpret_cast<const uint4*>(src + (size_t)r * D + c * 8) : make_uint4(0, 0, 0, 0);
-      Cvt<T>::unpack(raw, f);
-      *reinterpret_cast<float4*>(dst + r * LD + c * 8) = make_float4(f[0], f[1], f[2], f[3]);
-      *reinterpret_cast<float4*>(dst + r * LD + c * 8 + 4) = make_float4(f[4], f[5], f[6], f[7]);
-    }
+  for (int v = t; v < 32 * V; v += nthr) {
+    const int r = v / V, c = v % V;
+    const int bytes = r < n_rows ? 16 : 0;                 // 0: the 16 bytes are filled with zeros
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(dst + r * LD + c * 4)),
+                 "l"(src + (size_t)(r < n_rows ? r : 0) * D + c * 4), "r"(bytes) : "memory");
   }
 }
 
@@ -91,9 +50,9 @@ constexpr size_t simt_smem_bytes() {
   return sizeof(float) * ((size_t)kBQ * (D + 4) + kGroups * (2 * (size_t)kBK * (D + 4) + kBQ * (kBK + 4)));
 }
 
-template <typename T, int D>
+template <int D>
 __global__ void __launch_bounds__(kThreads)
-attend_simt_kernel(const StepArgs a, const T* __restrict__ q, T* __restrict__ out) {
+attend_simt_kernel(const StepArgs a, const float* __restrict__ q, float* __restrict__ out) {
   pdl_wait();
   constexpr int LD = D + 4, LP = kBK + 4;
   constexpr int CV = D / 32;                      // float4 columns per thread
@@ -109,16 +68,16 @@ attend_simt_kernel(const StepArgs a, const T* __restrict__ q, T* __restrict__ ou
   float* vs = ks + kBK * LD;
   float* ps = vs + kBK * LD;
 
-  const T* kp = static_cast<const T*>(a.k_plane) + (size_t)a.row_off[bh] * D;
-  const T* vp = static_cast<const T*>(a.v_plane) + (size_t)a.row_off[bh] * D;
+  const float* kp = static_cast<const float*>(a.k_plane) + (size_t)a.row_off[bh] * D;
+  const float* vp = static_cast<const float*>(a.v_plane) + (size_t)a.row_off[bh] * D;
   const int n_tiles = (len + kBK - 1) / kBK;
 
   auto group_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory"); };
 
-  stage_rows<T, D>(qs, q + ((size_t)bh * a.n_new + q0) * D, a.n_new - q0, tid, kThreads);
-  if (grp < n_tiles) stage_rows<T, D>(ks, kp + (size_t)grp * kBK * D, len - grp * kBK, gt, 64);
+  stage_rows<D>(qs, q + ((size_t)bh * a.n_new + q0) * D, a.n_new - q0, tid, kThreads);
+  if (grp < n_tiles) stage_rows<D>(ks, kp + (size_t)grp * kBK * D, len - grp * kBK, gt, 64);
   commit();
-  if (grp < n_tiles) stage_rows<T, D>(vs, vp + (size_t)grp * kBK * D, len - grp * kBK, gt, 64);
+  if (grp < n_tiles) stage_rows<D>(vs, vp + (size_t)grp * kBK * D, len - grp * kBK, gt, 64);
   commit();
   wait_group<1>();
   __syncthreads();
@@ -157,7 +116,7 @@ attend_simt_kernel(const StepArgs a, const T* __restrict__ q, T* __restrict__ ou
     }
     group_sync();                                 // both warps are done with the key tile
     if (t + kGroups < n_tiles)
-      stage_rows<T, D>(ks, kp + (size_t)(t + kGroups) * kBK * D, len - (t + kGroups) * kBK, gt, 64);
+      stage_rows<D>(ks, kp + (size_t)(t + kGroups) * kBK * D, len - (t + kGroups) * kBK, gt, 64);
     commit();
 
     float corr[4];
@@ -217,7 +176,7 @@ attend_simt_kernel(const StepArgs a, const T* __restrict__ q, T* __restrict__ ou
     }
     group_sync();                                 // both warps are done with the value tile
     if (t + kGroups < n_tiles)
-      stage_rows<T, D>(vs, vp + (size_t)(t + kGroups) * kBK * D, len - (t + kGroups) * kBK, gt, 64);
+      stage_rows<D>(vs, vp + (size_t)(t + kGroups) * kBK * D, len - (t + kGroups) * kBK, gt, 64);
     commit();
     wait_group<1>();                              // the next key tile has landed
     group_sync();
@@ -264,25 +223,24 @@ attend_simt_kernel(const StepArgs a, const T* __restrict__ q, T* __restrict__ ou
       acc.w = fmaf(w, f.w, acc.w);
     }
     const float inv = 1.f / sum;
-    Cvt<T>::store4(out + ((size_t)bh * a.n_new + q0 + r) * D + c * 4,
-                   make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv));
+    *reinterpret_cast<float4*>(out + ((size_t)bh * a.n_new + q0 + r) * D + c * 4) =
+        make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
   }
 }
 
-template <typename T, int D>
+template <int D>
 int launch_t(const StepArgs& a, const void* q, void* out, cudaStream_t st) {
-  if (!allow_dynamic_smem(attend_simt_kernel<T, D>, simt_smem_bytes<D>())) return -1;
+  if (!allow_dynamic_smem(attend_simt_kernel<D>, simt_smem_bytes<D>())) return -1;
   const dim3 grid((a.n_new + kBQ - 1) / kBQ, a.batch * a.n_heads);
-  launch_k(attend_simt_kernel<T, D>, grid, dim3(kThreads), simt_smem_bytes<D>(), st, a, static_cast<const T*>(q),
-           static_cast<T*>(out));
+  launch_k(attend_simt_kernel<D>, grid, dim3(kThreads), simt_smem_bytes<D>(), st, a, static_cast<const float*>(q),
+           static_cast<float*>(out));
   return launched(1);
 }
 
 }  // namespace
 
-int launch_attend_simt(const StepArgs& a, int dtype, const void* q, void* out, cudaStream_t st) {
-  if (dtype == HACK_F32) return a.head_dim == 64 ? launch_t<float, 64>(a, q, out, st) : launch_t<float, 128>(a, q, out, st);
-  return a.head_dim == 64 ? launch_t<__nv_bfloat16, 64>(a, q, out, st) : launch_t<__nv_bfloat16, 128>(a, q, out, st);
+int launch_attend_simt(const StepArgs& a, const void* q, void* out, cudaStream_t st) {
+  return a.head_dim == 64 ? launch_t<64>(a, q, out, st) : launch_t<128>(a, q, out, st);
 }
 
 }  // namespace hack

@@ -53,9 +53,9 @@ bool attend_tc_serves(const StepArgs& a, int dtype) {
 }
 
 int launch_attend(const StepArgs& a, int dtype, const void* q, void* out, cudaStream_t st) {
-  if (attend_tc_serves(a, dtype))
-    return launch_attend_tc(a, q, out, nullptr, nullptr, nullptr, st, 0);
-  return launch_attend_simt(a, dtype, q, out, st);
+  if (dtype == HACK_F32) return launch_attend_simt(a, q, out, st);
+  if (attend_small_serves(a)) return launch_attend_small(a, dtype, q, nullptr, nullptr, out, st);
+  return launch_attend_tc(a, q, out, nullptr, nullptr, nullptr, st, 0);
 }
 
 }  // namespace hack
@@ -679,7 +679,7 @@ hack_status_t hack_compact(hack_cache_t* c, int32_t layer, int32_t scale, const 
   return HACK_OK;
 }
 
-// fused: the arguments of a fused step whose tensor-core attention reads the new rows of the head types
+// fused: the arguments of a fused step whose attention reads the new rows of the head types
 // flagged in seg_new from the caller's tensors and appends them itself (compression_ctas: CTAs of the
 // step's compression launch, 0 if there is none).
 struct FusedAttend {
@@ -710,7 +710,9 @@ static hack_status_t attend_impl(hack_cache* c, int layer, int scale, const void
       n = m < 0 ? m : n + m;
     }
   } else if (fused) {
-    n = hack::launch_attend_tc(a, q, out, nullptr, fused->k_new, fused->v_new, st, fused->compression_ctas);
+    n = hack::attend_small_serves(a)
+            ? hack::launch_attend_small(a, c->cfg.dtype, q, fused->k_new, fused->v_new, out, st, fused->compression_ctas > 0)
+            : hack::launch_attend_tc(a, q, out, nullptr, fused->k_new, fused->v_new, st, fused->compression_ctas);
   } else {
     n = hack::launch_attend(a, c->cfg.dtype, q, out, st);
   }
@@ -773,21 +775,22 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
   hack::StepArgs a = make_args(c, layer, scale, p);
   const bool any = p.triggered_c || p.triggered_s;
   int n = 0, r;
-  // Tensor-core attention takes the rows of a head type that keeps the whole new scale straight
-  // from the caller's K/V and appends them itself: types that evict nothing in this step, and
+  // The bf16 attention kernels take the rows of a head type that keeps the whole new scale straight
+  // from the caller's K/V and append them themselves: types that evict nothing in this step, and
   // structural heads whose latest scale is protected (Eq. 11).  Contextual heads that evict rank the
   // new rows as well (Eq. 10) and are compacted first.  The final-scale merge keeps the separate
-  // compaction it is wrapped around.
+  // compaction it is wrapped around, and so do steps that evict with fewer new rows than one TMA box.
   const bool merge_step = c->cfg.merge_last && scale == c->cfg.n_scales - 1 && p.triggered_c;
-  const bool fused_append = hack::attend_tc_serves(a, c->cfg.dtype) && !merge_step;
+  const bool boxes = (long long)c->cfg.batch * c->cfg.n_heads * p.n_new >= 128;
+  const bool fused_append = c->cfg.dtype == HACK_BF16 && !merge_step && (!any || boxes);
   if (fused_append) {
     a.seg_new[0] = !p.triggered_s || a.protect_new;
     a.seg_new[1] = !p.triggered_c;
   }
-  if (!any && p.n_new <= hack::kSmallQueries) {
+  if (c->cfg.dtype == HACK_F32 && !any && p.n_new <= hack::kSmallQueries) {
     // nothing is evicted and the scale is small: one launch appends and attends
     StageScope ts(c, st, 3);
-    if ((r = hack::launch_append_attend_small(a, c->cfg.dtype, q, k, v, out, st)) < 0) return HACK_ERR_CUDA;
+    if ((r = hack::launch_attend_small(a, c->cfg.dtype, q, k, v, out, st)) < 0) return HACK_ERR_CUDA;
     ts.done(r);
     c->launches += r;
     advance_after_compact(c, layer, p);

@@ -96,7 +96,7 @@ int launch_compact(const StepArgs& a, int dtype, const int32_t* idx, int idx_all
                    const void* v_new, cudaStream_t st);
 int launch_attend(const StepArgs& a, int dtype, const void* q, void* out, cudaStream_t st);
 
-int launch_attend_simt(const StepArgs& a, int dtype, const void* q, void* out, cudaStream_t st);
+int launch_attend_simt(const StepArgs& a, const void* q, void* out, cudaStream_t st);   // fp32 caches
 // row_stats (optional, device [b*H, N_k, 2]): per query row the reference maximum m (raw logit
 // units; within the lazy-rescaling margin of the true maximum) and l = sum_j exp2(c (z_j - m)).
 // k_new / v_new (optional): the caller's K/V of this scale; head types with a.seg_new set then attend
@@ -117,12 +117,15 @@ bool attend_tc_serves(const StepArgs& a, int dtype);   // the tensor-core kernel
 // 2-D bf16 tensor map (128 x 64 boxes, 128-byte swizzle) over rows x head_dim; false on failure.
 bool make_rows_map(void* out_map, const void* base, uint64_t rows, int head_dim);
 
-// Untriggered step with at most kSmallQueries new tokens: append and attention in one SIMT launch.
-int launch_append_attend_small(const StepArgs& a, int dtype, const void* q, const void* k_new,
-                               const void* v_new, void* out, cudaStream_t st);
+// Attention of a small step in one launch that appends as well.  bf16: any step that attend_small_serves
+// (head types with a.seg_new read the caller's rows and append them; after_compression: the launch ahead in
+// the stream is the step's compression launch).  fp32: steps that evict nothing, at most kSmallQueries new tokens.
+int launch_attend_small(const StepArgs& a, int dtype, const void* q, const void* k_new, const void* v_new, void* out,
+                        cudaStream_t st, bool after_compression = false);
+bool attend_small_serves(const StepArgs& a);   // bf16: the small kernel is the one for this step's attention
 constexpr int kSmallQueries = 31;
 
-constexpr int kTcMinQueries = 32;   // below this the SIMT kernel serves bf16 as well
+constexpr int kTcMinQueries = 32;   // below this the small kernel serves every bf16 step
 
 void set_error(const std::string& msg);
 // Number of SMs of the current device (asked once per device); the grid heuristics size to it.
