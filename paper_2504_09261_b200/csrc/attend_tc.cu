@@ -3,7 +3,8 @@
 // compressed cache).
 //
 // One CTA serves one (batch, head) and up to two 128-row query tiles, which take turns on the
-// tensor pipe so that the softmax of one tile overlaps the MMAs of the other.
+// tensor pipe so that the softmax of one tile overlaps the MMAs of the other (T = 2); or, at head_dim
+// 64 and short caches, one tile on half an SM (T = 1: no warps 8-11, half the tensor memory).
 //   warp  0     : issuer of the Q K^T products; also owns the TMEM allocation
 //   warp  1     : TMA producer (K and V tiles of 128 cache rows through rings)
 //   warp  2     : issuer of the P V products (a single issuing thread for both products was the
@@ -57,6 +58,8 @@
 // flight, frees its TMEM and returns.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "hack_internal.h"
 #include "tc_ptx.cuh"
 
@@ -67,14 +70,23 @@ using namespace ptx;
 
 constexpr int kBM = 128;                 // query rows per tile
 constexpr int kBN = 128;                 // cache rows per K/V tile
-constexpr int kThreadsTc = 384;
 constexpr int kMmaWarp = 0, kProducerWarp = 1, kPvWarp = 2, kAppendWarp = 3;   // an issuer is the oldest warp of its scheduler
-constexpr int kSoftmaxRegs = 224, kOtherRegs = 56;   // 2*128*224 + 128*56 = 384*168 registers
+// A CTA of T tiles: four warps that issue and four softmax warps per tile.  Registers are moved from the
+// former to the latter: T = 2: 2*128*224 + 128*56 = 384*168 registers; T = 1: 128*200 + 128*56 = 256*128,
+// half an SM's, like its tensor memory and shared memory: two such CTAs per SM.
+template <int T> struct Shape;
+template <> struct Shape<2> {
+  static constexpr int kThreads = 384, kCtasPerSm = 1, kSoftmaxRegs = 224, kOtherRegs = 56;
+  static constexpr uint32_t kTmemCols = 512, kOutCol = 256, kCopyChunk = 16384;   // kCopyChunk: bytes per bulk copy of the append
+};
+template <> struct Shape<1> {
+  static constexpr int kThreads = 256, kCtasPerSm = 2, kSoftmaxRegs = 200, kOtherRegs = 56;
+  static constexpr uint32_t kTmemCols = 256, kOutCol = 192, kCopyChunk = 8192;
+};
 constexpr int kPolyOf8 = 0;              // pairs out of 8 whose 2^x runs on the FMA pipe
 constexpr int kKStages = 2;
 constexpr int kVStages = 2;
 constexpr uint32_t kSpinLimit = 1u << 22;          // polls while draining after an abort
-constexpr uint32_t kCopyChunk = 16384;             // bytes per bulk copy of the append
 constexpr float kRescaleThreshold = 32.0f;   // log2 units: p <= 2^32, far inside the bf16 / fp32 range
 
 struct TcParams {
@@ -136,8 +148,8 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Bars* b
   return false;
 }
 
-template <int D>
-__global__ void __launch_bounds__(kThreadsTc, 1)
+template <int D, int T>
+__global__ void __launch_bounds__(Shape<T>::kThreads, Shape<T>::kCtasPerSm)
 attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kn,
                  const __grid_constant__ CUtensorMap tm_vn, const __grid_constant__ CUtensorMap tm_o,
@@ -145,17 +157,20 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   constexpr int SUB = D / 64;                       // 64-column (128-byte) sub-tiles per row
   constexpr uint32_t SUB_BYTES = kBN * 128;         // one sub-tile: 128 rows x 128 bytes
   constexpr uint32_t TILE_BYTES = SUB * SUB_BYTES;
-  constexpr uint32_t S_COL = 0, P_COL = 128, O_COL = 256;
+  constexpr uint32_t S_COL = 0, P_COL = 128, O_COL = Shape<T>::kOutCol;
+  constexpr int kSoftmaxRegs = Shape<T>::kSoftmaxRegs, kOtherRegs = Shape<T>::kOtherRegs;
+  constexpr uint32_t kCopyChunk = Shape<T>::kCopyChunk;
+  static_assert(P_COL + T * 64 <= O_COL && O_COL + T * D <= Shape<T>::kTmemCols, "tensor memory plan");
 
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t raw = smem_u32(smem_dyn);
   const uint32_t base = (raw + 1023u) & ~1023u;     // 128-byte swizzle needs 1024-byte alignment
   unsigned char* sm = smem_dyn + (base - raw);
   const uint32_t q_sm = base;
-  const uint32_t k_sm = q_sm + 2 * TILE_BYTES;
+  const uint32_t k_sm = q_sm + T * TILE_BYTES;
   const uint32_t v_sm = k_sm + kKStages * TILE_BYTES;
   const uint32_t copy_sm = v_sm + kVStages * TILE_BYTES;           // 2 x kCopyChunk bytes: staging of the append
-  Bars* bars = reinterpret_cast<Bars*>(sm + (2 + kKStages + kVStages) * TILE_BYTES + 2 * kCopyChunk);
+  Bars* bars = reinterpret_cast<Bars*>(sm + (T + kKStages + kVStages) * TILE_BYTES + 2 * kCopyChunk);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // CTAs of the first head type, then those of the other one
@@ -170,7 +185,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   const int nblk_b = (len_b + kBN - 1) / kBN;             // the caller's rows come first: they may not have to wait
   const int nblk = nblk_b + (len_a + kBN - 1) / kBN;      // >= 1: a head never attends over nothing
   const int q0 = pair * p.tiles_per_cta[type] * kBM;
-  const int ntile = (p.tiles_per_cta[type] == 2 && q0 + kBM < p.n_new) ? 2 : 1;
+  const int ntile = T == 2 && p.tiles_per_cta[type] == 2 && q0 + kBM < p.n_new ? 2 : 1;
 
   const int qrow = bh * p.n_new + q0;
   const int krow = p.row_off[bh];
@@ -222,7 +237,6 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     };
     if (p.q_before_wait) load_queries();
     if (dep == kDepAll || (dep == kDepCache && nblk_b == 0)) pdl_grid_wait();
-    pdl_launch_dependents();
     if (!p.q_before_wait) load_queries();
     mbar_expect_tx(smem_u32(&bars->k_full[0]), TILE_BYTES);
     for (int c = 0; c < SUB; ++c) tma_load_2d(k_sm + c * SUB_BYTES, k_src(0), c * 64, tile_row(0), smem_u32(&bars->k_full[0]));
@@ -230,8 +244,11 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     for (int c = 0; c < SUB; ++c) tma_load_2d(v_sm + c * SUB_BYTES, v_src(0), c * 64, tile_row(0), smem_u32(&bars->v_full[0]));
   }
   if (warp == kMmaWarp) {
-    tmem_alloc(smem_u32(&bars->tmem_base), 512);
+    tmem_alloc(smem_u32(&bars->tmem_base), Shape<T>::kTmemCols);
     tmem_relinquish();
+    // the next launch may start once every CTA of this one holds its tensor memory: a CTA of the next
+    // launch that took the columns first would wait for this grid, and this CTA for the columns
+    pdl_launch_dependents();
   }
   tc_fence_before();
   __syncthreads();
@@ -357,7 +374,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     if (lane == 0) {
       constexpr uint32_t IDESC_S = idesc_bf16_f32(kBM, kBN, 0);        // A = Q, B = K (both K-major)
       // descriptors of the tile bases; a k-step only adds a constant to the address field
-      const uint64_t q_desc[2] = {smem_desc_sw128(q_sm, 16, 1024), smem_desc_sw128(q_sm + TILE_BYTES, 16, 1024)};
+      const uint64_t q_desc[2] = {smem_desc_sw128(q_sm, 16, 1024), smem_desc_sw128(q_sm + (T - 1) * TILE_BYTES, 16, 1024)};
       const uint64_t k_desc0 = smem_desc_sw128(k_sm, 16, 1024);
       bool ok = true;
       // S = Q_t K_j^T into the one logit buffer; `use` counts the products issued so far, and product
@@ -564,7 +581,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   __syncthreads();
   if (warp == kMmaWarp) {
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    tmem_dealloc(tmem, Shape<T>::kTmemCols);
   }
   // The launch behind this one relies on everything ahead of it being complete once this grid is, so
   // one CTA does not leave before the launch ahead has completed, whatever its heads depend on.
@@ -587,9 +604,9 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-template <int D>
+template <int D, int T>
 size_t tc_smem_bytes() {
-  return 1024 + (2 + kKStages + kVStages) * (size_t)(D / 64) * kBN * 128 + 2 * kCopyChunk + sizeof(Bars) + 64;
+  return 1024 + (T + kKStages + kVStages) * (size_t)(D / 64) * kBN * 128 + 2 * Shape<T>::kCopyChunk + sizeof(Bars) + 64;
 }
 
 }  // namespace
@@ -620,6 +637,18 @@ bool make_out_map(CUtensorMap* out_map, const void* base, int heads, int n_new, 
   return fn(out_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+}  // namespace
+
+namespace {
+template <int D, int T>
+int launch_tc(int grid, cudaStream_t st, const CUtensorMap& tm_q, const CUtensorMap& tk, const CUtensorMap& tv,
+              const CUtensorMap& tm_kn, const CUtensorMap& tm_vn, const CUtensorMap& tm_o, const TcParams& p) {
+  // two tiles of head_dim 64 ask for as much as head_dim 128: one CTA per SM, it owns all of tensor memory
+  const size_t smem = T == 2 ? tc_smem_bytes<128, 2>() : tc_smem_bytes<D, T>();
+  if (!allow_dynamic_smem(attend_tc_kernel<D, T>, smem)) return -1;
+  launch_k(attend_tc_kernel<D, T>, grid, Shape<T>::kThreads, smem, st, tm_q, tk, tv, tm_kn, tm_vn, tm_o, p);
+  return launched(1);
 }
 }  // namespace
 
@@ -671,11 +700,18 @@ int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_sta
   // One query tile per CTA while that still fits one wave (twice the CTAs, no idle SMs), else two.  A
   // type that does not wait for the compression has the SMs that launch does not hold.
   const int n_tiles = (a.n_new + kBM - 1) / kBM;
+  // head_dim 64: CTAs of one tile that take half an SM each.  Two of them hide each other's start and
+  // epilogue (4.5 us of a CTA), but read every K/V tile twice as often as one CTA of two tiles.  Behind a
+  // compression, 256 heads x 100 queries, 255 keys: 21.2 against 24.8 us per step, 240 heads x 324
+  // queries, 640 keys: 38.4 against 43.8, 1 024 queries, 1 045 keys: 128.0 against 128.7; without one, 256
+  // heads x 256 queries, 680 keys: 32.0 against 30.6, 128 heads x 4 096 queries, 6 401 keys: 1 138 against 1 044.
+  const int longest = (std::max(a.kept[0], a.kept[1]) + kBN - 1) / kBN;
+  const bool halves = a.head_dim == 64 && longest <= (compression_ctas > 0 ? 12 : 4);
   const bool apart = p.dep[p.first_type] == kDepNothing && p.dep[1 - p.first_type] != kDepNothing;   // one type runs after the other
   for (int t = 0; t < 2; ++t) {
     const int heads = apart ? a.heads_of[t] : a.heads_of[0] + a.heads_of[1];
     const int sms = sm_count() - (p.dep[t] == kDepNothing ? compression_ctas : 0);
-    p.tiles_per_cta[t] = n_tiles * heads <= sms ? 1 : 2;
+    p.tiles_per_cta[t] = halves || n_tiles * heads <= sms ? 1 : 2;
     p.n_pairs[t] = (n_tiles + p.tiles_per_cta[t] - 1) / p.tiles_per_cta[t];
   }
   p.first_ctas = p.n_pairs[p.first_type] * p.first_heads;
@@ -696,15 +732,9 @@ int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_sta
   p.out = static_cast<__nv_bfloat16*>(out);
   p.row_stats = row_stats;
   p.status = a.status;
-  if (a.head_dim == 128) {
-    if (!allow_dynamic_smem(attend_tc_kernel<128>, tc_smem_bytes<128>())) return -1;
-    launch_k(attend_tc_kernel<128>, grid, kThreadsTc, tc_smem_bytes<128>(), st, tm_q, tk, tv, tm_kn, tm_vn, tm_o, p);
-  } else {
-    if (!allow_dynamic_smem(attend_tc_kernel<64>, tc_smem_bytes<128>())) return -1;
-    // the larger request keeps it at one CTA per SM (the kernel owns all 512 TMEM columns)
-    launch_k(attend_tc_kernel<64>, grid, kThreadsTc, tc_smem_bytes<128>(), st, tm_q, tk, tv, tm_kn, tm_vn, tm_o, p);
-  }
-  return launched(1);
+  if (a.head_dim == 128) return launch_tc<128, 2>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, tm_o, p);
+  return halves ? launch_tc<64, 1>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, tm_o, p)
+                : launch_tc<64, 2>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, tm_o, p);
 }
 
 }  // namespace hack
