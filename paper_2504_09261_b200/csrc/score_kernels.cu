@@ -46,6 +46,25 @@ score_logits_kernel(const StepArgs a, const T* __restrict__ q, const T* __restri
       [&](int i) { return partials + (((size_t)bh * max_chunks + chunk) * kMaxObs + i) * 2; });
 }
 
+// Both passes in one launch of one cluster per head (PER: chunks per CTA, fp32 1).
+template <typename T, int D, int PER>
+__global__ void __launch_bounds__(simt::kFusedThreads)
+score_cluster_kernel(const StepArgs a, const T* __restrict__ q, const T* __restrict__ k_new, float* __restrict__ scores, int cl) {
+  pdl_wait();
+  const int bh = blockIdx.y;
+  const int ctx = a.is_ctx[bh % a.n_heads];
+  if (!a.trig[ctx]) return;                       // the whole cluster leaves together
+  const int stored = a.stored[ctx];
+  const T* kp = static_cast<const T*>(a.k_plane);
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  float* dst = scores + (size_t)bh * a.cand_stride;
+  auto obs = [&](int i) { return q + ((size_t)bh * a.n_new + obs_row(a, i)) * D; };
+  auto key = [&](int j) { return cand_row(a, kp, k_new, bh, stored, j); };
+  auto put = [&](int j, float s) { dst[j] = a.score_accumulate ? dst[j] + s : s; };
+  if constexpr (sizeof(T) == 4) simt::cluster_scores_f32<D>(smem_raw, cl, a.cand[ctx], a.n_obs_rows, a.sm_scale, obs, key, put);
+  else simt::cluster_scores_bf16<D, PER>(smem_raw, cl, a.cand[ctx], a.n_obs_rows, a.sm_scale, obs, key, put);
+}
+
 __global__ void __launch_bounds__(256)
 score_reduce_kernel(const StepArgs a, const float* __restrict__ logits,
                     const float* __restrict__ partials, int max_chunks, float* __restrict__ scores) {
@@ -73,6 +92,19 @@ int launch_score_t(const StepArgs& a, const void* q, const void* k_new, float* s
                    const Scratch& s, cudaStream_t st) {
   const int max_cand = a.cand[0] * a.trig[0] > a.cand[1] * a.trig[1] ? a.cand[0] : a.cand[1];
   const int bh = a.batch * a.n_heads;
+  int per = 0;
+  const int cl = simt::fused_cluster(max_cand, a.heads_of[0] * a.trig[0] + a.heads_of[1] * a.trig[1], sizeof(T) == 2, sm_count(), per);
+  if (cl > 0) {
+    auto go = [&](auto kern, size_t fused) {
+      if (!allow_dynamic_smem(kern, fused)) return -1;
+      simt::launch_cluster(kern, cl, bh, fused, st, a, static_cast<const T*>(q), static_cast<const T*>(k_new), scores, cl);
+      return launched(1);
+    };
+    if constexpr (sizeof(T) == 4) return go(score_cluster_kernel<T, D, 1>, simt::fused_f32_smem<D>());
+    else if (per == 1) return go(score_cluster_kernel<T, D, 1>, simt::fused_bf16_smem<D, 1>());
+    else if (per == 2) return go(score_cluster_kernel<T, D, 2>, simt::fused_bf16_smem<D, 2>());
+    else return go(score_cluster_kernel<T, D, 4>, simt::fused_bf16_smem<D, 4>());
+  }
   const size_t smem = simt::logits_smem_bytes<T, D>();
   if (!allow_dynamic_smem(score_logits_kernel<T, D>, smem)) return -1;
   dim3 g1((max_cand + kScoreChunk - 1) / kScoreChunk, bh);

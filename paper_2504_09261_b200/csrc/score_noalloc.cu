@@ -73,6 +73,21 @@ noalloc_reduce_kernel(const DenseArgs a, const float* __restrict__ logits,
     scores[(size_t)row * score_stride + blockIdx.x * 256 + threadIdx.x] = s;
 }
 
+// Both passes in one launch, no scratch (PER: chunks per CTA, fp32 1).
+template <typename T, int D, int PER>
+__global__ void __launch_bounds__(simt::kFusedThreads)
+noalloc_cluster_kernel(const DenseArgs a, const T* __restrict__ q, const T* __restrict__ k_cand, float* __restrict__ scores,
+                       int score_stride, int cl) {
+  pdl_wait();
+  const int row = blockIdx.y;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  auto obs = [&](int i) { return q + ((size_t)row * a.n_queries + (int)(((long long)i * a.n_queries) / a.n_obs_rows)) * D; };
+  auto key = [&](int j) { return k_cand + ((size_t)row * a.n_cand + j) * D; };
+  auto put = [&](int j, float s) { scores[(size_t)row * score_stride + j] = s; };
+  if constexpr (sizeof(T) == 4) simt::cluster_scores_f32<D>(smem_raw, cl, a.n_cand, a.n_obs_rows, a.sm_scale, obs, key, put);
+  else simt::cluster_scores_bf16<D, PER>(smem_raw, cl, a.n_cand, a.n_obs_rows, a.sm_scale, obs, key, put);
+}
+
 // One scratch address per device, resolved on the first call made with that device current.
 std::mutex g_setup_mutex;
 float* g_scratch_ptr[64] = {nullptr};
@@ -80,6 +95,19 @@ float* g_scratch_ptr[64] = {nullptr};
 template <typename T, int D>
 cudaError_t run(const DenseArgs& a, int n_rows, const void* q, const void* k, float* scratch,
                 float* scores, int score_stride, cudaStream_t st) {
+  int per = 0;
+  const int cl = simt::fused_cluster(a.n_cand, n_rows, sizeof(T) == 2, sm_count(), per);
+  if (cl > 0) {
+    auto go = [&](auto kern, size_t fused) {
+      if (!allow_dynamic_smem(kern, fused)) return cudaErrorInvalidValue;
+      simt::launch_cluster(kern, cl, n_rows, fused, st, a, static_cast<const T*>(q), static_cast<const T*>(k), scores, score_stride, cl);
+      return cudaGetLastError();
+    };
+    if constexpr (sizeof(T) == 4) return go(noalloc_cluster_kernel<T, D, 1>, simt::fused_f32_smem<D>());
+    else if (per == 1) return go(noalloc_cluster_kernel<T, D, 1>, simt::fused_bf16_smem<D, 1>());
+    else if (per == 2) return go(noalloc_cluster_kernel<T, D, 2>, simt::fused_bf16_smem<D, 2>());
+    else return go(noalloc_cluster_kernel<T, D, 4>, simt::fused_bf16_smem<D, 4>());
+  }
   const size_t smem = simt::logits_smem_bytes<T, D>();
   // opt-in to more than 48 KB of dynamic shared memory, once per (kernel, device)
   if (!allow_dynamic_smem(noalloc_logits_kernel<T, D>, smem)) return cudaErrorInvalidValue;

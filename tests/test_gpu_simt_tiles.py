@@ -52,11 +52,13 @@ def test_fp32_attention_over_ragged_tiles(sides, head_dim):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
-@pytest.mark.parametrize("n_cand,n_obs,head_dim", [(1, 1, 64), (127, 8, 128), (128, 31, 64), (129, 32, 128), (1153, 32, 64)])
+@pytest.mark.parametrize("n_cand,n_obs,head_dim", [(1, 1, 64), (127, 8, 128), (128, 31, 64), (129, 32, 128), (1153, 32, 64),
+                                                   (1100, 17, 128), (3000, 32, 64), (4096, 32, 128), (4097, 32, 128)])
 def test_dense_scores_over_ragged_chunks(n_cand, n_obs, head_dim, dtype):
-    """Chunks of 128 keys cut short, filled and exceeded by one; more chunks than the eight threads
-    that merge a row's statistics; observation rows that leave warps idle.  Bar as in the parity
-    tests of the scores: 1e-4 relative + 1e-7 (fp32 sums of at most 1153 terms)."""
+    """Chunks of 128 keys cut short, filled and exceeded by one; one, two and four chunks per CTA of a
+    cluster, clusters with idle CTAs, and the first size past one launch; observation rows that leave
+    warps idle.  Bar as in the parity tests of the scores: 1e-4 relative + 1e-7 (fp32 sums of at most
+    4097 terms)."""
     import torch
     import paper_2504_09261_b200 as hb
     rows, n_q = 3, 50
