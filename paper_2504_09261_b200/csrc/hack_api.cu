@@ -816,7 +816,11 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
   if (any && !compressed) {
     {
       StageScope ts(c, st, 0);
-      if ((r = hack::launch_score(a, c->cfg.dtype, q, k, c->scores, c->scratch, st)) < 0) return HACK_ERR_CUDA;   // text recorded by the launcher
+      // steps that need the scores in memory (the final-scale merge): still one cluster launch if it serves them
+      r = c->cfg.dtype == HACK_BF16 && boxes ? hack::launch_compress_cluster(a, q, k, nullptr, c->scores, st) : 0;
+      if (r > 0) r = 1;
+      if (r == 0) r = hack::launch_score(a, c->cfg.dtype, q, k, c->scores, c->scratch, st);
+      if (r < 0) return HACK_ERR_CUDA;   // text recorded by the launcher
       ts.done(r);
       n += r;
     }
