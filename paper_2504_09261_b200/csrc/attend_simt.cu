@@ -5,7 +5,9 @@
 // Bound: the FMA pipe.  A CTA serves 32 query rows of one head; its four groups of 64 threads walk
 // every fourth tile of 32 keys with a streaming softmax of their own and are merged at the end, so
 // that a launch with few query tiles (256 queries x 16 heads are 128 CTAs) still has eight warps per
-// SM at work.  Inside a group a thread forms 4 x 4 logits and 4 x D/8 outputs: eight 16-byte
+// SM at work.  With one CTA per SM the length of a launch is a matter of whole CTAs: the heads with
+// the longer cache go first, and clusters of 2 or 4 CTAs split the keys of a query tile further (merged
+// through distributed shared memory) where that evens out the last round.  Inside a group a thread forms 4 x 4 logits and 4 x D/8 outputs: eight 16-byte
 // shared-memory reads per 64 multiply-adds in Q K^T, twenty per 256 in P V, every read without bank
 // conflicts (rows are padded by 16 bytes; the lanes of a warp read 8 different rows or broadcast).
 // Both products run on packed pairs (fma.rn.f32x2).  The key buffer is refilled under the P V product
@@ -14,6 +16,8 @@
 // shared memory per 4 multiply-adds with a four-way bank conflict.  Decoding loop of two layers of 16
 // heads x 128, 2 240 tokens, stage calls: 13.8 -> 1.66 ms; one layer of 16 heads x 64, 680 tokens:
 // 0.531 -> 0.308 ms.)
+#include <algorithm>
+
 #include "hack_internal.h"
 #include "tc_ptx.cuh"
 
@@ -50,16 +54,19 @@ constexpr size_t simt_smem_bytes() {
   return sizeof(float) * ((size_t)kBQ * (D + 4) + kGroups * (2 * (size_t)kBK * (D + 4) + kBQ * (kBK + 4)));
 }
 
-template <int D>
-__global__ void __launch_bounds__(kThreads)
-attend_simt_kernel(const StepArgs a, const float* __restrict__ q, float* __restrict__ out) {
-  pdl_wait();
+template <int D, bool kCluster>
+__global__ void __launch_bounds__(kThreads, D == 64 && !kCluster ? 2 : 1)
+attend_simt_kernel(const StepArgs a, const float* __restrict__ q, float* __restrict__ out,
+                   const int32_t* __restrict__ order, int cluster) {
+  const int cl = kCluster ? cluster : 1;
   constexpr int LD = D + 4, LP = kBK + 4;
   constexpr int CV = D / 32;                      // float4 columns per thread
-  const int bh = blockIdx.y;
+  const int bh = order[blockIdx.y];               // tables written when the cache was created
+  const int rank = blockIdx.x % cl;
   const int len = a.kept[a.is_ctx[bh % a.n_heads]];
-  const int q0 = blockIdx.x * kBQ;
+  const int q0 = blockIdx.x / cl * kBQ;
   const int tid = threadIdx.x, grp = tid >> 6, gt = tid & 63;
+  const int first = rank * kGroups + grp, stride = cl * kGroups;   // key tiles of this group
   const int ty = gt >> 3, tx = gt & 7;            // rows ty + 8 i; keys tx + 8 j; columns 4 tx + 32 c
 
   extern __shared__ __align__(16) float smem[];
@@ -74,10 +81,11 @@ attend_simt_kernel(const StepArgs a, const float* __restrict__ q, float* __restr
 
   auto group_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory"); };
 
+  pdl_wait();
   stage_rows<D>(qs, q + ((size_t)bh * a.n_new + q0) * D, a.n_new - q0, tid, kThreads);
-  if (grp < n_tiles) stage_rows<D>(ks, kp + (size_t)grp * kBK * D, len - grp * kBK, gt, 64);
+  if (first < n_tiles) stage_rows<D>(ks, kp + (size_t)first * kBK * D, len - first * kBK, gt, 64);
   commit();
-  if (grp < n_tiles) stage_rows<D>(vs, vp + (size_t)grp * kBK * D, len - grp * kBK, gt, 64);
+  if (first < n_tiles) stage_rows<D>(vs, vp + (size_t)first * kBK * D, len - first * kBK, gt, 64);
   commit();
   wait_group<1>();
   __syncthreads();
@@ -92,7 +100,7 @@ attend_simt_kernel(const StepArgs a, const float* __restrict__ q, float* __restr
     for (int c = 0; c < CV; ++c) o[i][c][0] = o[i][c][1] = make_float2(0.f, 0.f);
   }
 
-  for (int t = grp; t < n_tiles; t += kGroups) {
+  for (int t = first; t < n_tiles; t += stride) {
     // logits: s[i][j] of query row ty + 8 i and key tx + 8 j, even and odd dimensions in the two halves
     float2 s[4][4];
 #pragma unroll
@@ -115,8 +123,8 @@ attend_simt_kernel(const StepArgs a, const float* __restrict__ q, float* __restr
         }
     }
     group_sync();                                 // both warps are done with the key tile
-    if (t + kGroups < n_tiles)
-      stage_rows<D>(ks, kp + (size_t)(t + kGroups) * kBK * D, len - (t + kGroups) * kBK, gt, 64);
+    if (t + stride < n_tiles)
+      stage_rows<D>(ks, kp + (size_t)(t + stride) * kBK * D, len - (t + stride) * kBK, gt, 64);
     commit();
 
     float corr[4];
@@ -175,16 +183,17 @@ attend_simt_kernel(const StepArgs a, const float* __restrict__ q, float* __restr
       }
     }
     group_sync();                                 // both warps are done with the value tile
-    if (t + kGroups < n_tiles)
-      stage_rows<D>(vs, vp + (size_t)(t + kGroups) * kBK * D, len - (t + kGroups) * kBK, gt, 64);
+    if (t + stride < n_tiles)
+      stage_rows<D>(vs, vp + (size_t)(t + stride) * kBK * D, len - (t + stride) * kBK, gt, 64);
     commit();
     wait_group<1>();                              // the next key tile has landed
     group_sync();
   }
   wait_group<0>();
 
-  // merge of the four groups: unnormalised outputs and (max, sum) of every row through shared memory
-  // (a group's own key tile holds its 32 x D outputs, its probability tile the row statistics)
+  // merge of the groups: unnormalised outputs and (max, sum) of every row through shared memory
+  // (a group's own key tile holds its 32 x D outputs, its probability tile the row statistics); the CTAs
+  // of a cluster each finish a share of the rows
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     float li = l[i];
@@ -197,43 +206,100 @@ attend_simt_kernel(const StepArgs a, const float* __restrict__ q, float* __restr
       *reinterpret_cast<float4*>(ks + (ty + 8 * i) * LD + 4 * tx + 32 * c) =
           make_float4(o[i][c][0].x, o[i][c][0].y, o[i][c][1].x, o[i][c][1].y);
   }
-  __syncthreads();
+  if (kCluster) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  else __syncthreads();
   constexpr int GSTRIDE = 2 * kBK * LD + kBQ * LP;
   const float* g0 = qs + kBQ * LD;
-  for (int v = tid; v < kBQ * (D / 4); v += kThreads) {
-    const int r = v / (D / 4), c = v % (D / 4);
+  const int rows = kBQ / cl;
+  for (int v = tid; v < rows * (D / 4); v += kThreads) {
+    const int r = rank * rows + v / (D / 4), c = v % (D / 4);
     if (q0 + r >= a.n_new) continue;
-    float2 st[kGroups];
-    float top = -INFINITY;
-#pragma unroll
-    for (int g = 0; g < kGroups; ++g) {
-      st[g] = *reinterpret_cast<const float2*>(g0 + g * GSTRIDE + 2 * kBK * LD + r * 2);
-      top = fmaxf(top, st[g].x);
-    }
-    float sum = 0.f;
+    float top = -INFINITY, sum = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int cta = 0; cta < cl; ++cta) {
+      uint32_t base = 0;
+      if (kCluster) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(base) : "r"(ptx::smem_u32(g0)), "r"(cta));
+      float2 st[kGroups];
+      float4 f[kGroups];
+      float mx = top;
 #pragma unroll
-    for (int g = 0; g < kGroups; ++g) {
-      const float w = expf(st[g].x - top);        // 0 for a group without keys
-      sum = fmaf(w, st[g].y, sum);
-      const float4 f = *reinterpret_cast<const float4*>(g0 + g * GSTRIDE + r * LD + c * 4);
-      acc.x = fmaf(w, f.x, acc.x);
-      acc.y = fmaf(w, f.y, acc.y);
-      acc.z = fmaf(w, f.z, acc.z);
-      acc.w = fmaf(w, f.w, acc.w);
+      for (int g = 0; g < kGroups; ++g) {
+        const int at_st = g * GSTRIDE + 2 * kBK * LD + r * 2, at_f = g * GSTRIDE + r * LD + c * 4;
+        if (kCluster) {
+          asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(st[g].x), "=f"(st[g].y) : "r"(base + 4u * at_st) : "memory");
+          asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                       : "=f"(f[g].x), "=f"(f[g].y), "=f"(f[g].z), "=f"(f[g].w) : "r"(base + 4u * at_f) : "memory");
+        } else {
+          st[g] = *reinterpret_cast<const float2*>(g0 + at_st);
+          f[g] = *reinterpret_cast<const float4*>(g0 + at_f);
+        }
+        mx = fmaxf(mx, st[g].x);
+      }
+      const float keep = expf(top - mx);          // 0 for the first CTA; every CTA before a later one has keys
+      top = mx;
+      sum *= keep;
+      acc.x *= keep; acc.y *= keep; acc.z *= keep; acc.w *= keep;
+#pragma unroll
+      for (int g = 0; g < kGroups; ++g) {
+        const float w = expf(st[g].x - top);      // 0 for a group without keys
+        sum = fmaf(w, st[g].y, sum);
+        acc.x = fmaf(w, f[g].x, acc.x);
+        acc.y = fmaf(w, f[g].y, acc.y);
+        acc.z = fmaf(w, f[g].z, acc.z);
+        acc.w = fmaf(w, f[g].w, acc.w);
+      }
     }
     const float inv = 1.f / sum;
     *reinterpret_cast<float4*>(out + ((size_t)bh * a.n_new + q0 + r) * D + c * 4) =
         make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
   }
+  // no CTA leaves while another may still read its shared memory
+  if (kCluster) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
 template <int D>
 int launch_t(const StepArgs& a, const void* q, void* out, cudaStream_t st) {
-  if (!allow_dynamic_smem(attend_simt_kernel<D>, simt_smem_bytes<D>())) return -1;
-  const dim3 grid((a.n_new + kBQ - 1) / kBQ, a.batch * a.n_heads);
-  launch_k(attend_simt_kernel<D>, grid, dim3(kThreads), simt_smem_bytes<D>(), st, a, static_cast<const float*>(q),
-           static_cast<float*>(out));
+  const int n_qt = (a.n_new + kBQ - 1) / kBQ, heads = a.batch * a.n_heads;
+  // Cluster size: the shortest estimate of the launch in key tiles of a group.  A CTA costs its share of
+  // the tiles and about three more (start, merge); a launch past one wave lasts as long as all of them
+  // spread over the SMs plus half of its longest CTA.  Steps of 16 heads x 100 queries x 64: 33.2 -> 30.8 us
+  // with two CTAs per query tile, 256 queries 49.5 -> 39.3; 324 queries x 128: 85 -> 75 by the order of the
+  // heads alone; 4 CTAs per tile 310 -> 464 where the launch is long anyway (1 024 queries, 1 717 keys).
+  const float sms = (float)sm_count();
+  int cl = 1;
+  float best = 0.f;
+  for (int c = 1; c <= 4; c *= 2) {
+    float total = 0.f, longest = 0.f;
+    for (int t = 0; t < 2; ++t) {
+      if (a.heads_of[t] == 0) continue;
+      const float one = 3.f + (float)(((a.kept[t] + kBK - 1) / kBK + c * kGroups - 1) / (c * kGroups));
+      total += one * a.heads_of[t] * n_qt * c;
+      longest = std::max(longest, one);
+    }
+    const float cost = n_qt * c * heads <= sms ? longest : std::max(longest, total / sms + 0.5f * longest);
+    if (c == 1 || cost < best) {
+      best = cost;
+      cl = c;
+    }
+  }
+  const int32_t* order = a.head_order + (a.kept[1] > a.kept[0] ? heads : 0);
+  auto kern = cl > 1 ? attend_simt_kernel<D, true> : attend_simt_kernel<D, false>;
+  if (!allow_dynamic_smem(kern, simt_smem_bytes<D>())) return -1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_qt * cl, heads);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = simt_smem_bytes<D>();
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cl;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cl > 1 ? 2 : 1;
+  cudaLaunchKernelEx(&cfg, kern, a, static_cast<const float*>(q), static_cast<float*>(out), order, cl);
   return launched(1);
 }
 

@@ -215,9 +215,8 @@ hack::StepArgs make_args(const hack_cache* c, int layer, int scale, const hack_s
   if (!c->k_maps.empty()) {
     a.k_map = &c->k_maps[layer];
     a.v_map = &c->v_maps[layer];
-    const int bh = c->cfg.batch * c->cfg.n_heads;
-    a.head_order = c->head_order + (size_t)layer * 2 * bh;
   }
+  a.head_order = c->head_order + (size_t)layer * 2 * c->cfg.batch * c->cfg.n_heads;
   return a;
 }
 
@@ -458,10 +457,9 @@ hack_status_t hack_init_cache(const hack_config_t* cfg, hack_cache_t** out) {
   HACK_TRY(cudaMalloc(&c->scratch.logits, (size_t)bh * hack::kMaxObs * c->limits.cand_stride * sizeof(float)));
   HACK_TRY(cudaMalloc(&c->scratch.partials, (size_t)bh * c->scratch.max_chunks * hack::kMaxObs * 2 * sizeof(float)));
   if (cfg->dtype == HACK_BF16) {
-    // tensor maps of every layer's planes and the two head orders of the tensor-core attention
+    // tensor maps of every layer's planes
     c->k_maps.resize(cfg->n_layers);
     c->v_maps.resize(cfg->n_layers);
-    std::vector<int32_t> order((size_t)cfg->n_layers * 2 * bh);
     for (int l = 0; l < cfg->n_layers; ++l) {
       const size_t rows = c->layer_rows[l] + (l + 1 == cfg->n_layers ? pad_rows : 0);
       if (!hack::make_rows_map(&c->k_maps[l], c->k_all + c->layer_row_base[l] * row_bytes, rows, cfg->head_dim) ||
@@ -469,6 +467,12 @@ hack_status_t hack_init_cache(const hack_config_t* cfg, hack_cache_t** out) {
         set_error("cuTensorMapEncodeTiled failed for a cache plane");
         return bail(HACK_ERR_CUDA);
       }
+    }
+  }
+  {
+    // the two head orders of the attention launches
+    std::vector<int32_t> order((size_t)cfg->n_layers * 2 * bh);
+    for (int l = 0; l < cfg->n_layers; ++l)
       for (int first = 0; first < 2; ++first) {
         int32_t* o = order.data() + ((size_t)l * 2 + first) * bh;
         int n = 0;
@@ -478,7 +482,6 @@ hack_status_t hack_init_cache(const hack_config_t* cfg, hack_cache_t** out) {
             if ((pass == 0) == (t == first)) o[n++] = i;
           }
       }
-    }
     HACK_TRY(cudaMalloc(&c->head_order, order.size() * sizeof(int32_t)));
     HACK_TRY(cudaMemcpy(c->head_order, order.data(), order.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
   }
