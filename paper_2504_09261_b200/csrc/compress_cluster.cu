@@ -23,8 +23,10 @@
 //      histogram of its own keys (the first one while it forms them) and publishes it in groups of 16
 //      bins; after a cluster barrier a thread adds one group over the cluster (4 bytes per CTA instead
 //      of 32), and one warp reads the bins of the group that holds the wanted rank, which also gives
-//      every CTA's counts and so its offset in the head's index list.  The select stops once all
-//      entries left in the located bin survive.  Ties at the threshold go to the lowest indices.
+//      every CTA's counts and so its offset in the head's index list.  Once at most kBinMax entries are
+//      left in the located bin they are ranked by comparison (a digit costs 1.3-2 us, the heads of a
+//      launch need one to three of them, and the slowest head sets its time).  The select stops early if
+//      all entries left survive.  Ties at the threshold go to the lowest indices.
 //   5. ascending index list by ballot counts; every entry goes straight into the shared memory of the
 //      CTA that will move it (the list never touches global memory).
 //   6. compaction in rounds: entry o of the list becomes row o of the head.  In a round every CTA
@@ -74,6 +76,7 @@ constexpr uint32_t kCkDrainSpins = 1u << 22;
 constexpr int kMaxStages = 4;              // key tiles in flight per CTA (deeper rings measured no faster)
 constexpr int kHistBins = 4096;            // bins of a 12-bit digit of the radix select
 constexpr int kHistWords = kHistBins / 2;  // 16-bit counters, two per word
+constexpr int kBinMax = 256;               // entries of the located bin that are ranked by comparison
 constexpr int kMaxStageRows = 512;         // rows (K and V) in a CTA's staging buffers of the compaction
 constexpr int kMoveBuffers = 3;            // staging buffers of the compaction: loads run two rounds ahead of the stores
 constexpr size_t kSmemBudget = 227 * 1024; // dynamic shared memory a CTA may ask for ...
@@ -81,6 +84,7 @@ constexpr size_t kSmemShared = 112 * 1024; // ... and half an SM's, for two CTAs
 constexpr float kLazyMax = 16.0f;          // log2 units a logit may exceed a thread's reference maximum
 static_assert(kHistBins == 16 * kWorkers, "a worker sums 16 bins of a histogram");
 static_assert(kMaxCpc * kCkChunk < 65536, "16-bit counters per CTA");
+static_assert(kBinMax < kCkThreads && 4 * (kBinMax + 1) <= kHistWords, "a thread per entry, two lists in a histogram's place");
 
 struct CkParams {
   int cluster;                // CTAs per head
@@ -107,6 +111,7 @@ struct CkShared {
   int abort_flag;
   int pub_abort;                              // read by the other CTAs of the cluster
   int digit, need_in_bin, bin_count;          // the located digit, the rank left inside its bin, the bin's count
+  int bin_n, bin_gt;                          // this CTA's entries in the located bin; the head's above the threshold there
   int cnt_gt[kMaxCluster], cnt_eq[kMaxCluster];   // per CTA: keys above the threshold, keys in the located bin
   int warp_sums[2][kCkWarps + 3];
   float2 pub_stats[4][kMaxObs];               // per lane quadrant (max, sum-exp) of every observation row; read by the cluster
@@ -145,6 +150,11 @@ __device__ __forceinline__ int ld_peer_i32(uint32_t addr) {
 __device__ __forceinline__ float2 ld_peer_f2(uint32_t addr) {
   float2 v;
   asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ unsigned long long ld_peer_u64(uint32_t addr) {
+  unsigned long long v;
+  asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
   return v;
 }
 __device__ __forceinline__ void st_peer_i32(uint32_t addr, int v) {
@@ -556,6 +566,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
     uint32_t prefix = 0, mask = 0;
     int need = n_rows;
     if (tid < CL) sh->cnt_gt[tid] = 0;
+    if (tid == 0) { sh->bin_n = 0; sh->bin_gt = 0; }
 #pragma unroll 1
     for (int pass = 0; pass < 3; ++pass) {
       const int shift = pass == 0 ? 20 : (pass == 1 ? 8 : 0);
@@ -661,7 +672,52 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
       prefix |= (uint32_t)sh->digit << shift;
       need = sh->need_in_bin;
       mask |= dmask << shift;
-      if (need == sh->bin_count) break;                       // the same in every CTA of the cluster
+      const int m = sh->bin_count;
+      if (need == m) break;                                   // the same in every CTA of the cluster
+      if (m <= kBinMax) {
+        // Few entries left: they are ranked by comparing each with all of them.  An entry is its key and,
+        // below it, its complemented index, so that among equals the lowest index ranks first.
+        unsigned long long* own = reinterpret_cast<unsigned long long*>(hist32 + ((pass & 1) ^ 1) * kHistWords);
+        unsigned long long* all = own + kBinMax;
+        for (int slot = tid; slot < n_slots; slot += kCkThreads) {
+          int j;
+          const uint32_t k = keys[slot];
+          if ((k & mask) == prefix && slot_info(slot, j)) own[atomicAdd(&sh->bin_n, 1)] = (unsigned long long)k << 32 | (uint32_t)~j;
+        }
+        cluster_sync(CL);
+        unsigned long long mine_e = 0;
+        int r = 0;                                            // the CTA that holds this thread's entry
+        if (tid < m) {
+          int e = tid;
+          while (e >= sh->cnt_eq[r]) e -= sh->cnt_eq[r++];
+          mine_e = CL == 1 ? own[e] : ld_peer_u64(peer_addr(&own[e], r));
+          all[tid] = mine_e;
+        } else if (tid == m) {
+          all[tid] = 0;                                       // the last pair may read one past the end
+        }
+        __syncthreads();
+        if (tid < CL) sh->cnt_eq[tid] = 0;
+        int before = 0;
+        if (tid < m) {
+#pragma unroll 4
+          for (int i = 0; i < m; i += 2) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(all + i);
+            before += (v.x > mine_e) + (v.y > mine_e);
+          }
+          if (before == need - 1) sh->digit = (int)(mine_e >> 32);
+        }
+        __syncthreads();
+        prefix = (uint32_t)sh->digit;
+        mask = 0xffffffffu;
+        if (tid < m) {
+          const uint32_t k = (uint32_t)(mine_e >> 32);
+          if (k > prefix) { atomicAdd(&sh->cnt_gt[r], 1); atomicAdd(&sh->bin_gt, 1); }
+          if (k == prefix) atomicAdd(&sh->cnt_eq[r], 1);
+        }
+        __syncthreads();
+        need -= sh->bin_gt;
+        break;
+      }
       __syncthreads();                                        // before the next pass writes what was just read
     }
     // ---------------------------------------------------------------- 5. ascending index list
