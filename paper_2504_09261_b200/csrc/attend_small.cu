@@ -9,6 +9,8 @@
 // value rows are read coalesced.  Keys below the stored length come from the cache planes, the
 // others straight from the caller's K/V tensors, so nothing depends on the append, which the
 // same CTAs perform afterwards on cache rows no one reads in this launch.
+#include <algorithm>
+
 #include "hack_internal.h"
 #include "tc_ptx.cuh"
 
@@ -147,9 +149,9 @@ append_attend_small_kernel(const StepArgs a, const T* __restrict__ q, const T* _
 
 // ------------------------------------------------------------------ bf16 caches
 // A CTA serves 16 queries of one head with warp-level matrix instructions (mma.m16n8k16; a 128-row
-// tcgen05 tile would be at most a quarter full here).  Its four warps take the keys in turns of 16 with
-// a streaming softmax of their own and are merged at the end, so that up to 64 keys are one trip to
-// memory: a warp fetches its 16 key and value rows (and the first time the queries) with cp.async,
+// tcgen05 tile would be at most a quarter full here).  Its W warps take the keys in turns of 16 with
+// a streaming softmax of their own and are merged at the end, so that up to 64 keys (W = 4; 128 with
+// eight warps, launches of few CTAs) are one trip to memory: a warp fetches its 16 key and value rows (and the first time the queries) with cp.async,
 // all of them in flight at once, and everything after that is registers and shared memory.  New rows
 // go from there to the cache as well.  The probabilities enter the second product as a sum of two
 // bf16 numbers (error 2^-17), so they are as good as the fp32 ones of a SIMT kernel.
@@ -158,7 +160,6 @@ append_attend_small_kernel(const StepArgs a, const T* __restrict__ q, const T* _
 // queries and 55 keys, 256 heads x 64: 5.4 us; 16 queries, 30 keys, 240 heads x 64: 3.4 us;
 // 16 queries, 21 keys, 32 heads x 128: 3.6 us (one warp per query row on the CUDA cores:
 // 27.5, 10.5 and 5.5 us).
-constexpr int kMmaWarps = 4;
 constexpr int kMmaRows = 16;                    // queries per CTA, keys per warp and turn
 
 // Two fp32 numbers as a sum of two packed pairs of bf16.
@@ -169,16 +170,21 @@ __device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint3
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-template <int D>
-__global__ void __launch_bounds__(kMmaWarps * 32)
+template <int D, int W>
+constexpr size_t mma_smem_bytes() {
+  // queries, then per warp a key and a value tile; the warp's two tiles later hold its 16 x D outputs
+  return (size_t)kMmaRows * D * 2 * (1 + 2 * W);
+}
+
+template <int D, int W>
+__global__ void __launch_bounds__(W * 32)
 append_attend_mma_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k_new,
                          const __nv_bfloat16* __restrict__ v_new, __nv_bfloat16* __restrict__ out, int after_compression) {
   constexpr int PIECES = D / 8;                 // 16-byte pieces per row
   constexpr uint32_t ROWB = D * 2;
   constexpr uint32_t TILE = kMmaRows * ROWB;    // 16 rows
-  // queries, then per warp a key and a value tile; the warp's two tiles later hold its 16 x D outputs
-  __shared__ __align__(128) unsigned char sm[TILE + kMmaWarps * 2 * TILE];
-  __shared__ float2 row_ml[kMmaWarps][kMmaRows];
+  extern __shared__ __align__(128) unsigned char sm[];
+  __shared__ float2 row_ml[W][kMmaRows];
 
   const int bh = blockIdx.y, q0 = blockIdx.x * kMmaRows;
   const int ctx = a.is_ctx[bh % a.n_heads];     // written when the cache was created, like row_off
@@ -203,8 +209,8 @@ append_attend_mma_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, 
 
   // rows past the last query or key repeat the last one: their results are not stored or weigh nothing
 #pragma unroll
-  for (int i = 0; i < kMmaRows * PIECES / (kMmaWarps * 32); ++i) {
-    const int v = tid + i * kMmaWarps * 32, r = v / PIECES, c = v % PIECES;
+  for (int v = tid; v < kMmaRows * PIECES; v += W * 32) {
+    const int r = v / PIECES, c = v % PIECES;
     fetch(q_sm + at(r, c), qn + (size_t)min(q0 + r, a.n_new - 1) * D + c * 8);
   }
   const bool appends = blockIdx.x == 0 && total > stored && dbg_ok(total <= a.cap[ctx], a.status, 6);
@@ -215,9 +221,9 @@ append_attend_mma_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, 
   for (int n = 0; n < D / 8; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
   uint32_t qa[D / 16][4];
 
-  const int turns = (total + kMmaWarps * kMmaRows - 1) / (kMmaWarps * kMmaRows);
+  const int turns = (total + W * kMmaRows - 1) / (W * kMmaRows);
   for (int t = 0; t < turns; ++t) {
-    const int j0 = (t * kMmaWarps + warp) * kMmaRows;
+    const int j0 = (t * W + warp) * kMmaRows;
     const bool any = j0 < total;
     if (any) {
 #pragma unroll
@@ -305,7 +311,7 @@ append_attend_mma_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, 
     __syncwarp();                               // the tiles are refilled, or hold the outputs below
   }
 
-  // merge of the four warps: unnormalised outputs in the warp's own tiles (pairs of columns spread over
+  // merge of the warps: unnormalised outputs in the warp's own tiles (pairs of columns spread over
   // the banks), (max, sum) of every row beside them
   const int g = lane >> 2;
   float* ob = reinterpret_cast<float*>(sm + TILE + warp * 2 * TILE);
@@ -323,18 +329,18 @@ append_attend_mma_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, 
   }
   __syncthreads();
 #pragma unroll
-  for (int i = 0; i < kMmaRows * PIECES / (kMmaWarps * 32); ++i) {
-    const int v = tid + i * kMmaWarps * 32, r = v / PIECES, c = v % PIECES;
-    float2 ml[kMmaWarps];
+  for (int v = tid; v < kMmaRows * PIECES; v += W * 32) {
+    const int r = v / PIECES, c = v % PIECES;
+    float2 ml[W];
     float top = -INFINITY;
 #pragma unroll
-    for (int w = 0; w < kMmaWarps; ++w) {
+    for (int w = 0; w < W; ++w) {
       ml[w] = row_ml[w][r];
       top = fmaxf(top, ml[w].x);
     }
     float sum = 0.f, acc[8] = {};
 #pragma unroll
-    for (int w = 0; w < kMmaWarps; ++w) {
+    for (int w = 0; w < W; ++w) {
       const float wt = exp2f(ml[w].x - top);    // 0 for a warp without keys
       sum = fmaf(wt, ml[w].y, sum);
       const float* src = reinterpret_cast<const float*>(sm + TILE + w * 2 * TILE) + r * D;
@@ -372,8 +378,8 @@ bool attend_small_serves(const StepArgs& a) {
   const int heads = a.batch * a.n_heads, keys = a.kept[0] > a.kept[1] ? a.kept[0] : a.kept[1];
   const float sms = (float)sm_count();
   const int ctas = heads * ((a.n_new + kMmaRows - 1) / kMmaRows);
-  const int turns = (keys + kMmaWarps * kMmaRows - 1) / (kMmaWarps * kMmaRows);
-  const float load = turns * (ctas > sms ? ctas / sms : 1.f);
+  const int turns = (keys + 4 * kMmaRows - 1) / (4 * kMmaRows);
+  const float load = ctas <= sms ? (turns + 1) / 2 : turns * (ctas / sms);
   const int tiles = heads * ((a.n_new + 127) / 128);
   const int waves = (tiles + sm_count() - 1) / sm_count();
   return 2.f + (a.head_dim == 128 ? 1.75f : 0.72f) * load < waves * (5.5f + 0.9f * ((keys + 127) / 128));
@@ -391,13 +397,22 @@ int launch_attend_small(const StepArgs& a, int dtype, const void* q, const void*
     if (a.head_dim == 64) launch_k(append_attend_small_kernel<float, 64>, grid, block, 0, st, a, qp, kp, vp, op);
     else launch_k(append_attend_small_kernel<float, 128>, grid, block, 0, st, a, qp, kp, vp, op);
   } else {
-    const dim3 grid((a.n_new + kMmaRows - 1) / kMmaRows, heads), block(kMmaWarps * 32);
+    const dim3 grid((a.n_new + kMmaRows - 1) / kMmaRows, heads);
     const __nv_bfloat16* qp = static_cast<const __nv_bfloat16*>(q);
     const __nv_bfloat16* kp = static_cast<const __nv_bfloat16*>(k_new);
     const __nv_bfloat16* vp = static_cast<const __nv_bfloat16*>(v_new);
     __nv_bfloat16* op = static_cast<__nv_bfloat16*>(out);
-    if (a.head_dim == 64) launch_k(append_attend_mma_kernel<64>, grid, block, 0, st, a, qp, kp, vp, op, (int)after_compression);
-    else launch_k(append_attend_mma_kernel<128>, grid, block, 0, st, a, qp, kp, vp, op, (int)after_compression);
+    auto go = [&](auto kern, int warps, size_t smem) {
+      if (!allow_dynamic_smem(kern, smem)) return -1;
+      launch_k(kern, grid, dim3(warps * 32), smem, st, a, qp, kp, vp, op, (int)after_compression);
+      return launched(1);
+    };
+    // eight warps once a CTA of four would need a second trip to memory, while that leaves every CTA an SM
+    // (64 queries, 121 keys, 32 heads x 128: 5.6 -> 5.4 us; 240 heads x 64, 36 queries, 66 keys: 9.0 -> 11.6)
+    const bool wide = std::max(a.kept[0], a.kept[1]) > 4 * kMmaRows && (int)(grid.x * grid.y) <= sm_count();
+    if (a.head_dim == 64)
+      return wide ? go(append_attend_mma_kernel<64, 8>, 8, mma_smem_bytes<64, 8>()) : go(append_attend_mma_kernel<64, 4>, 4, mma_smem_bytes<64, 4>());
+    return wide ? go(append_attend_mma_kernel<128, 8>, 8, mma_smem_bytes<128, 8>()) : go(append_attend_mma_kernel<128, 4>, 4, mma_smem_bytes<128, 4>());
   }
   return launched(1);
 }
