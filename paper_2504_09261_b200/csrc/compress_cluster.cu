@@ -9,8 +9,9 @@
 //
 //   1. scores, pass 1: each CTA streams its chunks through a TMA ring and forms their logits
 //      against the (at most 32) observation rows with tcgen05.mma, as score_tc.cu does, but every
-//      chunk keeps its own accumulator [128 lanes x 32 columns] in tensor memory (the ones that do not
-//      fit take turns on two bounce accumulators and go to shared memory if they are read again).
+//      chunk keeps its own accumulator [128 lanes x 32 columns] in tensor memory.  The ones that do not
+//      fit take turns on two bounce accumulators; the logits of ranked chunks among them go to shared
+//      memory, or, past that, are formed a second time in pass 2.
 //      Thread r of a consumer set owns key r of a chunk and keeps (reference maximum, sum-exp) of half
 //      of the softmax rows; the 32 keys of a warp are merged by exchanging halves between lanes.
 //   2. the CTAs publish their row statistics in shared memory; after a cluster barrier every CTA
@@ -69,8 +70,7 @@ constexpr int kIssueWarp = kWorkers / 32;
 constexpr int kCkChunk = 128;
 constexpr int kHalfObs = kMaxObs / 2;      // observation rows a consumer set takes in pass 1
 constexpr int kMaxSlots = 16;              // accumulators of 32 columns in 512 columns of tensor memory
-constexpr int kMaxOver = 7;                // chunks per CTA whose logits live in shared memory
-constexpr int kMaxCpc = 40;                // chunks per CTA
+constexpr int kMaxSeq = 80;                // products per CTA: its chunks, and those formed a second time
 constexpr int kMaxCluster = 8;
 constexpr uint32_t kCkDrainSpins = 1u << 22;
 constexpr int kMaxStages = 4;              // key tiles in flight per CTA (deeper rings measured no faster)
@@ -83,7 +83,7 @@ constexpr size_t kSmemBudget = 227 * 1024; // dynamic shared memory a CTA may as
 constexpr size_t kSmemShared = 112 * 1024; // ... and half an SM's, for two CTAs per SM
 constexpr float kLazyMax = 16.0f;          // log2 units a logit may exceed a thread's reference maximum
 static_assert(kHistBins == 16 * kWorkers, "a worker sums 16 bins of a histogram");
-static_assert(kMaxCpc * kCkChunk < 65536, "16-bit counters per CTA");
+static_assert(kMaxSeq * kCkChunk < 65536, "16-bit counters per CTA");
 static_assert(kBinMax < kCkThreads && 4 * (kBinMax + 1) <= kHistWords, "a thread per entry, two lists in a histogram's place");
 
 struct CkParams {
@@ -92,9 +92,9 @@ struct CkParams {
   int cpc_max;                // most chunks of any CTA
   int slots;                  // accumulators in tensor memory
   int direct;                 // chunks with an accumulator of their own; the others share the last two
-  int n_over;                 // chunks of shared-memory logits reserved per CTA
+  int n_over;                 // ranked chunks past the direct ones whose logits stay in shared memory; those of the rest are formed again
   int stages;                 // key tiles in the TMA ring (2 .. kMaxStages)
-  int region_bytes;           // front region of shared memory: ring, observation rows, overflow logits; later the row staging
+  int region_bytes;           // front region of shared memory: ring, observation rows, overflow logits, histograms; later the row staging
   int stage_rows;             // rows (K and V) a CTA stages in shared memory per round of the compaction
   int score_only;             // stop after the scores
   float* scores;              // [b*H, cand_stride] or nullptr
@@ -104,7 +104,7 @@ struct CkParams {
 
 struct CkShared {
   uint64_t full[kMaxStages], empty[kMaxStages];
-  uint64_t acc_full[kMaxCpc];
+  uint64_t acc_full[kMaxSeq];
   uint64_t acc_free[2];
   uint64_t drain;
   uint32_t tmem_base;
@@ -156,6 +156,9 @@ __device__ __forceinline__ unsigned long long ld_peer_u64(uint32_t addr) {
   unsigned long long v;
   asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
   return v;
+}
+__device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
 }
 __device__ __forceinline__ void st_peer_i32(uint32_t addr, int v) {
   asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
@@ -238,7 +241,9 @@ __device__ __forceinline__ int ck_block_scan(int v, int* sums, int& total) {
   return ck_warp_prefix(__shfl_sync(0xffffffffu, incl, 31), sums, total) + incl - v;
 }
 
-template <int D>
+// kAgain: some CTA holds ranked chunks whose logits are formed a second time (a form of its own: the code
+// for it costs a launch of few chunks 0.3 us).
+template <int D, bool kAgain>
 __global__ void __launch_bounds__(kCkThreads, 2)
 compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __grid_constant__ CUtensorMap tm_new,
                         const StepArgs a, const __nv_bfloat16* __restrict__ q, const CkParams p) {
@@ -247,7 +252,6 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   constexpr uint32_t Q_SUB_BYTES = kMaxObs * 128;
   constexpr uint32_t K_BYTES = SUB * K_SUB_BYTES;
   constexpr int PIECES = D * 2 / 16;                      // 16-byte pieces per row
-  static_assert(2 * K_BYTES >= 2 * kHistWords * sizeof(uint32_t), "two ring stages hold the histograms");
   const int STAGES = p.stages;
   const uint32_t RING_BYTES = (uint32_t)STAGES * K_BYTES;
 
@@ -273,6 +277,11 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   const int c_begin = rank * cpr, t_begin = rank * cpt;
   const int n_p = max(0, min(cpr, n_ranked - c_begin));
   const int n_run = n_p + (drop_new ? max(0, min(cpt, n_nc - t_begin)) : 0);      // <= p.cpc_max
+  // Ranked chunks whose logits are kept: with an accumulator of their own, then in shared memory.  The
+  // others go through the ring and the tensor pipe a second time once the statistics are known: product
+  // number n_run + x is chunk n_held + x.
+  const int n_held = kAgain ? min(n_p, p.direct + p.n_over) : n_p, n_seq = n_run + n_p - n_held;
+  auto chunk_of = [&](int seq) { return !kAgain || seq < n_run ? seq : n_held + seq - n_run; };
   const float zscale = a.sm_scale * 1.4426950408889634f;  // logits in log2 units
   const long long wlim = a.wait_cycles;
 
@@ -283,12 +292,12 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   const uint32_t k_sm = base;
   const uint32_t q_sm = base + RING_BYTES;
   float* over = reinterpret_cast<float*>(sm + RING_BYTES + SUB * Q_SUB_BYTES);            // [n_over][32][128]
+  uint32_t* hist32 = reinterpret_cast<uint32_t*>(over + (size_t)p.n_over * kMaxObs * kCkChunk);   // [2][kHistWords]
   const int S_ROWS = p.stage_rows;                          // rows a CTA holds in its staging buffers
   uint32_t* keys = reinterpret_cast<uint32_t*>(sm + p.region_bytes);                            // [p_max * 128]
   int32_t* pos_stage = reinterpret_cast<int32_t*>(keys + (size_t)p.p_max * kCkChunk);          // [S_ROWS]
   int32_t* src_all = pos_stage + S_ROWS;                    // [p_max * 128 + S_ROWS]: this CTA's list entries of every round
   CkShared* sh = reinterpret_cast<CkShared*>(src_all + (size_t)p.p_max * kCkChunk + S_ROWS);
-  uint32_t* hist32 = reinterpret_cast<uint32_t*>(sm);     // [2][kHistWords], reuses the ring once it is idle
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -309,7 +318,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   int issued = 0;                                           // issuing thread: key tiles on their way
   auto load_tile = [&](int i) {
     bool from_cache;
-    const int part = chunk_part(i, from_cache);
+    const int part = chunk_part(chunk_of(i), from_cache);
     const CUtensorMap* tm = from_cache ? &tm_cache : &tm_new;
     const int row = (from_cache ? a.row_off[bh] : bh * n_new) + part * kCkChunk;
     const int s = i % STAGES;
@@ -321,7 +330,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   };
   if (warp == kIssueWarp && lane == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(smem_u32(&sh->full[s]), 1); mbar_init(smem_u32(&sh->empty[s]), 1); }
-    for (int i = 0; i < n_run; ++i) mbar_init(smem_u32(&sh->acc_full[i]), 1);
+    for (int i = 0; i < n_seq; ++i) mbar_init(smem_u32(&sh->acc_full[i]), 1);
     mbar_init(smem_u32(&sh->acc_free[0]), kWorkers);
     mbar_init(smem_u32(&sh->acc_free[1]), kWorkers);
     mbar_init(smem_u32(&sh->drain), 1);
@@ -341,7 +350,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   if (warp == kIssueWarp) {
     // the first key tiles are on their way while the other warps fetch the observation rows
     if (lane == 0)
-      for (int i = 0; i < min(STAGES, n_run); ++i) load_tile(i);
+      for (int i = 0; i < min(STAGES, n_seq); ++i) load_tile(i);
     __syncwarp();
   } else {
     // observation rows into the swizzled B tile; unused rows are zero
@@ -366,18 +375,18 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   const uint32_t t_lane = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
   // Chunks past the `direct` ones take turns on the last two accumulators.
   auto acc_slot = [&](int i) { return i < p.direct ? i : p.slots - 2 + ((i - p.direct) & 1); };
-  if (warp == kIssueWarp) {
-    if (lane == 0) {
-      constexpr uint32_t IDESC = idesc_bf16_f32(kCkChunk, kMaxObs, 0);
-      const uint64_t q_desc = smem_desc_sw128(q_sm, 16, 1024);
-      bool ok = true;
-      for (int i = 0; i < n_run && ok; ++i) {
-        const int s = i % STAGES;
-        ok = ck_wait(&sh->full[s], (i / STAGES) & 1, sh, a.status, 52, wlim);
-        // a shared accumulator is free again once all consumers have read the chunk before
-        if (ok && i >= p.direct)
-          ok = ck_wait(&sh->acc_free[(i - p.direct) & 1], (((i - p.direct) >> 1) & 1) ^ 1, sh, a.status, 53, wlim);
-        if (!ok) break;
+  // Products [from, to) (issuing thread).
+  bool issue_ok = true;
+  auto issue = [&](int from, int to) {
+    constexpr uint32_t IDESC = idesc_bf16_f32(kCkChunk, kMaxObs, 0);
+    const uint64_t q_desc = smem_desc_sw128(q_sm, 16, 1024);
+    for (int i = from; i < to && issue_ok; ++i) {
+      const int s = i % STAGES;
+      bool ok = ck_wait(&sh->full[s], (i / STAGES) & 1, sh, a.status, 52, wlim);
+      // a shared accumulator is free again once all consumers have read the chunk before
+      if (ok && i >= p.direct)
+        ok = ck_wait(&sh->acc_free[(i - p.direct) & 1], (((i - p.direct) >> 1) & 1) ^ 1, sh, a.status, 53, wlim);
+      if (ok) {
         tc_fence_after();
         const uint64_t k_desc = smem_desc_sw128(k_sm + s * K_BYTES, 16, 1024);
         const uint32_t acc = tmem + acc_slot(i) * kMaxObs;
@@ -387,20 +396,27 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
         mma_commit(smem_u32(&sh->acc_full[i]));
         // the tile of the product before this one is free: refill its stage
         const int f = i - 1 + STAGES;
-        if (i > 0 && f < n_run) {
+        if (i > 0 && f < n_seq) {
           ok = ck_wait(&sh->empty[f % STAGES], (f / STAGES - 1) & 1, sh, a.status, 51, wlim);
           if (ok) load_tile(f);
         }
       }
-      if (!ok) {
-        // what is in flight gets a bounded chance to finish before the ring is reused
-        mma_commit(smem_u32(&sh->drain));
-        for (uint32_t it = 0; it < kCkDrainSpins && !mbar_try_wait(smem_u32(&sh->drain), 0); ++it) {}
-        for (int i = max(0, issued - STAGES); i < issued; ++i) {
-          const uint32_t bar = smem_u32(&sh->full[i % STAGES]);
-          for (uint32_t it = 0; it < kCkDrainSpins && !mbar_try_wait(bar, (i / STAGES) & 1); ++it) {}
-        }
-      }
+      issue_ok = ok;
+    }
+  };
+  // After a wait that gave up: what is in flight gets a bounded chance to finish before the ring is reused.
+  auto drain = [&]() {
+    mma_commit(smem_u32(&sh->drain));
+    for (uint32_t it = 0; it < kCkDrainSpins && !mbar_try_wait(smem_u32(&sh->drain), 0); ++it) {}
+    for (int i = max(0, issued - STAGES); i < issued; ++i) {
+      const uint32_t bar = smem_u32(&sh->full[i % STAGES]);
+      for (uint32_t it = 0; it < kCkDrainSpins && !mbar_try_wait(bar, (i / STAGES) & 1); ++it) {}
+    }
+  };
+  if (warp == kIssueWarp) {
+    if (lane == 0) {
+      issue(0, n_run);
+      if (!issue_ok) drain();
     }
     __syncwarp();
   } else {
@@ -422,7 +438,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
       if (i >= p.direct) {
         tc_fence_before();
         mbar_arrive(smem_u32(&sh->acc_free[(i - p.direct) & 1]));
-        if (i < n_p) {
+        if (i < n_held) {
           float* dst = over + ((size_t)(i - p.direct) * kMaxObs + set * kHalfObs) * kCkChunk + key_row;
 #pragma unroll
           for (int r = 0; r < kHalfObs; ++r) dst[r * kCkChunk] = __uint_as_float(acc[r]);
@@ -478,7 +494,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   }
   __syncthreads();
   if (tid == 0) sh->pub_abort = *reinterpret_cast<volatile int*>(&sh->abort_flag);
-  // the ring is idle from here on; its first 16 KB become the two histograms of the radix select
+  // the two histograms of the radix select
   if (tid < kWorkers) {
     uint4* z = reinterpret_cast<uint4*>(hist32 + 8 * tid);
     z[0] = z[1] = make_uint4(0, 0, 0, 0);
@@ -513,16 +529,35 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   const bool select = !aborted && !p.score_only && n_rows > 0;
 
   // ------------------------------------------------------------------ 3. scores, pass 2
-  if (!aborted && tid < kWorkers) {
+  if (kAgain && warp == kIssueWarp) {
+    if (lane == 0 && issue_ok) {
+      // (tiles of the second products may be on their way already)
+      if (!aborted) issue(n_run, n_seq);
+      if (aborted || !issue_ok) drain();
+    }
+    __syncwarp();
+  } else if (!aborted && warp != kIssueWarp) {
     const bool structural = ctx == 0;
+    bool ok = true;
     for (int i = set; i < n_p; i += 2) {                    // a set takes every other chunk here
+      const bool again = kAgain && i >= n_held;
+      const int seq = n_run + i - n_held;                   // the product that forms this chunk a second time
+      if (again) {
+        ok = __all_sync(0xffffffffu, ck_wait(&sh->acc_full[seq], 0, sh, a.status, 55, wlim)) && ok;
+        tc_fence_after();
+      }
       float s = 0.f;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         uint32_t acc[kHalfObs];
-        if (i < p.direct) {
-          tmem_ld16(t_lane + i * kMaxObs + h * kHalfObs, acc);
+        if (i < p.direct || again) {
+          tmem_ld16(t_lane + (again ? acc_slot(seq) : i) * kMaxObs + h * kHalfObs, acc);
           tmem_wait_ld();
+          if (again && h == 1) {
+            // the accumulator counts a release by every worker; the 128 of this set stand for all of them
+            tc_fence_before();
+            mbar_arrive_n(smem_u32(&sh->acc_free[(seq - p.direct) & 1]), kWorkers / 128);
+          }
         } else {
           const float* src = over + ((size_t)(i - p.direct) * kMaxObs + h * kHalfObs) * kCkChunk + key_row;
 #pragma unroll
@@ -880,11 +915,16 @@ template <int D>
 bool ck_size(CkParams& p, size_t budget) {
   const size_t k_bytes = (size_t)(D / 64) * kCkChunk * 128;
   const size_t row_bytes = 2 * (size_t)D * 2;                // a key row and a value row
-  const size_t q_over = (size_t)(D / 64) * kMaxObs * 128 + (size_t)p.n_over * kMaxObs * kCkChunk * sizeof(float);
+  const size_t over_bytes = (size_t)kMaxObs * kCkChunk * sizeof(float);
+  const size_t q_hist = (size_t)(D / 64) * kMaxObs * 128 + 2 * kHistWords * sizeof(uint32_t);
   p.stage_rows = kMaxStageRows;
   p.region_bytes = 0;
   const size_t other = ck_smem_bytes<D>(p);                   // everything but the front region
   const size_t room = budget > other ? budget - other : 0;
+  // logits past the accumulators stay in shared memory as far as they fit beside three key tiles
+  const size_t ring_min = std::min(3, std::max(p.cpc_max, 2)) * k_bytes;
+  p.n_over = std::max(0, std::min(p.p_max - p.direct, room > q_hist + ring_min ? (int)((room - q_hist - ring_min) / over_bytes) : 0));
+  const size_t q_over = q_hist + (size_t)p.n_over * over_bytes;
   const int fit = room > q_over ? (int)((room - q_over) / k_bytes) : 0;
   p.stages = std::max(2, std::min({fit, kMaxStages, std::max(p.cpc_max, 2)}));
   const size_t need = p.stages * k_bytes + q_over;
@@ -931,7 +971,7 @@ int ck_active_clusters(const StepArgs& a, const CkParams& p, int per_sm) {
   cudaLaunchConfig_t cfg = ck_config<D>(a, p, attr, nullptr);
   cfg.numAttrs = 2;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, compress_cluster_kernel<D>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, compress_cluster_kernel<D, false>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     n = 0;
   }
@@ -943,7 +983,11 @@ int ck_active_clusters(const StepArgs& a, const CkParams& p, int per_sm) {
 // that only enter the softmax denominators (the new scale of a head that keeps it whole).
 struct CkLists {
   int ranked[2], once[2];
+  int rows[2];                                               // survivors that are moved
 };
+
+// Ranked chunks of the longest CTA whose logits are formed a second time.
+int ck_again(const CkParams& p) { return std::max(0, p.p_max - p.direct - p.n_over); }
 
 // Shape of a launch with `cl` CTAs per head and `per_sm` CTAs per SM.  Two CTAs per SM share its tensor
 // memory (256 columns each) and shared memory; a CTA that takes all 512 columns asks for more than half
@@ -962,45 +1006,61 @@ bool ck_shape(CkParams& p, const CkLists& n, int cl, int per_sm) {
   p.slots = 1;
   while (p.slots < std::min(p.cpc_max, most)) p.slots *= 2;
   p.direct = p.cpc_max <= p.slots ? p.slots : p.slots - 2;
-  p.n_over = std::max(0, p.p_max - p.direct);
-  if (p.cpc_max > kMaxCpc || p.n_over > (per_sm == 2 ? 2 : kMaxOver)) return false;
   if (!ck_size<D>(p, per_sm == 2 ? kSmemShared : kSmemBudget)) return false;
+  if (p.cpc_max + ck_again(p) > kMaxSeq) return false;
   return p.slots <= kMaxSlots / 2 || ck_smem_bytes<D>(p) > kSmemShared + 4096;
 }
 
 // Device time of one cluster in microseconds, fitted to clock stamps inside the kernel over launches of
-// 1 to 50 chunks per head: 8 us of dependent round trips, 2.5 more where they cross CTAs, and per chunk
-// of a CTA its key tile, its two read-outs and its share of the row moves.  CTAs that share an SM slow
-// each other down.
+// 1 to 50 chunks per head: 7 us of dependent round trips, 2 to 6 more where they cross CTAs (a cluster of
+// eight also waits for eight SMs of one GPC); the key tiles of a CTA at no more than 75 GB/s and its share
+// of the memory's rate; a read-out per ranked chunk; the row moves.  CTAs that share an SM slow each
+// other down.
 template <int D>
-float ck_cluster_us(const CkLists& n, int cl, bool crowded) {
-  const float ranked_us = D == 128 ? 1.8f : 1.2f, once_us = D == 128 ? 1.0f : 0.6f;
+float ck_cluster_us(const CkParams& p, const CkLists& n, int cl, bool crowded, float ctas) {
+  const float tile_us = std::max(D / 128 * 0.43f + (D == 64 ? 0.25f : 0.f), ctas * kCkChunk * D * 2 / 6.0e6f);
   float most = 0.f;
-  for (int t = 0; t < 2; ++t)
-    most = std::max(most, ranked_us * ((n.ranked[t] + cl - 1) / cl) + once_us * ((n.once[t] + cl - 1) / cl));
-  return (cl > 1 ? 10.5f : 8.f) + (crowded ? 1.6f : 1.f) * most;
+  for (int t = 0; t < 2; ++t) {
+    const int ranked = (n.ranked[t] + cl - 1) / cl, once = (n.once[t] + cl - 1) / cl;
+    const int again = std::max(0, ranked - p.direct - p.n_over);
+    const float move = (float)n.rows[t] / cl * D * 8 / 65000.f;      // a key and a value row in, the same out, at 65 GB/s
+    most = std::max(most, (ranked + once + again) * tile_us + ranked * 0.3f + again * 0.2f + move);
+  }
+  const float fixed = cl == 1 ? 7.f : 8.4f + 0.35f * cl + (cl > 6 ? 2.f : 0.f);
+  return fixed + (crowded ? 1.5f : 1.f) * most;
 }
 
 template <int D>
 int launch_t(const StepArgs& a, const CUtensorMap& tm_cache, const CUtensorMap& tm_new, const void* q, CkParams p,
-             const CkLists& lists, int n_clusters, float beside_us, float behind_us, cudaStream_t st) {
+             const CkLists& lists, int n_clusters, float beside_us, float behind_us, uint16_t* shape, cudaStream_t st) {
   // the opt-in is made once per (kernel, device), so it asks for the most any launch can need
-  if (!allow_dynamic_smem(compress_cluster_kernel<D>, kSmemBudget)) return -1;
+  if (!allow_dynamic_smem(compress_cluster_kernel<D, false>, kSmemBudget) ||
+      !allow_dynamic_smem(compress_cluster_kernel<D, true>, kSmemBudget))
+    return -1;
   // CTAs per head and per SM: the step ends when this launch and the attention that needs it are done,
   // and not before the SMs have done all the work there is (larger clusters finish sooner and keep
-  // more SMs from the attention that could run beside them).
+  // more SMs from the attention that could run beside them).  A late launch also leaves the attention behind
+  // it a worse last round, hence the last term.  Measured per step (CTAs per head: us): 32 heads x 128,
+  // 2 304 queries 2: 144, 3: 131, 4: 133, 6: 144; 64 heads 1: 268, 2: 239, 3: 247, 4: 250; 240 heads x 64,
+  // 1 024 queries, one CTA per head: 127 with one per SM, 113 with two.
   const float sms = (float)sm_count();
   float best = 0.f;
   int best_cl = 0, best_per_sm = 0;
-  for (int per_sm = 1; per_sm <= 2; ++per_sm)
+  if (shape && *shape) {                                     // found when this step came by before
+    best_cl = *shape & 0xff;
+    best_per_sm = *shape >> 8;
+  }
+  for (int per_sm = 1; per_sm <= 2 && !(shape && *shape); ++per_sm)
     for (int cl = 1; cl <= kMaxCluster; ++cl) {
       if (!ck_shape<D>(p, lists, cl, per_sm)) continue;
       const int active = ck_active_clusters<D>(a, p, per_sm);
       if (active < 1) continue;
+      if (D == 128 && per_sm == 2 && n_clusters * cl <= sms) continue;    // the CTAs spread over as many SMs, and attention takes a whole one
       const int waves = (n_clusters + active - 1) / active;
-      const float us = waves * ck_cluster_us<D>(lists, cl, per_sm == 2 && std::min(n_clusters, active) * cl > sms);
+      const int at_once = std::min(n_clusters, active);
+      const float us = waves * ck_cluster_us<D>(p, lists, cl, per_sm == 2 && at_once * cl > sms, (float)at_once * cl);
       const float sm_us = n_clusters * cl * us / (waves * per_sm);
-      const float cost = std::max(us + behind_us / sms, (sm_us + beside_us + behind_us) / sms);
+      const float cost = std::max(us + behind_us / sms, (sm_us + beside_us + behind_us) / sms) + 0.6f * us;
       if (!best_cl || cost < best) {
         best = cost;
         best_cl = cl;
@@ -1008,10 +1068,11 @@ int launch_t(const StepArgs& a, const CUtensorMap& tm_cache, const CUtensorMap& 
       }
     }
   if (!best_cl) return 0;
+  if (shape) *shape = (uint16_t)(best_per_sm << 8 | best_cl);
   ck_shape<D>(p, lists, best_cl, best_per_sm);
   cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = ck_config<D>(a, p, attr, st);
-  cudaLaunchKernelEx(&cfg, compress_cluster_kernel<D>, tm_cache, tm_new, a, static_cast<const __nv_bfloat16*>(q), p);
+  cudaLaunchKernelEx(&cfg, ck_again(p) > 0 ? compress_cluster_kernel<D, true> : compress_cluster_kernel<D, false>, tm_cache, tm_new, a, static_cast<const __nv_bfloat16*>(q), p);
   return launched(n_clusters * p.cluster);
 }
 
@@ -1019,10 +1080,10 @@ int launch_t(const StepArgs& a, const CUtensorMap& tm_cache, const CUtensorMap& 
 
 // Scores only (scores != nullptr) or the whole compression of the step.  Returns the working CTAs of
 // its one launch, -1 on a launch error, or 0 when this step is outside what the kernel holds
-// (candidate lists beyond 8 x 21 chunks per head, the every-query scoring rounds): the caller then
+// (candidate lists far beyond 8 x 40 chunks per head, the every-query scoring rounds): the caller then
 // takes the separate scoring, selection and compaction launches.
 int launch_compress_cluster(const StepArgs& a, const void* q, const void* k_new, const void* v_new, float* scores,
-                            cudaStream_t st, float beside_us, float behind_us) {
+                            cudaStream_t st, float beside_us, float behind_us, uint16_t* shape) {
   if (!a.k_map || a.obs_full || a.score_accumulate) return 0;
   if (!a.trig[0] && !a.trig[1]) return 0;
   CkParams p{};
@@ -1037,6 +1098,7 @@ int launch_compress_cluster(const StepArgs& a, const void* q, const void* k_new,
       const bool drop_new = t == 0 && a.protect_new && !scores;
       lists.ranked[t] = (a.stored[t] + kCkChunk - 1) / kCkChunk + (drop_new ? 0 : n_new_chunks);
       lists.once[t] = drop_new ? n_new_chunks : 0;
+      lists.rows[t] = scores ? 0 : a.kept[t] - (drop_new ? a.n_new : 0);
     }
   // clusters that do work: the heads of the triggered types
   const int n_clusters = std::max(1, a.heads_of[0] * a.trig[0] + a.heads_of[1] * a.trig[1]);
@@ -1046,8 +1108,8 @@ int launch_compress_cluster(const StepArgs& a, const void* q, const void* k_new,
     return -1;
   }
   const CUtensorMap& tm_cache = *static_cast<const CUtensorMap*>(a.k_map);
-  return a.head_dim == 128 ? launch_t<128>(a, tm_cache, tm_new, q, p, lists, n_clusters, beside_us, behind_us, st)
-                           : launch_t<64>(a, tm_cache, tm_new, q, p, lists, n_clusters, beside_us, behind_us, st);
+  return a.head_dim == 128 ? launch_t<128>(a, tm_cache, tm_new, q, p, lists, n_clusters, beside_us, behind_us, shape, st)
+                           : launch_t<64>(a, tm_cache, tm_new, q, p, lists, n_clusters, beside_us, behind_us, shape, st);
 }
 
 }  // namespace hack

@@ -90,6 +90,7 @@ struct hack_cache {
   std::vector<size_t> layer_rows;               // rows per plane of each layer
   std::vector<size_t> layer_row_base;           // first row of each layer inside the big planes
   std::vector<int> n_ctx_heads;                 // contextual heads per layer
+  std::vector<uint16_t> compress_shape;         // [L][n_scales] shape of the compression launch, 0 until the step first needs one
   // device memory
   unsigned char* k_all = nullptr;
   unsigned char* v_all = nullptr;
@@ -417,6 +418,7 @@ hack_status_t hack_init_cache(const hack_config_t* cfg, hack_cache_t** out) {
     total_rows += rows;
   }
   c->row_off_host = row_off;
+  c->compress_shape.assign((size_t)cfg->n_layers * cfg->n_scales, 0);
   const size_t row_bytes = (size_t)cfg->head_dim * c->elt;
   const size_t pad_rows = 256;    // slack after the last layer so that tiled reads stay inside
   c->reserved_bytes = 2 * (total_rows - (size_t)kCanaryRows * cfg->n_layers * bh) * row_bytes;   // K and V rows proper
@@ -809,8 +811,14 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
     // nothing) on the SMs it leaves free.
     StageScope ts(c, st, 0);
     float beside_us = 0.f, behind_us = 0.f;
-    for (int t = 0; t < 2; ++t) (a.trig[t] ? behind_us : beside_us) += hack::attend_tc_sm_us(a, t);
-    if ((r = hack::launch_compress_cluster(a, q, k, v, nullptr, st, beside_us, behind_us)) < 0) return HACK_ERR_CUDA;
+    for (int t = 0; t < 2; ++t) {
+      // heads that keep the whole new scale attend over it first and need their survivors only at the end
+      const float us = hack::attend_tc_sm_us(a, t), free = !a.trig[t] ? 1.f : a.seg_new[t] ? (float)a.n_new / a.kept[t] : 0.f;
+      beside_us += free * us;
+      behind_us += (1.f - free) * us;
+    }
+    if ((r = hack::launch_compress_cluster(a, q, k, v, nullptr, st, beside_us, behind_us,
+                                           &c->compress_shape[(size_t)layer * c->cfg.n_scales + scale])) < 0) return HACK_ERR_CUDA;
     compression_ctas = r;
     ts.done(r > 0);
     n += r > 0;

@@ -87,9 +87,10 @@ int launch_select(const StepArgs& a, const float* scores, int32_t* idx, int32_t*
 // bf16 caches: scores only (scores != nullptr) or scoring, selection and in-place compaction of the step
 // in one launch of one thread-block cluster per head.  Its CTAs if launched; 0: the step is outside what
 // the kernel holds, take the separate launches; -1: launch error.  beside_us, behind_us: SM-microseconds
-// of the attention launch behind this one that can run beside it, and that need its result.
+// of the attention launch behind this one that can run beside it, and that need its result.  shape: the
+// launch shape of this step as found before (0: not yet), kept by the caller.
 int launch_compress_cluster(const StepArgs& a, const void* q, const void* k_new, const void* v_new, float* scores,
-                            cudaStream_t st, float beside_us = 0.f, float behind_us = 0.f);
+                            cudaStream_t st, float beside_us = 0.f, float behind_us = 0.f, uint16_t* shape = nullptr);
 // idx == nullptr: every head appends (keeps all candidates).  idx_all != 0: idx rows are valid for
 // heads that are not triggered as well (identity lists written by launch_select).
 int launch_compact(const StepArgs& a, int dtype, const int32_t* idx, int idx_all, const void* k_new,

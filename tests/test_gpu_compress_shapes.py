@@ -22,6 +22,7 @@ def _built():
     (1, 20, 16, (1, 2, 5, 9, 13, 16), 68, 400, 0),          # 320 heads of up to 6 chunks: two CTAs per SM
     (3, 30, 8, (1, 3, 7, 12, 19), 130, 257, 1),             # the same at head_dim 128, current scale competes
     (1, 15, 12, (1, 4, 9, 25, 41), 700, 1300, 0),           # 180 heads, lists past the accumulators of one CTA
+    (3, 30, 5, (1, 4, 13, 29, 37), 900, 2100, 0),           # the same at head_dim 128: logits formed a second time
     (3, 3, 1, (1, 4, 11, 17, 30), 257, 640, 1),             # 3 heads: large clusters, ragged last chunks
 ])
 def test_launch_shapes(base, heads, batch, sides, b_c, b_s, policy):
