@@ -7,7 +7,9 @@ arithmetic.  There is no fallback: if the shared library is missing, importing t
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
+import sysconfig
 from typing import Optional, Sequence
 
 # HACK_B200_CHECKED=1 selects the checked build of the same sources (bounds checks in the kernels,
@@ -108,6 +110,28 @@ def _load() -> C.CDLL:
 lib = _load()
 
 
+def _load_call():
+    """call(address, handle, layer, scale, *buffers) -> status: the compiled marshalling of the per-step
+    entry points, or the same through ctypes if the module was not built for this interpreter."""
+    path = os.path.join(os.path.dirname(_LIB_PATH), "_hackcall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
+    if os.path.exists(path):
+        spec = importlib.util.spec_from_file_location("_hackcall", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        return module.call
+    functions = {C.cast(getattr(lib, n), C.c_void_p).value: getattr(lib, n)
+                 for n in ("hack_score", "hack_select", "hack_compact", "hack_attend", "hack_attend_variance",
+                           "hack_scale_step", "hack_scale_step_host")}
+    return lambda address, handle, layer, scale, *buffers: functions[address](handle, layer, scale, *map(_ptr, buffers))
+
+
+_call = _load_call()
+_SCORE, _SELECT, _COMPACT, _ATTEND, _ATTEND_VARIANCE, _SCALE_STEP, _SCALE_STEP_HOST = (
+    C.cast(getattr(lib, n), C.c_void_p).value for n in (
+        "hack_score", "hack_select", "hack_compact", "hack_attend", "hack_attend_variance", "hack_scale_step",
+        "hack_scale_step_host"))
+
+
 def hack_last_error() -> str:
     return lib.hack_last_error().decode()
 
@@ -169,6 +193,7 @@ class HackCache:
                          budget_c, budget_s, n_obs, n_init_scales, sm_scale, overflow_policy, device,
                          obs_sampler, 1 if merge_last else 0)
         _check(lib.hack_init_cache(C.byref(cfg), C.byref(self._h)))
+        self._address = self._h.value
         self.n_layers, self.n_heads, self.head_dim, self.batch = n_layers, n_heads, head_dim, batch
         self.dtype = dtype
         self.elt = 4 if dtype == HACK_F32 else 2
@@ -188,6 +213,7 @@ class HackCache:
                     problem = f"{bad.value} guard rows overwritten: {hack_last_error()}"
             lib.hack_free_cache(self._h)
             self._h = C.c_void_p()
+            self._address = 0
             if problem:
                 raise HackError(HACK_ERR_STATE, problem)
 
@@ -215,26 +241,27 @@ class HackCache:
         return info
 
     def hack_score(self, layer, scale, q, k_new, scores, stream=None) -> None:
-        _check(lib.hack_score(self._h, layer, scale, _ptr(q), _ptr(k_new), _ptr(scores), _ptr(stream)))
+        _check(_call(_SCORE, self._address, layer, scale, q, k_new, scores, stream))
 
     def hack_select(self, layer, scale, scores, idx, kept_out=None, stream=None) -> None:
-        _check(lib.hack_select(self._h, layer, scale, _ptr(scores), _ptr(idx), _ptr(kept_out), _ptr(stream)))
+        _check(_call(_SELECT, self._address, layer, scale, scores, idx, kept_out, stream))
 
     def hack_compact(self, layer, scale, idx, k_new, v_new, stream=None) -> None:
-        _check(lib.hack_compact(self._h, layer, scale, _ptr(idx), _ptr(k_new), _ptr(v_new), _ptr(stream)))
+        _check(_call(_COMPACT, self._address, layer, scale, idx, k_new, v_new, stream))
 
     def hack_attend(self, layer, scale, q, out, stream=None) -> None:
-        _check(lib.hack_attend(self._h, layer, scale, _ptr(q), _ptr(out), _ptr(stream)))
+        _check(_call(_ATTEND, self._address, layer, scale, q, out, stream))
 
     def hack_attend_variance(self, layer, scale, q, out, sigma, stream=None) -> None:
-        _check(lib.hack_attend_variance(self._h, layer, scale, _ptr(q), _ptr(out), _ptr(sigma), _ptr(stream)))
+        _check(_call(_ATTEND_VARIANCE, self._address, layer, scale, q, out, sigma, stream))
 
     def hack_scale_step(self, layer, scale, q, k, v, out, stream=None) -> None:
-        _check(lib.hack_scale_step(self._h, layer, scale, _ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(stream)))
+        status = _call(_SCALE_STEP, self._address, layer, scale, q, k, v, out, stream)
+        if status:
+            _check(status)
 
     def hack_scale_step_host(self, layer, scale, q, k, v, out, stream=None) -> None:
-        _check(lib.hack_scale_step_host(self._h, layer, scale, _ptr(q), _ptr(k), _ptr(v), _ptr(out),
-                                        _ptr(stream)))
+        _check(_call(_SCALE_STEP_HOST, self._address, layer, scale, q, k, v, out, stream))
 
     def hack_get_lengths(self, layer: int):
         n = self.batch * self.n_heads

@@ -12,6 +12,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -21,6 +22,7 @@ BUILD = os.path.join(PKG, "_build")
 LIBDIR = os.path.join(PKG, "lib")
 LIB = os.path.join(LIBDIR, "libhack_b200.so")
 LIB_CHECKED = os.path.join(LIBDIR, "libhack_b200_checked.so")
+PYCALL = os.path.join(LIBDIR, "_hackcall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -40,6 +42,19 @@ def _newest_header() -> float:
     hdrs = glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
         glob.glob(os.path.join(ROOT, "include", "*.h"))
     return max(os.path.getmtime(h) for h in hdrs)
+
+
+def build_pycall(force: bool = False) -> None:
+    """The binding's marshalling module (csrc/pycall.c) for the running interpreter.  Where the
+    interpreter's headers are not installed the binding marshals with ctypes instead."""
+    src = os.path.join(CSRC, "pycall.c")
+    include = sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(include, "Python.h")) or not shutil.which("gcc"):
+        return
+    if not force and os.path.exists(PYCALL) and os.path.getmtime(PYCALL) >= os.path.getmtime(src):
+        return
+    os.makedirs(LIBDIR, exist_ok=True)
+    subprocess.run(["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", include, src, "-o", PYCALL], check=True)
 
 
 def build(force: bool = False, verbose: bool = False, checked: bool = False) -> str:
@@ -70,6 +85,7 @@ def build(force: bool = False, verbose: bool = False, checked: bool = False) -> 
             raise RuntimeError("nvcc failed:\n" + " ".join(cmd) + "\n" + res.stdout + res.stderr)
         return res.stderr
 
+    build_pycall(force)
     if jobs:
         with ThreadPoolExecutor(max_workers=min(8, len(jobs))) as ex:
             for log in ex.map(run, jobs):

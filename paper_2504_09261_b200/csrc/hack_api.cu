@@ -120,6 +120,7 @@ struct hack_cache {
   cudaEvent_t ev_in[kHostSlots] = {}, ev_step[kHostSlots] = {}, ev_out[kHostSlots] = {};
   uint64_t host_calls = 0;
   size_t reserved_bytes = 0, peak_bytes = 0;
+  long long live_rows = 0;                      // stored (batch, head) rows over all layers
   uint64_t launches = 0;
   long long wait_cycles = hack::kDefaultWaitCycles;   // limit of the kernels' bounded waits
   bool poisoned = false;                        // a launch failed after part of a step had been enqueued
@@ -221,15 +222,7 @@ hack::StepArgs make_args(const hack_cache* c, int layer, int scale, const hack_s
   return a;
 }
 
-size_t live_bytes(const hack_cache* c) {
-  size_t rows = 0;
-  for (int l = 0; l < c->cfg.n_layers; ++l) {
-    const LayerState& ls = c->layers[l];
-    rows += (size_t)c->cfg.batch * ((size_t)c->n_ctx_heads[l] * ls.len[1] +
-                                    (size_t)(c->cfg.n_heads - c->n_ctx_heads[l]) * ls.len[0]);
-  }
-  return rows * c->cfg.head_dim * c->elt * 2;
-}
+size_t live_bytes(const hack_cache* c) { return (size_t)c->live_rows * c->cfg.head_dim * c->elt * 2; }
 
 // Makes the cache's device current for the duration of an entry point and puts the caller's back.
 struct DeviceScope {
@@ -301,6 +294,8 @@ bool misaligned(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) !
 
 void advance_after_compact(hack_cache* c, int layer, const hack_step_info_t& p) {
   LayerState& ls = c->layers[layer];
+  c->live_rows += (long long)c->cfg.batch * ((long long)c->n_ctx_heads[layer] * (p.kept_c - ls.len[1]) +
+                                             (long long)(c->cfg.n_heads - c->n_ctx_heads[layer]) * (p.kept_s - ls.len[0]));
   ls.len[0] = p.kept_s;
   ls.len[1] = p.kept_c;
   ls.phase = 1;
@@ -585,6 +580,7 @@ hack_status_t hack_reset(hack_cache_t* c) {
   if (!c) return fail(HACK_ERR_INVALID_ARG, "cache is NULL");
   for (auto& ls : c->layers) ls = LayerState();
   c->peak_bytes = 0;
+  c->live_rows = 0;
   c->poisoned = false;
   return HACK_OK;
 }
