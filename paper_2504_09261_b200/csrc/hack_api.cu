@@ -820,6 +820,7 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
     n += r > 0;
   }
   const bool compressed = compression_ctas > 0;
+  bool moved = false;               // the selection launch has moved the rows as well
   if (any && !compressed) {
     {
       StageScope ts(c, st, 0);
@@ -831,14 +832,15 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
       ts.done(r);
       n += r;
     }
-    {
-      StageScope ts(c, st, 1);
-      if ((r = hack::launch_select(a, c->scores, c->idx, nullptr, st)) < 0) return poison(c);
-      ts.done(r);
-      n += r;
-    }
+    StageScope ts(c, st, 1);
+    r = merge_step || fused_append ? 0 : hack::launch_select_move(a, c->cfg.dtype, c->scores, k, v, st);
+    moved = r > 0;
+    if (r == 0) r = hack::launch_select(a, c->scores, c->idx, nullptr, st);
+    if (r < 0) return poison(c);
+    ts.done(r);
+    n += r;
   }
-  if ((any && !compressed) || !fused_append) {      // a step that only appends needs no launch ahead of the fused attention
+  if (((any && !compressed) || !fused_append) && !moved) {      // a step that only appends needs no launch ahead of the fused attention
     StageScope ts(c, st, 2);
     if ((r = compact_stage(c, a, p, scale, any ? c->idx : nullptr, any ? 1 : 0, k, v, st)) < 0) return any ? poison(c) : HACK_ERR_CUDA;
     ts.done(r);

@@ -84,6 +84,9 @@ int launch_score_tc(const StepArgs& a, const void* q, const void* k_new, float* 
                     cudaStream_t st);
 int launch_select(const StepArgs& a, const float* scores, int32_t* idx, int32_t* kept_out,
                   cudaStream_t st);
+// Selection and compaction of a step in one launch, for heads of few rows.  1: launched; 0: outside what
+// the kernel is for, take launch_select and launch_compact; -1: launch error.
+int launch_select_move(const StepArgs& a, int dtype, const float* scores, const void* k_new, const void* v_new, cudaStream_t st);
 // bf16 caches: scores only (scores != nullptr) or scoring, selection and in-place compaction of the step
 // in one launch of one thread-block cluster per head.  Its CTAs if launched; 0: the step is outside what
 // the kernel holds, take the separate launches; -1: launch error.  beside_us, behind_us: SM-microseconds

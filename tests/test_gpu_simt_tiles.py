@@ -75,3 +75,17 @@ def test_dense_scores_over_ragged_chunks(n_cand, n_obs, head_dim, dtype):
     got = scores[:, :n_cand].double()
     assert bool(((got - ref).abs() <= 1e-4 * torch.maximum(got.abs(), ref.abs()) + 1e-7).all())
     assert bool((scores[:, n_cand:] == -1.0).all())
+
+
+@pytest.mark.parametrize("head_dim,b_c,b_s,policy", [(64, 255, 257, 1), (64, 256, 512, 0), (128, 127, 129, 1), (128, 1, 383, 0)])
+def test_selection_that_moves_the_rows(head_dim, b_c, b_s, policy):
+    """fp32 steps small enough for selection and compaction in one launch, kept lengths around the rows of
+    its rounds (256 at head_dim 64, 128 at 128), against the oracle and the separate launches."""
+    from dataclasses import replace
+    from parity_util import run_parity
+    from workloads import get_config
+    cfg = replace(get_config(0), name=f"select-move-{head_dim}", n_heads=4, batch=2, head_dim=head_dim, sides=(1, 3, 9, 13, 17),
+                  budget_c=b_c, budget_s=b_s)
+    rep = run_parity(cfg, [0], fused=True, policy=policy)
+    assert rep.ok(), rep.problems[:5]
+    assert rep.compressed_heads > 0
