@@ -788,11 +788,17 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
     a.seg_new[0] = !p.triggered_s || a.protect_new;
     a.seg_new[1] = !p.triggered_c;
   }
-  if (c->cfg.dtype == HACK_F32 && !any && p.n_new <= hack::kSmallQueries) {
+  r = 0;
+  StageScope whole(c, st, 3);
+  if (c->cfg.dtype == HACK_F32 && !any && p.n_new <= hack::kSmallQueries)
     // nothing is evicted and the scale is small: one launch appends and attends
-    StageScope ts(c, st, 3);
-    if ((r = hack::launch_attend_small(a, c->cfg.dtype, q, k, v, out, st)) < 0) return HACK_ERR_CUDA;
-    ts.done(r);
+    r = hack::launch_attend_small(a, c->cfg.dtype, q, k, v, out, st);
+  else if (c->cfg.dtype == HACK_BF16 && any && !merge_step)
+    // heads of few candidates: one launch for the whole step
+    r = hack::launch_step_small(a, q, k, v, out, st);
+  if (r < 0) return HACK_ERR_CUDA;
+  if (r > 0) {
+    whole.done(r);
     c->launches += r;
     advance_after_compact(c, layer, p);
     LayerState& ls = c->layers[layer];

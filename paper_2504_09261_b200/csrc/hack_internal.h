@@ -129,6 +129,10 @@ int launch_attend_small(const StepArgs& a, int dtype, const void* q, const void*
 bool attend_small_serves(const StepArgs& a);   // bf16: the small kernel is the one for this step's attention
 constexpr int kSmallQueries = 31;
 
+// A whole step that evicts (scores, selection, attention, compaction) of a bf16 cache in one launch, for heads
+// that fit into shared memory.  1: launched; 0: outside what the kernel is for; -1: launch error.
+int launch_step_small(const StepArgs& a, const void* q, const void* k_new, const void* v_new, void* out, cudaStream_t st);
+
 constexpr int kTcMinQueries = 32;   // below this the small kernel serves every bf16 step
 
 void set_error(const std::string& msg);
@@ -172,7 +176,8 @@ __device__ __forceinline__ bool dbg_ok(bool, int*, int) { return true; }
 #endif
 // Query row that serves as observation row i (Eq. 9's subset Q~).
 __device__ __forceinline__ int obs_row(const StepArgs& a, int i) {
-  return a.obs_rows ? a.obs_rows[i] : a.obs_first + (int)(((long long)i * a.obs_span) / a.n_obs_rows);
+  // (i < 32 and obs_span <= N_k: the product fits 32 bits, whose division is a third of a 64-bit one's work)
+  return a.obs_rows ? a.obs_rows[i] : a.obs_first + (int)(((uint32_t)i * (uint32_t)a.obs_span) / (uint32_t)a.n_obs_rows);
 }
 __device__ __forceinline__ void pdl_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -39,3 +39,57 @@ def test_append_and_attend_over_ragged_tiles(sides, head_dim):
             assert cache.hack_read_head(0, b, h, which) == want
         assert np.array_equal(np.frombuffer(cache.hack_read_head(0, b, h, 2), dtype=np.int32), np.arange(total))
     cache.close()
+
+
+@pytest.mark.parametrize("base,heads,batch,sides,b_c,b_s,policy", [
+    (1, 5, 1, (1, 2, 3, 5, 7, 9), 47, 128, 0),              # up to 128 ranked candidates, every CTA one row tile
+    (1, 16, 1, (1, 2, 6, 10, 13), 87, 255, 1),              # 256 = two key tiles per warp; the current scale competes
+    (1, 8, 1, (1, 2, 7, 13, 15), 60, 287, 0),               # 512 = four, clusters of eight
+    (1, 4, 1, (1, 2, 9, 15, 19), 50, 407, 1),               # 768 = six
+    (1, 30, 8, (1, 2, 4, 6, 7), 39, 101, 0),                # 240 heads, two CTAs per SM
+    (1, 7, 3, (5, 5, 1, 1, 4), 20, 33, 1),                  # steps of a single token that evict
+    (3, 16, 1, (1, 3, 5, 8, 9), 33, 97, 0),                 # head_dim 128
+    (3, 9, 2, (1, 2, 8, 12), 1, 150, 1),                    # a contextual head keeps one row
+])
+def test_whole_step_in_one_launch(base, heads, batch, sides, b_c, b_s, policy):
+    from dataclasses import replace
+    from parity_util import run_parity
+    from workloads import get_config
+    cfg = replace(get_config(base, n_layers=1), name=f"small-{heads}x{batch}", n_heads=heads, batch=batch, sides=sides,
+                  budget_c=b_c, budget_s=b_s)
+    rep = run_parity(cfg, [0], fused=True, policy=policy)
+    assert rep.ok(), rep.problems[:5]
+    assert rep.compressed_heads > 0
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+def test_equal_scores_in_one_launch(head_dim):
+    """All keys zero: every entry lies in the located bin and the lowest candidate indices survive; the
+    outputs are the mean of the survivors' values (bar as above).  Every step is one launch."""
+    import torch
+    import paper_2504_09261_b200 as hb
+    sides, b_c, b_s, heads = (2, 3, 5, 9), 21, 100, 6
+    mask = np.array([[h % 2 for h in range(heads)]], dtype=np.uint8)
+    cache = hb.HackCache(1, heads, head_dim, 1, sides, hb.HACK_BF16, mask, b_c, b_s)
+    kept, total = [[], []], 0
+    for k, side in enumerate(sides):
+        n = side * side
+        z = torch.zeros((1, heads, n, head_dim), dtype=torch.bfloat16, device="cuda")
+        v = (torch.arange(total, total + n, device="cuda") / 128).bfloat16()[None, None, :, None].expand_as(z).contiguous()
+        out = torch.empty_like(z)
+        before = cache.hack_launch_count()
+        cache.hack_scale_step(0, k, torch.randn_like(z), z, v, out)
+        assert cache.hack_launch_count() == before + 1
+        new = list(range(total, total + n))
+        total += n
+        for t, budget in ((0, b_s), (1, b_c)):
+            cand = kept[t] + new
+            if len(cand) > budget and t == 0:               # the leading two scales and the new one are protected
+                cand = cand[:max(budget, 13 + n) - n] + new
+            kept[t] = cand if t == 0 else cand[:budget]
+        for h in range(heads):
+            t = int(mask[0, h])
+            assert np.array_equal(np.frombuffer(cache.hack_read_head(0, 0, h, 2), dtype=np.int32), kept[t])
+            mean = (torch.tensor(kept[t], device="cuda") / 128).bfloat16().double().mean()
+            assert (out[0, h].double() - mean).abs().max() <= 2e-2
+    cache.close()
