@@ -793,9 +793,9 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
   if (c->cfg.dtype == HACK_F32 && !any && p.n_new <= hack::kSmallQueries)
     // nothing is evicted and the scale is small: one launch appends and attends
     r = hack::launch_attend_small(a, c->cfg.dtype, q, k, v, out, st);
-  else if (c->cfg.dtype == HACK_BF16 && any && !merge_step)
+  else if (any && !merge_step)
     // heads of few candidates: one launch for the whole step
-    r = hack::launch_step_small(a, q, k, v, out, st);
+    r = hack::launch_step_small(a, c->cfg.dtype, q, k, v, out, st);
   if (r < 0) return HACK_ERR_CUDA;
   if (r > 0) {
     whole.done(r);

@@ -21,30 +21,17 @@
 #include <type_traits>
 
 #include "hack_internal.h"
+#include "step_small.cuh"
 #include "tc_ptx.cuh"
 
 namespace hack {
 namespace {
 
 using namespace ptx;
+using namespace small_step;
 
-constexpr int kStepWarps = 8;
-constexpr int kStepThreads = kStepWarps * 32;
 constexpr int kTile = 16;                       // queries per row tile, keys per warp and turn
-constexpr int kMaxTurns = 6;                    // key tiles of a warp whose logits it can hold
-constexpr int kMaxRows = kMaxTurns * kStepWarps * kTile;   // candidates of a head: 768
-constexpr int kMaxTiles = 8;                    // query tiles of a CTA
-constexpr int kMaxCtas = 8;                     // CTAs per head
-constexpr int kRangeBins = 256;                 // bins of the selection's histogram; one more for protected rows
-constexpr size_t kSmemCta = 222 * 1024;         // dynamic shared memory beside the static tables ...
-constexpr size_t kSmemHalf = 108 * 1024;        // ... and with two CTAs on an SM
-
-struct StepShape {
-  int ctas;        // CTAs per head
-  int tiles;       // query tiles per CTA: 1, 2, 4 or 8; the CTA's 8 warps share the keys of a tile 8 / tiles ways
-  int log_splits;  // log2(8 / tiles)
-  int rows;        // candidate rows shared memory has room for (multiple of 16)
-};
+constexpr int kMaxTurns = kMaxRows / (kStepWarps * kTile);   // key tiles of a warp whose logits it can hold: 6
 
 // Bytes in front of the small tables: K and V rows (later the warps' unnormalised outputs), observation
 // rows, queries.
@@ -55,11 +42,6 @@ __host__ __device__ constexpr size_t kv_bytes(int rows) {
 template <int D>
 size_t step_smem(const StepShape& s) {
   return kv_bytes<D>(s.rows) + (size_t)kMaxObs * D * 2 + (size_t)s.tiles * kTile * D * 2 + (size_t)s.rows * 3 * sizeof(int32_t);
-}
-
-__device__ __forceinline__ uint32_t order_key(float f) {     // larger float -> larger key, never the top one
-  const uint32_t u = __float_as_uint(f);
-  return min((u & 0x80000000u) ? ~u : (u | 0x80000000u), 0xfffffffeu);
 }
 
 // Two fp32 numbers as a sum of two packed pairs of bf16.
@@ -79,10 +61,7 @@ step_small_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, const _
   constexpr uint32_t ROWB = D * 2;
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ float2 stats[kStepWarps][kMaxObs];
-  __shared__ int hist[kRangeBins + 32];
-  __shared__ uint32_t range[2];
-  __shared__ int n_in;
-  __shared__ uint32_t words[kMaxRows / 32];
+  __shared__ PickShared ps;
   __shared__ float2 row_ml[kStepWarps][kTile];
 
   const int bh = a.head_order[blockIdx.y], rank = blockIdx.x;   // structural heads (the longer ones) first
@@ -106,8 +85,7 @@ step_small_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, const _
   auto fetch = [](uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
   };
-  for (int i = tid; i < kRangeBins + 32; i += kStepThreads) hist[i] = 0;
-  if (tid == 0) { range[0] = 0xffffffffu; range[1] = 0u; n_in = 0; }     // least and greatest key
+  pick_init(ps);
   pdl_wait();
 
   // ------------------------------------------------------------------ rows into shared memory
@@ -230,93 +208,14 @@ step_small_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, const _
         sc += __shfl_xor_sync(0xffffffffu, sc, 16);
         const int j = kt * kTile + (up ? 8 : 0) + 2 * (lane & 3) + (upper ? 1 : 0);
         if (lane < 16 && j < cand) {
-          const bool fixed = ctx == 0 && (j < a.t_init || (a.protect_new && j >= stored));
+          const bool fixed = is_protected(a, ctx, j);
           const uint32_t k = fixed ? 0xffffffffu : order_key(sc);
           key[j] = k;
           if (!fixed) { lo = min(lo, k); hi = max(hi, k); }
         }
       }
     }
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    if (lane == 0) {
-      atomicMin(&range[0], lo);
-      atomicMax(&range[1], hi);
-    }
-    __syncthreads();
-    // the n_keep greatest keys: one histogram over their range finds the bin of the last survivor, whose
-    // entries are ranked by comparison; protected rows have a bin of their own above all others
-    lo = range[0];
-    hi = range[1];
-    const int shift = hi <= lo ? 0 : max(0, 32 - __clz(hi - lo) - 8);
-    auto bin_of = [&](uint32_t k) { return k == 0xffffffffu ? kRangeBins : (int)((k - lo) >> shift); };
-    constexpr int MINE = (kTurns * kStepWarps * kTile + kStepThreads - 1) / kStepThreads;
-    uint32_t mine[MINE];
-#pragma unroll
-    for (int u = 0; u < MINE; ++u) {
-      const int j = tid + u * kStepThreads;
-      mine[u] = j < cand ? key[j] : 0u;
-      if (j < cand) atomicAdd(&hist[bin_of(mine[u])], 1);
-    }
-    __syncthreads();
-    int digit, need;                            // found by every warp for itself
-    {
-      constexpr int PER = (kRangeBins + 32) / 32;              // lane 0 has the top bins
-      int c[PER], sum = 0;
-#pragma unroll
-      for (int i = 0; i < PER; ++i) { c[i] = hist[kRangeBins + 31 - PER * lane - i]; sum += c[i]; }
-      int incl = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += n;
-      }
-      int cum = incl - sum, d = 0, rest = 0;
-      const bool here = cum < n_keep && n_keep <= incl;
-#pragma unroll
-      for (int i = 0; i < PER; ++i) {
-        if (cum < n_keep && n_keep <= cum + c[i]) { d = kRangeBins + 31 - PER * lane - i; rest = n_keep - cum; }
-        cum += c[i];
-      }
-      const int src = __ffs(__ballot_sync(0xffffffffu, here)) - 1;
-      digit = __shfl_sync(0xffffffffu, d, src);
-      need = __shfl_sync(0xffffffffu, rest, src);
-    }
-    int32_t* in = list;                         // the bin's entries, until the list is written
-#pragma unroll
-    for (int u = 0; u < MINE; ++u) {
-      const int j = tid + u * kStepThreads;
-      if (j < cand && bin_of(mine[u]) == digit) in[atomicAdd(&n_in, 1)] = j;
-    }
-    __syncthreads();
-    const int n_bin = n_in;
-    bool keep[MINE];
-#pragma unroll
-    for (int u = 0; u < MINE; ++u) {
-      const int j = tid + u * kStepThreads;
-      const int b = j < cand ? bin_of(mine[u]) : -1;
-      keep[u] = b >= digit;
-      if (b == digit && need < n_bin) {
-        int above = 0;                          // ties go to the lower candidate
-#pragma unroll 4
-        for (int i = 0; i < n_bin; ++i) {
-          const int o = in[i];
-          const uint32_t k = key[o];
-          above += k > mine[u] || (k == mine[u] && o < j);
-        }
-        keep[u] = above < need;
-      }
-      const uint32_t w = __ballot_sync(0xffffffffu, keep[u]);
-      if (lane == 0) words[u * kStepWarps + warp] = w;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < MINE; ++u) {
-      const int me = u * kStepWarps + warp;
-      const int before = __reduce_add_sync(0xffffffffu, lane < me ? __popc(words[lane]) : 0);
-      const int o = before + __popc(words[me] & ((1u << lane) - 1));
-      if (keep[u] && dbg_ok(o < n_keep, a.status, 12)) list[o] = tid + u * kStepThreads;
-    }
+    pick<(kTurns * kStepWarps * kTile + kStepThreads - 1) / kStepThreads>(a, ps, key, list, cand, n_keep, lo, hi);
   } else {
     for (int j = tid; j < n_keep; j += kStepThreads) list[j] = j;
   }
@@ -509,41 +408,12 @@ int launch_t(const StepArgs& a, const void* q, const void* k_new, const void* v_
   if (cand > kMaxRows || tiles > kMaxTiles * kMaxCtas) return 0;
   StepShape s;
   s.rows = (cand + kTile - 1) / kTile * kTile;
-  // as many CTAs per head as leave every CTA an SM, at least what its queries need; clusters of seven and eight
-  // only where they are few (16 clusters of 8 CTAs do not find a place at once beside each other: 100
-  // queries, 16 heads: 7 CTAs 8.5 us, 4 CTAs 7.9; 169 queries: 6 CTAs 8.2, 3 CTAs 10.3)
-  auto split_queries = [&](int most) {
-    const int want = std::max(1, std::min({sm_count() / heads, tiles, most}));
-    for (s.tiles = 1; s.tiles < kMaxTiles && s.tiles * want < tiles; s.tiles *= 2) {}
-    s.ctas = (tiles + s.tiles - 1) / s.tiles;
-  };
-  split_queries(kMaxCtas);
-  if (s.ctas > 6 && heads * s.ctas * 2 > sm_count()) split_queries(kMaxCtas / 2);
-  for (s.log_splits = 0; s.tiles << s.log_splits < kStepWarps; ++s.log_splits) {}
+  split_queries(s, heads, tiles);
   const size_t smem = step_smem<D>(s);
   const int ranked = std::max(a.trig[0] ? a.cand[0] : 0, a.trig[1] ? a.cand[1] : 0);
   const int turns = (ranked + kStepWarps * kTile - 1) / (kStepWarps * kTile);
   if (smem > kSmemCta || !step_small_pays<D>(a, s, D == 64 && turns <= 4 && smem <= kSmemHalf ? 2 : 1)) return 0;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(s.ctas, heads);
-  cfg.blockDim = dim3(kStepThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = s.ctas;
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = s.ctas > 1 ? 2 : 1;
-  auto go = [&](auto kern) {
-    if (!allow_dynamic_smem(kern, kSmemCta)) return -1;
-    cudaLaunchKernelEx(&cfg, kern, a, static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k_new),
-                       static_cast<const __nv_bfloat16*>(v_new), static_cast<__nv_bfloat16*>(out), s);
-    return launched(1);
-  };
+  auto go = [&](auto kern) { return launch_step<__nv_bfloat16>(kern, a, s, smem, q, k_new, v_new, out, st); };
   if (turns <= 1) return go(step_small_kernel<D, 1>);
   if (turns <= 2) return go(step_small_kernel<D, 2>);
   if (turns <= 4) return go(step_small_kernel<D, 4>);
@@ -552,8 +422,9 @@ int launch_t(const StepArgs& a, const void* q, const void* k_new, const void* v_
 
 }  // namespace
 
-int launch_step_small(const StepArgs& a, const void* q, const void* k_new, const void* v_new, void* out, cudaStream_t st) {
+int launch_step_small(const StepArgs& a, int dtype, const void* q, const void* k_new, const void* v_new, void* out, cudaStream_t st) {
   if (a.obs_full || a.score_accumulate || (!a.trig[0] && !a.trig[1])) return 0;
+  if (dtype == HACK_F32) return launch_step_small_f32(a, q, k_new, v_new, out, st);
   return a.head_dim == 128 ? launch_t<128>(a, q, k_new, v_new, out, st) : launch_t<64>(a, q, k_new, v_new, out, st);
 }
 
