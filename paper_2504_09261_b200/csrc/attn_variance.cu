@@ -11,11 +11,11 @@
 //   warps 2-5 : consumers of the first key block, warps 6-9 of the second; thread r owns key r: it reads
 //               its 128 logits with tcgen05.ld, forms p = exp2(c z - c m_i - log2 l_i) and adds p and
 //               p^2 to two registers
-// Two blocks per CTA halve the query traffic: with one block per CTA (two CTAs per SM) the launch ran at the
-// L2's rate of about 21 bytes per clock and SM.  32 heads x 4 096 queries x 10 521 keys x 128: 643 -> 610 us.
 // so the sums over the queries stay inside one thread and nothing of size N x T is stored.  At the
 // end the thread holds Var_i A[i, j] = sum p^2 / N - (sum p / N)^2 of its key; the CTA adds its 128
 // variances and a second, tiny kernel adds the blocks of a head in a fixed order.
+// Two blocks per CTA halve the query traffic: with one block per CTA (two CTAs per SM) the launch ran at the
+// L2's rate of about 21 bytes per clock and SM.  32 heads x 4 096 queries x 10 521 keys x 128: 643 -> 610 us.
 // Every mbarrier wait is bounded; on expiry the CTA raises the status word and winds down.
 #include <cuda.h>
 

@@ -1,6 +1,7 @@
 // Subset-attention importance scores (Eq. 9 and the TOPK argument of Eq. 10-11).
 //
-// Two launches per step.  Pass 1 walks the candidate keys once: each CTA takes 128 candidates of
+// One launch per step where the candidate lists fit the registers of a cluster (score_cluster_kernel, with
+// the bodies of score_simt.cuh).  Longer lists take two launches.  Pass 1 walks the candidate keys once: each CTA takes 128 candidates of
 // one head, stages them in shared memory with 16-byte coalesced loads, forms the logits against
 // the (at most 32) observation rows, stores them to scratch and publishes per-row (max, sum-exp)
 // partials for its chunk.  Pass 2 merges the partials into the row statistics of the full

@@ -5,8 +5,9 @@
 // simply fail), or a latency-critical decode loop where the implicit device-wide synchronisation
 // of cudaMalloc / cudaFree is not acceptable.  hack_init_cache allocates, so it is closed to them.
 // This entry point needs no cache object: the caller passes dense Q and candidate-key tensors and
-// an output buffer, and the two-pass scoring kernels keep their intermediate logits and row
-// statistics in a fixed array that lives in the library's own device image.
+// an output buffer.  Row-blocks that fit a cluster's registers are one launch without intermediates
+// (score_simt.cuh); for the others the two-pass scoring kernels keep their logits and row statistics in a
+// fixed array that lives in the library's own device image.
 //
 // The array (kScratchFloats floats, about 8.3 MiB) is part of the module: every GPU that loads
 // the library holds it until the process exits.  CUDA loads the module's device image lazily, so
