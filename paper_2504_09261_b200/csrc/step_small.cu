@@ -15,8 +15,11 @@
 // What bounds it is latency: launch, one trip to memory, some ten block barriers.  The two launches it
 // stands for (compression on tcgen05, then attention) wait for each other and each pay a launch, a trip to
 // memory and a tail.
-// Step of 16 heads x 64, 36 queries, 91 candidates: 12.6 -> 6.7 us (169 queries, 237 candidates: 14.6 -> 8.2);
-// 256 heads: 18.2 -> 9.7.  More work per head goes to the two launches (step_small_pays).
+// Step of 16 heads x 64, 36 queries, 91 candidates: 12.6 -> 5.9 us (169 queries, 237 candidates: 14.6 -> 7.6);
+// 256 heads: 18.2 -> 9.3.  More work per head goes to the two launches (step_small_pays).  The cluster
+// barrier without memory ordering took 0.45 us off a step, the merge in a form per number of warps 0.25.
+// Rounded probabilities (one product instead of two) where the larger kernel's would be rounded as well:
+// 5 to 15 % slower from eight turns on, the rounding costs more issue slots than the products.
 #include <algorithm>
 #include <type_traits>
 
@@ -221,8 +224,8 @@ step_small_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, const _
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  // this CTA has read what it needs of the cache
-  if (sp.ctas > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  // this CTA has read what it needs of the cache: its loads have landed, so no memory ordering is asked for
+  if (sp.ctas > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
   // ------------------------------------------------------------------ attention over the list
   const int splits = 1 << sp.log_splits, tile = warp >> sp.log_splits, split = warp & (splits - 1);
@@ -304,7 +307,7 @@ step_small_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, const _
   }
 
   // ------------------------------------------------------------------ survivors to their places in the cache
-  if (sp.ctas > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (sp.ctas > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   {
     const int share = (n_keep + sp.ctas - 1) / sp.ctas, r0 = rank * share, r1 = min(n_keep, r0 + share);
     uint4* kd = reinterpret_cast<uint4*>(kc);
@@ -337,47 +340,52 @@ step_small_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, const _
     }
   }
   __syncthreads();
-  for (int v = tid; v < sp.tiles * kTile * PIECES; v += kStepThreads) {
-    const int row = v / PIECES, c = v % PIECES, r = row % kTile, w0 = (row / kTile) << sp.log_splits;
-    if (q_first + row >= n_new) break;
-    float2 ml[kStepWarps];
-    float top = -INFINITY;
+  // four columns per thread; a form per number of warps, so that all loads of a row are in flight at once
+  auto combine = [&](auto splits_c) {
+    constexpr int S = decltype(splits_c)::value;
+    for (int v = tid; v < sp.tiles * kTile * (D / 4); v += kStepThreads) {
+      const int row = v / (D / 4), c = v % (D / 4), r = row % kTile, w0 = row / kTile * S;
+      if (q_first + row >= n_new) break;
+      float2 ml[S], f[S][2];
+      float top = -INFINITY, sum = 0.f, acc[4] = {};
 #pragma unroll
-    for (int w = 0; w < kStepWarps; ++w) {
-      ml[w] = w < splits ? row_ml[w0 + w][r] : make_float2(-INFINITY, 0.f);
-      top = fmaxf(top, ml[w].x);
-    }
-    float sum = 0.f, acc[8] = {};
+      for (int w = 0; w < S; ++w) {
+        ml[w] = row_ml[w0 + w][r];
+        const float* src = reinterpret_cast<const float*>(sm) + (size_t)(w0 + w) * kTile * D + r * D;
 #pragma unroll
-    for (int w = 0; w < kStepWarps; ++w) {
-      if (w >= splits) break;
-      const float wt = ex2(ml[w].x - top);      // 0 for a warp without keys
-      sum = fmaf(wt, ml[w].y, sum);
-      const float* src = reinterpret_cast<const float*>(sm) + (size_t)(w0 + w) * kTile * D + r * D;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 f = *reinterpret_cast<const float2*>(src + 2 * ((4 * c + e) ^ ((r & 3) << 2)));
-        acc[2 * e] = fmaf(wt, f.x, acc[2 * e]);
-        acc[2 * e + 1] = fmaf(wt, f.y, acc[2 * e + 1]);
+        for (int e = 0; e < 2; ++e) f[w][e] = *reinterpret_cast<const float2*>(src + 2 * ((2 * c + e) ^ ((r & 3) << 2)));
       }
-    }
-    const float inv = 1.f / sum;
-    uint32_t w[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const __nv_bfloat162 hh = __floats2bfloat162_rn(acc[2 * e] * inv, acc[2 * e + 1] * inv);
-      w[e] = *reinterpret_cast<const uint32_t*>(&hh);
+      for (int w = 0; w < S; ++w) top = fmaxf(top, ml[w].x);
+#pragma unroll
+      for (int w = 0; w < S; ++w) {
+        const float wt = ex2(ml[w].x - top);    // 0 for a warp without keys
+        sum = fmaf(wt, ml[w].y, sum);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          acc[2 * e] = fmaf(wt, f[w][e].x, acc[2 * e]);
+          acc[2 * e + 1] = fmaf(wt, f[w][e].y, acc[2 * e + 1]);
+        }
+      }
+      const float inv = 1.f / sum;
+      const __nv_bfloat162 h0 = __floats2bfloat162_rn(acc[0] * inv, acc[1] * inv), h1 = __floats2bfloat162_rn(acc[2] * inv, acc[3] * inv);
+      *reinterpret_cast<uint2*>(out + ((size_t)bh * n_new + q_first + row) * D + c * 4) =
+          make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
     }
-    *reinterpret_cast<uint4*>(out + ((size_t)bh * n_new + q_first + row) * D + c * 8) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
+  };
+  if (sp.log_splits == 3) combine(std::integral_constant<int, 8>());
+  else if (sp.log_splits == 2) combine(std::integral_constant<int, 4>());
+  else if (sp.log_splits == 1) combine(std::integral_constant<int, 2>());
+  else combine(std::integral_constant<int, 1>());
 }
 
 // Microseconds of this launch and of the two launches it stands for (compression, then attention).  Both
 // forms were fitted to 287 steps of 8 to 256 heads, 16 to 400 queries and 50 to 700 candidates (rms 8 and 6 %);
 // with the margin of a tenth no step of them is slower here, and none that gains a tenth is left out.
-// 16 heads x 64, 36 queries, 91 candidates: 6.7 against 12.6; 256 heads: 9.7 against 18.2; 100 queries,
-// 155 and 168 candidates: 9.0 against 12.8 (16 heads), 19.9 against 19.8 (256 heads: not taken);
-// 16 heads x 128, 36 queries, 91 candidates: 8.5 against 15.0; 256 heads: 18.8 against 25.2.
+// (Fitted before the last 0.7 us came off this side.)  16 heads x 64, 36 queries, 91 candidates: 5.9 against 12.6;
+// 256 heads: 9.3 against 18.2; 100 queries, 168 and 255 candidates: 7.3 against 12.8 (16 heads), 20.2 against
+// 19.9 (256 heads: not taken); 16 heads x 128, 36 queries, 91 candidates: 7.5 against 15.0; 256 heads: 18.6
+// against 25.2.
 template <int D>
 bool step_small_pays(const StepArgs& a, const StepShape& s, int per_sm) {
   const float sms = (float)sm_count(), heads = (float)(a.batch * a.n_heads), ctas = heads * s.ctas;

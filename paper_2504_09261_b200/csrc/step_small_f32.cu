@@ -233,8 +233,8 @@ step_small_f32_kernel(const StepArgs a, const float* __restrict__ q, const float
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  // this CTA has read what it needs of the cache
-  if (sp.ctas > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  // this CTA has read what it needs of the cache: its loads have landed, so no memory ordering is asked for
+  if (sp.ctas > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
   // ------------------------------------------------------------------ attention over the list
   const int splits = 1 << sp.log_splits, tile = warp >> sp.log_splits, split = warp & (splits - 1);
@@ -313,7 +313,7 @@ step_small_f32_kernel(const StepArgs a, const float* __restrict__ q, const float
   }
 
   // ------------------------------------------------------------------ survivors to their places in the cache
-  if (sp.ctas > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (sp.ctas > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   {
     const int share = (n_keep + sp.ctas - 1) / sp.ctas, r0 = rank * share, r1 = min(n_keep, r0 + share);
     for (int v = r0 * PIECES + tid; v < r1 * PIECES; v += kStepThreads) {
@@ -338,33 +338,40 @@ step_small_f32_kernel(const StepArgs a, const float* __restrict__ q, const float
     for (int p = 0; p < PAIRS; ++p) *reinterpret_cast<float2*>(ob + i * D + 2 * lane + 64 * p) = o[i][p];
   }
   __syncthreads();
-  for (int v = tid; v < sp.tiles * kRows * PIECES; v += kStepThreads) {
-    const int row = v / PIECES, c = v % PIECES, r = row % kRows, w0 = (row / kRows) << sp.log_splits;
-    if (q_first + row >= n_new) break;
-    float2 ml[kStepWarps];
-    float top = -INFINITY;
+  // a form per number of warps, so that all loads of a row are in flight at once
+  auto combine = [&](auto splits_c) {
+    constexpr int S = decltype(splits_c)::value;
+    for (int v = tid; v < sp.tiles * kRows * PIECES; v += kStepThreads) {
+      const int row = v / PIECES, c = v % PIECES, r = row % kRows, w0 = row / kRows * S;
+      if (q_first + row >= n_new) break;
+      float2 ml[S];
+      float4 f[S], acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      float top = -INFINITY, sum = 0.f;
 #pragma unroll
-    for (int w = 0; w < kStepWarps; ++w) {
-      ml[w] = w < splits ? row_ml[w0 + w][r] : make_float2(-INFINITY, 0.f);
-      top = fmaxf(top, ml[w].x);
-    }
-    float sum = 0.f;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int w = 0; w < S; ++w) {
+        ml[w] = row_ml[w0 + w][r];
+        f[w] = *reinterpret_cast<const float4*>(ks + ((size_t)(w0 + w) * kRows + r) * D + c * 4);
+      }
 #pragma unroll
-    for (int w = 0; w < kStepWarps; ++w) {
-      if (w >= splits) break;
-      const float wt = exp2f(ml[w].x - top);    // 0 for a warp without keys
-      sum = fmaf(wt, ml[w].y, sum);
-      const float4 f = *reinterpret_cast<const float4*>(ks + ((size_t)(w0 + w) * kRows + r) * D + c * 4);
-      acc.x = fmaf(wt, f.x, acc.x);
-      acc.y = fmaf(wt, f.y, acc.y);
-      acc.z = fmaf(wt, f.z, acc.z);
-      acc.w = fmaf(wt, f.w, acc.w);
+      for (int w = 0; w < S; ++w) top = fmaxf(top, ml[w].x);
+#pragma unroll
+      for (int w = 0; w < S; ++w) {
+        const float wt = exp2f(ml[w].x - top);  // 0 for a warp without keys
+        sum = fmaf(wt, ml[w].y, sum);
+        acc.x = fmaf(wt, f[w].x, acc.x);
+        acc.y = fmaf(wt, f[w].y, acc.y);
+        acc.z = fmaf(wt, f[w].z, acc.z);
+        acc.w = fmaf(wt, f[w].w, acc.w);
+      }
+      const float inv = 1.f / sum;
+      *reinterpret_cast<float4*>(out + ((size_t)bh * n_new + q_first + row) * D + c * 4) =
+          make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
     }
-    const float inv = 1.f / sum;
-    *reinterpret_cast<float4*>(out + ((size_t)bh * n_new + q_first + row) * D + c * 4) =
-        make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
-  }
+  };
+  if (sp.log_splits == 3) combine(std::integral_constant<int, 8>());
+  else if (sp.log_splits == 2) combine(std::integral_constant<int, 4>());
+  else if (sp.log_splits == 1) combine(std::integral_constant<int, 2>());
+  else combine(std::integral_constant<int, 1>());
 }
 
 template <int D>
