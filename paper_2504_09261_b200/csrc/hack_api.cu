@@ -790,12 +790,11 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
   }
   r = 0;
   StageScope whole(c, st, 3);
-  if (c->cfg.dtype == HACK_F32 && !any && p.n_new <= hack::kSmallQueries)
-    // nothing is evicted and the scale is small: one launch appends and attends
+  // heads of few candidates: one launch for the whole step
+  if (!merge_step) r = hack::launch_step_small(a, c->cfg.dtype, q, k, v, out, st);
+  // nothing is evicted and the scale is small: one launch appends and attends
+  if (r == 0 && c->cfg.dtype == HACK_F32 && !any && p.n_new <= hack::kSmallQueries)
     r = hack::launch_attend_small(a, c->cfg.dtype, q, k, v, out, st);
-  else if (any && !merge_step)
-    // heads of few candidates: one launch for the whole step
-    r = hack::launch_step_small(a, c->cfg.dtype, q, k, v, out, st);
   if (r < 0) return HACK_ERR_CUDA;
   if (r > 0) {
     whole.done(r);

@@ -129,8 +129,8 @@ int launch_attend_small(const StepArgs& a, int dtype, const void* q, const void*
 bool attend_small_serves(const StepArgs& a);   // bf16: the small kernel is the one for this step's attention
 constexpr int kSmallQueries = 31;
 
-// A whole step that evicts (scores, selection, attention, compaction) in one launch, for heads that fit into
-// shared memory.  1: launched; 0: outside what the kernels are for; -1: launch error.
+// A whole step (scores, selection, attention, compaction) in one launch, for heads that fit into shared memory:
+// steps that evict and, fp32, some that do not.  1: launched; 0: outside what the kernels are for; -1: launch error.
 int launch_step_small(const StepArgs& a, int dtype, const void* q, const void* k_new, const void* v_new, void* out, cudaStream_t st);
 int launch_step_small_f32(const StepArgs& a, const void* q, const void* k_new, const void* v_new, void* out, cudaStream_t st);
 

@@ -431,8 +431,10 @@ int launch_t(const StepArgs& a, const void* q, const void* k_new, const void* v_
 }  // namespace
 
 int launch_step_small(const StepArgs& a, int dtype, const void* q, const void* k_new, const void* v_new, void* out, cudaStream_t st) {
-  if (a.obs_full || a.score_accumulate || (!a.trig[0] && !a.trig[1])) return 0;
+  const bool any = a.trig[0] || a.trig[1];
+  if (a.score_accumulate || (any && a.obs_full)) return 0;
   if (dtype == HACK_F32) return launch_step_small_f32(a, q, k_new, v_new, out, st);
+  if (!any) return 0;                           // append_attend_mma_kernel has no list to go through
   return a.head_dim == 128 ? launch_t<128>(a, q, k_new, v_new, out, st) : launch_t<64>(a, q, k_new, v_new, out, st);
 }
 

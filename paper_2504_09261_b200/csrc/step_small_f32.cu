@@ -33,6 +33,11 @@ constexpr int kMaxTurns = 5;                    // groups of 32 keys of a warp w
 constexpr int kMaxCand = kMaxTurns * kKeyWarps * kKeys;   // 320
 constexpr float kLog2e = 1.4426950408889634f;
 
+// Steps that evict nothing: 16 heads x 64, 25 queries and 55 keys 9.1 -> 5.2 us, 64 heads 18.6 -> 6.2 (against a warp per
+// query); 36 queries, 91 keys 8.2 -> 5.7, 120 heads 12.9 -> 11.8 (against copy and attend_simt_kernel); 155 keys 9.8
+// against 9.3, 30 heads 10.3 against 10.8; 4 queries, 5 keys 3.2 against 4.1.
+constexpr int kMaxAppend = 96, kMinAppend = 12;
+
 template <int D>
 struct Layout {
   static constexpr int kKeyFloats = D + 4;      // padded key row
@@ -379,7 +384,7 @@ int launch_t(const StepArgs& a, const void* q, const void* k_new, const void* v_
   const int heads = a.batch * a.n_heads, tiles = (a.n_new + kRows - 1) / kRows;
   const int cand = std::max(a.heads_of[0] ? a.cand[0] : 0, a.heads_of[1] ? a.cand[1] : 0);
   const int ranked = std::max(a.trig[0] ? a.cand[0] : 0, a.trig[1] ? a.cand[1] : 0);
-  if (cand > kMaxCand || tiles > kMaxTiles * kMaxCtas) return 0;
+  if (cand > (ranked ? kMaxCand : kMaxAppend) || (!ranked && a.n_new < kMinAppend) || tiles > kMaxTiles * kMaxCtas) return 0;
   StepShape s;
   s.rows = (cand + 3) / 4 * 4;
   split_queries(s, heads, tiles);
