@@ -198,8 +198,9 @@ HACK_API hack_status_t hack_classify_heads(const double* sigma, int32_t n_layers
  * (section "KV Cache Compression for VAR": compress whenever the length exceeds the budget).
  * bf16 caches: at most two launches (one cluster launch that scores, selects and compacts, one
  * attention launch that also appends the rows of heads which keep the whole new scale).  The
- * attention of heads that do not depend on the compression runs beside it; `stream` orders everything
- * (also inside a stream capture). */
+ * attention of heads that do not depend on the compression runs beside it; steps whose heads fit into
+ * shared memory are one launch (fp32 caches too).  `stream` orders everything (also inside a stream
+ * capture). */
 HACK_API hack_status_t hack_scale_step(hack_cache_t* cache, int32_t layer, int32_t scale, const void* q,
                               const void* k, const void* v, void* out, void* stream);
 
@@ -257,7 +258,7 @@ HACK_API hack_status_t hack_stage_timing(hack_cache_t* cache, int32_t enable);
 /* Synchronises the device and returns the accumulated device time in ms and the number of kernel
  * launches per stage since timing was enabled: [0] score, [1] select, [2] compact, [3] attend.  In
  * hack_scale_step on a bf16 cache scoring, selection and compaction are one launch, counted under
- * [0]; while timing is on, the step does not run the two head types' work side by side. */
+ * [0], and a step that is one launch altogether is counted under [3]. */
 HACK_API hack_status_t hack_stage_times(hack_cache_t* cache, double* ms, uint64_t* launches);
 /* Synchronises `stream`, then reports the device status word: HACK_OK, or HACK_ERR_TIMEOUT if a
  * bounded device-side wait gave up (the word is cleared by the call). */
