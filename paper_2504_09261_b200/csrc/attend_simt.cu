@@ -94,7 +94,7 @@ attend_simt_kernel(const StepArgs a, const float* __restrict__ q, float* __restr
   float m[4], l[4];                               // l: this thread's share of the row sum
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    m[i] = -INFINITY;
+    m[i] = kNoLogit;
     l[i] = 0.f;
 #pragma unroll
     for (int c = 0; c < CV; ++c) o[i][c][0] = o[i][c][1] = make_float2(0.f, 0.f);

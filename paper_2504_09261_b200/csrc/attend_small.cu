@@ -215,7 +215,7 @@ append_attend_mma_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, 
   }
   const bool appends = blockIdx.x == 0 && total > stored && dbg_ok(total <= a.cap[ctx], a.status, 6);
   const float cs = a.sm_scale * 1.4426950408889634f;          // work in log2 units
-  float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};     // rows lane / 4 and lane / 4 + 8; l: this thread's share
+  float m[2] = {kNoLogit, kNoLogit}, l[2] = {0.f, 0.f};     // rows lane / 4 and lane / 4 + 8; l: this thread's share
   float o[D / 8][4];
 #pragma unroll
   for (int n = 0; n < D / 8; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;

@@ -426,7 +426,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       const uint32_t p_addr = tmem + lane_addr + P_COL + t * 64;
       const uint32_t o_addr = tmem + lane_addr + O_COL + t * D;
       const float c = p.scale_log2;
-      float m_used = -INFINITY, l = 0.f;
+      float m_used = kNoLogit, l = 0.f;
       bool ok = true;
       for (int j = 0; j < nblk; ++j) {
         ok = __all_sync(0xffffffffu, wait_bar(&bars->s_full[t], j & 1, bars, p.status, 8, wlim));

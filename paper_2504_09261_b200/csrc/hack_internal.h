@@ -134,6 +134,10 @@ constexpr int kSmallQueries = 31;
 int launch_step_small(const StepArgs& a, int dtype, const void* q, const void* k_new, const void* v_new, void* out, cudaStream_t st);
 int launch_step_small_f32(const StepArgs& a, const void* q, const void* k_new, const void* v_new, void* out, cudaStream_t st);
 
+// Start of a running softmax maximum.  Finite, so that logits of -inf (products that overflow) weigh nothing even
+// where they are all that a tile, or the share of a warp, has: -inf - (-inf) is no number.
+constexpr float kNoLogit = -3.402823466e38f;
+
 constexpr int kTcMinQueries = 32;   // below this the small kernel serves every bf16 step
 
 void set_error(const std::string& msg);

@@ -230,7 +230,7 @@ step_small_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, const _
   // ------------------------------------------------------------------ attention over the list
   const int splits = 1 << sp.log_splits, tile = warp >> sp.log_splits, split = warp & (splits - 1);
   const float cs = a.sm_scale * 1.4426950408889634f;
-  float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};     // rows lane / 4 and lane / 4 + 8; l: this thread's share
+  float m[2] = {kNoLogit, kNoLogit}, l[2] = {0.f, 0.f};     // rows lane / 4 and lane / 4 + 8; l: this thread's share
   float o[D / 8][4];
 #pragma unroll
   for (int n = 0; n < D / 8; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;

@@ -247,7 +247,7 @@ step_small_f32_kernel(const StepArgs a, const float* __restrict__ q, const float
   float2 o[kRows][PAIRS];
 #pragma unroll
   for (int i = 0; i < kRows; ++i) {
-    m[i] = -INFINITY;
+    m[i] = kNoLogit;
     l[i] = 0.f;                                 // this lane's share
 #pragma unroll
     for (int p = 0; p < PAIRS; ++p) o[i][p] = make_float2(0.f, 0.f);
