@@ -219,7 +219,7 @@ HACK_API hack_status_t hack_scale_step(hack_cache_t* cache, int32_t layer, int32
  * No cudaMalloc, cudaFree or other allocating call is made.  The first call on a device is a
  * set-up call: it resolves the array's address (cudaGetSymbolAddress) and, because CUDA loads a
  * module's device image lazily, it is also the moment the driver reserves those 8.3 MiB on that
- * device.  Make it at start-up, before the caller's own pool claims the rest of the memory and
+ * device and loads the kernels, those of every size and dtype.  Make it at start-up, before the caller's own pool claims the rest of the memory and
  * before any stream capture; every later call on that device leaves the device's memory as it is.
  * All calls share the array: calls that overlap on the GPU race, so keep them on one stream or
  * order them yourself.  Only enqueues; does not synchronise. */

@@ -10,9 +10,11 @@
 // fixed array that lives in the library's own device image.
 //
 // The array (kScratchFloats floats, about 8.3 MiB) is part of the module: every GPU that loads
-// the library holds it until the process exits.  CUDA loads the module's device image lazily, so
-// the driver reserves it on a device during the first call made there (the set-up call, to be made
-// at start-up); no later call changes the device's memory.  All calls share it and it keeps the previous
+// the library holds it until the process exits.  CUDA loads the module's data and every kernel of it
+// lazily, so the first call made on a device (the set-up call, to be made at start-up) asks for the
+// array and for all kernels of this file, whatever its own sizes and type need: which kernel a call
+// runs depends on both, and a kernel that is first used later would be loaded then.  No later call
+// changes the device's memory.  All calls share the array and it keeps the previous
 // call's contents; nothing in it has to start at zero because pass 1 overwrites every element
 // pass 2 reads.  Two calls that overlap on the GPU (different streams, or different host threads
 // without ordering) race on it: serialise them.
@@ -93,6 +95,34 @@ noalloc_cluster_kernel(const DenseArgs a, const T* __restrict__ q, const T* __re
 std::mutex g_setup_mutex;
 float* g_scratch_ptr[64] = {nullptr};
 
+// Set-up of one kernel on the current device: loaded, and its shared memory opted in to.
+template <typename F>
+bool load(F* kern, size_t smem) {
+  cudaFuncAttributes attr;
+  const cudaError_t e = cudaFuncGetAttributes(&attr, reinterpret_cast<const void*>(kern));
+  if (e != cudaSuccess) {
+    set_error(std::string("cudaFuncGetAttributes: ") + cudaGetErrorString(e));
+    return false;
+  }
+  return smem == 0 || allow_dynamic_smem(kern, smem);
+}
+// Every kernel a call with this type and head_dim can run.
+template <typename T, int D>
+bool load_kernels() {
+  if (!load(noalloc_logits_kernel<T, D>, simt::logits_smem_bytes<T, D>())) return false;
+  if constexpr (sizeof(T) == 4) {
+    return load(noalloc_cluster_kernel<T, D, 1>, simt::fused_f32_smem<D>());
+  } else {
+    return load(noalloc_cluster_kernel<T, D, 1>, simt::fused_bf16_smem<D, 1>()) &&
+           load(noalloc_cluster_kernel<T, D, 2>, simt::fused_bf16_smem<D, 2>()) &&
+           load(noalloc_cluster_kernel<T, D, 4>, simt::fused_bf16_smem<D, 4>());
+  }
+}
+bool load_all_kernels() {
+  return load(noalloc_reduce_kernel, 0) && load_kernels<float, 64>() && load_kernels<float, 128>() &&
+         load_kernels<__nv_bfloat16, 64>() && load_kernels<__nv_bfloat16, 128>();
+}
+
 template <typename T, int D>
 cudaError_t run(const DenseArgs& a, int n_rows, const void* q, const void* k, float* scratch,
                 float* scores, int score_stride, cudaStream_t st) {
@@ -154,7 +184,8 @@ extern "C" hack_status_t hack_score_noalloc(const void* q, const void* k_cand, f
   {
     std::lock_guard<std::mutex> lock(g_setup_mutex);
     if (!g_scratch_ptr[dev]) {
-      // set-up, once per device, with that device current: resolve the array's device address
+      // set-up, once per device, with that device current: load the kernels and resolve the array's address
+      if (!load_all_kernels()) return HACK_ERR_CUDA;       // text recorded
       float* ptr = nullptr;
       e = cudaGetSymbolAddress((void**)&ptr, g_noalloc_scratch);
       if (e != cudaSuccess || !ptr) {

@@ -9,6 +9,9 @@ in a row share the library's fixed scratch, so the second call also shows that s
 the first do no harm, and the device's free memory must not move across the second call.  Collected
 last so that a failure here cannot hide the result of any other test.
 """
+import os
+import subprocess
+import sys
 from dataclasses import replace
 
 import numpy as np
@@ -129,3 +132,60 @@ def test_noalloc_rejects_sizes_beyond_the_fixed_scratch():
     with pytest.raises(hb.HackError) as e:
         hb.hack_score_noalloc(q, None, q, 1, 1, 1, 1, 64, hb.HACK_F32)
     assert e.value.status == 1
+
+
+_OTHER_SIZES = """
+import sys
+import torch
+import paper_2504_09261_b200 as hb
+
+torch.cuda.set_device(0)
+stream = torch.cuda.Stream()
+sizes = [(14, 1100), (14, 2000), (14, 4097), (3, 600), (200, 320)]          # (row-blocks, candidates)
+work = []
+for dt, code in ((torch.bfloat16, hb.HACK_BF16), (torch.float32, hb.HACK_F32)):
+    for dim in (64, 128):
+        for rows, cand in sizes:
+            q = torch.randn((rows, 40, dim), device="cuda").to(dt)
+            k = torch.randn((rows, cand, dim), device="cuda").to(dt)
+            work.append((q, k, torch.zeros((rows, cand), device="cuda"), rows, 40, cand, cand, dim, code))
+
+def call(w, out=None):
+    hb.hack_score_noalloc(w[0], w[1], w[2] if out is None else out, *w[3:], stream=stream.cuda_stream)
+
+small = torch.zeros((2, 40, 64), device="cuda")
+call((small, small, torch.zeros((2, 40), device="cuda"), 2, 40, 40, 40, 64, hb.HACK_F32))      # the set-up call
+torch.cuda.synchronize()
+if sys.argv[1] == "plain":
+    # the figure is device-wide, so a change is given two more fresh processes before it counts
+    free = torch.cuda.mem_get_info()[0]
+    for w in work:
+        call(w)
+    torch.cuda.synchronize()
+    moved = free - torch.cuda.mem_get_info()[0]
+    print("moved", moved)
+    sys.exit(0 if moved == 0 else 3)
+graph = torch.cuda.CUDAGraph()
+with torch.cuda.graph(graph, stream=stream):
+    for w in work:
+        call(w)
+graph.replay()
+torch.cuda.synchronize()
+for w in work:
+    again = torch.zeros_like(w[2])
+    call(w, again)
+    torch.cuda.synchronize()
+    assert torch.equal(again, w[2])
+"""
+
+
+@pytest.mark.parametrize("mode", ["plain", "capture"])
+def test_the_first_call_sets_up_for_every_size_and_type(mode):
+    """A process whose first call is a small fp32 one: calls that run every other kernel of the entry
+    point leave the device's free memory as it is, and may be made for the first time inside a capture."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    for attempt in range(3 if mode == "plain" else 1):
+        res = subprocess.run([sys.executable, "-c", _OTHER_SIZES, mode], cwd=root, capture_output=True, text=True, timeout=300)
+        if res.returncode == 0:
+            break
+    assert res.returncode == 0, (res.stdout + res.stderr)[-2000:]
