@@ -376,6 +376,7 @@ append_attend_mma_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, 
 bool attend_small_serves(const StepArgs& a) {
   if (!attend_tc_serves(a, HACK_BF16)) return true;
   const int heads = a.batch * a.n_heads, keys = a.kept[0] > a.kept[1] ? a.kept[0] : a.kept[1];
+  if (heads > 65535) return false;              // the heads are the second dimension of its grid
   const float sms = (float)sm_count();
   const int ctas = heads * ((a.n_new + kMmaRows - 1) / kMmaRows);
   const int turns = (keys + 4 * kMmaRows - 1) / (4 * kMmaRows);
