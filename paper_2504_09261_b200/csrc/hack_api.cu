@@ -190,9 +190,11 @@ hack::StepArgs make_args(const hack_cache* c, int layer, int scale, const hack_s
   a.cand[0] = p.cand_s;     a.cand[1] = p.cand_c;
   a.kept[0] = p.kept_s;     a.kept[1] = p.kept_c;
   a.cap[0] = c->cap[0];     a.cap[1] = c->cap[1];
-  a.trig[0] = p.triggered_s; a.trig[1] = p.triggered_c;
   a.heads_of[1] = c->cfg.batch * c->n_ctx_heads[layer];
   a.heads_of[0] = c->cfg.batch * c->cfg.n_heads - a.heads_of[1];
+  // a type that has no heads in this layer evicts nothing, whatever its budget
+  a.trig[0] = p.triggered_s && a.heads_of[0] > 0;
+  a.trig[1] = p.triggered_c && a.heads_of[1] > 0;
   a.n_obs_rows = p.n_obs_rows;
   // the query subset of Eq. 9: uniform spacing, or one of the ablation's alternatives
   a.obs_first = c->cfg.obs_sampler == HACK_OBS_RECENT ? p.n_new - p.n_obs_rows : 0;
@@ -644,9 +646,9 @@ hack_status_t hack_select(hack_cache_t* c, int32_t layer, int32_t scale, const f
 
 // Compaction of one step; with merge_last, at the last scale, wrapped in the merge of what the
 // contextual heads discard.  Returns the number of launches, or -1.
-static int compact_stage(hack_cache* c, const hack::StepArgs& a, const hack_step_info_t& p, int scale,
+static int compact_stage(hack_cache* c, const hack::StepArgs& a, int scale,
                          const int32_t* idx, int idx_all, const void* k_new, const void* v_new, cudaStream_t st) {
-  const bool merge = c->cfg.merge_last && scale == c->cfg.n_scales - 1 && p.triggered_c && idx;
+  const bool merge = c->cfg.merge_last && scale == c->cfg.n_scales - 1 && a.trig[1] && idx;
   int n = 0, r;
   if (merge) {
     if ((r = hack::launch_merge_prepare(a, c->merge, idx, k_new, v_new, st)) < 0) return -1;
@@ -672,7 +674,7 @@ hack_status_t hack_compact(hack_cache_t* c, int32_t layer, int32_t scale, const 
   plan_step(c, c->layers[layer], scale, &p);
   const hack::StepArgs a = make_args(c, layer, scale, p);
   StageScope ts(c, (cudaStream_t)stream, 2);
-  const int n = compact_stage(c, a, p, scale, idx, 1, k_new, v_new, (cudaStream_t)stream);
+  const int n = compact_stage(c, a, scale, idx, 1, k_new, v_new, (cudaStream_t)stream);
   if (n < 0) return HACK_ERR_CUDA;   // text recorded by the launcher
   ts.done(n);
   c->launches += n;
@@ -774,19 +776,19 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
   if (c->cfg.obs_sampler == HACK_OBS_CALLER && (p.triggered_c || p.triggered_s) && !c->obs_rows_set[scale])
     return fail(HACK_ERR_STATE, "HACK_OBS_CALLER: no observation rows were set for this scale (hack_set_obs_rows)");
   hack::StepArgs a = make_args(c, layer, scale, p);
-  const bool any = p.triggered_c || p.triggered_s;
+  const bool any = a.trig[0] || a.trig[1];
   int n = 0, r;
   // The bf16 attention kernels take the rows of a head type that keeps the whole new scale straight
   // from the caller's K/V and append them themselves: types that evict nothing in this step, and
   // structural heads whose latest scale is protected (Eq. 11).  Contextual heads that evict rank the
   // new rows as well (Eq. 10) and are compacted first.  The final-scale merge keeps the separate
   // compaction it is wrapped around, and so do steps that evict with fewer new rows than one TMA box.
-  const bool merge_step = c->cfg.merge_last && scale == c->cfg.n_scales - 1 && p.triggered_c;
+  const bool merge_step = c->cfg.merge_last && scale == c->cfg.n_scales - 1 && a.trig[1];
   const bool boxes = (long long)c->cfg.batch * c->cfg.n_heads * p.n_new >= 128;
   const bool fused_append = c->cfg.dtype == HACK_BF16 && !merge_step && (!any || boxes);
   if (fused_append) {
-    a.seg_new[0] = !p.triggered_s || a.protect_new;
-    a.seg_new[1] = !p.triggered_c;
+    a.seg_new[0] = !a.trig[0] || a.protect_new;
+    a.seg_new[1] = !a.trig[1];
   }
   r = 0;
   StageScope whole(c, st, 3);
@@ -847,7 +849,7 @@ hack_status_t hack_scale_step(hack_cache_t* c, int32_t layer, int32_t scale, con
   }
   if (((any && !compressed) || !fused_append) && !moved) {      // a step that only appends needs no launch ahead of the fused attention
     StageScope ts(c, st, 2);
-    if ((r = compact_stage(c, a, p, scale, any ? c->idx : nullptr, any ? 1 : 0, k, v, st)) < 0) return any ? poison(c) : HACK_ERR_CUDA;
+    if ((r = compact_stage(c, a, scale, any ? c->idx : nullptr, any ? 1 : 0, k, v, st)) < 0) return any ? poison(c) : HACK_ERR_CUDA;
     ts.done(r);
     n += r;
   }
