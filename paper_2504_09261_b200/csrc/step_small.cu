@@ -381,8 +381,8 @@ step_small_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, const _
 
 // Microseconds of this launch and of the two launches it stands for (compression, then attention).  Both
 // forms were fitted to 287 steps of 8 to 256 heads, 16 to 400 queries and 50 to 700 candidates (rms 8 and 6 %);
-// with the margin of a tenth no step of them is slower here, and none that gains a tenth is left out.
-// (Fitted before the last 0.7 us came off this side.)  16 heads x 64, 36 queries, 91 candidates: 5.9 against 12.6;
+// with the margin of a tenth none of them was slower here.  The fit is from before the last 0.7 us came off
+// this side, so the line errs towards the two launches: steps just beyond it would gain up to a fifth here.  16 heads x 64, 36 queries, 91 candidates: 5.9 against 12.6;
 // 256 heads: 9.3 against 18.2; 100 queries, 168 and 255 candidates: 7.3 against 12.8 (16 heads), 20.2 against
 // 19.9 (256 heads: not taken); 16 heads x 128, 36 queries, 91 candidates: 7.5 against 15.0; 256 heads: 18.6
 // against 25.2.
@@ -424,8 +424,10 @@ int launch_t(const StepArgs& a, const void* q, const void* k_new, const void* v_
   auto go = [&](auto kern) { return launch_step<__nv_bfloat16>(kern, a, s, smem, q, k_new, v_new, out, st); };
   if (turns <= 1) return go(step_small_kernel<D, 1>);
   if (turns <= 2) return go(step_small_kernel<D, 2>);
-  if (turns <= 4) return go(step_small_kernel<D, 4>);
-  return go(step_small_kernel<D, kMaxTurns>);
+  if constexpr (D == 64) {                      // at head_dim 128 shared memory holds fewer rows than four turns rank
+    if (turns > 4) return go(step_small_kernel<D, kMaxTurns>);
+  }
+  return go(step_small_kernel<D, 4>);
 }
 
 }  // namespace

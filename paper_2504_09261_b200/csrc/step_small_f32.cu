@@ -394,8 +394,10 @@ int launch_t(const StepArgs& a, const void* q, const void* k_new, const void* v_
   if (smem > kSmemCta || (cand > 2 * kKeyWarps * kKeys && heads * s.ctas > sm_count())) return 0;
   auto go = [&](auto kern) { return launch_step<float>(kern, a, s, smem, q, k_new, v_new, out, st); };
   if (ranked <= 2 * kKeyWarps * kKeys) return go(step_small_f32_kernel<D, 2>);
-  if (ranked <= 4 * kKeyWarps * kKeys) return go(step_small_f32_kernel<D, 4>);
-  return go(step_small_f32_kernel<D, kMaxTurns>);
+  if constexpr (D == 64) {                      // at head_dim 128 shared memory holds fewer rows than four turns rank
+    if (ranked > 4 * kKeyWarps * kKeys) return go(step_small_f32_kernel<D, kMaxTurns>);
+  }
+  return go(step_small_f32_kernel<D, 4>);
 }
 
 }  // namespace
