@@ -37,6 +37,7 @@ class ParityReport:
     max_score_err: float = 0.0          # max of |d| / (max(|s|,|s^|) + atol/rtol)
     max_out_abs: float = 0.0
     max_out_abs_fused: float = 0.0
+    evicting_launches: List[int] = field(default_factory=list)   # launches of every fused step that evicts
     jaccard: List[float] = field(default_factory=list)   # free-running oracle vs GPU, per compressed (step, head)
     problems: List[str] = field(default_factory=list)
 
@@ -146,7 +147,10 @@ def run_parity(cfg: WorkloadConfig, layers: Sequence[int], fused: bool = False,
             staged.hack_attend(l, k, qd, out)
             if fused:
                 out_f = torch.full_like(qd, float("nan"))
+                before = twin.hack_launch_count()
                 twin.hack_scale_step(l, k, qd, kd, vd, out_f)
+                if info.triggered_c or info.triggered_s:
+                    rep.evicting_launches.append(twin.hack_launch_count() - before)
             torch.cuda.synchronize()
             staged.hack_poll_status()
             s_h = scores.cpu().numpy()

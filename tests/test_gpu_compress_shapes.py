@@ -1,6 +1,8 @@
-"""The compression launch in the shapes its dispatch rule can choose: two CTAs per SM (more heads than
-SMs), candidate lists past the accumulators in tensor memory (bounce accumulators, logits in shared
-memory), clusters that are not powers of two, and a select that has to settle ties in its last digit.
+"""The compression launch at sizes for which its dispatch rule has different shapes to choose from: more
+heads than SMs (two CTAs per SM), candidate lists past the accumulators in tensor memory (bounce accumulators,
+logits in shared memory or formed again), few heads of long lists (clusters), and a select that has to settle
+ties in its last digit.  That the compression launch is the one that runs is asserted (the last step is two launches);
+which shape the rule, a time model, takes for it is not visible from here.
 Oracle and bars are those of the parity tests."""
 from dataclasses import replace
 
@@ -19,7 +21,7 @@ def _built():
 
 
 @pytest.mark.parametrize("base,heads,batch,sides,b_c,b_s,policy", [
-    (1, 20, 16, (1, 2, 5, 9, 13, 16), 68, 400, 0),          # 320 heads of up to 6 chunks: two CTAs per SM
+    (1, 20, 16, (1, 2, 5, 9, 13, 16), 68, 400, 0),          # 320 heads of up to 6 chunks
     (3, 30, 8, (1, 3, 7, 12, 19), 130, 257, 1),             # the same at head_dim 128, current scale competes
     (1, 15, 12, (1, 4, 9, 25, 41), 700, 1300, 0),           # 180 heads, lists past the accumulators of one CTA
     (3, 30, 5, (1, 4, 13, 29, 37), 900, 2100, 0),           # the same at head_dim 128: logits formed a second time
@@ -32,6 +34,7 @@ def test_launch_shapes(base, heads, batch, sides, b_c, b_s, policy):
     rep = run_parity(cfg, [0], fused=True, heads_per_layer=6, policy=policy, gen_on_gpu=True)
     assert rep.ok(), rep.problems[:5]
     assert rep.compressed_heads > 0
+    assert rep.evicting_launches[-1] == 2, rep.evicting_launches
 
 
 @pytest.mark.parametrize("head_dim,heads", [(64, 2), (128, 200)])

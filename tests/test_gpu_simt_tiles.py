@@ -89,3 +89,4 @@ def test_selection_that_moves_the_rows(head_dim, b_c, b_s, policy):
     rep = run_parity(cfg, [0], fused=True, policy=policy)
     assert rep.ok(), rep.problems[:5]
     assert rep.compressed_heads > 0
+    assert rep.evicting_launches[-1] == 3, rep.evicting_launches      # scores, selection with the moves, attention

@@ -60,6 +60,7 @@ def test_whole_step_in_one_launch(base, heads, batch, sides, b_c, b_s, policy):
     rep = run_parity(cfg, [0], fused=True, policy=policy)
     assert rep.ok(), rep.problems[:5]
     assert rep.compressed_heads > 0
+    assert set(rep.evicting_launches) == {1}, rep.evicting_launches
 
 
 @pytest.mark.parametrize("head_dim", [64, 128])
@@ -98,7 +99,7 @@ def test_equal_scores_in_one_launch(head_dim):
 @pytest.mark.parametrize("head_dim,heads,batch,sides,b_c,b_s,policy", [
     (64, 5, 1, (1, 2, 3, 5, 7), 29, 63, 0),                 # up to two groups of 32 keys per warp, ragged last tile
     (64, 16, 1, (1, 2, 6, 10, 10), 87, 156, 1),             # 187 and 256 candidates: four groups
-    (64, 9, 2, (1, 2, 7, 11, 15), 95, 95, 0),               # 320 candidates: five, the largest served
+    (64, 9, 2, (1, 2, 7, 11, 15), 95, 95, 1),               # 320 candidates: five, the largest served
     (64, 30, 5, (1, 2, 4, 6), 39, 41, 0),                   # 150 heads, two CTAs per SM
     (64, 7, 3, (5, 5, 1, 1, 4), 20, 33, 1),                 # steps of a single token that evict
     (128, 6, 2, (1, 3, 5, 8, 9), 1, 97, 0),                 # head_dim 128; contextual heads keep one row
@@ -112,3 +113,4 @@ def test_whole_fp32_step_in_one_launch(head_dim, heads, batch, sides, b_c, b_s, 
     rep = run_parity(cfg, [0], fused=True, policy=policy)
     assert rep.ok(), rep.problems[:5]
     assert rep.compressed_heads > 0
+    assert set(rep.evicting_launches) == {1}, rep.evicting_launches
