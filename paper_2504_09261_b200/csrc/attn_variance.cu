@@ -15,7 +15,7 @@
 // end the thread holds Var_i A[i, j] = sum p^2 / N - (sum p / N)^2 of its key; the CTA adds its 128
 // variances and a second, tiny kernel adds the blocks of a head in a fixed order.
 // Two blocks per CTA halve the query traffic: with one block per CTA (two CTAs per SM) the launch ran at the
-// L2's rate of about 21 bytes per clock and SM.  32 heads x 4 096 queries x 10 521 keys x 128: 643 -> 610 us.
+// L2's rate of about 21 bytes per clock and SM.  32 heads x 4 096 queries x 10 521 keys x 128: 514 -> 482 us.
 // Every mbarrier wait is bounded; on expiry the CTA raises the status word and winds down.
 #include <cuda.h>
 
