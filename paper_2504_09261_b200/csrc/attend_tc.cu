@@ -4,7 +4,11 @@
 //
 // One CTA serves one (batch, head) and up to two 128-row query tiles, which take turns on the
 // tensor pipe so that the softmax of one tile overlaps the MMAs of the other (T = 2); or, at head_dim
-// 64 and short caches, one tile on half an SM (T = 1: no warps 8-11, half the tensor memory).
+// 64 and short caches, one tile on half an SM (T = 1: no warps 8-11, half the tensor memory).  A unit of work
+// is a head and its one or two tiles (heads whose keys are one block: several rounds of them); where there are
+// more units than CTAs run at once, a CTA that nears the end of its unit takes over one that has not
+// been launched yet (cluster launch control): its loads and first products run under the last softmax and the
+// epilogue of the unit before, and tensor memory, barriers and registers are set up once.
 //   warp  0     : issuer of the Q K^T products; also owns the TMEM allocation
 //   warp  1     : TMA producer (K and V tiles of 128 cache rows through rings)
 //   warp  2     : issuer of the P V products (a single issuing thread for both products was the
@@ -22,10 +26,13 @@
 //    softmax warps per scheduler, normally only one of them active) rather than more, lighter
 //    threads, and as few softmax instructions as possible: scale / sum / max work runs on packed
 //    or 3-input instructions.
-//  * Exponentials are scarce (16 per clock and SM against 8192 tensor flops): kPolyOf8 of every
-//    8 pairs can be evaluated with a cubic on the FMA pipe instead.  Two of eight made the loop
-//    2.4 % faster, but a probability from the cubic can round to the other bf16 neighbour than
-//    the one the row-sum correction below assumes, which cost 5e-3 of output accuracy: off.
+//  * The instruction cache: with every wait and every loop of the issuing warps unrolled the units made 82 KB of
+//    code and the warps waited for instructions 1.8 cycles per issue instead of 0.5 (head_dim 64: 112 -> 120 us
+//    a step).  Waits are small, the issuers' loops rolled, rare code is out of the way of the loop over the blocks.
+//  * Work for padding: the last block of a segment is formed and weighted in groups of 32 keys.
+// Measured (a step with its compression, before -> with units, groups of 32 and rolled loops): 240 heads x 64,
+// 1 024 queries, 1 045 keys 115 -> 110 us; 256 heads x 64, 256 queries, 612 keys 38.9 -> 37.4; 32 heads x 128,
+// 4 096 queries, 4 208 and 2 104 keys 191 -> 187.
 // TMEM (512 columns): S [0,128)  P0 [128,192)  P1 [192,256)  O0 [256,256+D)  O1 [256+D,256+2D).
 // There is ONE logit buffer, which the two tiles use in turn, and a probability buffer per tile.  A
 // softmax thread reads its whole logit row into registers first and hands the buffer back at once
@@ -51,9 +58,11 @@
 // launch gives it: heads of a type the step does not compress for nothing, heads that keep the whole
 // new scale for their stored survivors, which come last, and only evicting contextual heads for
 // everything.  Their CTAs lead the grid and start on the SMs the compression leaves free.
-// A tile's output rows leave through the shared memory of its query tile (free once the last Q K^T
-// product has read it) and one tiled store per 64 columns; the store's 3-D tensor map of the output
-// clips the rows behind a head's last query.
+// A thread writes its output row from tensor memory, a whole 32-byte sector an instruction: the query tile's shared
+// memory is free for the next unit's queries as soon as the last Q K^T product has read it.  (Tried: the output
+// of a unit under the first block of the next one, in the wait for P: 1 to 2 % slower, the loop carries the code.
+// Last units cut into pieces of their keys that the last one to finish adds up: 6 us per piece for the
+// exchange through memory, more than the shorter last round gains.)
 // Every mbarrier wait is bounded; on expiry the CTA raises the status word, drains what it has in
 // flight, frees its TMEM and returns.
 #include <cuda.h>
@@ -83,7 +92,6 @@ template <> struct Shape<1> {
   static constexpr int kThreads = 256, kCtasPerSm = 2, kSoftmaxRegs = 200, kOtherRegs = 56;
   static constexpr uint32_t kTmemCols = 256, kOutCol = 192, kCopyChunk = 8192;
 };
-constexpr int kPolyOf8 = 0;              // pairs out of 8 whose 2^x runs on the FMA pipe
 constexpr int kKStages = 2;
 constexpr int kVStages = 2;
 constexpr uint32_t kSpinLimit = 1u << 22;          // polls while draining after an abort
@@ -92,8 +100,11 @@ constexpr float kRescaleThreshold = 32.0f;   // log2 units: p <= 2^32, far insid
 struct TcParams {
   int n_new;
   int first_type, first_heads;           // the head type at the front of head_order and its heads
-  int first_ctas;                        // its CTAs; the other type's follow
-  int n_pairs[2], tiles_per_cta[2];      // per head type: CTAs per head, query tiles per CTA (2, or 1)
+  int first_units;                       // its units; the other type's follow
+  int units_per_head[2];                 // per head type
+  int tiles_per_cta[2];                  // per head type: query tiles of a round (2, or 1)
+  int rounds[2];                         // per head type: rounds of a unit (1 unless the keys are one block)
+  int steal;                             // more units than CTAs run at once: a CTA goes on with another one
   int len_a[2], len_b[2];                // per head type: rows read from the cache, rows read from the caller's K/V
   int append_new;                        // heads with len_b > 0 also store those rows behind their len_a cache rows
   int dep[2];                            // per head type: what lies behind the dependency wait (kDep*)
@@ -111,6 +122,7 @@ struct TcParams {
   const int32_t* row_off;
   const int32_t* head_order;             // the heads of first_type, then the others
   __nv_bfloat16* out;
+  int out_sectors;                       // the output starts on a 32-byte boundary
   float* row_stats;                      // optional [b*H, N_k, 2]: reference maximum and sum of every softmax row
   int* status;
 };
@@ -120,40 +132,45 @@ constexpr int kDepNothing = 0;           // nothing that launch touches: it comp
 constexpr int kDepCache = 1;             // the cache rows (and the place of the append); the new rows are the caller's
 constexpr int kDepAll = 2;
 
+// A piece of work: one head, some of its query tiles (`rounds` rounds of up to two).
+struct Unit { int bh, part, type, krow; };
+
 struct Bars {
-  uint64_t q_full[2];
+  uint4 answer;                                     // of cluster launch control
+  Unit unit[2];                                     // units of even and odd count; bh < 0: there is no more
+  uint64_t u_full[2], u_empty[2], asked;
+  uint64_t q_full[2], q_free[2];
   uint64_t k_full[kKStages], k_empty[kKStages];
   uint64_t v_full[kVStages], v_empty[kVStages];
-  uint64_t s_full[2], s_free, p_full[2], p_free[2], o_final[2];
+  uint64_t s_full[2], s_free, p_full[2], p_free[2];
   uint64_t copy_full[2];                            // append: a chunk of new rows has landed in its staging half
   uint64_t drain, drain2;
+  int2 out_at[8];                                   // per softmax warp
   uint32_t tmem_base;
-  int abort_flag;
+  int abort_code;                                   // of the wait that gave up
 };
 
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Bars* b, int* status, int code,
-                                         long long limit) {
+// Waits for a phase of a barrier; false once the limit has passed or another wait of the CTA has given up.  In
+// little code: the instruction cache bounds this kernel (with waits of 40 instructions, 82 instead of 40 KB in
+// all, the loop lost 40 % at head_dim 64).  The status word is written at the end, by one thread.
+__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Bars* b, int code, long long limit) {
   const uint32_t addr = smem_u32(bar);
-  if (mbar_try_wait(addr, parity)) return true;
+  if (__builtin_expect(mbar_try_wait(addr, parity), 1)) return true;
+  volatile int* const flag = &b->abort_code;
   const long long t0 = clock64();
-  for (uint32_t it = 0;; ++it) {
-    if (mbar_try_wait(addr, parity)) return true;
-    if ((it & 63u) == 63u) {
-      if (*reinterpret_cast<volatile int*>(&b->abort_flag)) return false;
-      if (clock64() - t0 > limit) break;
-    }
+#pragma unroll 1
+  while (!mbar_try_wait(addr, parity)) {
+    if (*flag) return false;
+    if (clock64() - t0 > limit) *flag = code;
   }
-  *reinterpret_cast<volatile int*>(&b->abort_flag) = 1;
-  atomicExch(status, code);
-  return false;
+  return true;
 }
 
 template <int D, int T>
 __global__ void __launch_bounds__(Shape<T>::kThreads, Shape<T>::kCtasPerSm)
 attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kn,
-                 const __grid_constant__ CUtensorMap tm_vn, const __grid_constant__ CUtensorMap tm_o,
-                 const TcParams p) {
+                 const __grid_constant__ CUtensorMap tm_vn, const TcParams p) {
   constexpr int SUB = D / 64;                       // 64-column (128-byte) sub-tiles per row
   constexpr uint32_t SUB_BYTES = kBN * 128;         // one sub-tile: 128 rows x 128 bytes
   constexpr uint32_t TILE_BYTES = SUB * SUB_BYTES;
@@ -173,75 +190,93 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   Bars* bars = reinterpret_cast<Bars*>(sm + (T + kKStages + kVStages) * TILE_BYTES + 2 * kCopyChunk);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // CTAs of the first head type, then those of the other one
-  const bool second = (int)blockIdx.x >= p.first_ctas;
-  const int type = second ? 1 - p.first_type : p.first_type;
-  const int cta = second ? blockIdx.x - p.first_ctas : blockIdx.x;
-  const int n_pairs = p.n_pairs[type];
-  const int bh = p.head_order[(second ? p.first_heads : 0) + cta / n_pairs];
-  const int pair = cta % n_pairs;
-  const int dep = p.dep[type];
-  const int len_a = p.len_a[type], len_b = p.len_b[type];
-  const int nblk_b = (len_b + kBN - 1) / kBN;             // the caller's rows come first: they may not have to wait
-  const int nblk = nblk_b + (len_a + kBN - 1) / kBN;      // >= 1: a head never attends over nothing
-  const int q0 = pair * p.tiles_per_cta[type] * kBM;
-  const int ntile = T == 2 && p.tiles_per_cta[type] == 2 && q0 + kBM < p.n_new ? 2 : 1;
-
-  const int qrow = bh * p.n_new + q0;
-  const int krow = p.row_off[bh];
-  const int nrow = bh * p.n_new;
   const long long wlim = p.wait_cycles;
-  // K / V tile j of this head: which tensor it comes from and its first row there
-  auto k_src = [&](int j) { return j < nblk_b ? &tm_kn : &tm_k; };
-  auto v_src = [&](int j) { return j < nblk_b ? &tm_vn : &tm_v; };
-  auto tile_row = [&](int j) { return j < nblk_b ? nrow + j * kBN : krow + (j - nblk_b) * kBN; };
+
+  // Unit number x of the launch: those of the first head type, then those of the other one.
+  auto make_unit = [&](int x) {
+    Unit u;
+    const bool second = x >= p.first_units;
+    u.type = second ? 1 - p.first_type : p.first_type;
+    const int at = second ? x - p.first_units : x, per = p.units_per_head[u.type];
+    const int head = at / per;
+    u.part = at - head * per;
+    u.bh = p.head_order[(second ? p.first_heads : 0) + head];
+    u.krow = p.row_off[u.bh];
+    return u;
+  };
+  // A role takes unit number n of this CTA (one thread; the arrival gives the slot back).
+  auto wait_unit = [&](int n) { return wait_bar(&bars->u_full[n & 1], (n >> 1) & 1, bars, 13, wlim); };
+  auto read_unit = [&](int n) {
+    const volatile Unit& v = bars->unit[n & 1];
+    return Unit{v.bh, v.part, v.type, v.krow};
+  };
+  auto give_unit = [&](int n) { mbar_arrive(smem_u32(&bars->u_empty[n & 1])); };
+  // Its rounds, and in a round: the first query row and the tiles
+  auto rounds_of = [&](const Unit& u) {
+    const int rows = p.tiles_per_cta[u.type] * kBM, left = p.n_new - u.part * p.rounds[u.type] * rows;
+    return min(p.rounds[u.type], (left + rows - 1) / rows);
+  };
+  auto first_row = [&](const Unit& u, int r) { return (u.part * p.rounds[u.type] + r) * p.tiles_per_cta[u.type] * kBM; };
+  auto tiles_of = [&](const Unit& u, int q0) { return T == 2 && p.tiles_per_cta[u.type] == 2 && q0 + kBM < p.n_new ? 2 : 1; };
+  // Blocks of 128 keys: the caller's rows come first (they may not have to wait), then the cache's; a head
+  // never attends over nothing.
+  auto blocks_b = [&](const Unit& u) { return (p.len_b[u.type] + kBN - 1) / kBN; };
+  auto blocks = [&](const Unit& u) { return blocks_b(u) + (p.len_a[u.type] + kBN - 1) / kBN; };
+  // Keys of the last block of a segment of `len` rows in groups of 32, the unit in which the products and the
+  // softmax leave out what is past the last key
+  auto last_groups = [](int len) { return (((len - 1) & (kBN - 1)) >> 5) + 1; };
+  // Loads of the producer: a tile of 128 rows (the queries of slot t, or K / V block j of the unit)
+  auto load_tile = [&](uint32_t dst, const CUtensorMap* tm, int row, uint64_t* bar) {
+    mbar_expect_tx(smem_u32(bar), TILE_BYTES);
+#pragma unroll 1
+    for (int c = 0; c < SUB; ++c) tma_load_2d(dst + c * SUB_BYTES, tm, c * 64, row, smem_u32(bar));
+  };
+  auto load_kv = [&](const Unit& u, int j, int nb, uint32_t slot, int kv) {
+    const bool b = j < nb;
+    load_tile((kv ? v_sm : k_sm) + slot * TILE_BYTES, kv ? (b ? &tm_vn : &tm_v) : (b ? &tm_kn : &tm_k),
+              b ? u.bh * p.n_new + j * kBN : u.krow + (j - nb) * kBN, kv ? &bars->v_full[slot] : &bars->k_full[slot]);
+  };
+
   if (warp == kProducerWarp && lane == 0) {
+#pragma unroll 1
     for (int t = 0; t < 2; ++t) {
+      mbar_init(smem_u32(&bars->u_full[t]), 1);
+      mbar_init(smem_u32(&bars->u_empty[t]), 3 + 4 * T);   // two issuers, the append, the softmax warps
       mbar_init(smem_u32(&bars->q_full[t]), 1);
+      mbar_init(smem_u32(&bars->q_free[t]), 1);
       mbar_init(smem_u32(&bars->s_full[t]), 1);
       mbar_init(smem_u32(&bars->p_full[t]), 4);     // one arrival per warp of the tile
       mbar_init(smem_u32(&bars->p_free[t]), 1);
-      mbar_init(smem_u32(&bars->o_final[t]), 1);
     }
     for (int s = 0; s < kKStages; ++s) { mbar_init(smem_u32(&bars->k_full[s]), 1); mbar_init(smem_u32(&bars->k_empty[s]), 1); }
     for (int s = 0; s < kVStages; ++s) { mbar_init(smem_u32(&bars->v_full[s]), 1); mbar_init(smem_u32(&bars->v_empty[s]), 1); }
+    mbar_init(smem_u32(&bars->asked), 1);
     mbar_init(smem_u32(&bars->s_free), 4);          // the four warps of the tile whose logits were in the buffer
     mbar_init(smem_u32(&bars->copy_full[0]), 1);
     mbar_init(smem_u32(&bars->copy_full[1]), 1);
     mbar_init(smem_u32(&bars->drain), 1);
     mbar_init(smem_u32(&bars->drain2), 1);
-    bars->abort_flag = 0;
+    bars->abort_code = 0;
     fence_barrier_init();
     fence_proxy_async();
     // the producer starts the first loads at once: they run under the TMEM allocation, the
     // block-wide synchronisation and the register reallocation below
-    prefetch_tensormap(&tm_q);
-    prefetch_tensormap(&tm_k);
-    prefetch_tensormap(&tm_v);
-    prefetch_tensormap(&tm_o);
-    if (len_b > 0) {
-      prefetch_tensormap(&tm_kn);
-      prefetch_tensormap(&tm_vn);
-    }
+    const Unit u = make_unit(blockIdx.x);
+    bars->unit[0] = u;
+    mbar_arrive(smem_u32(&bars->u_full[0]));
+    const int nb = blocks_b(u), dep = p.dep[u.type], q0 = first_row(u, 0), ntile = tiles_of(u, q0);
     // The queries, like the new rows, are the caller's input.  When the kernel ahead of this one in
     // the stream is the step's own compression launch, whatever produced them had completed before
     // that launch passed its own dependency wait, hence before any CTA of this launch started: they
     // are loaded ahead of the wait.
     auto load_queries = [&]() {
-      for (int t = 0; t < ntile; ++t) {
-        const uint32_t bar = smem_u32(&bars->q_full[t]);
-        mbar_expect_tx(bar, TILE_BYTES);
-        for (int c = 0; c < SUB; ++c)
-          tma_load_2d(q_sm + t * TILE_BYTES + c * SUB_BYTES, &tm_q, c * 64, qrow + t * kBM, bar);
-      }
+      for (int t = 0; t < ntile; ++t) load_tile(q_sm + t * TILE_BYTES, &tm_q, u.bh * p.n_new + q0 + t * kBM, &bars->q_full[t]);
     };
     if (p.q_before_wait) load_queries();
-    if (dep == kDepAll || (dep == kDepCache && nblk_b == 0)) pdl_grid_wait();
+    if (dep == kDepAll || (dep == kDepCache && nb == 0)) pdl_grid_wait();
     if (!p.q_before_wait) load_queries();
-    mbar_expect_tx(smem_u32(&bars->k_full[0]), TILE_BYTES);
-    for (int c = 0; c < SUB; ++c) tma_load_2d(k_sm + c * SUB_BYTES, k_src(0), c * 64, tile_row(0), smem_u32(&bars->k_full[0]));
-    mbar_expect_tx(smem_u32(&bars->v_full[0]), TILE_BYTES);
-    for (int c = 0; c < SUB; ++c) tma_load_2d(v_sm + c * SUB_BYTES, v_src(0), c * 64, tile_row(0), smem_u32(&bars->v_full[0]));
+    load_kv(u, 0, nb, 0, 0);
+    load_kv(u, 0, nb, 0, 1);
   }
   if (warp == kMmaWarp) {
     tmem_alloc(smem_u32(&bars->tmem_base), Shape<T>::kTmemCols);
@@ -265,20 +300,45 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       constexpr uint32_t IDESC_PV = idesc_bf16_f32(kBM, D, 1);         // A = P (TMEM), B = V (MN-major)
       const uint64_t v_desc0 = smem_desc_sw128(v_sm, SUB_BYTES, 1024);
       bool ok = true;
-      for (int j = 0; j < nblk && ok; ++j) {
-        const int vs = j % kVStages;
-        const uint64_t vd = v_desc0 + (uint64_t)((vs * TILE_BYTES) >> 4);
-        for (int t = 0; t < ntile && ok; ++t) {
-          ok = wait_bar(&bars->p_full[t], j & 1, bars, p.status, 5, wlim);
-          if (ok && t == 0) ok = wait_bar(&bars->v_full[vs], (j / kVStages) & 1, bars, p.status, 6, wlim);
-          if (!ok) break;
-          tc_fence_after();
-          mma_ts_chain4(tmem + O_COL + t * D, tmem + P_COL + t * 64, vd, IDESC_PV, j > 0);
-          mma_ts_chain4(tmem + O_COL + t * D, tmem + P_COL + t * 64 + 32, vd + 4 * 128, IDESC_PV, 1);
-          mma_commit(smem_u32(&bars->p_free[t]));             // P_t may be rewritten, O_t is up to date
-          if (t == ntile - 1) mma_commit(smem_u32(&bars->v_empty[vs]));
-          if (j + 1 == nblk) mma_commit(smem_u32(&bars->o_final[t]));
+      uint32_t g = 0, odd = 0;                                         // V tiles used up; per tile: products so far, parity
+#pragma unroll 1
+      for (int n = 0; ok; ++n) {
+        ok = wait_unit(n);
+        if (!ok) break;
+        const Unit u = read_unit(n);
+        give_unit(n);
+        if (u.bh < 0) break;
+        const int nb = blocks_b(u), nblk = blocks(u), nr = rounds_of(u);
+        const int kg_b = last_groups(p.len_b[u.type]), kg_a = last_groups(p.len_a[u.type]);
+#pragma unroll 1
+        for (int r = 0; r < nr && ok; ++r) {
+          const int ntile = tiles_of(u, first_row(u, r));
+#pragma unroll 1
+          for (int j = 0; j < nblk && ok; ++j) {
+            const uint32_t vs = (g + j) % kVStages;
+            const uint64_t vd = v_desc0 + (uint64_t)((vs * TILE_BYTES) >> 4);
+            const int kg = j == nb - 1 ? kg_b : j == nblk - 1 ? kg_a : 4;
+#pragma unroll 1
+            for (int t = 0; t < ntile; ++t) {
+              // (what comes last is the wait whose end something waits for)
+              if (t == 0 && r == 0) ok = wait_bar(&bars->v_full[vs], ((g + j) / kVStages) & 1, bars, 6, wlim);
+              const uint32_t o = tmem + O_COL + t * D, pa = tmem + P_COL + t * 64;
+              if (!ok || !wait_bar(&bars->p_full[t], (odd >> t) & 1, bars, 5, wlim)) { ok = false; break; }
+              tc_fence_after();
+              if (kg == 4) {
+                mma_ts_chain4(o, pa, vd, IDESC_PV, j > 0);
+                mma_ts_chain4(o, pa + 32, vd + 4 * 128, IDESC_PV, 1);
+              } else {
+#pragma unroll 1
+                for (int k = 0; k < 2 * kg; ++k) mma_ts(o, pa + 8 * k, vd + k * 128, IDESC_PV, j > 0 || k > 0);
+              }
+              mma_commit(smem_u32(&bars->p_free[t]));           // P_t may be rewritten, O_t is up to date
+              odd ^= 1u << t;
+              if (t == ntile - 1 && r == nr - 1) mma_commit(smem_u32(&bars->v_empty[vs]));
+            }
+          }
         }
+        g += nblk;
       }
       if (!ok) {
         mma_commit(smem_u32(&bars->drain2));
@@ -288,83 +348,133 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     }
   } else if (warp == kAppendWarp) {
     reg_dec<kOtherRegs>();
-    if (p.append_new && len_b > 0 && dbg_ok(len_a >= 0 && len_a + len_b <= p.cap[type], p.status, 7)) {
-      // Eq. 3 for this head: the new scale's rows go behind the len_a cache rows.  The rows are one
-      // contiguous run in the caller's tensor and in the cache plane; the CTAs of the head share
-      // them, and one thread moves this CTA's slice with bulk copies through two staging halves
-      // (global -> shared -> global), so the append costs no registers and no issue slots.
-      if (dep != kDepNothing) pdl_grid_wait();
-      const int per_cta = (len_b + n_pairs - 1) / n_pairs;
-      const int r0 = pair * per_cta, r1 = min(len_b, r0 + per_cta);
-      for (int r = r0 + lane; r < r1; r += 32) p.pos_plane[krow + len_a + r] = p.pos_base + r;
+    // Eq. 3 for the heads that keep the whole new scale: its rows go behind the len_a cache rows.  The rows are
+    // one contiguous run in the caller's tensor and in the cache plane; the units of the head share
+    // them, and one thread moves a unit's slice with bulk copies through two staging halves
+    // (global -> shared -> global), so the append costs no registers and no issue slots.
+    bool ok = true;
+    uint32_t chunks = 0;                             // chunk counter over planes and units
+#pragma unroll 1
+    for (int n = 0; ok; ++n) {
+      ok = __all_sync(0xffffffffu, wait_unit(n));
+      if (!ok) break;
+      const Unit u = read_unit(n);
+      __syncwarp();
+      if (lane == 0) give_unit(n);
+      if (u.bh < 0) break;
+      const int len_a = p.len_a[u.type], len_b = p.len_b[u.type];
+      if (!p.append_new || len_b == 0 || !dbg_ok(len_a >= 0 && len_a + len_b <= p.cap[u.type], p.status, 7)) continue;
+      if (p.dep[u.type] != kDepNothing) pdl_grid_wait();
+      const int per = (len_b + p.units_per_head[u.type] - 1) / p.units_per_head[u.type];
+      const int r0 = u.part * per, r1 = min(len_b, r0 + per);
+#pragma unroll 1
+      for (int r = r0 + lane; r < r1; r += 32) p.pos_plane[u.krow + len_a + r] = p.pos_base + r;
       if (lane == 0 && r1 > r0) {
         const uint32_t row_bytes = (uint32_t)p.head_dim_pieces * 16;
-        const size_t src_off = ((size_t)nrow + r0) * row_bytes, dst_off = ((size_t)krow + len_a + r0) * row_bytes;
+        const size_t src_off = ((size_t)u.bh * p.n_new + r0) * row_bytes, dst_off = ((size_t)u.krow + len_a + r0) * row_bytes;
         const uint32_t total = (uint32_t)(r1 - r0) * row_bytes;
         const uint32_t n_chunks = (total + kCopyChunk - 1) / kCopyChunk;
-        bool ok = true;
-        uint32_t n = 0;                              // chunk counter over both planes
+#pragma unroll 1
         for (int plane = 0; plane < 2 && ok; ++plane) {
           const unsigned char* src = reinterpret_cast<const unsigned char*>(plane == 0 ? p.k_new : p.v_new) + src_off;
           unsigned char* dst = reinterpret_cast<unsigned char*>(plane == 0 ? p.k_plane : p.v_plane) + dst_off;
-          for (uint32_t ch = 0; ch < n_chunks && ok; ++ch, ++n) {
-            const uint32_t half = n & 1;
+#pragma unroll 1
+          for (uint32_t ch = 0; ch < n_chunks && ok; ++ch, ++chunks) {
+            const uint32_t half = chunks & 1;
             const uint32_t bytes = min(kCopyChunk, total - ch * kCopyChunk);
             const uint32_t bar = smem_u32(&bars->copy_full[half]);
             bulk_wait_read<1>();                     // the store that last read this half (two chunks ago) is done with it
             mbar_expect_tx(bar, bytes);
             bulk_load(copy_sm + half * kCopyChunk, src + (size_t)ch * kCopyChunk, bytes, bar);
-            ok = wait_bar(&bars->copy_full[half], (n >> 1) & 1, bars, p.status, 12, wlim);
+            ok = wait_bar(&bars->copy_full[half], (chunks >> 1) & 1, bars, 12, wlim);
             if (!ok) break;
             bulk_store(dst + (size_t)ch * kCopyChunk, copy_sm + half * kCopyChunk, bytes);
             bulk_commit();
           }
         }
-        bulk_wait<0>();                              // every store has been performed before the CTA may leave
       }
+      ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
     }
+    if (lane == 0) bulk_wait<0>();                   // every store has been performed before the CTA may leave
   } else if (warp == kProducerWarp) {
-    // ------------------------------------------------------------------ TMA producer
+    // ------------------------------------------------------------------ TMA producer, and the CTA's next unit
     reg_dec<kOtherRegs>();
     if (lane == 0) {
-      int k_issued = 1, v_issued = 1;               // Q and tile 0 of K and V are already on their way
-      bool ok = true;
-      for (int j = 1; j < nblk && ok; ++j) {
-        if (dep == kDepCache && j == nblk_b) pdl_grid_wait();   // the head's stored survivors are in place
-        {
-          const int s = j % kKStages;
-          ok = wait_bar(&bars->k_empty[s], ((j / kKStages) & 1) ^ 1, bars, p.status, 1, wlim);
-          if (!ok) break;
-          const uint32_t bar = smem_u32(&bars->k_full[s]);
-          mbar_expect_tx(bar, TILE_BYTES);
-          for (int c = 0; c < SUB; ++c)
-            tma_load_2d(k_sm + s * TILE_BYTES + c * SUB_BYTES, k_src(j), c * 64, tile_row(j), bar);
-          ++k_issued;
+      bool ok = true, pending = false;              // pending: an answer of cluster launch control is on its way
+      uint32_t g = 0, issued_k = 1, issued_v = 1;   // K / V tiles of the units before this one; tiles on their way so far
+      uint32_t q_issued = 0, q_odd = 0, answers = 0;   // bit t: query slot t was filled, the parity of its fillings
+      Unit u = bars->unit[0];
+#pragma unroll 1
+      for (int n = 0;; ++n) {
+        const int nb = blocks_b(u), nblk = blocks(u), nr = rounds_of(u), dep = p.dep[u.type];
+        if (n > 0 && (dep == kDepAll || (dep == kDepCache && nb == 0))) pdl_grid_wait();
+        // K / V tiles of the unit in order, and the queries of round r ahead of step r's value tile
+#pragma unroll 1
+        for (int j = 0; j < max(nblk, nr) && ok; ++j) {
+          if (dep == kDepCache && j == nb && j < nblk) pdl_grid_wait();   // the head's stored survivors are in place
+          const bool fresh = n > 0 || j > 0;        // the first tiles and queries of the CTA are on their way already
+          const uint32_t gs = g + j;
+#pragma unroll 1
+          for (int kv = 0; kv < 2 && ok; ++kv) {
+            if (kv == 1 && j < nr) {
+              const int q0 = first_row(u, j), ntile = tiles_of(u, q0);
+#pragma unroll 1
+              for (int t = 0; t < ntile && ok; ++t) {
+                if (fresh) {
+                  if (q_issued >> t & 1) ok = wait_bar(&bars->q_free[t], ((q_odd >> t) & 1) ^ 1, bars, 14, wlim);
+                  if (!ok) break;
+                  load_tile(q_sm + t * TILE_BYTES, &tm_q, u.bh * p.n_new + q0 + t * kBM, &bars->q_full[t]);
+                }
+                q_issued |= 1u << t;
+                q_odd ^= 1u << t;
+              }
+            }
+            if (!ok || !fresh || j >= nblk) continue;
+            const uint32_t sl = gs % kKStages;      // (both rings have the same depth)
+            ok = wait_bar(kv ? &bars->v_empty[sl] : &bars->k_empty[sl], ((gs / kKStages) & 1) ^ 1, bars, 1 + kv, wlim);
+            if (!ok) break;
+            load_kv(u, j, nb, sl, kv);
+            if (kv) ++issued_v;
+            else ++issued_k;
+          }
         }
-        {
-          const int s = j % kVStages;
-          ok = wait_bar(&bars->v_empty[s], ((j / kVStages) & 1) ^ 1, bars, p.status, 2, wlim);
+        if (!ok) break;
+        g += nblk;
+        Unit next{-1, 0, 0, 0};
+        if (p.steal) {
+          // The next unit is asked for behind the last load of this one: three blocks earlier, it would be kept
+          // from CTAs that are idle by then (512 units of 5 blocks on 296 places: 43.0 against 37.4 us a step).
+          mbar_expect_tx(smem_u32(&bars->asked), 16);
+          clc_ask(smem_u32(&bars->answer), smem_u32(&bars->asked));
+          pending = true;
+          ok = wait_bar(&bars->asked, answers & 1, bars, 15, wlim);
           if (!ok) break;
-          const uint32_t bar = smem_u32(&bars->v_full[s]);
-          mbar_expect_tx(bar, TILE_BYTES);
-          for (int c = 0; c < SUB; ++c)
-            tma_load_2d(v_sm + s * TILE_BYTES + c * SUB_BYTES, v_src(j), c * 64, tile_row(j), bar);
-          ++v_issued;
+          pending = false;
+          ++answers;
+          const int x = clc_answer(smem_u32(&bars->answer));
+          fence_proxy_async();                       // the next answer overwrites what was just read
+          if (x >= 0) next = make_unit(x);
         }
+        if (n > 0) ok = wait_bar(&bars->u_empty[(n + 1) & 1], (((n + 1) >> 1) & 1) ^ 1, bars, 16, wlim);
+        if (!ok) break;
+        bars->unit[(n + 1) & 1] = next;
+        mbar_arrive(smem_u32(&bars->u_full[(n + 1) & 1]));
+        if (next.bh < 0) break;
+        u = next;
       }
       if (!ok) {
         // give the copies already in flight a bounded chance to land before the CTA leaves
-        for (int t = 0; t < ntile; ++t) {
-          const uint32_t bar = smem_u32(&bars->q_full[t]);
-          for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(bar, 0); ++it) {}
-        }
-        for (int i = max(0, k_issued - kKStages); i < k_issued; ++i) {
-          const uint32_t bar = smem_u32(&bars->k_full[i % kKStages]);
-          for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(bar, (i / kKStages) & 1); ++it) {}
-        }
-        for (int i = max(0, v_issued - kVStages); i < v_issued; ++i) {
-          const uint32_t bar = smem_u32(&bars->v_full[i % kVStages]);
-          for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(bar, (i / kVStages) & 1); ++it) {}
+        auto landed = [&](uint64_t* bar, uint32_t parity) {
+          for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(smem_u32(bar), parity); ++it) {}
+        };
+        if (pending) landed(&bars->asked, answers & 1);
+#pragma unroll 1
+        for (int t = 0; t < T; ++t)
+          if (q_issued >> t & 1) landed(&bars->q_full[t], ((q_odd >> t) & 1) ^ 1);
+#pragma unroll 1
+        for (uint32_t i = 0; i < kKStages; ++i) {
+          if (issued_k > i) landed(&bars->k_full[(issued_k - 1 - i) % kKStages], ((issued_k - 1 - i) / kKStages) & 1);
+          if (issued_v > i) landed(&bars->v_full[(issued_v - 1 - i) % kVStages], ((issued_v - 1 - i) / kVStages) & 1);
         }
       }
     }
@@ -372,42 +482,52 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     // ------------------------------------------------------------------ issuer of the Q K^T products
     reg_dec<kOtherRegs>();
     if (lane == 0) {
-      constexpr uint32_t IDESC_S = idesc_bf16_f32(kBM, kBN, 0);        // A = Q, B = K (both K-major)
+      constexpr uint32_t IDESC_0 = idesc_bf16_f32(kBM, 0, 0);          // A = Q, B = K (both K-major); N is added
       // descriptors of the tile bases; a k-step only adds a constant to the address field
-      const uint64_t q_desc[2] = {smem_desc_sw128(q_sm, 16, 1024), smem_desc_sw128(q_sm + (T - 1) * TILE_BYTES, 16, 1024)};
-      const uint64_t k_desc0 = smem_desc_sw128(k_sm, 16, 1024);
+      const uint64_t q_desc0 = smem_desc_sw128(q_sm, 16, 1024), k_desc0 = smem_desc_sw128(k_sm, 16, 1024);
       bool ok = true;
       // S = Q_t K_j^T into the one logit buffer; `use` counts the products issued so far, and product
-      // number use needs the logits of product use - 1 to have left the buffer (s_free phase use - 1)
-      int use = 0;
-      auto issue_s = [&](int t, int j) -> bool {
-        if (use > 0 && !wait_bar(&bars->s_free, (use - 1) & 1, bars, p.status, 10, wlim)) return false;
-        tc_fence_after();
-        const uint64_t kd = k_desc0 + (uint64_t)(((j % kKStages) * TILE_BYTES) >> 4);
-        if constexpr (D == 128) mma_ss_chain8(tmem + S_COL, q_desc[t], kd, IDESC_S, 0);
-        else mma_ss_chain4(tmem + S_COL, q_desc[t], kd, IDESC_S, 0);
-        mma_commit(smem_u32(&bars->s_full[t]));
-        ++use;
-        return true;
-      };
-      for (int t = 0; t < ntile && ok; ++t) ok = wait_bar(&bars->q_full[t], 0, bars, p.status, 3, wlim);
-      if (ok) ok = wait_bar(&bars->k_full[0], 0, bars, p.status, 4, wlim);
-      for (int t = 0; t < ntile && ok; ++t) ok = issue_s(t, 0);
-      if (ok) mma_commit(smem_u32(&bars->k_empty[0]));
-      for (int j = 0; j < nblk && ok; ++j) {
-        for (int t = 0; t < ntile && ok; ++t) {
-          // the next logits of this tile: they only wait for the buffer, not for this tile's
-          // softmax, and so run under it
-          if (j + 1 < nblk) {
-            if (t == 0) {
-              ok = wait_bar(&bars->k_full[(j + 1) % kKStages], ((j + 1) / kKStages) & 1, bars, p.status, 7, wlim);
-              if (!ok) break;
+      // number use needs the logits of product use - 1 to have left the buffer (s_free phase use - 1).  The
+      // next logits only wait for the buffer, not for the softmax of the tile or the end of a unit.
+      uint32_t use = 0, g = 0, q_odd = 0;
+#pragma unroll 1
+      for (int n = 0; ok; ++n) {
+        ok = wait_unit(n);
+        if (!ok) break;
+        const Unit u = read_unit(n);
+        give_unit(n);
+        if (u.bh < 0) break;
+        const int nb = blocks_b(u), nblk = blocks(u), nr = rounds_of(u);
+        const uint32_t idesc_b = IDESC_0 + ((uint32_t)(last_groups(p.len_b[u.type]) * 4) << 17);
+        const uint32_t idesc_a = IDESC_0 + ((uint32_t)(last_groups(p.len_a[u.type]) * 4) << 17);
+#pragma unroll 1
+        for (int r = 0; r < nr && ok; ++r) {
+          const int ntile = tiles_of(u, first_row(u, r));
+#pragma unroll 1
+          for (int j = 0; j < nblk && ok; ++j) {
+            const uint32_t ks = (g + j) % kKStages;
+            const uint64_t kd = k_desc0 + (uint64_t)((ks * TILE_BYTES) >> 4);
+            const uint32_t idesc = j == nb - 1 ? idesc_b : j == nblk - 1 ? idesc_a : IDESC_0 + ((kBN >> 3) << 17);
+#pragma unroll 1
+            for (int t = 0; t < ntile; ++t) {
+              if (j == 0) {
+                ok = wait_bar(&bars->q_full[t], (q_odd >> t) & 1, bars, 3, wlim);
+                q_odd ^= 1u << t;
+              }
+              if (ok && t == 0 && r == 0) ok = wait_bar(&bars->k_full[ks], ((g + j) / kKStages) & 1, bars, 4, wlim);
+              const uint64_t qd = q_desc0 + (uint64_t)((t * TILE_BYTES) >> 4);
+              if (!ok || !wait_bar(&bars->s_free, (use - 1) & 1, bars, 10, wlim)) { ok = false; break; }   // (a fresh barrier passes for odd)
+              tc_fence_after();
+              if constexpr (D == 128) mma_ss_chain8(tmem + S_COL, qd, kd, idesc, 0);
+              else mma_ss_chain4(tmem + S_COL, qd, kd, idesc, 0);
+              mma_commit(smem_u32(&bars->s_full[t]));
+              ++use;
+              if (j == nblk - 1) mma_commit(smem_u32(&bars->q_free[t]));
+              if (t == ntile - 1 && r == nr - 1) mma_commit(smem_u32(&bars->k_empty[ks]));
             }
-            ok = issue_s(t, j + 1);
-            if (!ok) break;
-            if (t == ntile - 1) mma_commit(smem_u32(&bars->k_empty[(j + 1) % kKStages]));
           }
         }
+        g += nblk;
       }
       if (!ok) {
         mma_commit(smem_u32(&bars->drain));
@@ -419,160 +539,238 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     // ------------------------------------------------------------------ softmax + epilogue
     reg_inc<kSoftmaxRegs>();
     const int t = (warp >> 2) - 1;                 // tile served by this warpgroup
-    if (t < ntile) {
-      const int r = tid & 127;                     // query row inside the tile == TMEM lane
-      const uint32_t lane_addr = static_cast<uint32_t>((warp & 3) * 32) << 16;
-      const uint32_t s_addr = tmem + lane_addr + S_COL;
-      const uint32_t p_addr = tmem + lane_addr + P_COL + t * 64;
-      const uint32_t o_addr = tmem + lane_addr + O_COL + t * D;
-      const float c = p.scale_log2;
-      float m_used = kNoLogit, l = 0.f;
-      bool ok = true;
-      for (int j = 0; j < nblk; ++j) {
-        ok = __all_sync(0xffffffffu, wait_bar(&bars->s_full[t], j & 1, bars, p.status, 8, wlim));
-        if (!ok) break;
-        tc_fence_after();
-        uint32_t sr[kBN];
-#pragma unroll
-        for (int ch = 0; ch < kBN / 32; ++ch) tmem_ld32(s_addr + ch * 32, sr + ch * 32);
+    const int row = tid & 127;                     // query row inside the tile == TMEM lane
+    const uint32_t lane_addr = static_cast<uint32_t>((warp & 3) * 32) << 16;
+    const uint32_t s_addr = tmem + lane_addr + S_COL;
+    const uint32_t p_addr = tmem + lane_addr + P_COL + t * 64;
+    const uint32_t o_addr = tmem + lane_addr + O_COL + t * D;
+    const float c = p.scale_log2;
+    float m_used = kNoLogit, l = 0.f;
+    uint32_t cnt = 0;                              // blocks of this tile so far
+    bool ok = true, pending = false;               // pending: a round's output is still in tensor memory
+    volatile int2* const out_at = &bars->out_at[warp - 4];   // of the round in work or pending: first row of its head, row of the tile
+    auto bar_all = [&](uint64_t* bar, uint32_t parity, int code) { return __all_sync(0xffffffffu, wait_bar(bar, parity, bars, code, wlim)) != 0; };
+    // Output of the round that ended.  A thread writes its own row, 32 bytes (a whole sector) an instruction,
+    // straight from tensor memory: through the query tile's shared memory and a tiled store, the next round's
+    // queries could not be on their way meanwhile.
+    auto flush = [&]() {
+      ok = bar_all(&bars->p_free[t], (cnt - 1) & 1, 9);        // the round's last product
+      if (!ok) return;
+      pending = false;
+      tc_fence_after();
+      const float inv = 1.f / l;
+      const int head_row = out_at->x, tile_row = out_at->y + row;
+      const bool out_live = tile_row < p.n_new;
+      const size_t out_row = (size_t)head_row + tile_row;
+      if (p.row_stats && out_live) *reinterpret_cast<float2*>(p.row_stats + out_row * 2) = make_float2(m_used, l);
+      unsigned char* dst = reinterpret_cast<unsigned char*>(p.out) + out_row * (D * 2);
+#pragma unroll 1
+      for (int ch = 0; ch < D / 16; ++ch) {
+        uint32_t orr[16], w[8];
+        tmem_ld16(o_addr + ch * 16, orr);
         tmem_wait_ld();
-        // the logits are in registers: the buffer goes back to the MMA warp at once
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&bars->s_free));
-        // live keys of this tile: fewer than 128 only in the last tile of either segment
-        const int valid = j < nblk_b ? len_b - j * kBN : len_a - (j - nblk_b) * kBN;
-        if (valid < kBN) {
 #pragma unroll
-          for (int i = 0; i < kBN; ++i)
-            if (i >= valid) sr[i] = 0xff800000u;   // -inf
+        for (int e = 0; e < 8; ++e) {
+          const __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(orr[2 * e]) * inv, __uint_as_float(orr[2 * e + 1]) * inv);
+          w[e] = *reinterpret_cast<const uint32_t*>(&hh);
         }
-        // row maximum, kept apart for the pairs whose exponential runs on the FMA pipe (pair index
-        // i with (i & 7) < kPolyOf8) and for the others: the row-sum correction below must form the
-        // largest probability with the same instructions the loop uses for that element
-        float mx_sfu[4], mx_fma[4];
+        if (out_live) st_global_32b(dst + ch * 32, w, p.out_sectors != 0);
+      }
+    };
+    // What a block adds to the reference maximum, the sum and, if the maximum grew, the factor of what is there
+    auto raise = [&](float mx, float& alpha) {
+      const bool grow = (mx - m_used) * c > kRescaleThreshold;     // always true in the first block
+      const bool any = __any_sync(0xffffffffu, grow);
+      alpha = 1.f;
+      if (any) {
+        const float m_new = grow ? mx : m_used;
+        alpha = grow ? ex2((m_used - m_new) * c) : 1.f;
+        l *= alpha;
+        m_used = m_new;
+      }
+      return any;
+    };
+    // The second MMA sees the probabilities rounded to bf16, the row sum does not.  With the
+    // lazily raised reference maximum even a dominant key's probability is no power of two,
+    // and its rounding error (up to 2^-9 of an output that can reach 4) would pass straight
+    // into O.  The block's largest probability is therefore entered into the sum as rounded,
+    // which makes the weight of a dominant key exact; what is left is bounded by the weight
+    // of the other keys.  Same instructions as the loops use for that element, hence the same bits.
+    auto top_rounding = [&](float mx, float nmc) {
+      const float p_top = ex2(fmaf(mx, c, nmc));
+      return __bfloat162float(__float2bfloat16_rn(p_top)) - p_top;
+    };
+    // P_t still feeds the product of the previous block, which also still adds to O_t
+    auto wait_p = [&](bool rescale, float alpha) {
+      ok = bar_all(&bars->p_free[t], (cnt - 1) & 1, 11);
+      if (!ok) return;
+      tc_fence_after();
+      if (rescale) {
+#pragma unroll 1
+        for (int ch = 0; ch < D / 8; ++ch) {               // rare path: kept light on registers
+          uint32_t orr[8];
+          tmem_ld8(o_addr + ch * 8, orr);
+          tmem_wait_ld();
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          mx_sfu[u] = -INFINITY;
-          mx_fma[u] = -INFINITY;
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float e0 = __uint_as_float(sr[u * 32 + 2 * i]), e1 = __uint_as_float(sr[u * 32 + 2 * i + 1]);
-            if ((i & 7) < kPolyOf8) mx_fma[u] = max3(mx_fma[u], e0, e1);
-            else mx_sfu[u] = max3(mx_sfu[u], e0, e1);
-          }
+          for (int i = 0; i < 8; ++i) orr[i] = __float_as_uint(__uint_as_float(orr[i]) * alpha);
+          tmem_st8(o_addr + ch * 8, orr);
         }
-        const float mxs = fmaxf(fmaxf(mx_sfu[0], mx_sfu[1]), fmaxf(mx_sfu[2], mx_sfu[3]));
-        const float mxf = fmaxf(fmaxf(mx_fma[0], mx_fma[1]), fmaxf(mx_fma[2], mx_fma[3]));
-        const float mx = fmaxf(mxs, mxf);
-        const bool grow = (mx - m_used) * c > kRescaleThreshold;     // always true in the first tile
-        const bool any_grow = __any_sync(0xffffffffu, grow);
-        float alpha = 1.f;
-        if (any_grow) {
-          const float m_new = grow ? mx : m_used;
-          alpha = grow ? ex2((m_used - m_new) * c) : 1.f;
-          l *= alpha;
-          m_used = m_new;
-        }
-        const float2 c2 = make_float2(c, c);
-        const float2 nmc2 = make_float2(-m_used * c, -m_used * c);
-        float2 sum4[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        uint32_t pk[kBN / 2];
+      }
+    };
+    auto give_p = [&]() {
+      tmem_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bars->p_full[t]));
+      ++cnt;
+    };
+    // A block of 65 to 128 keys.
+    auto block = [&](bool first, int valid) {
+      ok = bar_all(&bars->s_full[t], cnt & 1, 8);
+      if (!ok) return;
+      tc_fence_after();
+      uint32_t sr[kBN];
 #pragma unroll
-        for (int i = 0; i < kBN / 2; ++i) {
+      for (int ch = 0; ch < kBN / 32; ++ch) tmem_ld32(s_addr + ch * 32, sr + ch * 32);
+      tmem_wait_ld();
+      // the logits are in registers: the buffer goes back to the MMA warp at once
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bars->s_free));
+      if (__builtin_expect(valid < kBN, 0)) {
+#pragma unroll
+        for (int i = 64; i < kBN; ++i)
+          if (i >= valid) sr[i] = 0xff800000u;   // -inf
+      }
+      float mx4[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        mx4[u] = -INFINITY;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) mx4[u] = max3(mx4[u], __uint_as_float(sr[u * 32 + 2 * i]), __uint_as_float(sr[u * 32 + 2 * i + 1]));
+      }
+      const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+      float alpha;
+      const bool any_grow = raise(mx, alpha);
+      const float2 c2 = make_float2(c, c);
+      const float2 nmc2 = make_float2(-m_used * c, -m_used * c);
+      float2 sum4[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      uint32_t pk[kBN / 2];
+#pragma unroll
+      for (int i = 0; i < kBN / 2; ++i) {
+        const float2 x = fma2(make_float2(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1])), c2, nmc2);
+        float2 pr;
+        pr.x = ex2(x.x);
+        pr.y = ex2(x.y);
+        sum4[i & 3] = add2(sum4[i & 3], pr);
+        const __nv_bfloat162 hh = __floats2bfloat162_rn(pr.x, pr.y);
+        pk[i] = *reinterpret_cast<const uint32_t*>(&hh);
+      }
+      const float2 sum2 = add2(add2(sum4[0], sum4[1]), add2(sum4[2], sum4[3]));
+      l += sum2.x + sum2.y;
+      l += top_rounding(mx, nmc2.x);
+      if (cnt > 0) {
+        wait_p(any_grow && !first, alpha);
+        if (!ok) return;
+      }
+      tmem_st32(p_addr, pk);
+      tmem_st32(p_addr + 32, pk + 32);
+      give_p();
+    };
+    // The last block of a segment, up to 64 keys: 32 at a time and in little code, which reads the logits twice.  (With
+    // up to 127 keys this way, 126 units of 3 to 8 blocks took 34 instead of 33 us a step.)
+    auto tail = [&](bool first, int valid) {
+      ok = bar_all(&bars->s_full[t], cnt & 1, 8);
+      if (!ok) return;
+      tc_fence_after();
+      auto load = [&](int ch, uint32_t* sr) {
+        tmem_ld32(s_addr + ch, sr);
+        tmem_wait_ld();
+        if (valid - ch < 32) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (i >= valid - ch) sr[i] = 0xff800000u;   // -inf
+        }
+      };
+      float mx = -INFINITY;
+#pragma unroll 1
+      for (int ch = 0; ch < valid; ch += 32) {
+        uint32_t sr[32];
+        load(ch, sr);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) mx = max3(mx, __uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1]));
+      }
+      float alpha;
+      const bool any_grow = raise(mx, alpha);
+      const float2 c2 = make_float2(c, c);
+      const float2 nmc2 = make_float2(-m_used * c, -m_used * c);
+      if (cnt > 0) {
+        wait_p(any_grow && !first, alpha);
+        if (!ok) return;
+      }
+      float2 sum4[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll 1
+      for (int ch = 0; ch < valid; ch += 32) {
+        uint32_t sr[32], pk[16];
+        load(ch, sr);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
           const float2 x = fma2(make_float2(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1])), c2, nmc2);
           float2 pr;
-          if ((i & 7) < kPolyOf8) {
-            pr = ex2_poly2(x);
-          } else {
-            pr.x = ex2(x.x);
-            pr.y = ex2(x.y);
-          }
+          pr.x = ex2(x.x);
+          pr.y = ex2(x.y);
           sum4[i & 3] = add2(sum4[i & 3], pr);
           const __nv_bfloat162 hh = __floats2bfloat162_rn(pr.x, pr.y);
           pk[i] = *reinterpret_cast<const uint32_t*>(&hh);
         }
-        const float2 sum2 = add2(add2(sum4[0], sum4[1]), add2(sum4[2], sum4[3]));
-        l += sum2.x + sum2.y;
-        {
-          // The second MMA sees the probabilities rounded to bf16, the row sum does not.  With the
-          // lazily raised reference maximum even a dominant key's probability is no power of two,
-          // and its rounding error (up to 2^-9 of an output that can reach 4) would pass straight
-          // into O.  The tile's largest probability is therefore entered into the sum as rounded,
-          // which makes the weight of a dominant key exact; what is left is bounded by the weight
-          // of the other keys.  Same instructions as the loop above uses for that element, hence the same bits.
-          const float x_top = fmaf(mx, c, nmc2.x);
-          float p_top = ex2(x_top);
-          if (kPolyOf8 > 0 && mxf > mxs) p_top = ex2_poly2(make_float2(x_top, x_top)).x;
-          l += __bfloat162float(__float2bfloat16_rn(p_top)) - p_top;
-        }
-        if (j > 0) {
-          // P_t still feeds the product of the previous block, which also still adds to O_t
-          ok = __all_sync(0xffffffffu, wait_bar(&bars->p_free[t], (j - 1) & 1, bars, p.status, 11, wlim));
-          if (!ok) break;
-          tc_fence_after();
-          if (any_grow) {
-#pragma unroll 1
-            for (int ch = 0; ch < D / 8; ++ch) {             // rare path: kept light on registers
-              uint32_t orr[8];
-              tmem_ld8(o_addr + ch * 8, orr);
-              tmem_wait_ld();
-#pragma unroll
-              for (int i = 0; i < 8; ++i) orr[i] = __float_as_uint(__uint_as_float(orr[i]) * alpha);
-              tmem_st8(o_addr + ch * 8, orr);
-            }
-          }
-        }
-        tmem_st32(p_addr, pk);
-        tmem_st32(p_addr + 32, pk + 32);
-        tmem_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&bars->p_full[t]));
+        tmem_st16(p_addr + ch / 2, pk);
       }
-      if (ok) ok = __all_sync(0xffffffffu, wait_bar(&bars->o_final[t], 0, bars, p.status, 9, wlim));
-      // the four warps of the tile meet on a named barrier below, so they agree first on whether all of them got here
-      uint32_t all_ok;
-      asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.and.pred p, %2, 128, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                   : "=r"(all_ok) : "r"((uint32_t)ok), "r"(1 + t) : "memory");
-      if (all_ok) {
-        tc_fence_after();
-        const int row = q0 + t * kBM + r;
-        const float inv = 1.f / l;
-        if (p.row_stats && row < p.n_new)
-          *reinterpret_cast<float2*>(p.row_stats + (static_cast<size_t>(bh) * p.n_new + row) * 2) = make_float2(m_used, l);
-        // The tile's output goes through its query tile's shared memory (the last Q K^T product has
-        // read it), laid out as a tiled copy with the 128-byte swizzle expects it: thread r's 16-byte
-        // pieces of a store instruction fall into different banks, and one tiled store per 64
-        // columns writes whole rows (a thread storing its own row straight to memory wrote 32
-        // half-used sectors per instruction: 3 us per CTA against 1).  Rows past the head's last
-        // query lie outside the tensor and are not written.
-        const uint32_t o_sm = q_sm + t * TILE_BYTES + r * 128;
-#pragma unroll
-        for (int ch = 0; ch < D / 32; ++ch) {
-          uint32_t orr[32];
-          tmem_ld32(o_addr + ch * 32, orr);
-          tmem_wait_ld();
-#pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            uint32_t w[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(orr[v * 8 + 2 * e]) * inv,
-                                                              __uint_as_float(orr[v * 8 + 2 * e + 1]) * inv);
-              w[e] = *reinterpret_cast<const uint32_t*>(&hh);
-            }
-            const int piece = ch * 4 + v;                      // 16-byte piece of the row
-            st_shared_v4(o_sm + (piece >> 3) * SUB_BYTES + (((piece & 7) ^ (r & 7)) << 4), w[0], w[1], w[2], w[3]);
-          }
+      const float2 sum2 = add2(add2(sum4[0], sum4[1]), add2(sum4[2], sum4[3]));
+      l += sum2.x + sum2.y;
+      l += top_rounding(mx, nmc2.x);
+      give_p();                                            // (its fence orders the logits' reads as well)
+      if (lane == 0) mbar_arrive(smem_u32(&bars->s_free));
+    };
+    // (What a round needs is read where it is needed: registers that live through a block are scarce.)
+    int n = 0, r = 0;
+    ok = __all_sync(0xffffffffu, wait_unit(0)) != 0;
+#pragma unroll 1
+    while (ok) {
+      int left = 0, then = 0;                      // keys left of the caller's rows or the cache's; the cache's to follow
+      const Unit u = read_unit(n);
+      if (u.bh >= 0) {
+        if (r == rounds_of(u)) {
+          __syncwarp();
+          if (lane == 0) give_unit(n);
+          ++n;
+          r = 0;
+          ok = __all_sync(0xffffffffu, wait_unit(n)) != 0;
+          continue;
         }
-        fence_proxy_async();                                   // the tiled store reads what these threads wrote
-        asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
-        if (r == 0) {
-#pragma unroll
-          for (int cc = 0; cc < SUB; ++cc) tma_store_3d(&tm_o, cc * 64, q0 + t * kBM, bh, q_sm + t * TILE_BYTES + cc * SUB_BYTES);
-          bulk_commit();
-          bulk_wait_read<0>();                                 // shared memory is read out before the CTA leaves
+        if (t >= tiles_of(u, first_row(u, r))) { ++r; continue; }
+        left = p.len_b[u.type];
+        then = p.len_a[u.type];
+        if (left == 0) { left = then; then = 0; }
+      }
+      if (pending) flush();                        // the round before this one
+      if (left == 0 || !ok) break;                 // (the end: there is no other round without keys)
+      if (lane == 0) { out_at->x = u.bh * p.n_new; out_at->y = first_row(u, r) + t * kBM; }
+      __syncwarp();
+      ++r;
+      m_used = kNoLogit;
+      l = 0.f;
+      pending = true;
+      bool first = true;
+#pragma unroll 1
+      while (ok) {
+        if (left > 64) block(first, left);
+        else tail(first, left);
+        first = false;
+        left -= kBN;
+        if (left <= 0) {
+          left = then;
+          then = 0;
+          if (left == 0) break;
         }
       }
     }
@@ -583,9 +781,10 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     tc_fence_after();
     tmem_dealloc(tmem, Shape<T>::kTmemCols);
   }
+  if (tid == 0 && bars->abort_code) atomicExch(p.status, bars->abort_code);
   // The launch behind this one relies on everything ahead of it being complete once this grid is, so
-  // one CTA does not leave before the launch ahead has completed, whatever its heads depend on.
-  if (blockIdx.x == gridDim.x - 1 && tid == 0) pdl_grid_wait();
+  // no CTA leaves before the launch ahead has completed, whatever its heads depend on.
+  if (tid == 0) pdl_grid_wait();
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -625,29 +824,13 @@ bool make_rows_map(void* out_map, const void* base, uint64_t rows, int head_dim)
 }
 
 namespace {
-// 3-D bf16 tensor map over the output [heads, n_new, head_dim] (boxes of 128 rows x 64 columns of one
-// head, 128-byte swizzle): a tile that reaches past the head's last query row is clipped there.
-bool make_out_map(CUtensorMap* out_map, const void* base, int heads, int n_new, int head_dim) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn || heads <= 0 || n_new <= 0) return false;
-  const cuuint64_t dims[3] = {(cuuint64_t)head_dim, (cuuint64_t)n_new, (cuuint64_t)heads};
-  const cuuint64_t strides[2] = {(cuuint64_t)head_dim * 2, (cuuint64_t)n_new * head_dim * 2};
-  const cuuint32_t box[3] = {64, (cuuint32_t)kBM, 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  return fn(out_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-}  // namespace
-
-namespace {
 template <int D, int T>
 int launch_tc(int grid, cudaStream_t st, const CUtensorMap& tm_q, const CUtensorMap& tk, const CUtensorMap& tv,
-              const CUtensorMap& tm_kn, const CUtensorMap& tm_vn, const CUtensorMap& tm_o, const TcParams& p) {
+              const CUtensorMap& tm_kn, const CUtensorMap& tm_vn, const TcParams& p) {
   // two tiles of head_dim 64 ask for as much as head_dim 128: one CTA per SM, it owns all of tensor memory
   const size_t smem = T == 2 ? tc_smem_bytes<128, 2>() : tc_smem_bytes<D, T>();
   if (!allow_dynamic_smem(attend_tc_kernel<D, T>, smem)) return -1;
-  launch_k(attend_tc_kernel<D, T>, grid, Shape<T>::kThreads, smem, st, tm_q, tk, tv, tm_kn, tm_vn, tm_o, p);
+  launch_k(attend_tc_kernel<D, T>, grid, Shape<T>::kThreads, smem, st, tm_q, tk, tv, tm_kn, tm_vn, p);
   return launched(1);
 }
 }  // namespace
@@ -663,11 +846,6 @@ int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_sta
   CUtensorMap tm_q;
   if (!make_rows_map(&tm_q, q, (uint64_t)a.batch * a.n_heads * a.n_new, a.head_dim)) {
     set_error("attention: cuTensorMapEncodeTiled failed for the queries");
-    return -1;
-  }
-  CUtensorMap tm_o;
-  if (!make_out_map(&tm_o, out, a.batch * a.n_heads, a.n_new, a.head_dim)) {
-    set_error("attention: cuTensorMapEncodeTiled failed for the output");
     return -1;
   }
   TcParams p;
@@ -707,15 +885,19 @@ int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_sta
   // heads x 256 queries, 680 keys: 32.0 against 30.6, 128 heads x 4 096 queries, 6 401 keys: 1 138 against 1 044.
   const int longest = (std::max(a.kept[0], a.kept[1]) + kBN - 1) / kBN;
   const bool halves = a.head_dim == 64 && longest <= (compression_ctas > 0 ? 12 : 4);
+  const int slots = sm_count() * (halves ? 2 : 1);           // CTAs that run at once
   const bool apart = p.dep[p.first_type] == kDepNothing && p.dep[1 - p.first_type] != kDepNothing;   // one type runs after the other
   for (int t = 0; t < 2; ++t) {
     const int heads = apart ? a.heads_of[t] : a.heads_of[0] + a.heads_of[1];
     const int sms = sm_count() - (p.dep[t] == kDepNothing ? compression_ctas : 0);
     p.tiles_per_cta[t] = halves || n_tiles * heads <= sms ? 1 : 2;
-    p.n_pairs[t] = (n_tiles + p.tiles_per_cta[t] - 1) / p.tiles_per_cta[t];
+    const int parts = (n_tiles + p.tiles_per_cta[t] - 1) / p.tiles_per_cta[t];
+    p.rounds[t] = a.kept[t] <= kBN && (p.len_a[t] == 0 || p.len_b[t] == 0) ? std::min(parts, std::max(1, parts * a.heads_of[t] / slots)) : 1;
+    p.units_per_head[t] = (parts + p.rounds[t] - 1) / p.rounds[t];
   }
-  p.first_ctas = p.n_pairs[p.first_type] * p.first_heads;
-  const int grid = p.first_ctas + p.n_pairs[1 - p.first_type] * a.heads_of[1 - p.first_type];
+  p.first_units = p.units_per_head[p.first_type] * p.first_heads;
+  const int grid = p.first_units + p.units_per_head[1 - p.first_type] * a.heads_of[1 - p.first_type];
+  p.steal = grid > slots - compression_ctas / (halves ? 2 : 1);
   p.pos_base = a.pos_base;
   p.head_dim_pieces = a.head_dim * 2 / 16;
   p.cap[0] = a.cap[0];
@@ -730,11 +912,12 @@ int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_sta
   p.row_off = a.row_off;
   p.head_order = a.head_order + (size_t)p.first_type * a.batch * a.n_heads;
   p.out = static_cast<__nv_bfloat16*>(out);
+  p.out_sectors = reinterpret_cast<uintptr_t>(out) % 32 == 0;
   p.row_stats = row_stats;
   p.status = a.status;
-  if (a.head_dim == 128) return launch_tc<128, 2>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, tm_o, p);
-  return halves ? launch_tc<64, 1>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, tm_o, p)
-                : launch_tc<64, 2>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, tm_o, p);
+  if (a.head_dim == 128) return launch_tc<128, 2>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, p);
+  return halves ? launch_tc<64, 1>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, p)
+                : launch_tc<64, 2>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, p);
 }
 
 }  // namespace hack

@@ -64,15 +64,38 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
-// Tiled store of a shared-memory box into a 3-D tensor (bulk group completion); elements of the box
-// that fall outside the tensor are not written.  x * element size must be a multiple of 16 bytes.
-__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, int x, int y, int z, uint32_t src) {
-  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
-               ::"l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(src)
-               : "memory");
-}
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
+// 32 bytes of one thread's own: one whole sector (the address is a multiple of 32), or two halves (of 16).
+__device__ __forceinline__ void st_global_32b(void* dst, const uint32_t* w, bool whole) {
+  if (whole)
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+  else {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    reinterpret_cast<uint4*>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  }
+}
+
+// ---------------------------------------------------------------- cluster launch control: work stealing
+// Asks for a CTA of this grid that has not been launched yet; the 16-byte answer lands in shared memory
+// and completes 16 bytes of the barrier.  After an answer without a CTA there must be no further request.
+__device__ __forceinline__ void clc_ask(uint32_t answer, uint32_t bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+               ::"r"(answer), "r"(bar) : "memory");
+}
+// The CTA's blockIdx.x, or -1 if none was left.
+__device__ __forceinline__ int clc_answer(uint32_t answer) {
+  int x;
+  asm volatile(
+      "{\n\t.reg .b128 h;\n\t.reg .pred p;\n\t"
+      "mov.s32 %0, -1;\n\tld.shared.b128 h, [%1];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, h;\n\t}"
+      : "=&r"(x) : "r"(answer) : "memory");
+  return x;
 }
 
 // Untiled bulk copies (no multicast): a contiguous run of bytes, 16-byte aligned, size a multiple of 16.
@@ -144,6 +167,16 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
         "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
         "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
         "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+}
+
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+      ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
 
@@ -293,39 +326,10 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
   return d;
 }
-// rounds both sums towards minus infinity
-__device__ __forceinline__ float2 add2_rm(float2 a, float2 b) {
-  float2 d;
-  asm("{.reg .b64 ra, rb, rd;\n\t"
-      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
-      "add.rm.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;}"
-      : "=f"(d.x), "=f"(d.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return d;
-}
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
-}
-
-// 2^x for a pair of arguments on the FMA pipe: floor by a rounded-down add of 1.5 * 2^23, a cubic
-// for 2^frac on [0, 1) (minimax fit, relative error 7.5e-5: far below bf16 rounding) and the
-// integer part added into the exponent field.  Arguments are clamped at -126.
-__device__ __forceinline__ float2 ex2_poly2(float2 x) {
-  const float kMagic = 12582912.f;
-  x.x = fmaxf(x.x, -126.f);
-  x.y = fmaxf(x.y, -126.f);
-  const float2 t = add2_rm(x, make_float2(kMagic, kMagic));
-  const float2 nf = add2(t, make_float2(-kMagic, -kMagic));
-  const float2 fr = fma2(nf, make_float2(-1.f, -1.f), x);
-  float2 p = fma2(fr, make_float2(0.07802452892065048f, 0.07802452892065048f),
-                  make_float2(0.22606714069843292f, 0.22606714069843292f));
-  p = fma2(p, fr, make_float2(0.6958335638046265f, 0.6958335638046265f));
-  p = fma2(p, fr, make_float2(0.9999251961708069f, 0.9999251961708069f));
-  p.x = __uint_as_float(__float_as_uint(t.x) * 8388608u + __float_as_uint(p.x));   // one multiply-add
-  p.y = __uint_as_float(__float_as_uint(t.y) * 8388608u + __float_as_uint(p.y));
-  return p;
 }
 
 // 32 lanes x 8 consecutive 32-bit columns (for paths that must stay light on registers)

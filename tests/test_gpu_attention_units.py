@@ -1,0 +1,60 @@
+"""The tensor-core attention at the edges of its work split: last blocks of a segment of every number of 32-key
+groups (the caller's rows and the cache's), more units than CTAs run at once (a CTA takes over units that were not
+launched), and heads whose keys are one block (several rounds of query tiles per unit).  Heads are compared with
+64-bit attention over the rows the cache reports; bar 2e-2 max-abs as in the parity tests of bf16 outputs."""
+import math
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__ as ge
+    ge.build()
+
+
+def decode(dim, heads, batch, sides, b_c, b_s, sample):
+    import torch
+    import paper_2504_09261_b200 as hb
+    mask = (np.arange(heads) % 2).astype(np.uint8)[None]
+    cache = hb.HackCache(1, heads, dim, batch, sides, hb.HACK_BF16, mask, b_c, b_s)
+    g = torch.Generator(device="cuda").manual_seed(dim + heads)
+    ks, vs = [], []
+    for k, side in enumerate(sides):
+        q, kk, v = (torch.randn((batch, heads, side * side, dim), generator=g, device="cuda").bfloat16() for _ in range(3))
+        ks.append(kk)
+        vs.append(v)
+        out = torch.full_like(q, float("nan"))
+        cache.hack_scale_step(0, k, q, kk, v, out)
+        assert bool(torch.isfinite(out).all())
+        for b, h in sample:
+            pos = torch.from_numpy(np.frombuffer(cache.hack_read_head(0, b, h, 2), dtype=np.int32).copy()).long().cuda()
+            kc, vc = (torch.cat([t[b, h] for t in part])[pos].double() for part in (ks, vs))
+            ref = (q[b, h].double() @ kc.T / math.sqrt(dim)).softmax(-1) @ vc
+            err = (out[b, h].double() - ref).abs().max().item()
+            assert err <= 2e-2, (side, b, h, len(pos), err)
+    cache.hack_poll_status()
+    cache.close()
+
+
+# tokens modulo 128: 17 -> 16, 21 -> 57, 15 -> 97, 31 -> 65, 24 -> 64, 23 -> 17, 22 -> 100, 20 -> 16, 30 -> 4, 16 -> 0
+@pytest.mark.parametrize("dim,heads,batch,sides", [
+    (64, 3, 1, (15, 17, 31)), (64, 2, 2, (24, 23, 21)), (64, 5, 60, (15, 16, 17)),
+    (128, 3, 1, (15, 17, 31)), (128, 2, 2, (24, 23, 21)), (128, 9, 12, (22, 20, 30)), (128, 2, 100, (16, 31)),
+])
+def test_last_blocks_of_both_segments(dim, heads, batch, sides):
+    total = sum(s * s for s in sides)
+    decode(dim, heads, batch, sides, total, total, [(0, 0), (batch - 1, heads - 1)])
+
+
+@pytest.mark.parametrize("dim,heads,batch,sides,b_c,b_s", [
+    (64, 16, 16, (2, 8, 20, 32), 33, 1045),      # contextual heads of one short block, 6 rounds of one tile
+    (128, 12, 10, (2, 9, 33, 40), 100, 1700),    # the same on two tiles, an odd number of rounds
+    (64, 30, 12, (3, 9, 21, 24), 128, 700),      # a whole block
+    (128, 30, 8, (2, 7, 18, 29), 230, 900),      # more units than SMs, behind a compression
+])
+def test_rounds_and_units_that_change_hands(dim, heads, batch, sides, b_c, b_s):
+    decode(dim, heads, batch, sides, b_c, b_s, [(0, 0), (0, 1), (batch // 2, heads - 1), (batch - 1, heads - 2)])
