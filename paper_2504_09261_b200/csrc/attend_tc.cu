@@ -68,6 +68,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "hack_internal.h"
 #include "tc_ptx.cuh"
@@ -624,40 +625,41 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       if (lane == 0) mbar_arrive(smem_u32(&bars->p_full[t]));
       ++cnt;
     };
-    // A block of 65 to 128 keys.
-    auto block = [&](bool first, int valid) {
+    // A block of keys, the first `valid` of them live, in G groups of 32: 4, or (the last block of a segment) 2.
+    auto block = [&](auto groups_c, bool first, int valid) {
+      constexpr int G = decltype(groups_c)::value, N = 32 * G;
       ok = bar_all(&bars->s_full[t], cnt & 1, 8);
       if (!ok) return;
       tc_fence_after();
-      uint32_t sr[kBN];
+      uint32_t sr[N];
 #pragma unroll
-      for (int ch = 0; ch < kBN / 32; ++ch) tmem_ld32(s_addr + ch * 32, sr + ch * 32);
+      for (int ch = 0; ch < G; ++ch) tmem_ld32(s_addr + ch * 32, sr + ch * 32);
       tmem_wait_ld();
       // the logits are in registers: the buffer goes back to the MMA warp at once
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bars->s_free));
-      if (__builtin_expect(valid < kBN, 0)) {
+      if (__builtin_expect(valid < N, 0)) {
 #pragma unroll
-        for (int i = 64; i < kBN; ++i)
+        for (int i = G == 4 ? 64 : 0; i < N; ++i)
           if (i >= valid) sr[i] = 0xff800000u;   // -inf
       }
-      float mx4[4];
+      float mx4[G];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < G; ++u) {
         mx4[u] = -INFINITY;
 #pragma unroll
         for (int i = 0; i < 16; ++i) mx4[u] = max3(mx4[u], __uint_as_float(sr[u * 32 + 2 * i]), __uint_as_float(sr[u * 32 + 2 * i + 1]));
       }
-      const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+      const float mx = G == 4 ? fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[G - 2], mx4[G - 1])) : fmaxf(mx4[0], mx4[1]);
       float alpha;
       const bool any_grow = raise(mx, alpha);
       const float2 c2 = make_float2(c, c);
       const float2 nmc2 = make_float2(-m_used * c, -m_used * c);
       float2 sum4[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      uint32_t pk[kBN / 2];
+      uint32_t pk[N / 2];
 #pragma unroll
-      for (int i = 0; i < kBN / 2; ++i) {
+      for (int i = 0; i < N / 2; ++i) {
         const float2 x = fma2(make_float2(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1])), c2, nmc2);
         float2 pr;
         pr.x = ex2(x.x);
@@ -673,63 +675,9 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         wait_p(any_grow && !first, alpha);
         if (!ok) return;
       }
-      tmem_st32(p_addr, pk);
-      tmem_st32(p_addr + 32, pk + 32);
+#pragma unroll
+      for (int ch = 0; ch < G / 2; ++ch) tmem_st32(p_addr + ch * 32, pk + ch * 32);
       give_p();
-    };
-    // The last block of a segment, up to 64 keys: 32 at a time and in little code, which reads the logits twice.  (With
-    // up to 127 keys this way, 126 units of 3 to 8 blocks took 34 instead of 33 us a step.)
-    auto tail = [&](bool first, int valid) {
-      ok = bar_all(&bars->s_full[t], cnt & 1, 8);
-      if (!ok) return;
-      tc_fence_after();
-      auto load = [&](int ch, uint32_t* sr) {
-        tmem_ld32(s_addr + ch, sr);
-        tmem_wait_ld();
-        if (valid - ch < 32) {
-#pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if (i >= valid - ch) sr[i] = 0xff800000u;   // -inf
-        }
-      };
-      float mx = -INFINITY;
-#pragma unroll 1
-      for (int ch = 0; ch < valid; ch += 32) {
-        uint32_t sr[32];
-        load(ch, sr);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) mx = max3(mx, __uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1]));
-      }
-      float alpha;
-      const bool any_grow = raise(mx, alpha);
-      const float2 c2 = make_float2(c, c);
-      const float2 nmc2 = make_float2(-m_used * c, -m_used * c);
-      if (cnt > 0) {
-        wait_p(any_grow && !first, alpha);
-        if (!ok) return;
-      }
-      float2 sum4[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll 1
-      for (int ch = 0; ch < valid; ch += 32) {
-        uint32_t sr[32], pk[16];
-        load(ch, sr);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const float2 x = fma2(make_float2(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1])), c2, nmc2);
-          float2 pr;
-          pr.x = ex2(x.x);
-          pr.y = ex2(x.y);
-          sum4[i & 3] = add2(sum4[i & 3], pr);
-          const __nv_bfloat162 hh = __floats2bfloat162_rn(pr.x, pr.y);
-          pk[i] = *reinterpret_cast<const uint32_t*>(&hh);
-        }
-        tmem_st16(p_addr + ch / 2, pk);
-      }
-      const float2 sum2 = add2(add2(sum4[0], sum4[1]), add2(sum4[2], sum4[3]));
-      l += sum2.x + sum2.y;
-      l += top_rounding(mx, nmc2.x);
-      give_p();                                            // (its fence orders the logits' reads as well)
-      if (lane == 0) mbar_arrive(smem_u32(&bars->s_free));
     };
     // (What a round needs is read where it is needed: registers that live through a block are scarce.)
     int n = 0, r = 0;
@@ -763,8 +711,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       bool first = true;
 #pragma unroll 1
       while (ok) {
-        if (left > 64) block(first, left);
-        else tail(first, left);
+        if (left > 64) block(std::integral_constant<int, 4>(), first, left);
+        else block(std::integral_constant<int, 2>(), first, left);
         first = false;
         left -= kBN;
         if (left <= 0) {
