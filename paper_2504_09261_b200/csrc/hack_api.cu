@@ -106,6 +106,8 @@ struct hack_cache {
   hack::MergeScratch merge{};                   // merge_last: scratch of the final-scale merge
   TensorMapBox merge_ev_map;
   float* attn_row_stats = nullptr;              // bf16 caches: [b*H, max N_k, 2] softmax row statistics (Eq. 6 path)
+  float* simt_partial = nullptr;                // fp32 caches: scratch and counters of query tiles that CTAs share
+  int32_t* simt_arrived = nullptr;
   float* attn_block_var = nullptr;              // bf16 caches: [b*H, var_blocks] per key block variances
   int var_blocks = 0;
   int32_t* obs_rows = nullptr;                  // HACK_OBS_CALLER: [n_scales][kMaxObs] query rows of Q~
@@ -220,6 +222,8 @@ hack::StepArgs make_args(const hack_cache* c, int layer, int scale, const hack_s
     a.k_map = &c->k_maps[layer];
     a.v_map = &c->v_maps[layer];
   }
+  a.simt_partial = c->simt_partial;
+  a.simt_arrived = c->simt_arrived;
   a.head_order = c->head_order + (size_t)layer * 2 * c->cfg.batch * c->cfg.n_heads;
   return a;
 }
@@ -490,6 +494,12 @@ hack_status_t hack_init_cache(const hack_config_t* cfg, hack_cache_t** out) {
     HACK_TRY(cudaMalloc(&c->attn_row_stats, (size_t)bh * c->limits.max_new * 2 * sizeof(float)));
     HACK_TRY(cudaMalloc(&c->attn_block_var, (size_t)bh * c->var_blocks * sizeof(float)));
   }
+  if (cfg->dtype == HACK_F32) {
+    const size_t words = hack::simt_arrived_words(bh, c->limits.max_new);
+    HACK_TRY(cudaMalloc(&c->simt_partial, hack::simt_partial_floats(cfg->head_dim) * sizeof(float)));
+    HACK_TRY(cudaMalloc(&c->simt_arrived, words * sizeof(int32_t)));
+    HACK_TRY(cudaMemset(c->simt_arrived, 0, words * sizeof(int32_t)));
+  }
   if (cfg->merge_last) {
     // what the contextual heads discard at the last scale
     LayerState ls;
@@ -547,6 +557,8 @@ hack_status_t hack_free_cache(hack_cache_t* c) {
   cudaFree(c->merge.weight);
   cudaFree(c->attn_row_stats);
   cudaFree(c->attn_block_var);
+  cudaFree(c->simt_partial);
+  cudaFree(c->simt_arrived);
   cudaFree(c->obs_rows);
   for (int sl = 0; sl < hack_cache::kHostSlots; ++sl) {
     for (int i = 0; i < 4; ++i) cudaFree(c->stage[sl][i]);

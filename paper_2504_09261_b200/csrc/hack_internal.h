@@ -50,6 +50,8 @@ struct StepArgs {
   const void* k_map;
   const void* v_map;
   const int32_t* head_order;   // device, [2][batch*n_heads]: structural heads first, contextual heads first
+  float* simt_partial;         // fp32 attention: device scratch of query tiles that CTAs share (simt_partial_floats) ...
+  int32_t* simt_arrived;       // ... and their counters (simt_arrived_words), zero between launches
 };
 
 struct Scratch {
@@ -101,6 +103,9 @@ int launch_compact(const StepArgs& a, int dtype, const int32_t* idx, int idx_all
 int launch_attend(const StepArgs& a, int dtype, const void* q, void* out, cudaStream_t st);
 
 int launch_attend_simt(const StepArgs& a, const void* q, void* out, cudaStream_t st);   // fp32 caches
+// Its scratch of one cache, on the current device.
+size_t simt_partial_floats(int head_dim);
+size_t simt_arrived_words(int heads, int max_new);
 // row_stats (optional, device [b*H, N_k, 2]): per query row the reference maximum m (raw logit
 // units; within the lazy-rescaling margin of the true maximum) and l = sum_j exp2(c (z_j - m)).
 // k_new / v_new (optional): the caller's K/V of this scale; head types with a.seg_new set then attend

@@ -90,3 +90,35 @@ def test_selection_that_moves_the_rows(head_dim, b_c, b_s, policy):
     assert rep.ok(), rep.problems[:5]
     assert rep.compressed_heads > 0
     assert rep.evicting_launches[-1] == 3, rep.evicting_launches      # scores, selection with the moves, attention
+
+
+@pytest.mark.parametrize("head_dim,heads,batch,sides,b_c,b_s", [
+    (64, 16, 2, (2, 7, 18), 40, 377), (64, 13, 3, (3, 11, 17, 19), 33, 800), (128, 16, 1, (2, 9, 18, 21), 130, 850),
+    (128, 20, 1, (1, 16, 17), 545, 546), (128, 11, 2, (2, 23, 24), 1, 1000),
+])
+def test_query_tiles_that_ctas_share(head_dim, heads, batch, sides, b_c, b_s):
+    """More query tiles than SMs, heads of one and of two lengths: shares that begin and end inside a tile, in its
+    last round, and tiles of one round.  Against fp64 attention over the rows the cache reports."""
+    import numpy as np
+    import torch
+    import paper_2504_09261_b200 as hb
+    mask = (np.arange(heads) % 2).astype(np.uint8)[None]
+    cache = hb.HackCache(1, heads, head_dim, batch, sides, hb.HACK_F32, mask, b_c, b_s)
+    g = torch.Generator(device="cuda").manual_seed(heads * batch)
+    for _ in range(2):                                   # the second time on counters the first has left behind
+        cache.hack_reset()
+        ks, vs = [], []
+        for k, side in enumerate(sides):
+            q, kk, v = (torch.randn((batch, heads, side * side, head_dim), generator=g, device="cuda") for _ in range(3))
+            ks.append(kk)
+            vs.append(v)
+            out = torch.full_like(q, float("nan"))
+            cache.hack_scale_step(0, k, q, kk, v, out)
+            kc, vc = torch.cat(ks, 2).double(), torch.cat(vs, 2).double()
+            for b in range(batch):
+                for h in range(heads):
+                    pos = torch.from_numpy(np.frombuffer(cache.hack_read_head(0, b, h, 2), dtype=np.int32).copy()).long().cuda()
+                    z = q[b, h].double() @ kc[b, h, pos].T / math.sqrt(head_dim)
+                    ref = z.softmax(-1) @ vc[b, h, pos]
+                    assert (out[b, h].double() - ref).abs().max() <= 1e-5, (k, b, h)
+    cache.close()
