@@ -331,8 +331,8 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   if (warp == kIssueWarp && lane == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(smem_u32(&sh->full[s]), 1); mbar_init(smem_u32(&sh->empty[s]), 1); }
     for (int i = 0; i < n_seq; ++i) mbar_init(smem_u32(&sh->acc_full[i]), 1);
-    mbar_init(smem_u32(&sh->acc_free[0]), kWorkers);
-    mbar_init(smem_u32(&sh->acc_free[1]), kWorkers);
+    mbar_init(smem_u32(&sh->acc_free[0]), kWorkers / 32);   // a warp arrives once
+    mbar_init(smem_u32(&sh->acc_free[1]), kWorkers / 32);
     mbar_init(smem_u32(&sh->drain), 1);
     sh->abort_flag = 0;
     fence_barrier_init();
@@ -437,7 +437,8 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
       tmem_wait_ld();
       if (i >= p.direct) {
         tc_fence_before();
-        mbar_arrive(smem_u32(&sh->acc_free[(i - p.direct) & 1]));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&sh->acc_free[(i - p.direct) & 1]));
         if (i < n_held) {
           float* dst = over + ((size_t)(i - p.direct) * kMaxObs + set * kHalfObs) * kCkChunk + key_row;
 #pragma unroll
@@ -554,9 +555,10 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
           tmem_ld16(t_lane + (again ? acc_slot(seq) : i) * kMaxObs + h * kHalfObs, acc);
           tmem_wait_ld();
           if (again && h == 1) {
-            // the accumulator counts a release by every worker; the 128 of this set stand for all of them
+            // the accumulator counts a release by every worker warp; the four of this set stand for all of them
             tc_fence_before();
-            mbar_arrive_n(smem_u32(&sh->acc_free[(seq - p.direct) & 1]), kWorkers / 128);
+            __syncwarp();
+            if (lane == 0) mbar_arrive_n(smem_u32(&sh->acc_free[(seq - p.direct) & 1]), 2);
           }
         } else {
           const float* src = over + ((size_t)(i - p.direct) * kMaxObs + h * kHalfObs) * kCkChunk + key_row;
