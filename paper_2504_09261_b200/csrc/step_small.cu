@@ -380,9 +380,11 @@ step_small_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, const _
 }
 
 // Microseconds of this launch and of the two launches it stands for (compression, then attention).  Both
-// forms were fitted to 287 steps of 8 to 256 heads, 16 to 400 queries and 50 to 700 candidates (rms 8 and 6 %);
-// with the margin of a tenth none of them was slower here.  The fit is from before the last 0.7 us came off
-// this side, so the line errs towards the two launches: steps just beyond it would gain up to a fifth here.  16 heads x 64, 36 queries, 91 candidates: 5.9 against 12.6;
+// forms were fitted to 287 steps of 8 to 256 heads, 16 to 400 queries and 50 to 700 candidates (rms 8 and 6 %).
+// This side has become faster since the fit where every CTA has an SM and a cluster is smaller than eight, so there it
+// is taken up to a tenth past the line, to 256 queries: 13 heads x 128, 121 queries 20.5 -> 15.7 us, 36 heads, 169 queries
+// 22.2 -> 18.4, 52 heads x 64, 196 queries 22.5 -> 19.1.  Elsewhere it keeps a margin of a tenth (81 heads x 64, 169 queries
+// 20.5 against 24.6; 18 heads, 400 queries 21.2 against 22.5).  16 heads x 64, 36 queries, 91 candidates: 5.9 against 12.6;
 // 256 heads: 9.3 against 18.2; 100 queries, 168 and 255 candidates: 7.3 against 12.8 (16 heads), 20.2 against
 // 19.9 (256 heads: not taken); 16 heads x 128, 36 queries, 91 candidates: 7.5 against 15.0; 256 heads: 18.6
 // against 25.2.
@@ -406,7 +408,7 @@ bool step_small_pays(const StepArgs& a, const StepShape& s, int per_sm) {
                               ctas > sms * per_sm ? mean * (ctas / (sms * per_sm) * (per_sm == 2 ? 1.67f : 1.f) + 0.3f) : 0.f);
   const float apart = D == 64 ? 10.8f + (1.58f * heads + 0.92f * work) / sms + 1.57f * ranked
                               : 11.9f + (3.92f * heads + 1.13f * work) / sms + 1.94f * ranked;
-  return here * 1.1f < apart;
+  return here * (ctas <= sms && s.ctas < kMaxCtas && a.n_new <= 256 ? 0.9f : 1.1f) < apart;
 }
 
 template <int D>
