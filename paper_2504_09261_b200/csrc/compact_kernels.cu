@@ -17,6 +17,8 @@
 // Heads whose type evicts nothing keep every candidate, so their list is the identity and n_old = L; a step in
 // which no type evicts is the copy kernel alone (the moves of 32 heads that stay where they are took 36 us at 6 425
 // stored rows, 4 to 5 where there is next to nothing stored).
+#include <algorithm>
+
 #include "hack_internal.h"
 
 namespace hack {
@@ -114,15 +116,15 @@ compact_move_kernel(const StepArgs a, const int32_t* __restrict__ idx, int row_p
 }
 
 __global__ void __launch_bounds__(kThreads)
-compact_copy_kernel(const StepArgs a, const int32_t* __restrict__ idx, const uint4* __restrict__ k_new,
+compact_copy_kernel(const StepArgs a, const int32_t* __restrict__ idx, int idx_all, const uint4* __restrict__ k_new,
                     const uint4* __restrict__ v_new, int row_pieces) {
   pdl_wait();
   const int bh = blockIdx.z;
   const int ctx = a.is_ctx[bh % a.n_heads];
   if (a.seg_new[ctx]) return;                      // the attention launch appends this type's new rows
   const int stored = a.stored[ctx], n_keep = a.kept[ctx];
-  const int32_t* list = idx ? idx + (size_t)bh * a.kept_stride : nullptr;
-  const int n_old = list ? a.n_old[bh] : stored;
+  const int32_t* list = idx && (idx_all || ctx) ? idx + (size_t)bh * a.kept_stride : nullptr;
+  const int n_old = list ? a.n_old[bh] : n_keep - a.n_new;   // no list: all new rows, behind what the head keeps of the stored ones
   const int plane_id = blockIdx.y;                 // 0: K (also writes the positions), 1: V
   const size_t off = a.row_off[bh];
   const int tid = threadIdx.x;
@@ -141,7 +143,7 @@ compact_copy_kernel(const StepArgs a, const int32_t* __restrict__ idx, const uin
       const int r = c0 + u * rows_per_pass + rsub;
       ok[u] = false;
       if (r < n_keep) {
-        const int src = (list ? list[r] : r) - stored;
+        const int src = list ? list[r] - stored : r - n_old;
         ok[u] = dbg_ok(src >= 0 && src < a.n_new && r < a.cap[ctx], a.status, 3);
         if (!ok[u]) continue;
         val[u] = fresh[(size_t)src * row_pieces + piece];
@@ -160,7 +162,6 @@ compact_copy_kernel(const StepArgs a, const int32_t* __restrict__ idx, const uin
 
 int launch_compact(const StepArgs& a, int dtype, const int32_t* idx, int idx_all, const void* k_new,
                    const void* v_new, cudaStream_t st) {
-  (void)idx_all;                                    // an index list, when given, covers every head
   const int elt = dtype == HACK_F32 ? 4 : 2;
   const int row_pieces = a.head_dim * elt / 16;    // 8, 16 or 32
   const int heads = a.batch * a.n_heads;
@@ -177,12 +178,12 @@ int launch_compact(const StepArgs& a, int dtype, const int32_t* idx, int idx_all
   if (idx) {
     most = 0;
     for (int t = 0; t < 2; ++t)
-      if (!a.seg_new[t] && a.kept[t] > most) most = a.kept[t];
+      if (!a.seg_new[t]) most = std::max(most, idx_all || t == 1 ? a.kept[t] : a.n_new);
   }
   int n_copy = (most + rows_per_cta - 1) / rows_per_cta;
   const int cap = (16 * sm_count() + 2 * heads - 1) / (2 * heads);
   n_copy = n_copy < 1 ? 1 : (n_copy > cap ? cap : n_copy);
-  launch_k(compact_copy_kernel, dim3(n_copy, 2, heads), dim3(kThreads), 0, st, a, idx,
+  launch_k(compact_copy_kernel, dim3(n_copy, 2, heads), dim3(kThreads), 0, st, a, idx, idx_all,
            static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), row_pieces);
   return launched(n + 1);
 }

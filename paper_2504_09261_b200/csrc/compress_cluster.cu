@@ -35,6 +35,7 @@
 //      own rows, at or behind its destination; a surviving new row from the caller's K/V) into shared
 //      memory, the cluster meets, and the run goes out with bulk stores.  The destinations of a round
 //      lie at or before its own cache sources and before those of every later round: in place.
+//      (Contextual heads of a step that merges: the list and its complement go to memory, nothing moves.)
 //   7. heads that keep the whole new scale stop behind their stored survivors; the attention
 //      launch reads their new rows from the caller's tensors and appends them itself.
 //
@@ -98,6 +99,9 @@ struct CkParams {
   int stage_rows;             // rows (K and V) a CTA stages in shared memory per round of the compaction
   int score_only;             // stop after the scores
   float* scores;              // [b*H, cand_stride] or nullptr
+  int32_t* kept_list;         // contextual heads: their list goes here, [b*H, kept_stride], and the rest of the
+  int32_t* gone_list;         // candidates here, [b*H, gone_stride], and no row is moved; or both nullptr
+  int gone_stride;
   const uint4* k_new;         // caller's K/V of this scale (compaction of heads whose new rows compete)
   const uint4* v_new;
 };
@@ -243,7 +247,8 @@ __device__ __forceinline__ int ck_block_scan(int v, int* sums, int& total) {
 
 // kAgain: some CTA holds ranked chunks whose logits are formed a second time (a form of its own: the code
 // for it costs a launch of few chunks 0.3 us).
-template <int D, bool kAgain>
+// kLists: a step that merges (kept_list, gone_list).
+template <int D, bool kAgain, bool kLists = false>
 __global__ void __launch_bounds__(kCkThreads, 2)
 compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __grid_constant__ CUtensorMap tm_new,
                         const StepArgs a, const __nv_bfloat16* __restrict__ q, const CkParams p) {
@@ -791,6 +796,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
     // o / S and o / RS by a multiplication: exact for o < 65 536 and divisors up to 65 536
     const uint32_t inv_s = 0xffffffffu / (uint32_t)S + 1u, inv_rs = 0xffffffffu / (uint32_t)RS + 1u;
     const uint32_t lower = (1u << lane) - 1u;
+    const bool lists = kLists && ctx;
     for (int g = g_begin; g < g_end; ++g) {
       const int slot = g * 32 + lane;
       int j;
@@ -800,7 +806,14 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
       const uint32_t m_gt = __ballot_sync(0xffffffffu, is_gt), m_eq = __ballot_sync(0xffffffffu, is_eq);
       const int eq_rank = eq_before + __popc(m_eq & lower);
       const int o = gt_before + __popc(m_gt & lower) + min(eq_rank, need);
-      if ((is_gt || (is_eq && eq_rank < need)) && dbg_ok(o >= 0 && o < n_rows, a.status, 9)) {
+      if (lists) {
+        // (as many survivors as o are ahead of an entry, whether it is one itself or not)
+        if (is_gt || (is_eq && eq_rank < need)) {
+          if (dbg_ok(o >= 0 && o < a.kept_stride, a.status, 9)) p.kept_list[(size_t)bh * a.kept_stride + o] = j;
+        } else if (live && dbg_ok(j - o >= 0 && j - o < p.gone_stride, a.status, 9)) {
+          p.gone_list[(size_t)bh * p.gone_stride + (j - o)] = j;
+        }
+      } else if ((is_gt || (is_eq && eq_rank < need)) && dbg_ok(o >= 0 && o < n_rows, a.status, 9)) {
         const int t = RS == 1 ? o : (int)__umulhi((uint32_t)o, inv_rs), w = o - t * RS;
         const int rk = S == 1 ? w : (int)__umulhi((uint32_t)w, inv_s), lr = w - rk * S;
         st_peer_i32(peer_addr(&src_all[t * S + lr], rk), j);
@@ -860,9 +873,12 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
       }
       cp_async_commit();                                      // one group per round, empty or not
     };
-    issue_loads(0);
-    issue_loads(1);
-    for (int t = 0; t < n_rounds; ++t) {
+    const int n_moves = lists ? 0 : n_rounds;
+    if (n_moves > 0) {
+      issue_loads(0);
+      issue_loads(1);
+    }
+    for (int t = 0; t < n_moves; ++t) {
       cp_async_wait_group<1>();                               // the loads of round t (all but the latest group) have landed
       fence_proxy_async();                                    // the bulk stores below read what these threads wrote
       cluster_sync_relaxed(CL);                               // every source of this round has been read
@@ -1037,7 +1053,8 @@ int launch_t(const StepArgs& a, const CUtensorMap& tm_cache, const CUtensorMap& 
              const CkLists& lists, int n_clusters, float beside_us, float behind_us, uint16_t* shape, cudaStream_t st) {
   // the opt-in is made once per (kernel, device), so it asks for the most any launch can need
   if (!allow_dynamic_smem(compress_cluster_kernel<D, false>, kSmemBudget) ||
-      !allow_dynamic_smem(compress_cluster_kernel<D, true>, kSmemBudget))
+      !allow_dynamic_smem(compress_cluster_kernel<D, true>, kSmemBudget) ||
+      !allow_dynamic_smem(compress_cluster_kernel<D, true, true>, kSmemBudget))
     return -1;
   // CTAs per head and per SM: the step ends when this launch and the attention that needs it are done,
   // and not before the SMs have done all the work there is (larger clusters finish sooner and keep
@@ -1074,7 +1091,7 @@ int launch_t(const StepArgs& a, const CUtensorMap& tm_cache, const CUtensorMap& 
   ck_shape<D>(p, lists, best_cl, best_per_sm);
   cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = ck_config<D>(a, p, attr, st);
-  cudaLaunchKernelEx(&cfg, ck_again(p) > 0 ? compress_cluster_kernel<D, true> : compress_cluster_kernel<D, false>, tm_cache, tm_new, a, static_cast<const __nv_bfloat16*>(q), p);
+  cudaLaunchKernelEx(&cfg, p.kept_list ? compress_cluster_kernel<D, true, true> : ck_again(p) > 0 ? compress_cluster_kernel<D, true> : compress_cluster_kernel<D, false>, tm_cache, tm_new, a, static_cast<const __nv_bfloat16*>(q), p);
   return launched(n_clusters * p.cluster);
 }
 
@@ -1085,12 +1102,16 @@ int launch_t(const StepArgs& a, const CUtensorMap& tm_cache, const CUtensorMap& 
 // (candidate lists far beyond 8 x 40 chunks per head, the every-query scoring rounds): the caller then
 // takes the separate scoring, selection and compaction launches.
 int launch_compress_cluster(const StepArgs& a, const void* q, const void* k_new, const void* v_new, float* scores,
-                            cudaStream_t st, float beside_us, float behind_us, uint16_t* shape) {
+                            cudaStream_t st, float beside_us, float behind_us, uint16_t* shape, int32_t* kept_list, int32_t* gone_list,
+                            int gone_stride) {
   if (!a.k_map || a.obs_full || a.score_accumulate) return 0;
   if (!a.trig[0] && !a.trig[1]) return 0;
   CkParams p{};
   p.score_only = scores != nullptr;
   p.scores = scores;
+  p.kept_list = kept_list;
+  p.gone_list = gone_list;
+  p.gone_stride = gone_stride;
   p.k_new = static_cast<const uint4*>(k_new);
   p.v_new = static_cast<const uint4*>(v_new);
   CkLists lists = {};
@@ -1100,7 +1121,7 @@ int launch_compress_cluster(const StepArgs& a, const void* q, const void* k_new,
       const bool drop_new = t == 0 && a.protect_new && !scores;
       lists.ranked[t] = (a.stored[t] + kCkChunk - 1) / kCkChunk + (drop_new ? 0 : n_new_chunks);
       lists.once[t] = drop_new ? n_new_chunks : 0;
-      lists.rows[t] = scores ? 0 : a.kept[t] - (drop_new ? a.n_new : 0);
+      lists.rows[t] = scores || (t == 1 && kept_list) ? 0 : a.kept[t] - (drop_new ? a.n_new : 0);
     }
   // clusters that do work: the heads of the triggered types
   const int n_clusters = std::max(1, a.heads_of[0] * a.trig[0] + a.heads_of[1] * a.trig[1]);

@@ -73,8 +73,8 @@ struct MergeScratch {
   float* weight;               // [b*H, stride] max(cosine similarity, 0)
   const void* ev_map;          // host pointer to the 128-byte tensor map over ev_k
 };
-// Before the compaction of the step (idx = the kept lists of launch_select) and after it.
-int launch_merge_prepare(const StepArgs& a, const MergeScratch& ms, const int32_t* idx, const void* k_new,
+// Before the compaction of the step (idx = the kept lists; listed: ms.ev_idx holds their complements already) and after it.
+int launch_merge_prepare(const StepArgs& a, const MergeScratch& ms, const int32_t* idx, bool listed, const void* k_new,
                          const void* v_new, cudaStream_t st);
 int launch_merge_finish(const StepArgs& a, const MergeScratch& ms, cudaStream_t st);
 
@@ -93,11 +93,13 @@ int launch_select_move(const StepArgs& a, int dtype, const float* scores, const 
 // in one launch of one thread-block cluster per head.  Its CTAs if launched; 0: the step is outside what
 // the kernel holds, take the separate launches; -1: launch error.  beside_us, behind_us: SM-microseconds
 // of the attention launch behind this one that can run beside it, and that need its result.  shape: the
-// launch shape of this step as found before (0: not yet), kept by the caller.
+// launch shape of this step as found before (0: not yet), kept by the caller.  kept_list, gone_list: the lists of
+// the contextual heads and their complements go there, ascending, and their rows stay where they are (a step that merges).
 int launch_compress_cluster(const StepArgs& a, const void* q, const void* k_new, const void* v_new, float* scores,
-                            cudaStream_t st, float beside_us = 0.f, float behind_us = 0.f, uint16_t* shape = nullptr);
-// idx == nullptr: every head appends (keeps all candidates).  idx_all != 0: idx rows are valid for
-// heads that are not triggered as well (identity lists written by launch_select).
+                            cudaStream_t st, float beside_us = 0.f, float behind_us = 0.f, uint16_t* shape = nullptr,
+                            int32_t* kept_list = nullptr, int32_t* gone_list = nullptr, int gone_stride = 0);
+// idx == nullptr: every head appends (keeps all candidates).  idx_all: there is a list for every head; 0: for the contextual
+// ones, and the stored rows that the others keep are in place already (a.trig[0] must be 0).
 int launch_compact(const StepArgs& a, int dtype, const int32_t* idx, int idx_all, const void* k_new,
                    const void* v_new, cudaStream_t st);
 int launch_attend(const StepArgs& a, int dtype, const void* q, void* out, cudaStream_t st);

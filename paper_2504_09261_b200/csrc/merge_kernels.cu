@@ -209,7 +209,7 @@ merge_assign_kernel(const __grid_constant__ CUtensorMap tm_e, const __grid_const
   if (tid == 0) {
     mbar_init(smem_u32(&bars->e_full), 1);
     for (int s = 0; s < kRing; ++s) { mbar_init(smem_u32(&bars->k_full[s]), 1); mbar_init(smem_u32(&bars->k_empty[s]), 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&bars->acc_full[b]), 1); mbar_init(smem_u32(&bars->acc_free[b]), kTileM); }
+    for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&bars->acc_full[b]), 1); mbar_init(smem_u32(&bars->acc_free[b]), kTileM / 32); }
     mbar_init(smem_u32(&bars->drain), 1);
     bars->abort_flag = 0;
     fence_barrier_init();
@@ -282,12 +282,18 @@ merge_assign_kernel(const __grid_constant__ CUtensorMap tm_e, const __grid_const
     const int quad = warp & 3;                                // TMEM lane quadrant this warp may read
     const int my_row = eb * kTileM + quad * 32 + lane;        // discarded entry this thread owns
     const uint32_t t_lane = tmem + (static_cast<uint32_t>(quad * 32) << 16);
-    // Issue slots bound this: the running maximum is compared with the largest of four columns, and only
-    // where that is a new maximum is the column looked for (7 instead of 16 instructions per four
-    // columns).  The norms are fetched one tile ahead.
+    // Bound by the latency of a reading warp's chain of instructions (0.9 us per tile and CTA, 1.3 with two on the SM):
+    // the largest of 32 columns is formed as a tree, the 32 columns that hold the best one so far are kept
+    // without a branch, and which of them it is is looked up once, at the end.  The next columns and norms are
+    // on their way meanwhile.  (Four columns at a time, looked up at once: 62 us, now 55.  Two tiles of discarded rows that share
+    // the retained tiles, or eight reading warps per tile: no faster.)
     float best = -INFINITY;
-    int arg = 0;
-    bool ok = true;
+    int arg = 0;                                              // first of the 32 columns with the best one ...
+    float2 won[16];                                           // ... and those columns
+#pragma unroll
+    for (int i = 0; i < 16; ++i) won[i] = make_float2(-INFINITY, -INFINITY);
+    int last = 0;
+    bool ok = true, single = false;
     // Every warp keeps its own copy of a tile's norms, so that the warps do not meet inside the loop.
     float inv[4];
     auto fetch = [&](int t) {
@@ -309,29 +315,54 @@ merge_assign_kernel(const __grid_constant__ CUtensorMap tm_e, const __grid_const
       if (!ok) break;
       tc_fence_after();
       const int n_valid = min(kTileM, kept - t * kTileM);
+      uint32_t acc2[2][32];                                    // the next 32 columns are on their way under these
+      tmem_ld32(t_lane + b * kTileM, acc2[0]);
 #pragma unroll
       for (int ch = 0; ch < kTileM / 32; ++ch) {
-        uint32_t acc[32];
-        tmem_ld32(t_lane + b * kTileM + ch * 32, acc);
+        uint32_t* acc = acc2[ch & 1];
         tmem_wait_ld();
-        if (ch == kTileM / 32 - 1) {
+        if (ch < kTileM / 32 - 1) {
+          tmem_ld32(t_lane + b * kTileM + (ch + 1) * 32, acc2[(ch + 1) & 1]);
+        } else {
           tc_fence_before();
-          mbar_arrive(smem_u32(&bars->acc_free[b]));
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&bars->acc_free[b]));
         }
         if (n_valid == kTileM) {
+          float2 v[16];
+          float top4[4];
 #pragma unroll
-          for (int i = 0; i < 32; i += 4) {
-            const float4 ic = *reinterpret_cast<const float4*>(&inv_tile[ch * 32 + i]);
-            const float2 v01 = mul2(make_float2(__uint_as_float(acc[i]), __uint_as_float(acc[i + 1])), make_float2(ic.x, ic.y));
-            const float2 v23 = mul2(make_float2(__uint_as_float(acc[i + 2]), __uint_as_float(acc[i + 3])), make_float2(ic.z, ic.w));
-            const float top = fmaxf(max3(v01.x, v01.y, v23.x), v23.y);
-            // strict comparisons in ascending column order: the lowest index wins among equals
-            if (top > best) {
-              best = top;
-              arg = t * kTileM + ch * 32 + i + (v01.x == top ? 0 : v01.y == top ? 1 : v23.x == top ? 2 : 3);
-            }
+          for (int i = 0; i < 16; i += 2) {
+            const float4 ic = *reinterpret_cast<const float4*>(&inv_tile[ch * 32 + 2 * i]);
+            v[i] = mul2(make_float2(__uint_as_float(acc[2 * i]), __uint_as_float(acc[2 * i + 1])), make_float2(ic.x, ic.y));
+            v[i + 1] = mul2(make_float2(__uint_as_float(acc[2 * i + 2]), __uint_as_float(acc[2 * i + 3])), make_float2(ic.z, ic.w));
           }
-        } else {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            top4[u] = fmaxf(v[4 * u].x, v[4 * u].y);
+#pragma unroll
+            for (int i = 1; i < 4; ++i) top4[u] = max3(top4[u], v[4 * u + i].x, v[4 * u + i].y);
+          }
+          const float top = fmaxf(fmaxf(top4[0], top4[1]), fmaxf(top4[2], top4[3]));
+          // strict comparison, and of the equal columns the lowest: the lowest index wins among equals
+          const bool more = top > best;
+          best = more ? top : best;
+          arg = more ? t * kTileM + ch * 32 : arg;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            won[i].x = more ? v[i].x : won[i].x;
+            won[i].y = more ? v[i].y : won[i].y;
+          }
+        } else if (ch * 32 < n_valid) {
+          if (ch == 0) {                                      // the last tile, a column at a time: from here on arg is the column itself
+#pragma unroll
+            for (int i = 15; i >= 0; --i) {
+              if (won[i].y == best) last = arg + 2 * i + 1;
+              if (won[i].x == best) last = arg + 2 * i;
+            }
+            arg = last;
+            single = true;
+          }
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
             const float val = __uint_as_float(acc[i]) * inv_tile[ch * 32 + i];
@@ -342,6 +373,14 @@ merge_assign_kernel(const __grid_constant__ CUtensorMap tm_e, const __grid_const
           }
         }
       }
+    }
+    if (!single) {
+#pragma unroll
+      for (int i = 15; i >= 0; --i) {
+        if (won[i].y == best) last = arg + 2 * i + 1;
+        if (won[i].x == best) last = arg + 2 * i;
+      }
+      arg = last;
     }
     if (ok && my_row < n_evict) {
       const size_t o = (size_t)bh * ms.stride + my_row;
@@ -504,18 +543,18 @@ size_t assign_smem_bytes() {
 
 }  // namespace
 
-int launch_merge_prepare(const StepArgs& a, const MergeScratch& ms, const int32_t* idx, const void* k_new,
+int launch_merge_prepare(const StepArgs& a, const MergeScratch& ms, const int32_t* idx, bool listed, const void* k_new,
                          const void* v_new, cudaStream_t st) {
   const int bh = a.batch * a.n_heads;
   const int rows = a.cand[1];                                  // discarded + retained entries of a contextual head
-  launch_k(merge_evicted_index_kernel, bh, kIdxThreads, 0, st, a, ms, idx);
+  if (!listed) launch_k(merge_evicted_index_kernel, bh, kIdxThreads, 0, st, a, ms, idx);
   constexpr int kEntries = kPrepThreads / 32 * kPrepRows;      // per CTA
   const dim3 grid((rows + kEntries - 1) / kEntries, bh);
   const __nv_bfloat16* kn = static_cast<const __nv_bfloat16*>(k_new);
   const __nv_bfloat16* vn = static_cast<const __nv_bfloat16*>(v_new);
   if (a.head_dim == 128) launch_k(merge_prepare_kernel<128>, grid, kPrepThreads, 0, st, a, ms, idx, kn, vn);
   else launch_k(merge_prepare_kernel<64>, grid, kPrepThreads, 0, st, a, ms, idx, kn, vn);
-  return launched(2);
+  return launched(listed ? 1 : 2);
 }
 
 int launch_merge_finish(const StepArgs& a, const MergeScratch& ms, cudaStream_t st) {
