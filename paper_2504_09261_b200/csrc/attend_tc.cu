@@ -260,8 +260,19 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     bars->abort_code = 0;
     fence_barrier_init();
     fence_proxy_async();
+  }
+  if (T == 2 && warp == kProducerWarp) {
+    // The barriers are ready; the producer does not wait for the others, nor they for its wait for the launch ahead:
+    // with all of them behind that wait, their code came in from L2 only then (3.0 instead of 2.1 us from the end of the
+    // compression to the first logits).  Not on half an SM, whose other half may be a CTA of the launch ahead that
+    // their polling slows down (240 heads x 64, 1 045 keys: 110 against 114 us a step).
+    __syncwarp();
+    asm volatile("bar.arrive 1, %0;" ::"n"(Shape<T>::kThreads) : "memory");
+    reg_dec<kOtherRegs>();
+  }
+  if (warp == kProducerWarp && lane == 0) {
     // the producer starts the first loads at once: they run under the TMEM allocation, the
-    // block-wide synchronisation and the register reallocation below
+    // synchronisation and the register reallocation below
     const Unit u = make_unit(blockIdx.x);
     bars->unit[0] = u;
     mbar_arrive(smem_u32(&bars->u_full[0]));
@@ -287,7 +298,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     pdl_launch_dependents();
   }
   tc_fence_before();
-  __syncthreads();
+  if (T == 1) __syncthreads();
+  else if (warp != kProducerWarp) asm volatile("bar.sync 1, %0;" ::"n"(Shape<T>::kThreads) : "memory");
   tc_fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&bars->tmem_base);
   // Everything above overlaps the tail of the previous kernel.  What waits for that kernel is the
@@ -399,7 +411,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     if (lane == 0) bulk_wait<0>();                   // every store has been performed before the CTA may leave
   } else if (warp == kProducerWarp) {
     // ------------------------------------------------------------------ TMA producer, and the CTA's next unit
-    reg_dec<kOtherRegs>();
+    if (T == 1) reg_dec<kOtherRegs>();
     if (lane == 0) {
       bool ok = true, pending = false;              // pending: an answer of cluster launch control is on its way
       uint32_t g = 0, issued_k = 1, issued_v = 1;   // K / V tiles of the units before this one; tiles on their way so far
