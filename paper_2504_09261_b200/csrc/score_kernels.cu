@@ -94,7 +94,7 @@ int launch_score_t(const StepArgs& a, const void* q, const void* k_new, float* s
   const int max_cand = a.cand[0] * a.trig[0] > a.cand[1] * a.trig[1] ? a.cand[0] : a.cand[1];
   const int bh = a.batch * a.n_heads;
   int per = 0;
-  const int cl = simt::fused_cluster(max_cand, a.heads_of[0] * a.trig[0] + a.heads_of[1] * a.trig[1], sizeof(T) == 2, sm_count(), per);
+  const int cl = simt::fused_cluster(max_cand, a.heads_of[0] * a.trig[0] + a.heads_of[1] * a.trig[1], sizeof(T) == 2, D, sm_count(), per);
   if (cl > 0) {
     auto go = [&](auto kern, size_t fused) {
       if (!allow_dynamic_smem(kern, fused)) return -1;

@@ -127,7 +127,7 @@ template <typename T, int D>
 cudaError_t run(const DenseArgs& a, int n_rows, const void* q, const void* k, float* scratch,
                 float* scores, int score_stride, cudaStream_t st) {
   int per = 0;
-  const int cl = simt::fused_cluster(a.n_cand, n_rows, sizeof(T) == 2, sm_count(), per);
+  const int cl = simt::fused_cluster(a.n_cand, n_rows, sizeof(T) == 2, D, sm_count(), per);
   if (cl > 0) {
     auto go = [&](auto kern, size_t fused) {
       if (!allow_dynamic_smem(kern, fused)) return cudaErrorInvalidValue;

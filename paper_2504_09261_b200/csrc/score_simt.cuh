@@ -220,15 +220,19 @@ __device__ __forceinline__ void cluster_scores_bf16(unsigned char* smem_raw, int
         fetch(k_sm + p * kChunk * D * 2 + at(r, c), key_ptr(min(first + p * kChunk + r, n_cand - 1)) + c * 8, 16);
       }
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");     // a group per chunk: its logits are formed while the next ones arrive
   }
-  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-  __syncthreads();
   // z[p][n][e]: key 16 warp + lane / 4 + 8 (e / 2) of chunk p, observation row 8 n + 2 (lane % 4) + e % 2
   float z[PER][4][4];
   const int key = 16 * warp + (lane >> 2);
 #pragma unroll
   for (int p = 0; p < PER; ++p) {
     const int j0 = first + p * kChunk;
+    if (PER - 1 - p == 3) asm volatile("cp.async.wait_group 3;" ::: "memory");
+    else if (PER - 1 - p == 2) asm volatile("cp.async.wait_group 2;" ::: "memory");
+    else if (PER - 1 - p == 1) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
 #pragma unroll
     for (int n = 0; n < 4; ++n) z[p][n][0] = z[p][n][1] = z[p][n][2] = z[p][n][3] = 0.f;
     if (j0 < n_cand) {
@@ -302,12 +306,16 @@ __device__ __forceinline__ void cluster_scores_bf16(unsigned char* smem_raw, int
 // CTAs per row-block (0: two launches) and chunks per CTA of the one-launch form.  fp32: one chunk per
 // CTA, and one CTA per SM or few CTAs per row-block (past that the two launches stream more: 32 rows x
 // 1 024 candidates x 64 10.3 us against 11.1).
-inline int fused_cluster(int n_cand, int rows, bool bf16, int sms, int& per) {
+// bf16, head_dim 128: as many chunks per CTA as leave one CTA per SM, if four do (32 rows x 2 000 candidates 11.2 us with
+// two, 9.7 with four; at head_dim 64 7.7 and 8.7).  A group of copies per chunk: 16 rows x 4 000 candidates 18.5 -> 17.3.
+inline int fused_cluster(int n_cand, int rows, bool bf16, int head_dim, int sms, int& per) {
   const int n = (n_cand + kChunk - 1) / kChunk;
   per = (n + kFusedCluster - 1) / kFusedCluster;
   if (bf16) {
     if (per > 4) return 0;
     if (per == 3) per = 4;
+    if (head_dim == 128 && rows * ((n + 3) / 4) <= sms)
+      while (per < 4 && rows * ((n + per - 1) / per) > sms) per *= 2;
     return (n + per - 1) / per;
   }
   return per == 1 && (rows * n <= sms || n <= 4) ? n : 0;
