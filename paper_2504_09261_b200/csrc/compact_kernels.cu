@@ -123,8 +123,6 @@ compact_copy_kernel(const StepArgs a, const int32_t* __restrict__ idx, int idx_a
   const int ctx = a.is_ctx[bh % a.n_heads];
   if (a.seg_new[ctx]) return;                      // the attention launch appends this type's new rows
   const int stored = a.stored[ctx], n_keep = a.kept[ctx];
-  const int32_t* list = idx && (idx_all || ctx) ? idx + (size_t)bh * a.kept_stride : nullptr;
-  const int n_old = list ? a.n_old[bh] : n_keep - a.n_new;   // no list: all new rows, behind what the head keeps of the stored ones
   const int plane_id = blockIdx.y;                 // 0: K (also writes the positions), 1: V
   const size_t off = a.row_off[bh];
   const int tid = threadIdx.x;
@@ -134,27 +132,38 @@ compact_copy_kernel(const StepArgs a, const int32_t* __restrict__ idx, int idx_a
   const int rows_per_pass = kThreads / row_pieces;
   const int piece = tid % row_pieces;
   const int rsub = tid / row_pieces;
-  for (int c0 = n_old + blockIdx.x * rows_per_pass * kCopyUnroll; c0 < n_keep;
-       c0 += gridDim.x * rows_per_pass * kCopyUnroll) {
-    uint4 val[kCopyUnroll];
-    bool ok[kCopyUnroll];
+  // Row r from n_old on takes row source(r) of the new scale.  (A form for heads with a list and one for heads without:
+  // rows that are looked up in a list that may not be there are no longer all in flight at once, 3 us of a step.)
+  auto copy = [&](int n_old, auto source) {
+    for (int c0 = n_old + blockIdx.x * rows_per_pass * kCopyUnroll; c0 < n_keep;
+         c0 += gridDim.x * rows_per_pass * kCopyUnroll) {
+      uint4 val[kCopyUnroll];
+      bool ok[kCopyUnroll];
 #pragma unroll
-    for (int u = 0; u < kCopyUnroll; ++u) {
-      const int r = c0 + u * rows_per_pass + rsub;
-      ok[u] = false;
-      if (r < n_keep) {
-        const int src = list ? list[r] - stored : r - n_old;
-        ok[u] = dbg_ok(src >= 0 && src < a.n_new && r < a.cap[ctx], a.status, 3);
-        if (!ok[u]) continue;
-        val[u] = fresh[(size_t)src * row_pieces + piece];
-        if (plane_id == 0 && piece == 0) pos[r] = a.pos_base + src;
+      for (int u = 0; u < kCopyUnroll; ++u) {
+        const int r = c0 + u * rows_per_pass + rsub;
+        ok[u] = false;
+        if (r < n_keep) {
+          const int src = source(r);
+          ok[u] = dbg_ok(src >= 0 && src < a.n_new && r < a.cap[ctx], a.status, 3);
+          if (!ok[u]) continue;
+          val[u] = fresh[(size_t)src * row_pieces + piece];
+          if (plane_id == 0 && piece == 0) pos[r] = a.pos_base + src;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kCopyUnroll; ++u) {
+        const int r = c0 + u * rows_per_pass + rsub;
+        if (r < n_keep && ok[u]) plane[(size_t)r * row_pieces + piece] = val[u];
       }
     }
-#pragma unroll
-    for (int u = 0; u < kCopyUnroll; ++u) {
-      const int r = c0 + u * rows_per_pass + rsub;
-      if (r < n_keep && ok[u]) plane[(size_t)r * row_pieces + piece] = val[u];
-    }
+  };
+  if (idx && (idx_all || ctx)) {
+    const int32_t* list = idx + (size_t)bh * a.kept_stride;
+    copy(a.n_old[bh], [=](int r) { return list[r] - stored; });
+  } else {                                         // all new rows, behind what the head keeps of the stored ones
+    const int n_old = n_keep - a.n_new;
+    copy(n_old, [=](int r) { return r - n_old; });
   }
 }
 
