@@ -66,7 +66,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int& 
 
 // Warp 0 finds the digit d (scanning from 255 down) at which the running count reaches `need`:
 // sum_{b > d} hist[b] < need <= sum_{b >= d} hist[b].  Returns through shared memory.
-__device__ __forceinline__ void locate_digit(const int* hist, int need, int* sh_digit, int* sh_need) {
+__device__ __forceinline__ void locate_digit(const int* hist, int need, int* sh_digit, int* sh_need, int* sh_count) {
   const int lane = threadIdx.x & 31;
   // lane l owns bins 255 - 8l ... 248 - 8l (descending), so lane order == descending bin order
   int c[8];
@@ -84,7 +84,7 @@ __device__ __forceinline__ void locate_digit(const int* hist, int need, int* sh_
     int cum = before;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      if (cum < need && need <= cum + c[i]) { *sh_digit = 255 - 8 * lane - i; *sh_need = need - cum; }
+      if (cum < need && need <= cum + c[i]) { *sh_digit = 255 - 8 * lane - i; *sh_need = need - cum; *sh_count = c[i]; }
       cum += c[i];
     }
   }
@@ -102,7 +102,7 @@ __device__ __forceinline__ void select_list(const StepArgs& a, const float* scor
   HeadView hv{scores + (size_t)bh * a.cand_stride, cand, a.stored[ctx], a.t_init, a.protect_new, ctx == 0};
 
   __shared__ int hist[256];
-  __shared__ int sh_digit, sh_need;
+  __shared__ int sh_digit, sh_need, sh_count;
   __shared__ int warp_sums[33];
 
   // thread t owns candidates [t*E, t*E + E)
@@ -125,13 +125,15 @@ __device__ __forceinline__ void select_list(const StepArgs& a, const float* scor
       if (in && lane == __ffs(peers) - 1) atomicAdd(&hist[digit], __popc(peers));
     }
     __syncthreads();
-    if (tid < 32) locate_digit(hist, need, &sh_digit, &sh_need);
+    if (tid < 32) locate_digit(hist, need, &sh_digit, &sh_need, &sh_count);
     __syncthreads();
     prefix |= (uint32_t)sh_digit << shift;
     need = sh_need;
     mask |= 255u << shift;
+    // every entry of the located bin survives: those above prefix and, at most `need`, those equal to it
+    if (need == sh_count) break;
   }
-  // prefix = key of the n_keep-th largest element; `need` of the entries equal to it survive
+  // prefix = key of the n_keep-th largest element (or its digits so far); `need` of the entries equal to it survive
   const uint32_t thr = prefix;
   int gt = 0, eq = 0;
 #pragma unroll
@@ -174,15 +176,17 @@ select_reg_kernel(const StepArgs a, const float* __restrict__ scores, int32_t* _
 // before those of every later round, so reading a round before writing it is enough.  Three launches of 3
 // to 5 us that wait for each other become one where a head's rows are a few microseconds for one SM
 // (kSmallMoveBytes); step of 16 fp32 heads x 64, 374 kept rows: 36.0 against 40.4 us, 34 rows 20.4 against 24.6.
+// Where there are SMs to spare a cluster of up to four CTAs moves a head's rows (one CTA reads and writes its own at 40 GB/s);
+// each forms the whole list for itself.  Steps of 169 and 256 queries 33.8 -> 32.3 and 33.3 us.
 constexpr int kMoveRun = 4;
 constexpr size_t kSmallMoveBytes = 384 * 1024;   // K and V rows of a head
 
 template <int E>
 __global__ void __launch_bounds__(kSelThreads)
 select_move_kernel(const StepArgs a, const float* __restrict__ scores, const uint4* __restrict__ k_new,
-                   const uint4* __restrict__ v_new, int row_pieces) {
+                   const uint4* __restrict__ v_new, int row_pieces, int cl) {
   pdl_wait();
-  const int bh = blockIdx.x;
+  const int bh = blockIdx.x / cl, rank = blockIdx.x % cl;
   const int ctx = a.is_ctx[bh % a.n_heads];
   const int stored = a.stored[ctx], n_keep = a.kept[ctx];
   extern __shared__ int32_t list[];               // [largest kept length]
@@ -197,13 +201,13 @@ select_move_kernel(const StepArgs a, const float* __restrict__ scores, const uin
   int32_t* pos = a.pos_plane + off;
   const int piece = tid % row_pieces, rsub = tid / row_pieces, rows = kSelThreads / row_pieces;   // row_pieces divides kSelThreads
   // stored rows that stay where they are need not be touched
-  for (int c0 = 0; c0 < n_keep; c0 += rows * kMoveRun) {
+  for (int c0 = 0; c0 < n_keep; c0 += cl * rows * kMoveRun) {
     uint4 kv[kMoveRun], vv[kMoveRun];
     int p[kMoveRun];
     bool mv[kMoveRun];
 #pragma unroll
     for (int u = 0; u < kMoveRun; ++u) {
-      const int r = c0 + u * rows + rsub;
+      const int r = c0 + (u * cl + rank) * rows + rsub;
       mv[u] = false;
       if (r < n_keep) {
         const int src = list[r];
@@ -217,11 +221,13 @@ select_move_kernel(const StepArgs a, const float* __restrict__ scores, const uin
         }
       }
     }
-    __syncthreads();
+    // every source of the round has been read (with memory ordering: the loads need not have landed in registers)
+    if (cl > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else __syncthreads();
 #pragma unroll
     for (int u = 0; u < kMoveRun; ++u) {
       if (mv[u]) {
-        const int r = c0 + u * rows + rsub;
+        const int r = c0 + (u * cl + rank) * rows + rsub;
         kp[(size_t)r * row_pieces + piece] = kv[u];
         vp[(size_t)r * row_pieces + piece] = vv[u];
         if (piece == 0) pos[r] = p[u];
@@ -248,7 +254,7 @@ select_kernel(const StepArgs a, const float* __restrict__ scores, int32_t* __res
   HeadView hv{scores + (size_t)bh * a.cand_stride, cand, a.stored[ctx], a.t_init, a.protect_new, ctx == 0};
 
   __shared__ int hist[256];
-  __shared__ int sh_digit, sh_need;
+  __shared__ int sh_digit, sh_need, sh_count;
   __shared__ int warp_sums[33];
 
   uint32_t prefix = 0, mask = 0;
@@ -266,7 +272,7 @@ select_kernel(const StepArgs a, const float* __restrict__ scores, int32_t* __res
       if (in && lane == __ffs(peers) - 1) atomicAdd(&hist[digit], __popc(peers));
     }
     __syncthreads();
-    if (tid < 32) locate_digit(hist, need, &sh_digit, &sh_need);
+    if (tid < 32) locate_digit(hist, need, &sh_digit, &sh_need, &sh_count);
     __syncthreads();
     prefix |= (uint32_t)sh_digit << shift;
     need = sh_need;
@@ -298,8 +304,24 @@ int launch_select_move(const StepArgs& a, int dtype, const float* scores, const 
   const int max_cand = a.cand[0] > a.cand[1] ? a.cand[0] : a.cand[1], max_keep = a.kept[0] > a.kept[1] ? a.kept[0] : a.kept[1];
   const int row_pieces = a.head_dim * (dtype == HACK_F32 ? 4 : 2) / 16;
   if (max_cand > 4 * kSelThreads || (size_t)max_keep * row_pieces * 32 > kSmallMoveBytes) return 0;
-  launch_k(select_move_kernel<4>, dim3(a.batch * a.n_heads), dim3(kSelThreads), (size_t)max_cand * sizeof(int32_t), st, a, scores,
-           static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), row_pieces);
+  const int heads = a.batch * a.n_heads;
+  int cl = 1;
+  while (cl < 4 && heads * cl * 2 <= sm_count()) cl *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(heads * cl);
+  cfg.blockDim = dim3(kSelThreads);
+  cfg.dynamicSmemBytes = (size_t)max_cand * sizeof(int32_t);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cl;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  cudaLaunchKernelEx(&cfg, select_move_kernel<4>, a, scores, static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), row_pieces, cl);
   return launched(1);
 }
 
