@@ -46,6 +46,9 @@
 // and 44 us; 7 us per digit where that traffic met the attention of the other heads.)  One CTA per
 // head where the GPU is full of heads, two CTAs per SM where there are more heads than SMs: 256 heads of
 // 680 candidates 51 -> 40 us per step, attention included.
+// Its code runs once from front to back, right behind the attention kernel's, so every line of it comes in from L2:
+// loops of unknown length are not unrolled, waits are small and a round's loads stand in one place (97 -> 69 KB of
+// code; 21 heads x 128, 121 to 2 025 queries: 818 -> 798 us a layer, 256 heads x 64 37.9 -> 36.9 us a step).
 // In score-only mode the kernel stops after step 3 and writes the fp32 scores (hack_score).
 // Every mbarrier wait is bounded; a CTA whose wait gives up raises the status word, and the
 // cluster agrees at the first exchange to skip the rest, so that every CTA still reaches every
@@ -176,24 +179,22 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-__device__ __forceinline__ bool ck_wait(uint64_t* bar, uint32_t parity, CkShared* sh, int* status, int code,
-                                        long long limit) {
+// False once the limit has passed or another wait of the CTA has given up (in little code; one thread writes the status word
+// at the end).
+__device__ __forceinline__ bool ck_wait(uint64_t* bar, uint32_t parity, CkShared* sh, int code, long long limit) {
   const uint32_t addr = smem_u32(bar);
   // a limit of a few cycles (a test's way to make a wait run out) is taken literally: the barrier is
   // tested without blocking and the clock is read after every test
   const bool brief = limit < 65536;
-  if (brief ? mbar_test_wait(addr, parity) : mbar_try_wait(addr, parity)) return true;
+  if (__builtin_expect(!brief && mbar_try_wait(addr, parity), 1)) return true;
+  volatile int* const flag = &sh->abort_flag;
   const long long t0 = clock64();
-  for (uint32_t it = 0;; ++it) {
-    if (brief ? mbar_test_wait(addr, parity) : mbar_try_wait(addr, parity)) return true;
-    if ((it & 63u) == 63u || brief) {
-      if (*reinterpret_cast<volatile int*>(&sh->abort_flag)) return false;
-      if (clock64() - t0 > limit) break;
-    }
+#pragma unroll 1
+  while (!(brief ? mbar_test_wait(addr, parity) : mbar_try_wait(addr, parity))) {
+    if (*flag) return false;
+    if (clock64() - t0 > limit) *flag = code;
   }
-  *reinterpret_cast<volatile int*>(&sh->abort_flag) = 1;
-  atomicExch(status, code);
-  return false;
+  return true;
 }
 
 // Order-preserving map from fp32 bits to unsigned (larger float -> larger key).
@@ -334,7 +335,9 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
     ++issued;
   };
   if (warp == kIssueWarp && lane == 0) {
+#pragma unroll 1
     for (int s = 0; s < STAGES; ++s) { mbar_init(smem_u32(&sh->full[s]), 1); mbar_init(smem_u32(&sh->empty[s]), 1); }
+#pragma unroll 1
     for (int i = 0; i < n_seq; ++i) mbar_init(smem_u32(&sh->acc_full[i]), 1);
     mbar_init(smem_u32(&sh->acc_free[0]), kWorkers / 32);   // a warp arrives once
     mbar_init(smem_u32(&sh->acc_free[1]), kWorkers / 32);
@@ -355,6 +358,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   if (warp == kIssueWarp) {
     // the first key tiles are on their way while the other warps fetch the observation rows
     if (lane == 0)
+#pragma unroll 1
       for (int i = 0; i < min(STAGES, n_seq); ++i) load_tile(i);
     __syncwarp();
   } else {
@@ -385,12 +389,13 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   auto issue = [&](int from, int to) {
     constexpr uint32_t IDESC = idesc_bf16_f32(kCkChunk, kMaxObs, 0);
     const uint64_t q_desc = smem_desc_sw128(q_sm, 16, 1024);
+#pragma unroll 1
     for (int i = from; i < to && issue_ok; ++i) {
       const int s = i % STAGES;
-      bool ok = ck_wait(&sh->full[s], (i / STAGES) & 1, sh, a.status, 52, wlim);
+      bool ok = ck_wait(&sh->full[s], (i / STAGES) & 1, sh, 52, wlim);
       // a shared accumulator is free again once all consumers have read the chunk before
       if (ok && i >= p.direct)
-        ok = ck_wait(&sh->acc_free[(i - p.direct) & 1], (((i - p.direct) >> 1) & 1) ^ 1, sh, a.status, 53, wlim);
+        ok = ck_wait(&sh->acc_free[(i - p.direct) & 1], (((i - p.direct) >> 1) & 1) ^ 1, sh, 53, wlim);
       if (ok) {
         tc_fence_after();
         const uint64_t k_desc = smem_desc_sw128(k_sm + s * K_BYTES, 16, 1024);
@@ -402,7 +407,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
         // the tile of the product before this one is free: refill its stage
         const int f = i - 1 + STAGES;
         if (i > 0 && f < n_seq) {
-          ok = ck_wait(&sh->empty[f % STAGES], (f / STAGES - 1) & 1, sh, a.status, 51, wlim);
+          ok = ck_wait(&sh->empty[f % STAGES], (f / STAGES - 1) & 1, sh, 51, wlim);
           if (ok) load_tile(f);
         }
       }
@@ -412,9 +417,12 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   // After a wait that gave up: what is in flight gets a bounded chance to finish before the ring is reused.
   auto drain = [&]() {
     mma_commit(smem_u32(&sh->drain));
+#pragma unroll 1
     for (uint32_t it = 0; it < kCkDrainSpins && !mbar_try_wait(smem_u32(&sh->drain), 0); ++it) {}
+#pragma unroll 1
     for (int i = max(0, issued - STAGES); i < issued; ++i) {
       const uint32_t bar = smem_u32(&sh->full[i % STAGES]);
+#pragma unroll 1
       for (uint32_t it = 0; it < kCkDrainSpins && !mbar_try_wait(bar, (i / STAGES) & 1); ++it) {}
     }
   };
@@ -433,8 +441,9 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
 #pragma unroll
     for (int i = 0; i < kHalfObs; ++i) { rm[i] = -INFINITY; rl[i] = 0.f; }
     bool ok = true, first = true;
+#pragma unroll 1
     for (int i = 0; i < n_run; ++i) {
-      ok = __all_sync(0xffffffffu, ck_wait(&sh->acc_full[i], 0, sh, a.status, 54, wlim));
+      ok = __all_sync(0xffffffffu, ck_wait(&sh->acc_full[i], 0, sh, 54, wlim));
       if (!ok) break;
       tc_fence_after();
       uint32_t acc[kHalfObs];
@@ -545,11 +554,12 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   } else if (!aborted && warp != kIssueWarp) {
     const bool structural = ctx == 0;
     bool ok = true;
+#pragma unroll 1
     for (int i = set; i < n_p; i += 2) {                    // a set takes every other chunk here
       const bool again = kAgain && i >= n_held;
       const int seq = n_run + i - n_held;                   // the product that forms this chunk a second time
       if (again) {
-        ok = __all_sync(0xffffffffu, ck_wait(&sh->acc_full[seq], 0, sh, a.status, 55, wlim)) && ok;
+        ok = __all_sync(0xffffffffu, ck_wait(&sh->acc_full[seq], 0, sh, 55, wlim)) && ok;
         tc_fence_after();
       }
       float s = 0.f;
@@ -615,6 +625,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
       const uint32_t dmask = pass == 2 ? 255u : 4095u;
       uint32_t* hist = hist32 + (pass & 1) * kHistWords;
       if (pass > 0) {
+#pragma unroll 1
         for (int slot = tid; slot < n_slots; slot += kCkThreads) {
           int j;
           const uint32_t k = keys[slot];
@@ -721,6 +732,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
         // below it, its complemented index, so that among equals the lowest index ranks first.
         unsigned long long* own = reinterpret_cast<unsigned long long*>(hist32 + ((pass & 1) ^ 1) * kHistWords);
         unsigned long long* all = own + kBinMax;
+#pragma unroll 1
         for (int slot = tid; slot < n_slots; slot += kCkThreads) {
           int j;
           const uint32_t k = keys[slot];
@@ -774,6 +786,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
     const int n_groups = n_slots / 32, per = (n_groups + kCkWarps - 1) / kCkWarps;
     const int g_begin = min(n_groups, warp * per), g_end = min(n_groups, g_begin + per);
     int gt = 0, eq = 0;
+#pragma unroll 1
     for (int g = g_begin; g < g_end; ++g) {
       const int slot = g * 32 + lane;
       int j;
@@ -797,6 +810,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
     const uint32_t inv_s = 0xffffffffu / (uint32_t)S + 1u, inv_rs = 0xffffffffu / (uint32_t)RS + 1u;
     const uint32_t lower = (1u << lane) - 1u;
     const bool lists = kLists && ctx;
+#pragma unroll 1
     for (int g = g_begin; g < g_end; ++g) {
       const int slot = g * 32 + lane;
       int j;
@@ -854,6 +868,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
         const int32_t* srcs = src_all + t * S;
         const uint32_t kb = base + (uint32_t)(t % kMoveBuffers) * buf_bytes, vb = kb + (uint32_t)S * ROWB;
         int32_t* ps = pos_stage + (t % kMoveBuffers) * s_cap;
+#pragma unroll 2
         for (int v = tid; v < rows * PIECES; v += kCkThreads) {
           const int lr = v / PIECES, piece = v % PIECES;
           int src = srcs[lr];
@@ -865,6 +880,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
           cp_async16(kb + (uint32_t)lr * ROWB + piece * 16, ks + piece);
           cp_async16(vb + (uint32_t)lr * ROWB + piece * 16, vs + piece);
         }
+#pragma unroll 1
         for (int lr = tid; lr < rows; lr += kCkThreads) {
           const int src = srcs[lr];
           if (src < stored) cp_async4(smem_u32(&ps[lr]), pos + max(src, 0));
@@ -874,39 +890,42 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
       cp_async_commit();                                      // one group per round, empty or not
     };
     const int n_moves = lists ? 0 : n_rounds;
-    if (n_moves > 0) {
-      issue_loads(0);
-      issue_loads(1);
-    }
-    for (int t = 0; t < n_moves; ++t) {
-      cp_async_wait_group<1>();                               // the loads of round t (all but the latest group) have landed
-      fence_proxy_async();                                    // the bulk stores below read what these threads wrote
-      cluster_sync_relaxed(CL);                               // every source of this round has been read
-      const bool moving = slice_moves(t);
-      if (moving) {
-        const int first = slice_first(t), rows = slice_rows(t);
-        const uint32_t kb = base + (uint32_t)(t % kMoveBuffers) * buf_bytes, vb = kb + (uint32_t)S * ROWB;
-        if (tid == 0) {
-          constexpr uint32_t kPiece = 32768;                  // bytes per bulk store
-          const uint32_t bytes = (uint32_t)rows * ROWB;
-          for (uint32_t o = 0; o < bytes; o += kPiece) {
-            const uint32_t n = min(kPiece, bytes - o);
-            bulk_store(reinterpret_cast<unsigned char*>(kp + (size_t)first * PIECES) + o, kb + o, n);
-            bulk_store(reinterpret_cast<unsigned char*>(vp + (size_t)first * PIECES) + o, vb + o, n);
+    // (the two rounds ahead of the first only issue their loads: one place in the code for them)
+#pragma unroll 1
+    for (int t = n_moves > 0 ? -2 : 0; t < n_moves; ++t) {
+      if (t >= 0) {
+        cp_async_wait_group<1>();                               // the loads of round t (all but the latest group) have landed
+        fence_proxy_async();                                    // the bulk stores below read what these threads wrote
+        cluster_sync_relaxed(CL);                               // every source of this round has been read
+        const bool moving = slice_moves(t);
+        if (moving) {
+          const int first = slice_first(t), rows = slice_rows(t);
+          const uint32_t kb = base + (uint32_t)(t % kMoveBuffers) * buf_bytes, vb = kb + (uint32_t)S * ROWB;
+          if (tid == 0) {
+            constexpr uint32_t kPiece = 32768;                  // bytes per bulk store
+            const uint32_t bytes = (uint32_t)rows * ROWB;
+#pragma unroll 1
+            for (uint32_t o = 0; o < bytes; o += kPiece) {
+              const uint32_t n = min(kPiece, bytes - o);
+              bulk_store(reinterpret_cast<unsigned char*>(kp + (size_t)first * PIECES) + o, kb + o, n);
+              bulk_store(reinterpret_cast<unsigned char*>(vp + (size_t)first * PIECES) + o, vb + o, n);
+            }
           }
+          const int32_t* ps = pos_stage + (t % kMoveBuffers) * s_cap;
+#pragma unroll 1
+          for (int lr = tid; lr < rows; lr += kCkThreads) pos[first + lr] = ps[lr];
         }
-        const int32_t* ps = pos_stage + (t % kMoveBuffers) * s_cap;
-        for (int lr = tid; lr < rows; lr += kCkThreads) pos[first + lr] = ps[lr];
+        if (tid == 0) {
+          bulk_commit();                                        // one group per round, empty or not
+          bulk_wait_read<1>();                                  // round t - 1 has left its buffer, which round t + 2 fills
+        }
+        __syncthreads();
       }
-      if (tid == 0) {
-        bulk_commit();                                        // one group per round, empty or not
-        bulk_wait_read<1>();                                  // round t - 1 has left its buffer, which round t + 2 fills
-      }
-      __syncthreads();
       issue_loads(t + 2);
     }
     if (tid == 0) bulk_wait_read<0>();                        // shared memory is read out before the CTA leaves
   }
+  if (tid == 0 && sh->abort_flag) atomicExch(a.status, sh->abort_flag);
   // no CTA leaves while another may still read its shared memory (past the list nobody does)
   if (!select) cluster_sync(CL);
   if (warp == 0) {
