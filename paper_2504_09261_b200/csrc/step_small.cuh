@@ -79,6 +79,7 @@ struct PickShared {
   uint32_t words[kMaxRows / 32];
 };
 __device__ __forceinline__ void pick_init(PickShared& ps) {
+#pragma unroll 1
   for (int i = threadIdx.x; i < kRangeBins + 32; i += kStepThreads) ps.hist[i] = 0;
   if (threadIdx.x == 0) { ps.range[0] = 0xffffffffu; ps.range[1] = 0u; ps.n_in = 0; }
 }

@@ -120,22 +120,26 @@ step_small_f32_kernel(const StepArgs a, const float* __restrict__ q, const float
   pdl_wait();
 
   // ------------------------------------------------------------------ rows into shared memory
+#pragma unroll 2
   for (int v = tid; v < cand * PIECES; v += kStepThreads) {
     const int r = v / PIECES, c = v % PIECES;
     fetch(ks + r * KF + c * 4, (r < stored ? kc + (size_t)r * D : kn + (size_t)(r - stored) * D) + c * 4);
   }
   if (evicts) {
+#pragma unroll 1
     for (int v = tid; v < kMaxObs * PIECES; v += kStepThreads) {
       const int r = v / PIECES, c = v % PIECES;                // rows past the last repeat it and weigh nothing
       fetch(os + v * 4, qn + (size_t)obs_row(a, min(r, a.n_obs_rows - 1)) * D + c * 4);
     }
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
+#pragma unroll 2
   for (int v = tid; v < cand * PIECES; v += kStepThreads) {
     const int r = v / PIECES, c = v % PIECES;
     fetch(vs + v * 4, (r < stored ? vc + (size_t)r * D : vn + (size_t)(r - stored) * D) + c * 4);
   }
   const int q_first = rank * sp.tiles * kRows;
+#pragma unroll 1
   for (int v = tid; v < sp.tiles * kRows * PIECES; v += kStepThreads) {
     const int r = v / PIECES, c = v % PIECES;
     fetch(qs + v * 4, qn + (size_t)min(q_first + r, n_new - 1) * D + c * 4);
@@ -145,6 +149,7 @@ step_small_f32_kernel(const StepArgs a, const float* __restrict__ q, const float
 
   // ------------------------------------------------------------------ scores and list
   if (evicts) {
+#pragma unroll 1
     for (int j = tid; j < cand; j += kStepThreads) pos[j] = j < stored ? a.pos_plane[off + j] : a.pos_base + (j - stored);
     asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();
@@ -223,6 +228,7 @@ step_small_f32_kernel(const StepArgs a, const float* __restrict__ q, const float
     }
     __syncthreads();
     uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll 1
     for (int j = tid; j < cand; j += kStepThreads) {
       float s = 0.f;
 #pragma unroll
@@ -234,6 +240,7 @@ step_small_f32_kernel(const StepArgs a, const float* __restrict__ q, const float
     }
     pick<(kTurns * kKeyWarps * kKeys + kStepThreads - 1) / kStepThreads>(a, ps, key, list, cand, n_keep, lo, hi);
   } else {
+#pragma unroll 1
     for (int j = tid; j < n_keep; j += kStepThreads) list[j] = j;
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -321,6 +328,7 @@ step_small_f32_kernel(const StepArgs a, const float* __restrict__ q, const float
   if (sp.ctas > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   {
     const int share = (n_keep + sp.ctas - 1) / sp.ctas, r0 = rank * share, r1 = min(n_keep, r0 + share);
+#pragma unroll 2
     for (int v = r0 * PIECES + tid; v < r1 * PIECES; v += kStepThreads) {
       const int r = v / PIECES, c = v % PIECES, src = list[r];
       // stored rows that stay where they are need not be touched
@@ -346,6 +354,7 @@ step_small_f32_kernel(const StepArgs a, const float* __restrict__ q, const float
   // a form per number of warps, so that all loads of a row are in flight at once
   auto combine = [&](auto splits_c) {
     constexpr int S = decltype(splits_c)::value;
+#pragma unroll 1
     for (int v = tid; v < sp.tiles * kRows * PIECES; v += kStepThreads) {
       const int row = v / PIECES, c = v % PIECES, r = row % kRows, w0 = row / kRows * S;
       if (q_first + row >= n_new) break;
