@@ -67,7 +67,9 @@ attn_colstats_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
   constexpr uint32_t TILE_BYTES = SUB * SUB_BYTES;
 
   pdl_wait();
-  const int bh = blockIdx.y, kb0 = blockIdx.x * kVarSets;
+  // All heads' first blocks come first and the last ones, which may be one block instead of two, last: 32 heads of 83 blocks
+  // are 1 344 CTAs on 148 SMs, and a tenth round for twelve of them is short this way.
+  const int bh = blockIdx.x, kb0 = blockIdx.y * kVarSets;
   const int len = a.kept[a.is_ctx[bh % a.n_heads]];
   if (kb0 * kVarTile >= len) return;
   const int n_sets = (kb0 + 1) * kVarTile < len ? 2 : 1;
@@ -89,7 +91,7 @@ attn_colstats_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     mbar_init(smem_u32(&bars->k_full), 1);
     for (int s = 0; s < kQStages; ++s) { mbar_init(smem_u32(&bars->q_full[s]), 1); mbar_init(smem_u32(&bars->q_empty[s]), 1); }
     for (int i = 0; i < kVarSets; ++i)
-      for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&bars->acc_full[i][b]), 1); mbar_init(smem_u32(&bars->acc_free[i][b]), kVarTile); }
+      for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&bars->acc_full[i][b]), 1); mbar_init(smem_u32(&bars->acc_free[i][b]), kVarTile / 32); }
     mbar_init(smem_u32(&bars->drain), 1);
     bars->abort_flag = 0;
     fence_barrier_init();
@@ -203,7 +205,8 @@ attn_colstats_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
           tmem_ld32(t_lane + b * kVarTile + (ch + 1) * 32, acc[(ch + 1) & 1]);
         } else {
           tc_fence_before();
-          mbar_arrive(smem_u32(&bars->acc_free[set][b]));
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&bars->acc_free[set][b]));
         }
         const uint32_t* z = acc[ch & 1];
 #pragma unroll
@@ -281,7 +284,7 @@ int launch_attention_variance(const StepArgs& a, const void* q, const float* row
     set_error("attention variance: cache longer than the scratch area");
     return -1;
   }
-  const dim3 grid((n_blocks + kVarSets - 1) / kVarSets, bh);
+  const dim3 grid(bh, (n_blocks + kVarSets - 1) / kVarSets);
   if (a.head_dim == 128) {
     if (!allow_dynamic_smem(attn_colstats_kernel<128>, var_smem_bytes<128>())) return -1;
     launch_k(attn_colstats_kernel<128>, grid, kVarThreads, var_smem_bytes<128>(), st, tm_q, tk, a, row_stats, block_var, max_blocks);
