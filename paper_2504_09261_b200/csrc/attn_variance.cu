@@ -8,14 +8,17 @@
 //   warp 0    : TMA producer (the key blocks once, the query tiles through a ring)
 //   warp 1    : tcgen05.mma issuer; S^T = K_blk Q_tile^T, keys on the 128 TMEM lanes, queries on
 //               128 columns, two accumulators per key block so that the next MMA runs under the read-out
-//   warps 2-5 : consumers of the first key block, warps 6-9 of the second; thread r owns key r: it reads
-//               its 128 logits with tcgen05.ld, forms p = exp2(c z - c m_i - log2 l_i) and adds p and
+//   warps 2-9 : consumers of the first key block, warps 10-17 of the second; two threads own key r: each reads
+//               its 64 of the 128 logits with tcgen05.ld, forms p = exp2(c z - c m_i - log2 l_i) and adds p and
 //               p^2 to two registers
-// so the sums over the queries stay inside one thread and nothing of size N x T is stored.  At the
-// end the thread holds Var_i A[i, j] = sum p^2 / N - (sum p / N)^2 of its key; the CTA adds its 128
-// variances and a second, tiny kernel adds the blocks of a head in a fixed order.
+// so the sums over the queries stay inside a thread and nothing of size N x T is stored.  At the
+// end the two have Var_i A[i, j] = sum p^2 / N - (sum p / N)^2 of their key; the CTA adds its 128
+// variances and a second, tiny kernel adds the blocks of a head in a fixed order.  Bound by the special-function unit:
+// 2 048 cycles for the two tiles of a step.  With one thread per key (two warps per scheduler, each waiting for its own
+// tcgen05.ld and barriers) 32 heads x 4 096 queries x 10 521 keys took 472 us, some 3 150 cycles a step; now 451 us.
 // Two blocks per CTA halve the query traffic: with one block per CTA (two CTAs per SM) the launch ran at the
-// L2's rate of about 21 bytes per clock and SM.  32 heads x 4 096 queries x 10 521 keys x 128: 514 -> 482 us.
+// L2's rate of about 21 bytes per clock and SM.  32 heads x 4 096 queries x 10 521 keys x 128: 514 -> 482 us, short last blocks
+// last in the order of the CTAs: -> 472 us.
 // Every mbarrier wait is bounded; on expiry the CTA raises the status word and winds down.
 #include <cuda.h>
 
@@ -28,8 +31,11 @@ namespace {
 using namespace ptx;
 
 constexpr int kVarSets = 2;             // key blocks per CTA
-constexpr int kVarThreads = 64 + 128 * kVarSets;
+constexpr int kVarParts = 2;            // threads per key, each with its part of a tile's queries
+constexpr int kVarWarps = 4 * kVarSets * kVarParts;   // consumers
+constexpr int kVarThreads = 64 + 32 * kVarWarps;
 constexpr int kVarTile = 128;            // keys per block, queries per tile
+constexpr int kVarPart = kVarTile / kVarParts;
 constexpr int kQStages = 3;
 constexpr uint32_t kVarDrainSpins = 1u << 22;
 
@@ -83,15 +89,16 @@ attn_colstats_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
   const uint32_t k_sm = base;
   const uint32_t q_sm = base + kVarSets * TILE_BYTES;
   VarBars* bars = reinterpret_cast<VarBars*>(sm + (kVarSets + kQStages) * TILE_BYTES);
-  __shared__ __align__(16) float stat[4 * kVarSets][2][kVarTile];   // -c m_i - log2 l_i of the query tile in accumulator b
+  __shared__ __align__(16) float stat[kVarWarps][2][kVarPart];   // -c m_i - log2 l_i of the query tile in accumulator b
   __shared__ float red[4 * kVarSets];
+  __shared__ float2 other[kVarSets][kVarTile];                      // sums of the second thread of every key
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     mbar_init(smem_u32(&bars->k_full), 1);
     for (int s = 0; s < kQStages; ++s) { mbar_init(smem_u32(&bars->q_full[s]), 1); mbar_init(smem_u32(&bars->q_empty[s]), 1); }
     for (int i = 0; i < kVarSets; ++i)
-      for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&bars->acc_full[i][b]), 1); mbar_init(smem_u32(&bars->acc_free[i][b]), kVarTile / 32); }
+      for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&bars->acc_full[i][b]), 1); mbar_init(smem_u32(&bars->acc_free[i][b]), 4 * kVarParts); }
     mbar_init(smem_u32(&bars->drain), 1);
     bars->abort_flag = 0;
     fence_barrier_init();
@@ -165,21 +172,21 @@ attn_colstats_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         for (uint32_t it = 0; it < kVarDrainSpins && !mbar_try_wait(smem_u32(&bars->drain), 0); ++it) {}
       }
     }
-  } else if ((warp - 2) / 4 < n_sets) {
+  } else if ((warp - 2) / (4 * kVarParts) < n_sets) {
     // ------------------------------------------------------------------ consumers
-    const int set = (warp - 2) / 4, kb = kb0 + set;
+    const int set = (warp - 2) / (4 * kVarParts), part = (warp - 2) / 4 % kVarParts, kb = kb0 + set;
     const int quad = warp & 3;                                // TMEM lane quadrant this warp may read
     const int key_row = quad * 32 + lane;                     // key of the block this thread owns
-    const uint32_t t_lane = tmem + (static_cast<uint32_t>(quad * 32) << 16) + 2 * set * kVarTile;
+    const uint32_t t_lane = tmem + (static_cast<uint32_t>(quad * 32) << 16) + 2 * set * kVarTile + part * kVarPart;
     float2 sum_p[2] = {}, sum_p2[2] = {};                     // queries apart by their index modulo 4
     bool ok = true;
     // Statistics of a tile's queries, fetched one tile ahead; every warp keeps its own copy, so that the
     // warps do not meet inside the loop.  Queries past the end of the scale get weight 0: exp2(-inf) = 0.
-    float2 ml[4];
+    float2 ml[kVarPart / 32];
     auto fetch = [&](int t) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int qi = t * kVarTile + u * 32 + lane;
+      for (int u = 0; u < kVarPart / 32; ++u) {
+        const int qi = t * kVarTile + part * kVarPart + u * 32 + lane;
         ml[u] = qi < a.n_new ? *reinterpret_cast<const float2*>(row_stats + ((size_t)bh * a.n_new + qi) * 2) : make_float2(INFINITY, 1.f);
       }
     };
@@ -189,7 +196,7 @@ attn_colstats_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
       float* st_tile = stat[warp - 2][b];
       // p = exp2(c z - c m - log2 l): the division is in the exponent
 #pragma unroll
-      for (int u = 0; u < 4; ++u) st_tile[u * 32 + lane] = -ml[u].x * c - __log2f(ml[u].y);
+      for (int u = 0; u < kVarPart / 32; ++u) st_tile[u * 32 + lane] = -ml[u].x * c - __log2f(ml[u].y);
       __syncwarp();
       fetch(t + 1);
       ok = __all_sync(0xffffffffu, var_wait(&bars->acc_full[set][b], (t >> 1) & 1, bars, a.status, 35, a.wait_cycles));
@@ -199,9 +206,9 @@ attn_colstats_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
       uint32_t acc[2][32];
       tmem_ld32(t_lane + b * kVarTile, acc[0]);
 #pragma unroll
-      for (int ch = 0; ch < kVarTile / 32; ++ch) {
+      for (int ch = 0; ch < kVarPart / 32; ++ch) {
         tmem_wait_ld();
-        if (ch + 1 < kVarTile / 32) {
+        if (ch + 1 < kVarPart / 32) {
           tmem_ld32(t_lane + b * kVarTile + (ch + 1) * 32, acc[(ch + 1) & 1]);
         } else {
           tc_fence_before();
@@ -226,17 +233,26 @@ attn_colstats_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     // Var_i A[i, j] of this thread's key; keys past the end of the head count nothing (their sums
     // come from rows of another head and may have overflowed)
     const float inv_n = 1.f / (float)a.n_new;
+    const float2 s1 = add2(sum_p[0], sum_p[1]), s2 = add2(sum_p2[0], sum_p2[1]);
+    float sp = s1.x + s1.y, sp2 = s2.x + s2.y;
+    if (part == 1) other[set][key_row] = make_float2(sp, ok ? sp2 : -1.f);   // < 0: this warp gave up
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + set), "n"(128 * kVarParts) : "memory");
     float var = 0.f;
-    if (ok && kb * kVarTile + key_row < len) {
-      const float2 s1 = add2(sum_p[0], sum_p[1]), s2 = add2(sum_p2[0], sum_p2[1]);
-      const float mean = (s1.x + s1.y) * inv_n;
-      var = fmaxf(fmaf(-mean, mean, (s2.x + s2.y) * inv_n), 0.f);
-    }
+    if (part == 0) {
+      const float2 o = other[set][key_row];
+      sp += o.x;
+      sp2 += o.y;
+      ok = __all_sync(0xffffffffu, ok && !(o.y < 0.f));
+      if (ok && kb * kVarTile + key_row < len) {
+        const float mean = sp * inv_n;
+        var = fmaxf(fmaf(-mean, mean, sp2 * inv_n), 0.f);
+      }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) var += __shfl_xor_sync(0xffffffffu, var, o);
-    if (lane == 0) red[warp - 2] = ok ? var : NAN;           // a warp that gave up poisons the block's sum
-    asm volatile("bar.sync %0, 128;" ::"r"(1 + set) : "memory");
-    if (tid == 64 + 128 * set && ok)
+      for (int o2 = 16; o2 > 0; o2 >>= 1) var += __shfl_xor_sync(0xffffffffu, var, o2);
+      if (lane == 0) red[4 * set + (warp - 2) % 4] = ok ? var : NAN;         // a warp that gave up poisons the block's sum
+    }
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + set), "n"(128 * kVarParts) : "memory");
+    if (part == 0 && (warp - 2) % 4 == 0 && lane == 0 && ok)
       block_var[(size_t)bh * max_blocks + kb] = (red[4 * set] + red[4 * set + 1]) + (red[4 * set + 2] + red[4 * set + 3]);
   }
   tc_fence_before();
