@@ -1091,7 +1091,13 @@ int launch_t(const StepArgs& a, const CUtensorMap& tm_cache, const CUtensorMap& 
   for (int per_sm = 1; per_sm <= 2 && !(shape && *shape); ++per_sm)
     for (int cl = 1; cl <= kMaxCluster; ++cl) {
       if (!ck_shape<D>(p, lists, cl, per_sm)) continue;
-      const int active = ck_active_clusters<D>(a, p, per_sm);
+      // Clusters of an odd size that are placed while the launch ahead drains do not pack as tightly as on an empty chip:
+      // of 44 clusters of 3, where 45 fit, one to three often started only when the first ones had ended, 12 us
+      // late.  So a fifteenth of their places is not counted on: 45 heads x 128, 529 queries 42.7 -> 33.8 us a step, 43
+      // heads 33.6 -> 31.1, 26 heads 32.3 -> 27.3; 42 and 24 heads are as fast with 3 and 5 CTAs as with any other number.
+      // Even sizes need no reserve (33 heads, clusters of 4: 30.0, with one 31.0; 74 heads, of 2: 40.6, with one 47.4).
+      const int fit = ck_active_clusters<D>(a, p, per_sm);
+      const int active = per_sm == 1 && cl > 1 && cl % 2 == 1 ? fit - (fit + 14) / 15 : fit;
       if (active < 1) continue;
       if (D == 128 && per_sm == 2 && n_clusters * cl <= sms) continue;    // the CTAs spread over as many SMs, and attention takes a whole one
       const int waves = (n_clusters + active - 1) / active;
