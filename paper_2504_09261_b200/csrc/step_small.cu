@@ -418,12 +418,15 @@ int launch_t(const StepArgs& a, const void* q, const void* k_new, const void* v_
   if (cand > kMaxRows || tiles > kMaxTiles * kMaxCtas) return 0;
   StepShape s;
   s.rows = (cand + kTile - 1) / kTile * kTile;
-  split_queries(s, heads, tiles);
-  const size_t smem = step_smem<D>(s);
   const int ranked = std::max(a.trig[0] ? a.cand[0] : 0, a.trig[1] ? a.cand[1] : 0);
   const int turns = (ranked + kStepWarps * kTile - 1) / (kStepWarps * kTile);
-  if (smem > kSmemCta || !step_small_pays<D>(a, s, D == 64 && turns <= 4 && smem <= kSmemHalf ? 2 : 1)) return 0;
-  auto go = [&](auto kern) { return launch_step<__nv_bfloat16>(kern, a, s, smem, q, k_new, v_new, out, st); };
+  auto go = [&](auto kern) {
+    if (!allow_dynamic_smem(kern, kSmemCta)) return -1;
+    split_and_place(s, heads, tiles, reinterpret_cast<const void*>(kern), step_smem<D>);
+    const size_t smem = step_smem<D>(s);
+    if (smem > kSmemCta || !step_small_pays<D>(a, s, D == 64 && turns <= 4 && smem <= kSmemHalf ? 2 : 1)) return 0;
+    return launch_step<__nv_bfloat16>(kern, a, s, smem, q, k_new, v_new, out, st);
+  };
   if (turns <= 1) return go(step_small_kernel<D, 1>);
   if (turns <= 2) return go(step_small_kernel<D, 2>);
   if constexpr (D == 64) {                      // at head_dim 128 shared memory holds fewer rows than four turns rank

@@ -1,4 +1,5 @@
-"""Compression of as many heads as clusters of an odd size would just find places for (45 of 3 CTAs, 26 of 5, 15 of 7 on
+"""Small steps in one launch of more heads than clusters of the size that would spread them best find a place (46 of 3
+CTAs, 35 of 4, 24 of 6 on 148 SMs), and compression of as many heads as clusters of an odd size would just find places for (45 of 3 CTAs, 26 of 5, 15 of 7 on
 148 SMs) and of one more than they may take: the cluster size changes there.  Protocol and bars are those of the parity tests."""
 from dataclasses import replace
 
@@ -21,5 +22,17 @@ def test_heads_at_the_line_of_a_cluster_size(base, heads):
     cfg = replace(get_config(base, n_layers=1), name=f"places-{heads}", n_heads=heads, batch=1, sides=(1, 2, 5, 9, 14, 23),
                   budget_c=260, budget_s=520)
     rep = run_parity(cfg, [0], fused=True, heads_per_layer=4, policy=1, gen_on_gpu=True)
+    assert rep.ok(), rep.problems[:5]
+    assert rep.compressed_heads > 0
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("head_dim,heads", [(128, 45), (128, 46), (64, 35), (128, 35), (64, 24), (128, 23)])
+def test_heads_at_the_places_of_small_clusters(head_dim, heads, dtype):
+    from parity_util import run_parity
+    base = get_config(0) if dtype == "fp32" else get_config(3 if head_dim == 128 else 1, n_layers=1)
+    cfg = replace(base, name=f"small-{heads}", n_heads=heads, batch=1, head_dim=head_dim, sides=(1, 2, 3, 5, 7, 9, 11),
+                  budget_c=60, budget_s=100)
+    rep = run_parity(cfg, [0], fused=True, heads_per_layer=4, policy=1)
     assert rep.ok(), rep.problems[:5]
     assert rep.compressed_heads > 0
