@@ -145,7 +145,7 @@ struct Bars {
   uint64_t v_full[kVStages], v_empty[kVStages];
   uint64_t s_full[2], s_free, p_full[2], p_free[2];
   uint64_t copy_full[2];                            // append: a chunk of new rows has landed in its staging half
-  uint64_t drain, drain2;
+  uint64_t drain;
   int2 out_at[8];                                   // per softmax warp
   uint32_t tmem_base;
   int abort_code;                                   // of the wait that gave up
@@ -255,8 +255,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     mbar_init(smem_u32(&bars->s_free), 4);          // the four warps of the tile whose logits were in the buffer
     mbar_init(smem_u32(&bars->copy_full[0]), 1);
     mbar_init(smem_u32(&bars->copy_full[1]), 1);
-    mbar_init(smem_u32(&bars->drain), 1);
-    mbar_init(smem_u32(&bars->drain2), 1);
+    mbar_init(smem_u32(&bars->drain), 2);           // the two issuers
     bars->abort_code = 0;
     fence_barrier_init();
     fence_proxy_async();
@@ -353,11 +352,6 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         }
         g += nblk;
       }
-      if (!ok) {
-        mma_commit(smem_u32(&bars->drain2));
-        const uint32_t bar = smem_u32(&bars->drain2);
-        for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(bar, 0); ++it) {}
-      }
     }
   } else if (warp == kAppendWarp) {
     reg_dec<kOtherRegs>();
@@ -400,7 +394,11 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             mbar_expect_tx(bar, bytes);
             bulk_load(copy_sm + half * kCopyChunk, src + (size_t)ch * kCopyChunk, bytes, bar);
             ok = wait_bar(&bars->copy_full[half], (chunks >> 1) & 1, bars, 12, wlim);
-            if (!ok) break;
+            if (!ok) {                               // the copy gets a bounded chance to land before the CTA leaves
+#pragma unroll 1
+              for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(bar, (chunks >> 1) & 1); ++it) {}
+              break;
+            }
             bulk_store(dst + (size_t)ch * kCopyChunk, copy_sm + half * kCopyChunk, bytes);
             bulk_commit();
           }
@@ -541,11 +539,6 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           }
         }
         g += nblk;
-      }
-      if (!ok) {
-        mma_commit(smem_u32(&bars->drain));
-        const uint32_t bar = smem_u32(&bars->drain);
-        for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(bar, 0); ++it) {}
       }
     }
   } else {
@@ -737,6 +730,15 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   }
   tc_fence_before();
   __syncthreads();
+  if (bars->abort_code) {
+    // after a wait that gave up: the products in flight, of either issuer, get a bounded chance to end before tensor memory is freed
+    if ((warp == kMmaWarp || warp == kPvWarp) && lane == 0) {
+      mma_commit(smem_u32(&bars->drain));
+#pragma unroll 1
+      for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(smem_u32(&bars->drain), 0); ++it) {}
+    }
+    __syncthreads();
+  }
   if (warp == kMmaWarp) {
     tc_fence_after();
     tmem_dealloc(tmem, Shape<T>::kTmemCols);

@@ -167,10 +167,6 @@ attn_colstats_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         }
         if (ok) mma_commit(smem_u32(&bars->q_empty[s]));
       }
-      if (!ok) {
-        mma_commit(smem_u32(&bars->drain));
-        for (uint32_t it = 0; it < kVarDrainSpins && !mbar_try_wait(smem_u32(&bars->drain), 0); ++it) {}
-      }
     }
   } else if ((warp - 2) / (4 * kVarParts) < n_sets) {
     // ------------------------------------------------------------------ consumers
@@ -258,6 +254,11 @@ attn_colstats_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
+    if (lane == 0 && bars->abort_flag) {             // what was issued gets a bounded chance to end, so that tensor memory can be freed
+      mma_commit(smem_u32(&bars->drain));
+      for (uint32_t it = 0; it < kVarDrainSpins && !mbar_try_wait(smem_u32(&bars->drain), 0); ++it) {}
+    }
+    __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem, 2 * kVarSets * kVarTile);
   }

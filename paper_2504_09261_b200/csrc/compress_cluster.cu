@@ -414,7 +414,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
       issue_ok = ok;
     }
   };
-  // After a wait that gave up: what is in flight gets a bounded chance to finish before the ring is reused.
+  // After a wait that gave up: what is in flight gets a bounded chance to finish before the ring is reused and tensor memory freed.
   auto drain = [&]() {
     mma_commit(smem_u32(&sh->drain));
 #pragma unroll 1
@@ -427,10 +427,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
     }
   };
   if (warp == kIssueWarp) {
-    if (lane == 0) {
-      issue(0, n_run);
-      if (!issue_ok) drain();
-    }
+    if (lane == 0) issue(0, n_run);
     __syncwarp();
   } else {
     // Thread r of a set owns key r of every chunk and keeps (reference maximum, sum-exp) of the set's 16
@@ -545,11 +542,7 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
 
   // ------------------------------------------------------------------ 3. scores, pass 2
   if (kAgain && warp == kIssueWarp) {
-    if (lane == 0 && issue_ok) {
-      // (tiles of the second products may be on their way already)
-      if (!aborted) issue(n_run, n_seq);
-      if (aborted || !issue_ok) drain();
-    }
+    if (lane == 0 && issue_ok && !aborted) issue(n_run, n_seq);
     __syncwarp();
   } else if (!aborted && warp != kIssueWarp) {
     const bool structural = ctx == 0;
@@ -605,6 +598,8 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
   }
   tc_fence_before();
   __syncthreads();
+  // (whichever thread's wait it was; tiles of the second products may be on their way when another CTA gives up)
+  if (warp == kIssueWarp && lane == 0 && (aborted || sh->abort_flag)) drain();
 
   if (select) {
     // ---------------------------------------------------------------- 4. radix select over the cluster

@@ -272,10 +272,6 @@ merge_assign_kernel(const __grid_constant__ CUtensorMap tm_e, const __grid_const
         mma_commit(smem_u32(&bars->k_empty[s]));
         mma_commit(smem_u32(&bars->acc_full[b]));
       }
-      if (!ok) {
-        mma_commit(smem_u32(&bars->drain));
-        for (uint32_t it = 0; it < kMergeDrainSpins && !mbar_try_wait(smem_u32(&bars->drain), 0); ++it) {}
-      }
     }
   } else {
     // ------------------------------------------------------------------ consumers
@@ -391,6 +387,11 @@ merge_assign_kernel(const __grid_constant__ CUtensorMap tm_e, const __grid_const
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
+    if (lane == 0 && bars->abort_flag) {             // what was issued gets a bounded chance to end, so that tensor memory can be freed
+      mma_commit(smem_u32(&bars->drain));
+      for (uint32_t it = 0; it < kMergeDrainSpins && !mbar_try_wait(smem_u32(&bars->drain), 0); ++it) {}
+    }
+    __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem, 2 * kTileM);
   }

@@ -202,11 +202,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_cache, const __grid_const
         mma_commit(smem_u32(&bars->empty[s]));
         mma_commit(smem_u32(&bars->acc_full[b]));
       }
-      if (!ok) {
-        // wait (bounded) for what was issued, so that TMEM can be released safely
-        mma_commit(smem_u32(&bars->drain));
-        for (uint32_t it = 0; it < kDrainSpins && !mbar_try_wait(smem_u32(&bars->drain), 0); ++it) {}
-      }
     }
   } else {
     // ------------------------------------------------------------------ consumers
@@ -306,6 +301,11 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tm_cache, const __grid_const
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
+    if (lane == 0 && bars->abort_flag) {             // what was issued gets a bounded chance to end, so that tensor memory can be freed
+      mma_commit(smem_u32(&bars->drain));
+      for (uint32_t it = 0; it < kDrainSpins && !mbar_try_wait(smem_u32(&bars->drain), 0); ++it) {}
+    }
+    __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem, kAccBufs * kMaxObs);
   }

@@ -62,3 +62,59 @@ def test_scoring_wait_runs_out_and_the_cache_stays_usable(head_dim):
     assert rep.ok(), rep.summary() + "\n" + "\n".join(rep.problems)
     assert rep.compressed_heads > 0
     cache.close()
+
+
+def _aborted_last_step(head_dim, sides, budget_c, budget_s, heads=6, batch=1, merge=False):
+    """A decode whose last step runs with a limit of one cycle; then a clean decode on the same cache and
+    on a fresh one, whose rows, positions and outputs have to be the same."""
+    import numpy as np
+    import paper_2504_09261_b200 as hb
+    mask = (np.arange(heads) % 2).astype(np.uint8)[None]
+    dev = torch.device("cuda:0")
+    g = torch.Generator(device=dev).manual_seed(head_dim + len(sides))
+    steps = [tuple(torch.randn((batch, heads, s * s, head_dim), generator=g, device=dev).bfloat16() for _ in range(3)) for s in sides]
+    caches = [hb.HackCache(1, heads, head_dim, batch, sides, hb.HACK_BF16, mask, budget_c, budget_s, merge_last=merge) for _ in range(2)]
+
+    def decode(cache, last_limit=0):
+        cache.hack_reset()
+        for k, (q, kk, v) in enumerate(steps):
+            if k == len(steps) - 1:
+                cache.hack_poll_status()
+                cache.hack_set_wait_limit(last_limit)
+            out = torch.full_like(q, float("nan"))
+            cache.hack_scale_step(0, k, q, kk, v, out)
+        return out
+
+    decode(caches[0], 1)
+    status = 0
+    try:
+        caches[0].hack_poll_status()
+    except hb.HackError as e:
+        status = e.status
+    caches[0].hack_set_wait_limit(0)
+    outs = [decode(c) for c in caches]
+    for c in caches:
+        c.hack_poll_status()
+    assert torch.equal(outs[0].view(torch.int16), outs[1].view(torch.int16))
+    for h in range(heads):
+        for which in (0, 1, 2):
+            assert caches[0].hack_read_head(0, batch - 1, h, which) == caches[1].hack_read_head(0, batch - 1, h, which)
+    for c in caches:
+        c.close()
+    return status
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("sides,budget_c,budget_s", [
+    ((1, 2, 4, 12, 26), 300, 760),      # both types evict; at head_dim 64 two CTAs of the attention share an SM
+    ((1, 2, 14, 24, 40), 2000, 2300),   # the same where a CTA takes two query tiles
+    ((1, 2, 4, 12, 26), 300, 2000),     # structural heads append beside the compression of the others
+])
+def test_a_step_that_evicts_gives_up_and_the_cache_stays_usable(head_dim, sides, budget_c, budget_s):
+    assert _aborted_last_step(head_dim, sides, budget_c, budget_s) == 6    # HACK_ERR_TIMEOUT
+
+
+@pytest.mark.parametrize("head_dim,sides", [(64, (1, 2, 20)), (64, (1, 20, 40)), (128, (1, 20, 40))])
+def test_an_appending_step_with_a_short_limit(head_dim, sides):
+    """The attention blocks in its waits for a while before it looks at the clock, so that it may well get through."""
+    assert _aborted_last_step(head_dim, sides, 4000, 4000, heads=40) in (0, 6)
