@@ -919,6 +919,14 @@ compress_cluster_kernel(const __grid_constant__ CUtensorMap tm_cache, const __gr
       issue_loads(t + 2);
     }
     if (tid == 0) bulk_wait_read<0>();                        // shared memory is read out before the CTA leaves
+  } else if (kLists && ctx) {
+    // After a wait that gave up: the launches behind this one read rows through the lists all the same, so these hold
+    // candidates of the head, each of them once.
+#pragma unroll 1
+    for (int j = rank * kCkThreads + tid; j < stored + n_new; j += CL * kCkThreads) {
+      if (j < n_rows) p.kept_list[(size_t)bh * a.kept_stride + j] = j;
+      else p.gone_list[(size_t)bh * p.gone_stride + (j - n_rows)] = j;
+    }
   }
   if (tid == 0 && sh->abort_flag) atomicExch(a.status, sh->abort_flag);
   // no CTA leaves while another may still read its shared memory (past the list nobody does)

@@ -118,3 +118,10 @@ def test_a_step_that_evicts_gives_up_and_the_cache_stays_usable(head_dim, sides,
 def test_an_appending_step_with_a_short_limit(head_dim, sides):
     """The attention blocks in its waits for a while before it looks at the clock, so that it may well get through."""
     assert _aborted_last_step(head_dim, sides, 4000, 4000, heads=40) in (0, 6)
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("budget_s", [760, 2000])
+def test_a_merging_step_that_gives_up_reads_rows_of_its_heads_only(head_dim, budget_s):
+    """Its lists of kept and discarded rows are not formed then, and the launches behind read rows through them."""
+    assert _aborted_last_step(head_dim, (1, 2, 4, 12, 26), 300, budget_s, merge=True) == 6
