@@ -68,6 +68,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <limits>
 #include <type_traits>
 
 #include "hack_internal.h"
@@ -113,7 +114,8 @@ struct TcParams {
   int pos_base;                          // global position of the new scale's first token
   int head_dim_pieces;                   // 16-byte pieces per row
   int cap[2];                            // rows a head of each type owns (checked builds)
-  long long wait_cycles;                 // limit of every mbarrier wait
+  long long wait_cycles;                 // limit of every mbarrier wait ...
+  long long unit_cycles;                 // ... but those for another role to be done with a unit of work
   uint4* k_plane;                        // cache planes of this layer (append only)
   uint4* v_plane;
   int32_t* pos_plane;
@@ -149,20 +151,24 @@ struct Bars {
   int2 out_at[8];                                   // per softmax warp
   uint32_t tmem_base;
   int abort_code;                                   // of the wait that gave up
+  int held;                                         // the producer waits for the launch ahead
 };
 
 // Waits for a phase of a barrier; false once the limit has passed or another wait of the CTA has given up.  In
 // little code: the instruction cache bounds this kernel (with waits of 40 instructions, 82 instead of 40 KB in
-// all, the loop lost 40 % at head_dim 64).  The status word is written at the end, by one thread.
+// all, the loop lost 40 % at head_dim 64).  The status word is written at the end, by one thread.  Time in which the
+// producer waits for the launch ahead does not count: that is not this launch's.
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Bars* b, int code, long long limit) {
   const uint32_t addr = smem_u32(bar);
   if (__builtin_expect(mbar_try_wait(addr, parity), 1)) return true;
   volatile int* const flag = &b->abort_code;
-  const long long t0 = clock64();
+  long long t0 = clock64();
 #pragma unroll 1
   while (!mbar_try_wait(addr, parity)) {
     if (*flag) return false;
-    if (clock64() - t0 > limit) *flag = code;
+    const long long now = clock64();
+    if (*static_cast<volatile int*>(&b->held)) t0 = now;
+    else if (now - t0 > limit) *flag = code;
   }
   return true;
 }
@@ -206,7 +212,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     return u;
   };
   // A role takes unit number n of this CTA (one thread; the arrival gives the slot back).
-  auto wait_unit = [&](int n) { return wait_bar(&bars->u_full[n & 1], (n >> 1) & 1, bars, 13, wlim); };
+  auto wait_unit = [&](int n) { return wait_bar(&bars->u_full[n & 1], (n >> 1) & 1, bars, 13, p.unit_cycles); };
   auto read_unit = [&](int n) {
     const volatile Unit& v = bars->unit[n & 1];
     return Unit{v.bh, v.part, v.type, v.krow};
@@ -226,6 +232,13 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   // Keys of the last block of a segment of `len` rows in groups of 32, the unit in which the products and the
   // softmax leave out what is past the last key
   auto last_groups = [](int len) { return (((len - 1) & (kBN - 1)) >> 5) + 1; };
+  // The producer's wait for the launch ahead
+  auto wait_ahead = [&]() {
+    volatile int* const held = &bars->held;
+    *held = 1;
+    pdl_grid_wait();
+    *held = 0;
+  };
   // Loads of the producer: a tile of 128 rows (the queries of slot t, or K / V block j of the unit)
   auto load_tile = [&](uint32_t dst, const CUtensorMap* tm, int row, uint64_t* bar) {
     mbar_expect_tx(smem_u32(bar), TILE_BYTES);
@@ -257,6 +270,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     mbar_init(smem_u32(&bars->copy_full[1]), 1);
     mbar_init(smem_u32(&bars->drain), 2);           // the two issuers
     bars->abort_code = 0;
+    bars->held = 1;                                 // until the first loads are on their way
     fence_barrier_init();
     fence_proxy_async();
   }
@@ -285,6 +299,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     };
     if (p.q_before_wait) load_queries();
     if (dep == kDepAll || (dep == kDepCache && nb == 0)) pdl_grid_wait();
+    *static_cast<volatile int*>(&bars->held) = 0;
     if (!p.q_before_wait) load_queries();
     load_kv(u, 0, nb, 0, 0);
     load_kv(u, 0, nb, 0, 1);
@@ -418,11 +433,11 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 #pragma unroll 1
       for (int n = 0;; ++n) {
         const int nb = blocks_b(u), nblk = blocks(u), nr = rounds_of(u), dep = p.dep[u.type];
-        if (n > 0 && (dep == kDepAll || (dep == kDepCache && nb == 0))) pdl_grid_wait();
+        if (n > 0 && (dep == kDepAll || (dep == kDepCache && nb == 0))) wait_ahead();
         // K / V tiles of the unit in order, and the queries of round r ahead of step r's value tile
 #pragma unroll 1
         for (int j = 0; j < max(nblk, nr) && ok; ++j) {
-          if (dep == kDepCache && j == nb && j < nblk) pdl_grid_wait();   // the head's stored survivors are in place
+          if (dep == kDepCache && j == nb && j < nblk) wait_ahead();   // the head's stored survivors are in place
           const bool fresh = n > 0 || j > 0;        // the first tiles and queries of the CTA are on their way already
           const uint32_t gs = g + j;
 #pragma unroll 1
@@ -466,7 +481,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           fence_proxy_async();                       // the next answer overwrites what was just read
           if (x >= 0) next = make_unit(x);
         }
-        if (n > 0) ok = wait_bar(&bars->u_empty[(n + 1) & 1], (((n + 1) >> 1) & 1) ^ 1, bars, 16, wlim);
+        if (n > 0) ok = wait_bar(&bars->u_empty[(n + 1) & 1], (((n + 1) >> 1) & 1) ^ 1, bars, 16, p.unit_cycles);
         if (!ok) break;
         bars->unit[(n + 1) & 1] = next;
         mbar_arrive(smem_u32(&bars->u_full[(n + 1) & 1]));
@@ -865,6 +880,11 @@ int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_sta
   p.cap[0] = a.cap[0];
   p.cap[1] = a.cap[1];
   p.wait_cycles = a.wait_cycles;
+  // a block takes a role no more than eight waits
+  long long unit_waits = 0;
+  for (int t = 0; t < 2; ++t)
+    unit_waits = std::max<long long>(unit_waits, 8ll * p.rounds[t] * ((p.len_a[t] + kBN - 1) / kBN + (p.len_b[t] + kBN - 1) / kBN + 1));
+  p.unit_cycles = a.wait_cycles > std::numeric_limits<long long>::max() / unit_waits ? a.wait_cycles : a.wait_cycles * unit_waits;
   p.k_plane = static_cast<uint4*>(a.k_plane);
   p.v_plane = static_cast<uint4*>(a.v_plane);
   p.pos_plane = a.pos_plane;

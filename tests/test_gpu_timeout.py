@@ -125,3 +125,26 @@ def test_an_appending_step_with_a_short_limit(head_dim, sides):
 def test_a_merging_step_that_gives_up_reads_rows_of_its_heads_only(head_dim, budget_s):
     """Its lists of kept and discarded rows are not formed then, and the launches behind read rows through them."""
     assert _aborted_last_step(head_dim, (1, 2, 4, 12, 26), 300, budget_s, merge=True) == 6
+
+
+def test_the_limit_counts_neither_the_launch_ahead_nor_whole_units_of_work():
+    """Two attention launches of three rounds of CTAs, back to back: a CTA of the second one waits for the first for as
+    long as that launch's last CTAs take, and a unit is 83 blocks of 128 keys, 130 us.  The limit lies below either, at
+    about 40 us, far above what a wait inside the loop takes (a block is 1.6 us)."""
+    import paper_2504_09261_b200 as hb
+    dev = torch.device("cuda:0")
+    sides, heads, batch, dim = (1, 2, 80, 64), 16, 2, 128
+    cache = hb.HackCache(2, heads, dim, batch, sides, hb.HACK_BF16, [0, 1] * heads, 20000, 20000)
+    g = torch.Generator(device=dev).manual_seed(5)
+    steps = [tuple(torch.randn((batch, heads, s * s, dim), generator=g, device=dev).bfloat16() for _ in range(3)) for s in sides]
+    outs = [torch.empty_like(steps[-1][0]) for _ in range(4)]
+    for limit in (0, 75000):
+        cache.hack_reset()
+        for k, (q, kk, v) in enumerate(steps):
+            cache.hack_set_wait_limit(limit if k == len(steps) - 1 else 0)
+            for layer in range(2):
+                cache.hack_scale_step(layer, k, q, kk, v, outs[layer + (2 if limit else 0)] if k == len(steps) - 1 else torch.empty_like(q))
+        cache.hack_poll_status()                   # raises if a wait ran out
+    assert torch.equal(outs[0].view(torch.int16), outs[2].view(torch.int16))
+    assert torch.equal(outs[1].view(torch.int16), outs[3].view(torch.int16))
+    cache.close()
