@@ -73,7 +73,8 @@ __host__ __device__ __forceinline__ int tile_begin(const Shares& sh, int tile) {
   return n * (2 * sh.rounds[0] + 1) + (tile - n) * (2 * sh.rounds[1] + 1);
 }
 
-// One query tile per CTA, or per cluster, or equal shares (a form of its own: its bookkeeping costs the others registers).
+// One query tile per CTA, or per cluster, or equal shares (a form of its own: its bookkeeping costs the others registers;
+// at head_dim 64, with two CTAs on an SM, it spills 24 bytes, which the plain form does not).
 enum { kOne, kClustered, kShared };
 
 template <int D, int MODE>
@@ -155,7 +156,7 @@ attend_simt_kernel(const StepArgs a, const float* __restrict__ q, float* __restr
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) s[i][j] = make_float2(0.f, 0.f);
-#pragma unroll (D == 128 ? 8 : 4)
+#pragma unroll (D == 128 || MODE == kOne ? 8 : 4)
       for (int d = 0; d < D; d += 4) {
         float4 qf[4], kf[4];
 #pragma unroll
