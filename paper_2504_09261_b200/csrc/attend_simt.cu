@@ -22,19 +22,16 @@
 // shared memory per 4 multiply-adds with a four-way bank conflict.  Decoding loop of two layers of 16
 // heads x 128, 2 240 tokens, stage calls: 13.8 -> 1.66 ms; one layer of 16 heads x 64, 680 tokens:
 // 0.531 -> 0.308 ms.)
-#include <algorithm>
-
 #include "hack_internal.h"
+#include "launch_plans.h"
 #include "tc_ptx.cuh"
 
 namespace hack {
 namespace {
 
 using ptx::fma2;
+using namespace simt;
 
-constexpr int kBQ = 32;              // query rows per CTA
-constexpr int kBK = 32;              // keys per tile
-constexpr int kGroups = 4;           // groups of 64 threads, each with its own key tiles
 constexpr int kThreads = kGroups * 64;
 
 // 32 rows of D floats from global memory (rows at or past n_rows read as zero) into padded rows by
@@ -58,19 +55,6 @@ template <int D>
 constexpr size_t simt_smem_bytes() {
   // query rows, then per group a key tile, a value tile and a probability tile
   return sizeof(float) * ((size_t)kBQ * (D + 4) + kGroups * (2 * (size_t)kBK * (D + 4) + kBQ * (kBK + 8)));
-}
-
-// A launch whose query tiles are shared out evenly: the tiles of the first type's heads, then the others', laid
-// end to end, a tile of r rounds (a key tile per group each) as 2 r + 1 half rounds, the first of which stands for its
-// loads and its merge.  CTA i takes the half rounds [i * span, (i + 1) * span).
-struct Shares {
-  int n_qt, n_first;              // query tiles per head; of the first type's heads together
-  int rounds[2];                  // of a query tile of the first type, of the other one
-  int span, total;                // half rounds of a CTA, of the launch
-};
-__host__ __device__ __forceinline__ int tile_begin(const Shares& sh, int tile) {
-  const int n = tile < sh.n_first ? tile : sh.n_first;
-  return n * (2 * sh.rounds[0] + 1) + (tile - n) * (2 * sh.rounds[1] + 1);
 }
 
 // One query tile per CTA, or per cluster, or equal shares (a form of its own: its bookkeeping costs the others registers;
@@ -358,76 +342,17 @@ attend_simt_kernel(const StepArgs a, const float* __restrict__ q, float* __restr
   if (kCluster) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
-// Rounds until `slots` CTAs at a time have done the tiles one by one, those of the first type first.
-float rounds_one_by_one(const Shares& sh, int tiles, int slots) {
-  struct Group { float at; int n; } g[16] = {{0.f, slots}};
-  int groups = 1;
-  float end = 0.f;
-  for (int type = 0; type < 2; ++type)
-    for (int left = type == 0 ? sh.n_first : tiles - sh.n_first; left > 0;) {
-      int e = 0;                                             // the places that are free first
-      for (int i = 1; i < groups; ++i)
-        if (g[i].at < g[e].at) e = i;
-      const int take = std::min(left, g[e].n);
-      const float at = g[e].at + sh.rounds[type] + 0.5f;
-      g[e].n -= take;
-      if (g[e].n == 0) g[e] = g[--groups];
-      if (groups == 16) return 1e30f;
-      g[groups++] = {at, take};
-      end = std::max(end, at);
-      left -= take;
-    }
-  return end;
-}
-
 template <int D>
 int launch_t(const StepArgs& a, const void* q, void* out, cudaStream_t st) {
   const int n_qt = (a.n_new + kBQ - 1) / kBQ, heads = a.batch * a.n_heads;
-  // Cluster size: the shortest estimate of the launch in key tiles of a group.  A CTA costs its share of
-  // the tiles and about three more (start, merge); a launch past one wave lasts as long as all of them
-  // spread over the SMs plus half of its longest CTA.  Steps of 16 heads x 100 queries x 64: 33.2 -> 30.8 us
-  // with two CTAs per query tile, 256 queries 49.5 -> 39.3; 324 queries x 128: 85 -> 75 by the order of the
-  // heads alone; 4 CTAs per tile 310 -> 464 where the launch is long anyway (1 024 queries, 1 717 keys).
-  const float sms = (float)sm_count();
-  int cl = 1;
-  float best = 0.f;
-  for (int c = 1; c <= 4; c *= 2) {
-    float total = 0.f, longest = 0.f;
-    for (int t = 0; t < 2; ++t) {
-      if (a.heads_of[t] == 0) continue;
-      const float one = 3.f + (float)(((a.kept[t] + kBK - 1) / kBK + c * kGroups - 1) / (c * kGroups));
-      total += one * a.heads_of[t] * n_qt * c;
-      longest = std::max(longest, one);
-    }
-    const float cost = n_qt * c * heads <= sms ? longest : std::max(longest, total / sms + 0.5f * longest);
-    if (c == 1 || cost < best) {
-      best = cost;
-      cl = c;
-    }
-  }
-  const int first_type = a.kept[1] > a.kept[0];
-  const int32_t* order = a.head_order + (first_type ? heads : 0);
-  Shares sh{};
-  bool shared = false;
-  if (cl == 1) {
-    const int slots = sm_count() * (D == 64 ? 2 : 1);
-    sh.n_qt = n_qt;
-    sh.n_first = n_qt * a.heads_of[first_type];
-    for (int i = 0; i < 2; ++i) {
-      const int type = i == 0 ? first_type : 1 - first_type;
-      sh.rounds[i] = ((a.kept[type] + kBK - 1) / kBK + kGroups - 1) / kGroups;
-    }
-    // A query tile per CTA, the longer ones first, or equal shares, whichever ends earlier; parts of a tile that meet
-    // in memory cost about a round.  16 heads x 128, us a step: 324 queries (176 tiles) 70 against 77, 576 queries
-    // (288 tiles) 170 against 138, 1 024 queries (512 tiles) 300 against 267.
-    sh.total = tile_begin(sh, n_qt * heads);
-    sh.span = (sh.total + slots - 1) / slots;
-    shared = n_qt * heads > sm_count() && rounds_one_by_one(sh, n_qt * heads, slots) > 0.5f * sh.span + 1.f;
-  }
-  auto kern = cl > 1 ? attend_simt_kernel<D, kClustered> : shared ? attend_simt_kernel<D, kShared> : attend_simt_kernel<D, kOne>;
+  const SimtPlan plan = simt_plan(D, a.n_new, a.kept, a.heads_of, sm_count());
+  const Shares& sh = plan.sh;
+  const int cl = plan.cluster;
+  const int32_t* order = a.head_order + (a.kept[1] > a.kept[0] ? heads : 0);
+  auto kern = cl > 1 ? attend_simt_kernel<D, kClustered> : plan.shared ? attend_simt_kernel<D, kShared> : attend_simt_kernel<D, kOne>;
   if (!allow_dynamic_smem(kern, simt_smem_bytes<D>())) return -1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = shared ? dim3((sh.total + sh.span - 1) / sh.span) : dim3(n_qt * cl, heads);
+  cfg.gridDim = plan.shared ? dim3(plan.ctas) : dim3(n_qt * cl, heads);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = simt_smem_bytes<D>();
   cfg.stream = st;

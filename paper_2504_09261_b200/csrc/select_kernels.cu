@@ -12,6 +12,7 @@
 // digit holding the wanted rank is located by one warp, and the index list is produced with a
 // single block scan.  Longer candidate lists take the general path that re-reads the scores.
 #include "hack_internal.h"
+#include "launch_plans.h"
 
 namespace hack {
 namespace {
@@ -179,7 +180,6 @@ select_reg_kernel(const StepArgs a, const float* __restrict__ scores, int32_t* _
 // Where there are SMs to spare a cluster of up to four CTAs moves a head's rows (one CTA reads and writes its own at 40 GB/s);
 // each forms the whole list for itself.  Steps of 169 and 256 queries 33.8 -> 32.3 and 33.3 us.
 constexpr int kMoveRun = 4;
-constexpr size_t kSmallMoveBytes = 384 * 1024;   // K and V rows of a head
 
 template <int E>
 __global__ void __launch_bounds__(kSelThreads)

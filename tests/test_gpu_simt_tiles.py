@@ -122,3 +122,10 @@ def test_query_tiles_that_ctas_share(head_dim, heads, batch, sides, b_c, b_s):
                     ref = z.softmax(-1) @ vc[b, h, pos]
                     assert (out[b, h].double() - ref).abs().max() <= 1e-5, (k, b, h)
     cache.close()
+
+
+@pytest.mark.parametrize("heads,batch,sides", [(16, 1, (2, 24, 18)), (13, 2, (5, 22, 19))])
+def test_query_tiles_that_ctas_share_at_head_dim_64(heads, batch, sides):
+    """Sizes that head_dim 64 serves in shares: 176 tiles of 8 rounds, 312 of 7."""
+    total = sum(s * s for s in sides)
+    test_query_tiles_that_ctas_share(64, heads, batch, sides, total, total)
