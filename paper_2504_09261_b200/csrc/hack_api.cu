@@ -1,6 +1,7 @@
 // Host side of the C ABI: argument checks, the per-layer state machine, the deterministic length
 // plan of every step, cache and scratch allocation, and the launch sequence of the step.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -45,6 +46,36 @@ int sm_count() {
     count[dev] = n;
   }
   return count[dev];
+}
+
+int cluster_places(const void* kern, int ctas, int threads, size_t smem) {
+  if (ctas == 1) return INT_MAX;
+  struct Known { const void* kern; int dev, ctas; size_t smem; int n; };
+  static std::mutex mu;
+  static std::vector<Known> known;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lock(mu);
+  for (const Known& k : known)
+    if (k.kern == kern && k.dev == dev && k.ctas == ctas && k.smem == smem) return k.n;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ctas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    n = INT_MAX;                                // no answer: no limit
+  }
+  known.push_back({kern, dev, ctas, smem, n});
+  return n;
 }
 
 bool attend_tc_serves(const StepArgs& a, int dtype) {

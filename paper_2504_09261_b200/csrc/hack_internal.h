@@ -150,6 +150,9 @@ constexpr int kTcMinQueries = 32;   // below this the small kernel serves every 
 void set_error(const std::string& msg);
 // Number of SMs of the current device (asked once per device); the grid heuristics size to it.
 int sm_count();
+// Clusters of `ctas` CTAs of a kernel that find a place at once on an empty chip (asked once per kernel, size and device; its
+// opt-in to the shared memory comes first).
+int cluster_places(const void* kern, int ctas, int threads, size_t smem);
 
 // Every kernel of the step is launched with programmatic stream serialisation: its CTAs may start
 // while the previous kernel of the stream drains, and stop at pdl_wait() until that kernel has

@@ -10,6 +10,23 @@ namespace hack {
 // K and V rows of a head up to which the selection moves the rows itself (select_kernels.cu).
 constexpr size_t kSmallMoveBytes = 384 * 1024;
 
+// ---------------------------------------------------------------- selection with the moves (select_kernels.cu)
+// CTAs per head.  A cluster moves a head's rows faster than one CTA, which reads and writes its own at 40 GB/s, but every
+// cluster has to find a place at once (148 SMs take 33 of 4 CTAs: 37 heads x 64, 324 queries 67.8 us a step with one CTA, 72.2 with
+// four).  The CTAs of the attention behind it take their SMs while it runs.  At head_dim 128 an SM holds one of them either way
+// (us a step with one, two and four CTAs: 16 heads, 324 queries 50.4, 48.1 and 45.8, 26 heads 67.3, 65.1 and 63.0, 37 heads 80.4,
+// 77.9 and, in a second wave, 81.5).  At head_dim 64 two of them meet on an SM if the launch leaves too few, so there it
+// leaves one each of attention_ctas (8 heads, 196 queries, 64 CTAs 23.0, 23.0 and 21.5; 16 heads, 112 CTAs 33.3, 31.7 and 36.4, 256
+// queries, 128 CTAs 28.4, 30.5 and 30.0; 26 heads, 182 CTAs 28.4, 32.3 and 34.3), unless there are two for every SM anyway (33
+// heads, 324 queries, 363 CTAs 60.2, 56.3 and 55.5; 45 heads, 256 queries, 360 CTAs 57.7 and 55.2).
+template <typename Places>
+int move_ctas(int heads, int attention_ctas, int sms, Places places) {
+  int cl = 1;
+  const int beside = attention_ctas < 2 * sms ? attention_ctas : 0;
+  while (cl < 4 && heads * cl * 2 + beside <= sms && heads <= places(2 * cl)) cl *= 2;
+  return cl;
+}
+
 // ---------------------------------------------------------------- attention of fp32 caches (attend_simt.cu)
 namespace simt {
 

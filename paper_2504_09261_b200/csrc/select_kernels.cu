@@ -177,8 +177,8 @@ select_reg_kernel(const StepArgs a, const float* __restrict__ scores, int32_t* _
 // before those of every later round, so reading a round before writing it is enough.  Three launches of 3
 // to 5 us that wait for each other become one where a head's rows are a few microseconds for one SM
 // (kSmallMoveBytes); step of 16 fp32 heads x 64, 374 kept rows: 36.0 against 40.4 us, 34 rows 20.4 against 24.6.
-// Where there are SMs to spare a cluster of up to four CTAs moves a head's rows (one CTA reads and writes its own at 40 GB/s);
-// each forms the whole list for itself.  Steps of 169 and 256 queries 33.8 -> 32.3 and 33.3 us.
+// Where there are SMs to spare a cluster of up to four CTAs moves a head's rows (move_ctas); each forms the whole list for
+// itself.
 constexpr int kMoveRun = 4;
 
 template <int E>
@@ -305,8 +305,10 @@ int launch_select_move(const StepArgs& a, int dtype, const float* scores, const 
   const int row_pieces = a.head_dim * (dtype == HACK_F32 ? 4 : 2) / 16;
   if (max_cand > 4 * kSelThreads || (size_t)max_keep * row_pieces * 32 > kSmallMoveBytes) return 0;
   const int heads = a.batch * a.n_heads;
-  int cl = 1;
-  while (cl < 4 && heads * cl * 2 <= sm_count()) cl *= 2;
+  const int beside = dtype == HACK_F32 && a.head_dim == 64 ? simt::simt_plan(64, a.n_new, a.kept, a.heads_of, sm_count()).ctas : 0;
+  const int cl = move_ctas(heads, beside, sm_count(), [](int ctas) {
+    return cluster_places(reinterpret_cast<const void*>(select_move_kernel<4>), ctas, kSelThreads, 4 * kSelThreads * sizeof(int32_t));
+  });
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(heads * cl);
   cfg.blockDim = dim3(kSelThreads);

@@ -2,10 +2,6 @@
 // a launch and the selection of a head's survivors by one block.
 #pragma once
 
-#include <climits>
-#include <mutex>
-#include <vector>
-
 #include "hack_internal.h"
 
 namespace hack {
@@ -43,38 +39,6 @@ inline void split_queries(StepShape& s, int heads, int tiles, int at_most = kMax
   for (s.log_splits = 0; s.tiles << s.log_splits < kStepWarps; ++s.log_splits) {}
 }
 
-// Clusters of `ctas` CTAs that find a place at once on an empty chip (asked once per kernel, size and device).
-inline int cluster_places(const void* kern, int ctas, size_t smem) {
-  if (ctas == 1) return INT_MAX;
-  struct Known { const void* kern; int dev, ctas; bool half; int n; };
-  static std::mutex mu;
-  static std::vector<Known> known;
-  const bool half = smem <= kSmemHalf;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  std::lock_guard<std::mutex> lock(mu);
-  for (const Known& k : known)
-    if (k.kern == kern && k.dev == dev && k.ctas == ctas && k.half == half) return k.n;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ctas);
-  cfg.blockDim = dim3(kStepThreads);
-  cfg.dynamicSmemBytes = half ? kSmemHalf : kSmemCta;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = ctas;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
-    cudaGetLastError();
-    n = INT_MAX;                                // no answer: no limit
-  }
-  known.push_back({kern, dev, ctas, half, n});
-  return n;
-}
-
 // split_queries, with smaller clusters where those meant to run at once would not all find a place (the SMs of a
 // processing cluster are no multiple of every size: 148 SMs take 45 clusters of 3, 33 of 4, 22 of 6).  A second wave doubles
 // the step: 46 heads x 128, 81 queries 17.1 -> 12.3 us; 35 heads, 121 queries 17.4 -> 13.0; 24 heads, 81
@@ -82,7 +46,7 @@ inline int cluster_places(const void* kern, int ctas, size_t smem) {
 template <typename Smem>
 void split_and_place(StepShape& s, int heads, int tiles, const void* kern, Smem smem) {
   split_queries(s, heads, tiles);
-  for (int most = s.ctas - 1; most >= 1 && heads * s.ctas <= sm_count() && heads > cluster_places(kern, s.ctas, smem(s)); --most)
+  for (int most = s.ctas - 1; most >= 1 && heads * s.ctas <= sm_count() && heads > cluster_places(kern, s.ctas, kStepThreads, smem(s) <= kSmemHalf ? kSmemHalf : kSmemCta); --most)
     split_queries(s, heads, tiles, most);
 }
 

@@ -129,3 +129,16 @@ def test_query_tiles_that_ctas_share_at_head_dim_64(heads, batch, sides):
     """Sizes that head_dim 64 serves in shares: 176 tiles of 8 rounds, 312 of 7."""
     total = sum(s * s for s in sides)
     test_query_tiles_that_ctas_share(64, heads, batch, sides, total, total)
+
+
+@pytest.mark.parametrize("head_dim,heads", [(128, 33), (128, 36), (128, 80), (64, 9), (64, 40)])
+def test_selection_that_moves_the_rows_in_clusters_of_every_size(head_dim, heads):
+    """Four, two and one CTA per head at head_dim 128; at head_dim 64 as many as leave the attention its SMs."""
+    from dataclasses import replace
+    from parity_util import run_parity
+    from workloads import get_config
+    cfg = replace(get_config(0), name=f"select-move-{head_dim}-{heads}", n_heads=heads, batch=1, head_dim=head_dim, sides=(1, 3, 9, 13, 17),
+                  budget_c=150, budget_s=380)
+    rep = run_parity(cfg, [0], fused=True, heads_per_layer=6, policy=1)
+    assert rep.ok(), rep.problems[:5]
+    assert rep.evicting_launches[-1] <= 4, rep.evicting_launches      # scores in one or two launches, selection with the moves, attention

@@ -15,6 +15,9 @@ extern "C" void attention(int dim, int n_new, int kept_s, int kept_c, int heads_
   const hack::simt::SimtPlan p = hack::simt::simt_plan(dim, n_new, kept, heads, 148);
   out[0] = p.cluster; out[1] = p.shared; out[2] = p.ctas;
 }
+// clusters of 2, 4 CTAs that 148 SMs take at once
+static int places(int ctas) { return ctas == 1 ? 1 << 30 : ctas == 2 ? 74 : 33; }
+extern "C" int move_ctas(int heads, int attention_ctas) { return hack::move_ctas(heads, attention_ctas, 148, places); }
 """
 
 
@@ -60,3 +63,18 @@ def test_query_tiles_in_shares_at_head_dim_128(plans, queries, kept_s, kept_c, s
     out = (ctypes.c_int * 3)()
     plans.attention(128, queries, kept_s, kept_c, 10, 6, out)
     assert bool(out[1]) == (shares < apart), list(out)
+
+
+# selection with the moves: us a step with 1, 2 and 4 CTAs per head
+@pytest.mark.parametrize("dim,heads,queries,kept_s,kept_c,us", [
+    (64, 8, 196, 216, 40, (23.0, 23.0, 21.5)), (64, 16, 196, 380, 190, (33.3, 31.7, 36.4)), (64, 16, 256, 276, 40, (28.4, 30.5, 30.0)),
+    (64, 26, 196, 216, 40, (28.4, 32.3, 34.3)), (64, 37, 196, 250, 120, (36.9, 36.9, 42.0)), (128, 16, 324, 344, 40, (50.4, 48.1, 45.8)),
+    (128, 33, 256, 380, 190, (77.1, 74.0, 70.9)), (128, 37, 144, 250, 120, (47.4, 45.1, 50.0)), (128, 45, 324, 344, 40, (90.5, 88.2, None)),
+    (128, 80, 324, 344, 40, (135.0, None, None)), (64, 33, 324, 380, 190, (60.2, 56.3, 55.5)), (64, 45, 256, 380, 190, (57.7, 55.2, None)),
+])
+def test_ctas_that_move_the_rows_of_a_head(plans, dim, heads, queries, kept_s, kept_c, us):
+    out = (ctypes.c_int * 3)()
+    plans.attention(dim, queries, kept_s, kept_c, heads - heads // 2, heads // 2, out)
+    cl = plans.move_ctas(heads, out[2] if dim == 64 else 0)
+    best = min(t for t in us if t is not None)
+    assert us[{1: 0, 2: 1, 4: 2}[cl]] <= 1.02 * best, (cl, list(out))
