@@ -138,4 +138,159 @@ inline SimtPlan simt_plan(int head_dim, int n_new, const int* kept, const int* h
 }
 
 }  // namespace simt
+
+// ---------------------------------------------------------------- small steps in one launch (step_small.cu, step_small_f32.cu)
+namespace small_step {
+
+constexpr int kStepWarps = 8;
+constexpr int kStepThreads = kStepWarps * 32;
+constexpr int kMaxRows = 768;                   // candidates of a head, at most
+constexpr int kMaxTiles = 8;                    // query tiles of a CTA
+constexpr int kMaxCtas = 8;                     // CTAs per head
+constexpr size_t kSmemCta = 216 * 1024;         // dynamic shared memory beside the static tables ...
+constexpr size_t kSmemHalf = 108 * 1024;        // ... and with two CTAs on an SM
+
+struct StepShape {
+  int ctas;        // CTAs per head
+  int tiles;       // query tiles per CTA: 1, 2, 4 or 8; the CTA's 8 warps share the keys of a tile 8 / tiles ways
+  int log_splits;  // log2(8 / tiles)
+  int rows;        // candidate rows shared memory has room for
+};
+
+// What the rules know of a step; arrays by head type, structural heads first (as the launches take them).
+struct StepSizes {
+  int head_dim, n_new;
+  const int *heads_of, *cand, *kept, *trig;
+  int sms;
+};
+
+// The CTAs of a head and their query tiles: as many CTAs per head as leave every CTA an SM, at least what its
+// queries need; clusters of seven and eight only where they are few (16 clusters of 8 CTAs do not find a
+// place at once beside each other: 100 queries, 16 heads, bf16: 7 CTAs 8.5 us, 4 CTAs 7.9; 169 queries:
+// 6 CTAs 8.2, 3 CTAs 10.3).
+inline void split_queries(StepShape& s, int heads, int tiles, int sms, int at_most = kMaxCtas) {
+  auto split = [&](int most) {
+    int want = sms / heads < tiles ? sms / heads : tiles;
+    want = want < 1 ? 1 : want > most ? most : want;
+    for (s.tiles = 1; s.tiles < kMaxTiles && s.tiles * want < tiles; s.tiles *= 2) {}
+    s.ctas = (tiles + s.tiles - 1) / s.tiles;
+  };
+  split(at_most);
+  if (s.ctas > 6 && heads * s.ctas * 2 > sms) split(kMaxCtas / 2);
+  for (s.log_splits = 0; s.tiles << s.log_splits < kStepWarps; ++s.log_splits) {}
+}
+
+// The clusters of split_queries are meant to run at once, but may not all find a place (the SMs of a processing cluster are
+// no multiple of every size: 148 SMs take 45 clusters of 3, 33 of 4, 22 of 6).  Returns the heads that have to wait for a
+// first one to end; if there are any, `smaller` is the shape of the largest clusters that all find a place and fit shared
+// memory (ctas 0: there is none, -1: it does not fit).
+template <typename Smem, typename Places>
+int split_and_place(StepShape& s, StepShape& smaller, int heads, int tiles, int sms, Smem smem, Places places) {
+  auto missing = [&](const StepShape& of) {
+    const size_t bytes = smem(of);
+    if (heads * of.ctas > sms || bytes > kSmemCta) return 0;
+    const int n = places(of.ctas, bytes <= kSmemHalf ? kSmemHalf : kSmemCta);
+    return heads > n ? heads - n : 0;
+  };
+  split_queries(s, heads, tiles, sms);
+  smaller = s;
+  const int waiting = missing(s);
+  bool found = false, fits = true;
+  for (int most = s.ctas - 1; waiting > 0 && most >= 1 && !found && fits; --most) {
+    split_queries(smaller, heads, tiles, sms, most);
+    fits = smem(smaller) <= kSmemCta;
+    found = fits && smaller.ctas < s.ctas && missing(smaller) == 0;
+  }
+  if (!found) smaller.ctas = fits ? 0 : -1;
+  return waiting;
+}
+
+// Microseconds of a bf16 step in one launch and in the two it stands for (compression, then attention).  Both forms were
+// fitted to 287 steps of 8 to 256 heads, 16 to 400 queries and 50 to 700 candidates (rms 8 and 6 %).  two_waves: the same in one
+// launch of which `waiting` heads, the last ones, start when the first clusters end (23 to 49 heads, 81 to 361 queries,
+// within 10 % where shared memory holds one CTA).
+struct StepTimes { float here, two_waves, apart; };
+inline StepTimes step_times(const StepSizes& z, const StepShape& s, int per_sm, int waiting) {
+  constexpr int kTile = 16;                     // keys a warp weighs at a time
+  const float sms = (float)z.sms, heads = (float)(z.heads_of[0] + z.heads_of[1]), ctas = heads * s.ctas;
+  const float turn = z.head_dim == 64 ? 0.92f : 1.81f;
+  const int keys = 2 * kTile << s.log_splits;   // of a turn
+  float longest = 0.f, mean = 0.f, work = 0.f, ranked = 0.f, last = 0.f;
+  for (int t = 0; t < 2; ++t) {
+    if (z.heads_of[t] == 0) continue;
+    const float start = 2.1f + (z.trig[t] && z.kept[t] < z.cand[t] ? 3.5f : 0.f) + 0.031f * (z.cand[t] * z.head_dim * 4 / 1000.f);
+    const float us = start + turn * ((z.kept[t] + keys - 1) / keys);
+    longest = std::max(longest, us);
+    mean += us * z.heads_of[t] / heads;
+    work += (float)z.heads_of[t] * ((z.n_new + 127) / 128) * (1 + (z.kept[t] + 127) / 128);
+    if (z.trig[t]) ranked = std::max(ranked, z.cand[t] / 128.f);
+    if (t == 0 || z.heads_of[1] >= waiting) last = start + turn * z.kept[t] / keys;
+  }
+  StepTimes us;
+  // two CTAs on an SM slow each other down by two thirds
+  us.here = std::max(longest * (per_sm == 2 ? 1.f + 0.67f * std::min(1.f, std::max(0.f, ctas / sms - 1.f)) : 1.f),
+                     ctas > sms * per_sm ? mean * (ctas / (sms * per_sm) * (per_sm == 2 ? 1.67f : 1.f) + 0.3f) : 0.f);
+  us.two_waves = std::max(longest, 1.8f * last);
+  us.apart = z.head_dim == 64 ? 10.8f + (1.58f * heads + 0.92f * work) / sms + 1.57f * ranked
+                              : 11.9f + (3.92f * heads + 1.13f * work) / sms + 1.94f * ranked;
+  return us;
+}
+
+// The shape of a bf16 step in one launch (s.rows is given); false: two launches are the faster ones.  turns: key tiles of a warp.
+// This side has become faster since the fit where every CTA has an SM and a cluster is smaller than eight, so there it
+// is taken up to a tenth past the line, to 256 queries: 13 heads x 128, 121 queries 20.5 -> 15.7 us, 36 heads, 169 queries
+// 22.2 -> 18.4, 52 heads x 64, 196 queries 22.5 -> 19.1.  Elsewhere it keeps a margin of a tenth (81 heads x 64, 169 queries
+// 20.5 against 24.6; 18 heads, 400 queries 21.2 against 22.5).  16 heads x 64, 36 queries, 91 candidates: 5.9 against 12.6;
+// 256 heads: 9.3 against 18.2; 100 queries, 168 and 255 candidates: 7.3 against 12.8 (16 heads), 20.2 against
+// 19.9 (256 heads: not taken); 16 heads x 128, 36 queries, 91 candidates: 7.5 against 15.0; 256 heads: 18.6
+// against 25.2.
+// Where clusters would have to wait, smaller ones usually are faster (46 heads x 128, 81 queries 17.1 -> 12.3 us; 35 heads, 121
+// queries 17.4 -> 13.0; 24 heads, 81 queries 16.0 -> 10.2), but not if the heads that wait are contextual ones of few
+// keys: 46 heads x 128, 144 queries, 174 candidates, clusters of 3, of 2, two launches: 16.1, 17.9 and 17.4 us with 23 keys, 17.1,
+// 17.9 and 17.7 with 43, 19.5, 17.9 and 18.9 with 87.  (At head_dim 64 with a margin: 24 heads, 324 queries, 435 candidates 18.0
+// against 16.4 for two launches.)
+template <typename Smem, typename Places>
+bool step_shape_bf16(const StepSizes& z, StepShape& s, int tiles, int turns, Smem smem, Places places) {
+  const int heads = z.heads_of[0] + z.heads_of[1];
+  StepShape smaller;
+  const int waiting = split_and_place(s, smaller, heads, tiles, z.sms, smem, places);
+  auto times = [&](const StepShape& of) { return step_times(z, of, z.head_dim == 64 && turns <= 4 && smem(of) <= kSmemHalf ? 2 : 1, waiting); };
+  if (smem(s) > kSmemCta) return false;
+  if (waiting > 0) {
+    const StepTimes us = times(s);
+    if (smaller.ctas <= 0 || us.two_waves < 0.95f * times(smaller).here) return us.two_waves * (z.head_dim == 64 ? 1.1f : 1.f) < us.apart;
+    s = smaller;
+  }
+  const StepTimes us = times(s);
+  return us.here * (heads * s.ctas <= z.sms && s.ctas < kMaxCtas && z.n_new <= 256 ? 0.9f : 1.1f) < us.apart;
+}
+
+// The same for a step of an fp32 cache: every head of up to 128 candidates; longer ones only where every CTA has an SM to itself
+// (120 heads x 64, 260 candidates, 240 CTAs: 37.0 against 42.1 us; 120 heads, 155 candidates, 120 CTAs: 30.7 -> 19.0).
+// Where clusters would have to wait, both shapes by lines through what they took (23 to 48 heads, 81 to 169 queries, 102 to 311
+// candidates; 4 %): 23 heads x 64, 169 queries, 311 candidates, clusters of 6 and of 3: 26.7 and 39.9 us with 24 keys in the heads that
+// wait, 35.3 and 39.9 with 103, 41.0 and 40.2 with 155; 36 heads x 128, 100 queries, clusters of 4 and of 2: 30.2 and 32.5 with
+// 18 keys, 42.6 and 32.8 with 90.  Where the smaller ones do not fit shared memory the launches of their own are faster (27
+// heads x 128, 144 queries 35.1 against 35 to 47).
+template <typename Smem, typename Places>
+bool step_shape_f32(const StepSizes& z, StepShape& s, int tiles, Smem smem, Places places) {
+  const int heads = z.heads_of[0] + z.heads_of[1], cand = std::max(z.heads_of[0] ? z.cand[0] : 0, z.heads_of[1] ? z.cand[1] : 0);
+  StepShape smaller;
+  const int waiting = split_and_place(s, smaller, heads, tiles, z.sms, smem, places);
+  if (waiting > 0) {
+    const int kept = std::max(z.heads_of[0] ? z.kept[0] : 0, z.heads_of[1] ? z.kept[1] : 0);
+    const int last = z.kept[z.heads_of[1] >= waiting ? 1 : 0];
+    const int keys = 32 << s.log_splits, keys_smaller = 32 << smaller.log_splits;   // of a turn of the warps
+    const int more = (last + keys - 1) / keys - 1, turns = (kept + keys_smaller - 1) / keys_smaller;
+    const float part = (float)last / keys, past = cand > 128 ? 3.f : 0.f;
+    const float two_waves = z.head_dim == 64 ? 18.3f + 0.02f * cand + 4.5f * part + 3.f * more : 27.7f + 6.7f * part + 4.5f * more + 2.f * past;
+    const float one_wave = z.head_dim == 64 ? 9.3f + 3.05f * turns : 15.3f + 4.3f * turns + past;
+    const bool evicts = z.trig[0] || z.trig[1];
+    if (smaller.ctas < 0) return false;
+    if (smaller.ctas > 0 && (!evicts || 1.03f * two_waves > one_wave)) s = smaller;
+  }
+  return smem(s) <= kSmemCta && (cand <= 128 || heads * s.ctas <= z.sms);
+}
+
+}  // namespace small_step
 }  // namespace hack

@@ -16,7 +16,7 @@
 // stands for (compression on tcgen05, then attention) wait for each other and each pay a launch, a trip to
 // memory and a tail.
 // Step of 16 heads x 64, 36 queries, 91 candidates: 12.6 -> 5.9 us (169 queries, 237 candidates: 14.6 -> 7.6);
-// 256 heads: 18.2 -> 9.3.  More work per head goes to the two launches (step_small_pays).  The cluster
+// 256 heads: 18.2 -> 9.3.  More work per head goes to the two launches (step_shape_bf16).  The cluster
 // barrier without memory ordering took 0.45 us off a step, the merge in a form per number of warps 0.25.
 // Rounded probabilities (one product instead of two) where the larger kernel's would be rounded as well:
 // 5 to 15 % slower from eight turns on, the rounding costs more issue slots than the products.
@@ -379,38 +379,6 @@ step_small_kernel(const StepArgs a, const __nv_bfloat16* __restrict__ q, const _
   else combine(std::integral_constant<int, 1>());
 }
 
-// Microseconds of this launch and of the two launches it stands for (compression, then attention).  Both
-// forms were fitted to 287 steps of 8 to 256 heads, 16 to 400 queries and 50 to 700 candidates (rms 8 and 6 %).
-// This side has become faster since the fit where every CTA has an SM and a cluster is smaller than eight, so there it
-// is taken up to a tenth past the line, to 256 queries: 13 heads x 128, 121 queries 20.5 -> 15.7 us, 36 heads, 169 queries
-// 22.2 -> 18.4, 52 heads x 64, 196 queries 22.5 -> 19.1.  Elsewhere it keeps a margin of a tenth (81 heads x 64, 169 queries
-// 20.5 against 24.6; 18 heads, 400 queries 21.2 against 22.5).  16 heads x 64, 36 queries, 91 candidates: 5.9 against 12.6;
-// 256 heads: 9.3 against 18.2; 100 queries, 168 and 255 candidates: 7.3 against 12.8 (16 heads), 20.2 against
-// 19.9 (256 heads: not taken); 16 heads x 128, 36 queries, 91 candidates: 7.5 against 15.0; 256 heads: 18.6
-// against 25.2.
-template <int D>
-bool step_small_pays(const StepArgs& a, const StepShape& s, int per_sm) {
-  const float sms = (float)sm_count(), heads = (float)(a.batch * a.n_heads), ctas = heads * s.ctas;
-  const int splits = 1 << s.log_splits;
-  float longest = 0.f, mean = 0.f, work = 0.f, ranked = 0.f;
-  for (int t = 0; t < 2; ++t) {
-    if (a.heads_of[t] == 0) continue;
-    const int turns = (a.kept[t] + 2 * kTile * splits - 1) / (2 * kTile * splits);
-    const float us = 2.1f + (a.trig[t] && a.kept[t] < a.cand[t] ? 3.5f : 0.f) + 0.031f * (a.cand[t] * D * 4 / 1000.f) +
-                     (D == 64 ? 0.92f : 1.81f) * turns;
-    longest = std::max(longest, us);
-    mean += us * a.heads_of[t] / heads;
-    work += (float)a.heads_of[t] * ((a.n_new + 127) / 128) * (1 + (a.kept[t] + 127) / 128);
-    if (a.trig[t]) ranked = std::max(ranked, a.cand[t] / 128.f);
-  }
-  // two CTAs on an SM slow each other down by two thirds
-  const float here = std::max(longest * (per_sm == 2 ? 1.f + 0.67f * std::min(1.f, std::max(0.f, ctas / sms - 1.f)) : 1.f),
-                              ctas > sms * per_sm ? mean * (ctas / (sms * per_sm) * (per_sm == 2 ? 1.67f : 1.f) + 0.3f) : 0.f);
-  const float apart = D == 64 ? 10.8f + (1.58f * heads + 0.92f * work) / sms + 1.57f * ranked
-                              : 11.9f + (3.92f * heads + 1.13f * work) / sms + 1.94f * ranked;
-  return here * (ctas <= sms && s.ctas < kMaxCtas && a.n_new <= 256 ? 0.9f : 1.1f) < apart;
-}
-
 template <int D>
 int launch_t(const StepArgs& a, const void* q, const void* k_new, const void* v_new, void* out, cudaStream_t st) {
   const int heads = a.batch * a.n_heads, tiles = (a.n_new + kTile - 1) / kTile;
@@ -420,12 +388,12 @@ int launch_t(const StepArgs& a, const void* q, const void* k_new, const void* v_
   s.rows = (cand + kTile - 1) / kTile * kTile;
   const int ranked = std::max(a.trig[0] ? a.cand[0] : 0, a.trig[1] ? a.cand[1] : 0);
   const int turns = (ranked + kStepWarps * kTile - 1) / (kStepWarps * kTile);
+  const StepSizes sizes{D, a.n_new, a.heads_of, a.cand, a.kept, a.trig, sm_count()};
   auto go = [&](auto kern) {
     if (!allow_dynamic_smem(kern, kSmemCta)) return -1;
-    split_and_place(s, heads, tiles, reinterpret_cast<const void*>(kern), step_smem<D>);
-    const size_t smem = step_smem<D>(s);
-    if (smem > kSmemCta || !step_small_pays<D>(a, s, D == 64 && turns <= 4 && smem <= kSmemHalf ? 2 : 1)) return 0;
-    return launch_step<__nv_bfloat16>(kern, a, s, smem, q, k_new, v_new, out, st);
+    const auto places = [&](int ctas, size_t smem) { return cluster_places(reinterpret_cast<const void*>(kern), ctas, kStepThreads, smem); };
+    if (!step_shape_bf16(sizes, s, tiles, turns, step_smem<D>, places)) return 0;
+    return launch_step<__nv_bfloat16>(kern, a, s, step_smem<D>(s), q, k_new, v_new, out, st);
   };
   if (turns <= 1) return go(step_small_kernel<D, 1>);
   if (turns <= 2) return go(step_small_kernel<D, 2>);

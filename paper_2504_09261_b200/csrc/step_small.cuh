@@ -3,52 +3,12 @@
 #pragma once
 
 #include "hack_internal.h"
+#include "launch_plans.h"
 
 namespace hack {
 namespace small_step {
 
-constexpr int kStepWarps = 8;
-constexpr int kStepThreads = kStepWarps * 32;
-constexpr int kMaxRows = 768;                   // candidates of a head, at most
-constexpr int kMaxTiles = 8;                    // query tiles of a CTA
-constexpr int kMaxCtas = 8;                     // CTAs per head
 constexpr int kRangeBins = 256;                 // bins of the selection's histogram; one more for protected rows
-constexpr size_t kSmemCta = 216 * 1024;         // dynamic shared memory beside the static tables ...
-constexpr size_t kSmemHalf = 108 * 1024;        // ... and with two CTAs on an SM
-
-struct StepShape {
-  int ctas;        // CTAs per head
-  int tiles;       // query tiles per CTA: 1, 2, 4 or 8; the CTA's 8 warps share the keys of a tile 8 / tiles ways
-  int log_splits;  // log2(8 / tiles)
-  int rows;        // candidate rows shared memory has room for
-};
-
-// The CTAs of a head and their query tiles: as many CTAs per head as leave every CTA an SM, at least what its
-// queries need; clusters of seven and eight only where they are few (16 clusters of 8 CTAs do not find a
-// place at once beside each other: 100 queries, 16 heads, bf16: 7 CTAs 8.5 us, 4 CTAs 7.9; 169 queries:
-// 6 CTAs 8.2, 3 CTAs 10.3).
-inline void split_queries(StepShape& s, int heads, int tiles, int at_most = kMaxCtas) {
-  auto split = [&](int most) {
-    int want = sm_count() / heads < tiles ? sm_count() / heads : tiles;
-    want = want < 1 ? 1 : want > most ? most : want;
-    for (s.tiles = 1; s.tiles < kMaxTiles && s.tiles * want < tiles; s.tiles *= 2) {}
-    s.ctas = (tiles + s.tiles - 1) / s.tiles;
-  };
-  split(at_most);
-  if (s.ctas > 6 && heads * s.ctas * 2 > sm_count()) split(kMaxCtas / 2);
-  for (s.log_splits = 0; s.tiles << s.log_splits < kStepWarps; ++s.log_splits) {}
-}
-
-// split_queries, with smaller clusters where those meant to run at once would not all find a place (the SMs of a
-// processing cluster are no multiple of every size: 148 SMs take 45 clusters of 3, 33 of 4, 22 of 6).  A second wave doubles
-// the step: 46 heads x 128, 81 queries 17.1 -> 12.3 us; 35 heads, 121 queries 17.4 -> 13.0; 24 heads, 81
-// queries 16.0 -> 10.2 (fp32 37.2 -> 25.9).
-template <typename Smem>
-void split_and_place(StepShape& s, int heads, int tiles, const void* kern, Smem smem) {
-  split_queries(s, heads, tiles);
-  for (int most = s.ctas - 1; most >= 1 && heads * s.ctas <= sm_count() && heads > cluster_places(kern, s.ctas, kStepThreads, smem(s) <= kSmemHalf ? kSmemHalf : kSmemCta); --most)
-    split_queries(s, heads, tiles, most);
-}
 
 template <typename T, typename... KArgs>
 int launch_step(void (*kern)(KArgs...), const StepArgs& a, const StepShape& s, size_t smem, const void* q, const void* k_new,

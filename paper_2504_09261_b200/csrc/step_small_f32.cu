@@ -396,15 +396,13 @@ int launch_t(const StepArgs& a, const void* q, const void* k_new, const void* v_
   if (cand > (ranked ? kMaxCand : kMaxAppend) || (!ranked && a.n_new < kMinAppend) || tiles > kMaxTiles * kMaxCtas) return 0;
   StepShape s;
   s.rows = (cand + 3) / 4 * 4;
-  // launches of longer heads only where every CTA has an SM to itself (120 heads x 64, 260 candidates, 240 CTAs:
-  // 37.0 against 42.1 us; 120 heads, 155 candidates, 120 CTAs: 30.7 -> 19.0)
+  const StepSizes sizes{D, a.n_new, a.heads_of, a.cand, a.kept, a.trig, sm_count()};
   auto go = [&](auto kern) {
     if (!allow_dynamic_smem(kern, kSmemCta)) return -1;
     const auto bytes = [](const StepShape& of) -> size_t { return Layout<D>(of.rows, of.tiles).total; };
-    split_and_place(s, heads, tiles, reinterpret_cast<const void*>(kern), bytes);
-    const size_t smem = bytes(s);
-    if (smem > kSmemCta || (cand > 2 * kKeyWarps * kKeys && heads * s.ctas > sm_count())) return 0;
-    return launch_step<float>(kern, a, s, smem, q, k_new, v_new, out, st);
+    const auto places = [&](int ctas, size_t smem) { return cluster_places(reinterpret_cast<const void*>(kern), ctas, kStepThreads, smem); };
+    if (!step_shape_f32(sizes, s, tiles, bytes, places)) return 0;
+    return launch_step<float>(kern, a, s, bytes(s), q, k_new, v_new, out, st);
   };
   if (ranked <= 2 * kKeyWarps * kKeys) return go(step_small_f32_kernel<D, 2>);
   if constexpr (D == 64) {                      // at head_dim 128 shared memory holds fewer rows than four turns rank

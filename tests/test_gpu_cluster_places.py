@@ -36,3 +36,16 @@ def test_heads_at_the_places_of_small_clusters(head_dim, heads, dtype):
     rep = run_parity(cfg, [0], fused=True, heads_per_layer=4, policy=1)
     assert rep.ok(), rep.problems[:5]
     assert rep.compressed_heads > 0
+
+
+@pytest.mark.parametrize("dtype,head_dim,heads,sides,b_c,b_s", [
+    ("bf16", 128, 46, (1, 2, 5, 12), 20, 166), ("fp32", 64, 24, (1, 2, 4, 7, 13), 24, 231), ("fp32", 128, 36, (1, 2, 4, 10), 18, 113),
+])
+def test_contextual_heads_that_wait_for_the_first_clusters(dtype, head_dim, heads, sides, b_c, b_s):
+    """One launch whose last clusters, contextual heads of few keys, start when the first ones have ended."""
+    from parity_util import run_parity
+    base = get_config(0) if dtype == "fp32" else get_config(3 if head_dim == 128 else 1, n_layers=1)
+    cfg = replace(base, name=f"waiting-{heads}", n_heads=heads, batch=1, head_dim=head_dim, sides=sides, budget_c=b_c, budget_s=b_s)
+    rep = run_parity(cfg, [0], fused=True, heads_per_layer=8, policy=1)
+    assert rep.ok(), rep.problems[:5]
+    assert rep.evicting_launches[-1] == 1, rep.evicting_launches
