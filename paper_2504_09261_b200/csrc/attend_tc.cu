@@ -147,28 +147,27 @@ struct Bars {
   uint64_t v_full[kVStages], v_empty[kVStages];
   uint64_t s_full[2], s_free, p_full[2], p_free[2];
   uint64_t copy_full[2];                            // append: a chunk of new rows has landed in its staging half
-  uint64_t drain;
+  uint64_t drain[2];                                // the issuers' last products
   int2 out_at[8];                                   // per softmax warp
   uint32_t tmem_base;
   int abort_code;                                   // of the wait that gave up
-  int held;                                         // the producer waits for the launch ahead
+  long long limit[2];                               // of a wait, and of one for a unit of work; none while the producer is held up
 };
 
 // Waits for a phase of a barrier; false once the limit has passed or another wait of the CTA has given up.  In
 // little code: the instruction cache bounds this kernel (with waits of 40 instructions, 82 instead of 40 KB in
-// all, the loop lost 40 % at head_dim 64).  The status word is written at the end, by one thread.  Time in which the
-// producer waits for the launch ahead does not count: that is not this launch's.
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Bars* b, int code, long long limit) {
+// all, the loop lost 40 % at head_dim 64).  The status word is written at the end, by one thread.  The limit is read anew in
+// every turn: there is none while the producer waits for the launch ahead, whose time is not this launch's (the same
+// with that time taken off in here, 20 more instructions a wait: 33.6 -> 35.0 us a step of 256 heads x 64).
+__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Bars* b, int code, const volatile long long* limit) {
   const uint32_t addr = smem_u32(bar);
   if (__builtin_expect(mbar_try_wait(addr, parity), 1)) return true;
   volatile int* const flag = &b->abort_code;
-  long long t0 = clock64();
+  const long long t0 = clock64();
 #pragma unroll 1
   while (!mbar_try_wait(addr, parity)) {
     if (*flag) return false;
-    const long long now = clock64();
-    if (*static_cast<volatile int*>(&b->held)) t0 = now;
-    else if (now - t0 > limit) *flag = code;
+    if (clock64() - t0 > *limit) *flag = code;
   }
   return true;
 }
@@ -197,7 +196,6 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   Bars* bars = reinterpret_cast<Bars*>(sm + (T + kKStages + kVStages) * TILE_BYTES + 2 * kCopyChunk);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long wlim = p.wait_cycles;
 
   // Unit number x of the launch: those of the first head type, then those of the other one.
   auto make_unit = [&](int x) {
@@ -212,7 +210,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     return u;
   };
   // A role takes unit number n of this CTA (one thread; the arrival gives the slot back).
-  auto wait_unit = [&](int n) { return wait_bar(&bars->u_full[n & 1], (n >> 1) & 1, bars, 13, p.unit_cycles); };
+  auto wait_unit = [&](int n) { return wait_bar(&bars->u_full[n & 1], (n >> 1) & 1, bars, 13, &bars->limit[1]); };
   auto read_unit = [&](int n) {
     const volatile Unit& v = bars->unit[n & 1];
     return Unit{v.bh, v.part, v.type, v.krow};
@@ -232,12 +230,15 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   // Keys of the last block of a segment of `len` rows in groups of 32, the unit in which the products and the
   // softmax leave out what is past the last key
   auto last_groups = [](int len) { return (((len - 1) & (kBN - 1)) >> 5) + 1; };
-  // The producer's wait for the launch ahead
-  auto wait_ahead = [&]() {
-    volatile int* const held = &bars->held;
-    *held = 1;
-    pdl_grid_wait();
-    *held = 0;
+  // The producer's wait for the launch ahead lifts the limits; afterwards a wait that began before it has as much more time.
+  auto set_limits = [&](long long held) {
+    volatile Bars* const v = bars;
+    v->limit[0] = p.wait_cycles + held;
+    v->limit[1] = p.unit_cycles + held;
+  };
+  auto lift_limits = [&]() {
+    volatile Bars* const v = bars;
+    v->limit[0] = v->limit[1] = std::numeric_limits<long long>::max();
   };
   // Loads of the producer: a tile of 128 rows (the queries of slot t, or K / V block j of the unit)
   auto load_tile = [&](uint32_t dst, const CUtensorMap* tm, int row, uint64_t* bar) {
@@ -268,9 +269,11 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     mbar_init(smem_u32(&bars->s_free), 4);          // the four warps of the tile whose logits were in the buffer
     mbar_init(smem_u32(&bars->copy_full[0]), 1);
     mbar_init(smem_u32(&bars->copy_full[1]), 1);
-    mbar_init(smem_u32(&bars->drain), 2);           // the two issuers
+    mbar_init(smem_u32(&bars->drain[0]), 1);
+    mbar_init(smem_u32(&bars->drain[1]), 1);
     bars->abort_code = 0;
-    bars->held = 1;                                 // until the first loads are on their way
+    if (T == 2) lift_limits();                      // (the other warps run ahead of the wait for the first loads)
+    else set_limits(0);
     fence_barrier_init();
     fence_proxy_async();
   }
@@ -298,11 +301,13 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       for (int t = 0; t < ntile; ++t) load_tile(q_sm + t * TILE_BYTES, &tm_q, u.bh * p.n_new + q0 + t * kBM, &bars->q_full[t]);
     };
     if (p.q_before_wait) load_queries();
+    const long long t0 = clock64();
     if (dep == kDepAll || (dep == kDepCache && nb == 0)) pdl_grid_wait();
-    *static_cast<volatile int*>(&bars->held) = 0;
+    const long long t1 = clock64();
     if (!p.q_before_wait) load_queries();
     load_kv(u, 0, nb, 0, 0);
     load_kv(u, 0, nb, 0, 1);
+    if (T == 2) set_limits(t1 - t0);
   }
   if (warp == kMmaWarp) {
     tmem_alloc(smem_u32(&bars->tmem_base), Shape<T>::kTmemCols);
@@ -319,6 +324,12 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   // Everything above overlaps the tail of the previous kernel.  What waits for that kernel is the
   // producer (and so everything behind the tiles it loads) and the append.
 
+  // An issuer leaves when its last product has ended, or after a while: a softmax thread that gave up waits for none.
+  auto drained = [&](uint64_t* bar) {
+    mma_commit(smem_u32(bar));
+#pragma unroll 1
+    for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(smem_u32(bar), 0); ++it) {}
+  };
   if (warp == kPvWarp) {
     // ------------------------------------------------------------------ issuer of the P V products
     // (a thread of its own: one thread issuing both products was the bottleneck of the CTA)
@@ -348,9 +359,9 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 #pragma unroll 1
             for (int t = 0; t < ntile; ++t) {
               // (what comes last is the wait whose end something waits for)
-              if (t == 0 && r == 0) ok = wait_bar(&bars->v_full[vs], ((g + j) / kVStages) & 1, bars, 6, wlim);
+              if (t == 0 && r == 0) ok = wait_bar(&bars->v_full[vs], ((g + j) / kVStages) & 1, bars, 6, &bars->limit[0]);
               const uint32_t o = tmem + O_COL + t * D, pa = tmem + P_COL + t * 64;
-              if (!ok || !wait_bar(&bars->p_full[t], (odd >> t) & 1, bars, 5, wlim)) { ok = false; break; }
+              if (!ok || !wait_bar(&bars->p_full[t], (odd >> t) & 1, bars, 5, &bars->limit[0])) { ok = false; break; }
               tc_fence_after();
               if (kg == 4) {
                 mma_ts_chain4(o, pa, vd, IDESC_PV, j > 0);
@@ -367,6 +378,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         }
         g += nblk;
       }
+      drained(&bars->drain[1]);
     }
   } else if (warp == kAppendWarp) {
     reg_dec<kOtherRegs>();
@@ -408,7 +420,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             bulk_wait_read<1>();                     // the store that last read this half (two chunks ago) is done with it
             mbar_expect_tx(bar, bytes);
             bulk_load(copy_sm + half * kCopyChunk, src + (size_t)ch * kCopyChunk, bytes, bar);
-            ok = wait_bar(&bars->copy_full[half], (chunks >> 1) & 1, bars, 12, wlim);
+            ok = wait_bar(&bars->copy_full[half], (chunks >> 1) & 1, bars, 12, &bars->limit[0]);
             if (!ok) {                               // the copy gets a bounded chance to land before the CTA leaves
 #pragma unroll 1
               for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(bar, (chunks >> 1) & 1); ++it) {}
@@ -433,11 +445,18 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 #pragma unroll 1
       for (int n = 0;; ++n) {
         const int nb = blocks_b(u), nblk = blocks(u), nr = rounds_of(u), dep = p.dep[u.type];
-        if (n > 0 && (dep == kDepAll || (dep == kDepCache && nb == 0))) wait_ahead();
+        bool ahead = n > 0 && (dep == kDepAll || (dep == kDepCache && nb == 0));   // the launch ahead has to be done first
         // K / V tiles of the unit in order, and the queries of round r ahead of step r's value tile
 #pragma unroll 1
         for (int j = 0; j < max(nblk, nr) && ok; ++j) {
-          if (dep == kDepCache && j == nb && j < nblk) wait_ahead();   // the head's stored survivors are in place
+          ahead = ahead || (dep == kDepCache && j == nb && j < nblk);   // (the head's stored survivors are in place then)
+          if (ahead) {
+            const long long t0 = clock64();
+            lift_limits();
+            pdl_grid_wait();
+            set_limits(clock64() - t0);
+            ahead = false;
+          }
           const bool fresh = n > 0 || j > 0;        // the first tiles and queries of the CTA are on their way already
           const uint32_t gs = g + j;
 #pragma unroll 1
@@ -447,7 +466,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 #pragma unroll 1
               for (int t = 0; t < ntile && ok; ++t) {
                 if (fresh) {
-                  if (q_issued >> t & 1) ok = wait_bar(&bars->q_free[t], ((q_odd >> t) & 1) ^ 1, bars, 14, wlim);
+                  if (q_issued >> t & 1) ok = wait_bar(&bars->q_free[t], ((q_odd >> t) & 1) ^ 1, bars, 14, &bars->limit[0]);
                   if (!ok) break;
                   load_tile(q_sm + t * TILE_BYTES, &tm_q, u.bh * p.n_new + q0 + t * kBM, &bars->q_full[t]);
                 }
@@ -457,7 +476,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             }
             if (!ok || !fresh || j >= nblk) continue;
             const uint32_t sl = gs % kKStages;      // (both rings have the same depth)
-            ok = wait_bar(kv ? &bars->v_empty[sl] : &bars->k_empty[sl], ((gs / kKStages) & 1) ^ 1, bars, 1 + kv, wlim);
+            ok = wait_bar(kv ? &bars->v_empty[sl] : &bars->k_empty[sl], ((gs / kKStages) & 1) ^ 1, bars, 1 + kv, &bars->limit[0]);
             if (!ok) break;
             load_kv(u, j, nb, sl, kv);
             if (kv) ++issued_v;
@@ -473,7 +492,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           mbar_expect_tx(smem_u32(&bars->asked), 16);
           clc_ask(smem_u32(&bars->answer), smem_u32(&bars->asked));
           pending = true;
-          ok = wait_bar(&bars->asked, answers & 1, bars, 15, wlim);
+          ok = wait_bar(&bars->asked, answers & 1, bars, 15, &bars->limit[0]);
           if (!ok) break;
           pending = false;
           ++answers;
@@ -481,7 +500,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           fence_proxy_async();                       // the next answer overwrites what was just read
           if (x >= 0) next = make_unit(x);
         }
-        if (n > 0) ok = wait_bar(&bars->u_empty[(n + 1) & 1], (((n + 1) >> 1) & 1) ^ 1, bars, 16, p.unit_cycles);
+        if (n > 0) ok = wait_bar(&bars->u_empty[(n + 1) & 1], (((n + 1) >> 1) & 1) ^ 1, bars, 16, &bars->limit[1]);
         if (!ok) break;
         bars->unit[(n + 1) & 1] = next;
         mbar_arrive(smem_u32(&bars->u_full[(n + 1) & 1]));
@@ -537,12 +556,12 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 #pragma unroll 1
             for (int t = 0; t < ntile; ++t) {
               if (j == 0) {
-                ok = wait_bar(&bars->q_full[t], (q_odd >> t) & 1, bars, 3, wlim);
+                ok = wait_bar(&bars->q_full[t], (q_odd >> t) & 1, bars, 3, &bars->limit[0]);
                 q_odd ^= 1u << t;
               }
-              if (ok && t == 0 && r == 0) ok = wait_bar(&bars->k_full[ks], ((g + j) / kKStages) & 1, bars, 4, wlim);
+              if (ok && t == 0 && r == 0) ok = wait_bar(&bars->k_full[ks], ((g + j) / kKStages) & 1, bars, 4, &bars->limit[0]);
               const uint64_t qd = q_desc0 + (uint64_t)((t * TILE_BYTES) >> 4);
-              if (!ok || !wait_bar(&bars->s_free, (use - 1) & 1, bars, 10, wlim)) { ok = false; break; }   // (a fresh barrier passes for odd)
+              if (!ok || !wait_bar(&bars->s_free, (use - 1) & 1, bars, 10, &bars->limit[0])) { ok = false; break; }   // (a fresh barrier passes for odd)
               tc_fence_after();
               if constexpr (D == 128) mma_ss_chain8(tmem + S_COL, qd, kd, idesc, 0);
               else mma_ss_chain4(tmem + S_COL, qd, kd, idesc, 0);
@@ -555,6 +574,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         }
         g += nblk;
       }
+      drained(&bars->drain[0]);
     }
   } else {
     // ------------------------------------------------------------------ softmax + epilogue
@@ -570,7 +590,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     uint32_t cnt = 0;                              // blocks of this tile so far
     bool ok = true, pending = false;               // pending: a round's output is still in tensor memory
     volatile int2* const out_at = &bars->out_at[warp - 4];   // of the round in work or pending: first row of its head, row of the tile
-    auto bar_all = [&](uint64_t* bar, uint32_t parity, int code) { return __all_sync(0xffffffffu, wait_bar(bar, parity, bars, code, wlim)) != 0; };
+    auto bar_all = [&](uint64_t* bar, uint32_t parity, int code) { return __all_sync(0xffffffffu, wait_bar(bar, parity, bars, code, &bars->limit[0])) != 0; };
     // Output of the round that ended.  A thread writes its own row, 32 bytes (a whole sector) an instruction,
     // straight from tensor memory: through the query tile's shared memory and a tiled store, the next round's
     // queries could not be on their way meanwhile.
@@ -745,15 +765,6 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   }
   tc_fence_before();
   __syncthreads();
-  if (bars->abort_code) {
-    // after a wait that gave up: the products in flight, of either issuer, get a bounded chance to end before tensor memory is freed
-    if ((warp == kMmaWarp || warp == kPvWarp) && lane == 0) {
-      mma_commit(smem_u32(&bars->drain));
-#pragma unroll 1
-      for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(smem_u32(&bars->drain), 0); ++it) {}
-    }
-    __syncthreads();
-  }
   if (warp == kMmaWarp) {
     tc_fence_after();
     tmem_dealloc(tmem, Shape<T>::kTmemCols);
@@ -879,12 +890,13 @@ int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_sta
   p.head_dim_pieces = a.head_dim * 2 / 16;
   p.cap[0] = a.cap[0];
   p.cap[1] = a.cap[1];
-  p.wait_cycles = a.wait_cycles;
+  constexpr long long kMost = std::numeric_limits<long long>::max() / 4;
+  p.wait_cycles = std::min(a.wait_cycles, kMost);
   // a block takes a role no more than eight waits
   long long unit_waits = 0;
   for (int t = 0; t < 2; ++t)
     unit_waits = std::max<long long>(unit_waits, 8ll * p.rounds[t] * ((p.len_a[t] + kBN - 1) / kBN + (p.len_b[t] + kBN - 1) / kBN + 1));
-  p.unit_cycles = a.wait_cycles > std::numeric_limits<long long>::max() / unit_waits ? a.wait_cycles : a.wait_cycles * unit_waits;
+  p.unit_cycles = p.wait_cycles > kMost / unit_waits ? kMost : p.wait_cycles * unit_waits;
   p.k_plane = static_cast<uint4*>(a.k_plane);
   p.v_plane = static_cast<uint4*>(a.v_plane);
   p.pos_plane = a.pos_plane;
