@@ -265,8 +265,9 @@ HACK_API hack_status_t hack_stage_times(hack_cache_t* cache, double* ms, uint64_
 HACK_API hack_status_t hack_poll_status(hack_cache_t* cache, void* stream);
 /* Limit, in SM clock cycles, of every bounded device-side wait (mbarrier waits of the tensor-core
  * kernels) in launches made through this cache from now on; 0 restores the default of about one
- * second.  What counts is a launch's own time: not that in which it waits for the launch ahead of it in the
- * stream, and waits for a whole unit of work of the attention get the limit once per wait in it.  A wait that outlasts the limit raises the status word (hack_poll_status then returns
+ * second.  What counts is a launch's own time, not that in which it waits for the launch ahead of it
+ * in the stream; waits for a whole unit of work of the attention get the limit once per wait in it.
+ * A wait that outlasts the limit raises the status word (hack_poll_status then returns
  * HACK_ERR_TIMEOUT), the CTA drains what it has in flight, frees its tensor memory and returns; the
  * results of that launch are undefined and the cache should be reset.  Meant for tests of that path
  * (a limit of a few cycles makes the first wait that is not already satisfied give up) and for

@@ -97,6 +97,7 @@ template <> struct Shape<1> {
 constexpr int kKStages = 2;
 constexpr int kVStages = 2;
 constexpr uint32_t kSpinLimit = 1u << 22;          // polls while draining after an abort
+constexpr uint32_t kWaitPolls = 1u << 28;          // polls of a wait without a clock, minutes
 constexpr float kRescaleThreshold = 32.0f;   // log2 units: p <= 2^32, far inside the bf16 / fp32 range
 
 struct TcParams {
@@ -114,8 +115,8 @@ struct TcParams {
   int pos_base;                          // global position of the new scale's first token
   int head_dim_pieces;                   // 16-byte pieces per row
   int cap[2];                            // rows a head of each type owns (checked builds)
-  long long wait_cycles;                 // limit of every mbarrier wait ...
-  long long unit_cycles;                 // ... but those for another role to be done with a unit of work
+  long long wait_cycles;                 // limit of the producer's waits ...
+  long long unit_cycles;                 // ... but those for other roles to be done with a unit of work
   uint4* k_plane;                        // cache planes of this layer (append only)
   uint4* v_plane;
   int32_t* pos_plane;
@@ -151,15 +152,26 @@ struct Bars {
   int2 out_at[8];                                   // per softmax warp
   uint32_t tmem_base;
   int abort_code;                                   // of the wait that gave up
-  long long limit[2];                               // of a wait, and of one for a unit of work; none while the producer is held up
 };
 
-// Waits for a phase of a barrier; false once the limit has passed or another wait of the CTA has given up.  In
-// little code: the instruction cache bounds this kernel (with waits of 40 instructions, 82 instead of 40 KB in
-// all, the loop lost 40 % at head_dim 64).  The status word is written at the end, by one thread.  The limit is read anew in
-// every turn: there is none while the producer waits for the launch ahead, whose time is not this launch's (the same
-// with that time taken off in here, 20 more instructions a wait: 33.6 -> 35.0 us a step of 256 heads x 64).
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Bars* b, int code, const volatile long long* limit) {
+// Waits for a phase of a barrier; false once a wait of the CTA has given up.  In little code: the instruction cache bounds
+// this kernel (with waits of 40 instructions, 82 instead of 40 KB in all, the loop lost 40 % at head_dim 64).  The producer keeps the
+// time: whatever else stands still, one of its own waits soon does too, and while it waits for the launch ahead, whose time is not this
+// launch's, nobody's counts.  (A clock in every wait that leaves that time out: 33.6 -> 35.0 us a step of 256 heads x 64.)  The status
+// word is written at the end, by one thread.
+__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Bars* b, int code) {
+  const uint32_t addr = smem_u32(bar);
+  if (__builtin_expect(mbar_try_wait(addr, parity), 1)) return true;
+  volatile int* const flag = &b->abort_code;
+#pragma unroll 1
+  for (uint32_t polls = kWaitPolls; !mbar_try_wait(addr, parity); --polls) {
+    if (*flag) return false;
+    if (polls == 0) *flag = code;
+  }
+  return true;
+}
+// The same with a limit in clock cycles.
+__device__ __forceinline__ bool wait_timed(uint64_t* bar, uint32_t parity, Bars* b, int code, long long limit) {
   const uint32_t addr = smem_u32(bar);
   if (__builtin_expect(mbar_try_wait(addr, parity), 1)) return true;
   volatile int* const flag = &b->abort_code;
@@ -167,7 +179,7 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Bars* b
 #pragma unroll 1
   while (!mbar_try_wait(addr, parity)) {
     if (*flag) return false;
-    if (clock64() - t0 > *limit) *flag = code;
+    if (clock64() - t0 > limit) *flag = code;
   }
   return true;
 }
@@ -210,7 +222,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     return u;
   };
   // A role takes unit number n of this CTA (one thread; the arrival gives the slot back).
-  auto wait_unit = [&](int n) { return wait_bar(&bars->u_full[n & 1], (n >> 1) & 1, bars, 13, &bars->limit[1]); };
+  auto wait_unit = [&](int n) { return wait_bar(&bars->u_full[n & 1], (n >> 1) & 1, bars, 13); };
   auto read_unit = [&](int n) {
     const volatile Unit& v = bars->unit[n & 1];
     return Unit{v.bh, v.part, v.type, v.krow};
@@ -230,16 +242,6 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   // Keys of the last block of a segment of `len` rows in groups of 32, the unit in which the products and the
   // softmax leave out what is past the last key
   auto last_groups = [](int len) { return (((len - 1) & (kBN - 1)) >> 5) + 1; };
-  // The producer's wait for the launch ahead lifts the limits; afterwards a wait that began before it has as much more time.
-  auto set_limits = [&](long long held) {
-    volatile Bars* const v = bars;
-    v->limit[0] = p.wait_cycles + held;
-    v->limit[1] = p.unit_cycles + held;
-  };
-  auto lift_limits = [&]() {
-    volatile Bars* const v = bars;
-    v->limit[0] = v->limit[1] = std::numeric_limits<long long>::max();
-  };
   // Loads of the producer: a tile of 128 rows (the queries of slot t, or K / V block j of the unit)
   auto load_tile = [&](uint32_t dst, const CUtensorMap* tm, int row, uint64_t* bar) {
     mbar_expect_tx(smem_u32(bar), TILE_BYTES);
@@ -272,8 +274,6 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     mbar_init(smem_u32(&bars->drain[0]), 1);
     mbar_init(smem_u32(&bars->drain[1]), 1);
     bars->abort_code = 0;
-    if (T == 2) lift_limits();                      // (the other warps run ahead of the wait for the first loads)
-    else set_limits(0);
     fence_barrier_init();
     fence_proxy_async();
   }
@@ -301,13 +301,10 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       for (int t = 0; t < ntile; ++t) load_tile(q_sm + t * TILE_BYTES, &tm_q, u.bh * p.n_new + q0 + t * kBM, &bars->q_full[t]);
     };
     if (p.q_before_wait) load_queries();
-    const long long t0 = clock64();
     if (dep == kDepAll || (dep == kDepCache && nb == 0)) pdl_grid_wait();
-    const long long t1 = clock64();
     if (!p.q_before_wait) load_queries();
     load_kv(u, 0, nb, 0, 0);
     load_kv(u, 0, nb, 0, 1);
-    if (T == 2) set_limits(t1 - t0);
   }
   if (warp == kMmaWarp) {
     tmem_alloc(smem_u32(&bars->tmem_base), Shape<T>::kTmemCols);
@@ -359,9 +356,9 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 #pragma unroll 1
             for (int t = 0; t < ntile; ++t) {
               // (what comes last is the wait whose end something waits for)
-              if (t == 0 && r == 0) ok = wait_bar(&bars->v_full[vs], ((g + j) / kVStages) & 1, bars, 6, &bars->limit[0]);
+              if (t == 0 && r == 0) ok = wait_bar(&bars->v_full[vs], ((g + j) / kVStages) & 1, bars, 6);
               const uint32_t o = tmem + O_COL + t * D, pa = tmem + P_COL + t * 64;
-              if (!ok || !wait_bar(&bars->p_full[t], (odd >> t) & 1, bars, 5, &bars->limit[0])) { ok = false; break; }
+              if (!ok || !wait_bar(&bars->p_full[t], (odd >> t) & 1, bars, 5)) { ok = false; break; }
               tc_fence_after();
               if (kg == 4) {
                 mma_ts_chain4(o, pa, vd, IDESC_PV, j > 0);
@@ -420,7 +417,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             bulk_wait_read<1>();                     // the store that last read this half (two chunks ago) is done with it
             mbar_expect_tx(bar, bytes);
             bulk_load(copy_sm + half * kCopyChunk, src + (size_t)ch * kCopyChunk, bytes, bar);
-            ok = wait_bar(&bars->copy_full[half], (chunks >> 1) & 1, bars, 12, &bars->limit[0]);
+            ok = wait_timed(&bars->copy_full[half], (chunks >> 1) & 1, bars, 12, p.wait_cycles);
             if (!ok) {                               // the copy gets a bounded chance to land before the CTA leaves
 #pragma unroll 1
               for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(bar, (chunks >> 1) & 1); ++it) {}
@@ -445,18 +442,11 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 #pragma unroll 1
       for (int n = 0;; ++n) {
         const int nb = blocks_b(u), nblk = blocks(u), nr = rounds_of(u), dep = p.dep[u.type];
-        bool ahead = n > 0 && (dep == kDepAll || (dep == kDepCache && nb == 0));   // the launch ahead has to be done first
+        if (n > 0 && (dep == kDepAll || (dep == kDepCache && nb == 0))) pdl_grid_wait();
         // K / V tiles of the unit in order, and the queries of round r ahead of step r's value tile
 #pragma unroll 1
         for (int j = 0; j < max(nblk, nr) && ok; ++j) {
-          ahead = ahead || (dep == kDepCache && j == nb && j < nblk);   // (the head's stored survivors are in place then)
-          if (ahead) {
-            const long long t0 = clock64();
-            lift_limits();
-            pdl_grid_wait();
-            set_limits(clock64() - t0);
-            ahead = false;
-          }
+          if (dep == kDepCache && j == nb && j < nblk) pdl_grid_wait();   // the head's stored survivors are in place
           const bool fresh = n > 0 || j > 0;        // the first tiles and queries of the CTA are on their way already
           const uint32_t gs = g + j;
 #pragma unroll 1
@@ -466,7 +456,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 #pragma unroll 1
               for (int t = 0; t < ntile && ok; ++t) {
                 if (fresh) {
-                  if (q_issued >> t & 1) ok = wait_bar(&bars->q_free[t], ((q_odd >> t) & 1) ^ 1, bars, 14, &bars->limit[0]);
+                  if (q_issued >> t & 1) ok = wait_timed(&bars->q_free[t], ((q_odd >> t) & 1) ^ 1, bars, 14, p.wait_cycles);
                   if (!ok) break;
                   load_tile(q_sm + t * TILE_BYTES, &tm_q, u.bh * p.n_new + q0 + t * kBM, &bars->q_full[t]);
                 }
@@ -476,7 +466,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             }
             if (!ok || !fresh || j >= nblk) continue;
             const uint32_t sl = gs % kKStages;      // (both rings have the same depth)
-            ok = wait_bar(kv ? &bars->v_empty[sl] : &bars->k_empty[sl], ((gs / kKStages) & 1) ^ 1, bars, 1 + kv, &bars->limit[0]);
+            ok = wait_timed(kv ? &bars->v_empty[sl] : &bars->k_empty[sl], ((gs / kKStages) & 1) ^ 1, bars, 1 + kv, p.wait_cycles);
             if (!ok) break;
             load_kv(u, j, nb, sl, kv);
             if (kv) ++issued_v;
@@ -492,7 +482,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           mbar_expect_tx(smem_u32(&bars->asked), 16);
           clc_ask(smem_u32(&bars->answer), smem_u32(&bars->asked));
           pending = true;
-          ok = wait_bar(&bars->asked, answers & 1, bars, 15, &bars->limit[0]);
+          ok = wait_timed(&bars->asked, answers & 1, bars, 15, p.wait_cycles);
           if (!ok) break;
           pending = false;
           ++answers;
@@ -500,11 +490,14 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           fence_proxy_async();                       // the next answer overwrites what was just read
           if (x >= 0) next = make_unit(x);
         }
-        if (n > 0) ok = wait_bar(&bars->u_empty[(n + 1) & 1], (((n + 1) >> 1) & 1) ^ 1, bars, 16, &bars->limit[1]);
+        if (n > 0) ok = wait_timed(&bars->u_empty[(n + 1) & 1], (((n + 1) >> 1) & 1) ^ 1, bars, 16, p.unit_cycles);
         if (!ok) break;
         bars->unit[(n + 1) & 1] = next;
         mbar_arrive(smem_u32(&bars->u_full[(n + 1) & 1]));
-        if (next.bh < 0) break;
+        if (next.bh < 0) {                           // the roles leave on time as well
+          ok = wait_timed(&bars->u_empty[n & 1], (n >> 1) & 1, bars, 17, p.unit_cycles);
+          break;
+        }
         u = next;
       }
       if (!ok) {
@@ -556,12 +549,12 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 #pragma unroll 1
             for (int t = 0; t < ntile; ++t) {
               if (j == 0) {
-                ok = wait_bar(&bars->q_full[t], (q_odd >> t) & 1, bars, 3, &bars->limit[0]);
+                ok = wait_bar(&bars->q_full[t], (q_odd >> t) & 1, bars, 3);
                 q_odd ^= 1u << t;
               }
-              if (ok && t == 0 && r == 0) ok = wait_bar(&bars->k_full[ks], ((g + j) / kKStages) & 1, bars, 4, &bars->limit[0]);
+              if (ok && t == 0 && r == 0) ok = wait_bar(&bars->k_full[ks], ((g + j) / kKStages) & 1, bars, 4);
               const uint64_t qd = q_desc0 + (uint64_t)((t * TILE_BYTES) >> 4);
-              if (!ok || !wait_bar(&bars->s_free, (use - 1) & 1, bars, 10, &bars->limit[0])) { ok = false; break; }   // (a fresh barrier passes for odd)
+              if (!ok || !wait_bar(&bars->s_free, (use - 1) & 1, bars, 10)) { ok = false; break; }   // (a fresh barrier passes for odd)
               tc_fence_after();
               if constexpr (D == 128) mma_ss_chain8(tmem + S_COL, qd, kd, idesc, 0);
               else mma_ss_chain4(tmem + S_COL, qd, kd, idesc, 0);
@@ -590,7 +583,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     uint32_t cnt = 0;                              // blocks of this tile so far
     bool ok = true, pending = false;               // pending: a round's output is still in tensor memory
     volatile int2* const out_at = &bars->out_at[warp - 4];   // of the round in work or pending: first row of its head, row of the tile
-    auto bar_all = [&](uint64_t* bar, uint32_t parity, int code) { return __all_sync(0xffffffffu, wait_bar(bar, parity, bars, code, &bars->limit[0])) != 0; };
+    auto bar_all = [&](uint64_t* bar, uint32_t parity, int code) { return __all_sync(0xffffffffu, wait_bar(bar, parity, bars, code)) != 0; };
     // Output of the round that ended.  A thread writes its own row, 32 bytes (a whole sector) an instruction,
     // straight from tensor memory: through the query tile's shared memory and a tiled store, the next round's
     // queries could not be on their way meanwhile.
