@@ -184,7 +184,8 @@ __device__ __forceinline__ bool wait_timed(uint64_t* bar, uint32_t parity, Bars*
   return true;
 }
 
-template <int D, int T>
+// kAhead: the other warps do not wait behind the producer's wait for the launch ahead.
+template <int D, int T, bool kAhead = T == 2>
 __global__ void __launch_bounds__(Shape<T>::kThreads, Shape<T>::kCtasPerSm)
 attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kn,
@@ -277,11 +278,10 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (T == 2 && warp == kProducerWarp) {
+  if (kAhead && warp == kProducerWarp) {
     // The barriers are ready; the producer does not wait for the others, nor they for its wait for the launch ahead:
     // with all of them behind that wait, their code came in from L2 only then (3.0 instead of 2.1 us from the end of the
-    // compression to the first logits).  Not on half an SM, whose other half may be a CTA of the launch ahead that
-    // their polling slows down (240 heads x 64, 1 045 keys: 110 against 114 us a step).
+    // compression to the first logits).  On half an SM only where heads are few and short (launch_attend_tc).
     __syncwarp();
     asm volatile("bar.arrive 1, %0;" ::"n"(Shape<T>::kThreads) : "memory");
     reg_dec<kOtherRegs>();
@@ -314,7 +314,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     pdl_launch_dependents();
   }
   tc_fence_before();
-  if (T == 1) __syncthreads();
+  if (!kAhead) __syncthreads();
   else if (warp != kProducerWarp) asm volatile("bar.sync 1, %0;" ::"n"(Shape<T>::kThreads) : "memory");
   tc_fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&bars->tmem_base);
@@ -433,7 +433,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     if (lane == 0) bulk_wait<0>();                   // every store has been performed before the CTA may leave
   } else if (warp == kProducerWarp) {
     // ------------------------------------------------------------------ TMA producer, and the CTA's next unit
-    if (T == 1) reg_dec<kOtherRegs>();
+    if (!kAhead) reg_dec<kOtherRegs>();
     if (lane == 0) {
       bool ok = true, pending = false;              // pending: an answer of cluster launch control is on its way
       uint32_t g = 0, issued_k = 1, issued_v = 1;   // K / V tiles of the units before this one; tiles on their way so far
@@ -805,13 +805,13 @@ bool make_rows_map(void* out_map, const void* base, uint64_t rows, int head_dim)
 }
 
 namespace {
-template <int D, int T>
+template <int D, int T, bool kAhead = T == 2>
 int launch_tc(int grid, cudaStream_t st, const CUtensorMap& tm_q, const CUtensorMap& tk, const CUtensorMap& tv,
               const CUtensorMap& tm_kn, const CUtensorMap& tm_vn, const TcParams& p) {
   // two tiles of head_dim 64 ask for as much as head_dim 128: one CTA per SM, it owns all of tensor memory
   const size_t smem = T == 2 ? tc_smem_bytes<128, 2>() : tc_smem_bytes<D, T>();
-  if (!allow_dynamic_smem(attend_tc_kernel<D, T>, smem)) return -1;
-  launch_k(attend_tc_kernel<D, T>, grid, Shape<T>::kThreads, smem, st, tm_q, tk, tv, tm_kn, tm_vn, p);
+  if (!allow_dynamic_smem(attend_tc_kernel<D, T, kAhead>, smem)) return -1;
+  launch_k(attend_tc_kernel<D, T, kAhead>, grid, Shape<T>::kThreads, smem, st, tm_q, tk, tv, tm_kn, tm_vn, p);
   return launched(1);
 }
 }  // namespace
@@ -903,6 +903,12 @@ int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_sta
   p.row_stats = row_stats;
   p.status = a.status;
   if (a.head_dim == 128) return launch_tc<128, 2>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, p);
+  // Half an SM: a CTA's other warps run ahead of the wait for the compression if all CTAs run at once and heads have a
+  // few blocks (34 heads, 400 queries, 430 keys 22.4 -> 21.8 us a step, 60 heads 24.2 -> 23.6); beside a compression on the
+  // other half of their SMs their polling would slow that down (240 heads, 1 045 keys 110 -> 114; 120 heads, 576 queries, 918
+  // candidates 42.9 -> 43.5; 256 heads of 4 blocks 27.3 -> 28.2).
+  if (halves && compression_ctas > 0 && !p.steal && longest <= 5)
+    return launch_tc<64, 1, true>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, p);
   return halves ? launch_tc<64, 1>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, p)
                 : launch_tc<64, 2>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, p);
 }

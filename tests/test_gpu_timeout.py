@@ -109,6 +109,7 @@ def _aborted_last_step(head_dim, sides, budget_c, budget_s, heads=6, batch=1, me
     ((1, 2, 4, 12, 26), 300, 760),      # both types evict; at head_dim 64 two CTAs of the attention share an SM
     ((1, 2, 14, 24, 40), 2000, 2300),   # the same where a CTA takes two query tiles
     ((1, 2, 4, 12, 26), 300, 2000),     # structural heads append beside the compression of the others
+    ((1, 2, 6, 12, 22), 300, 600),      # lists of few blocks
 ])
 def test_a_step_that_evicts_gives_up_and_the_cache_stays_usable(head_dim, sides, budget_c, budget_s):
     assert _aborted_last_step(head_dim, sides, budget_c, budget_s) == 6    # HACK_ERR_TIMEOUT
