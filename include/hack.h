@@ -197,7 +197,8 @@ HACK_API hack_status_t hack_classify_heads(const double* sigma, int32_t n_layers
  * candidate count does not exceed their budget skip scoring and selection and keep everything
  * (section "KV Cache Compression for VAR": compress whenever the length exceeds the budget).
  * bf16 caches: at most two launches (one cluster launch that scores, selects and compacts, one
- * attention launch that also appends the rows of heads which keep the whole new scale).  The
+ * attention launch that also appends the rows of heads which keep the whole new scale); a step that
+ * merges takes seven, one whose candidate lists are beyond a cluster the launches of the stages.  The
  * attention of heads that do not depend on the compression runs beside it; steps whose heads fit into
  * shared memory are one launch (fp32 caches too).  `stream` orders everything (also inside a stream
  * capture). */

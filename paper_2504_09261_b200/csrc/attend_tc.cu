@@ -26,9 +26,9 @@
 //    softmax warps per scheduler, normally only one of them active) rather than more, lighter
 //    threads, and as few softmax instructions as possible: scale / sum / max work runs on packed
 //    or 3-input instructions.
-//  * The instruction cache: with every wait and every loop of the issuing warps unrolled the units made 82 KB of
-//    code and the warps waited for instructions 1.8 cycles per issue instead of 0.5 (head_dim 64: 112 -> 120 us
-//    a step).  Waits are small, the issuers' loops rolled, rare code is out of the way of the loop over the blocks.
+//  * The instruction cache: with every wait and every loop of the issuing warps unrolled the units made 91 KB of
+//    code and the warps waited for instructions 1.8 cycles per issue instead of 0.5 (6 % slower).  Waits are small,
+//    the issuers' loops rolled, rare code is out of the way of the loop over the blocks.
 //  * Work for padding: the last block of a segment is formed and weighted in groups of 32 keys.
 // Measured (a step with its compression, before -> with units, groups of 32 and rolled loops): 240 heads x 64,
 // 1 024 queries, 1 045 keys 115 -> 110 us; 256 heads x 64, 256 queries, 612 keys 38.9 -> 37.4; 32 heads x 128,
@@ -155,10 +155,9 @@ struct Bars {
 };
 
 // Waits for a phase of a barrier; false once a wait of the CTA has given up.  In little code: the instruction cache bounds
-// this kernel (with waits of 40 instructions, 82 instead of 40 KB in all, the loop lost 40 % at head_dim 64).  The producer keeps the
-// time: whatever else stands still, one of its own waits soon does too, and while it waits for the launch ahead, whose time is not this
-// launch's, nobody's counts.  (A clock in every wait that leaves that time out: 33.6 -> 35.0 us a step of 256 heads x 64.)  The status
-// word is written at the end, by one thread.
+// this kernel.  The producer keeps the time: whatever else stands still, one of its own waits soon does too, and while
+// it waits for the launch ahead, whose time is not this launch's, nobody's counts.  (A clock in every wait that leaves that time
+// out: 33.6 -> 35.0 us a step of 256 heads x 64.)  The status word is written at the end, by one thread.
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Bars* b, int code) {
   const uint32_t addr = smem_u32(bar);
   if (__builtin_expect(mbar_try_wait(addr, parity), 1)) return true;
@@ -817,7 +816,8 @@ int launch_tc(int grid, cudaStream_t st, const CUtensorMap& tm_q, const CUtensor
 }  // namespace
 
 float attend_tc_sm_us(const StepArgs& a, int type) {
-  // 4.5 us around the steps of a CTA; a step of 128 keys is bound by the exponentials at head_dim 64
+  // 4.5 us around the steps of a CTA (of a unit: a CTA that goes on with another one hides part of it); a step of 128 keys
+  // is bound by the exponentials at head_dim 64
   const float step_us = a.head_dim == 128 ? 1.6f : 1.2f;
   return (float)a.heads_of[type] * ((a.n_new + 2 * kBM - 1) / (2 * kBM)) * (4.5f + step_us * ((a.kept[type] + kBN - 1) / kBN));
 }

@@ -66,8 +66,8 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int& 
 }
 
 // Warp 0 finds the digit d (scanning from 255 down) at which the running count reaches `need`:
-// sum_{b > d} hist[b] < need <= sum_{b >= d} hist[b].  Returns through shared memory.
-__device__ __forceinline__ void locate_digit(const int* hist, int need, int* sh_digit, int* sh_need, int* sh_count) {
+// sum_{b > d} hist[b] < need <= sum_{b >= d} hist[b].  Returns through shared memory (sh_count: the entries of bin d, if asked for).
+__device__ __forceinline__ void locate_digit(const int* hist, int need, int* sh_digit, int* sh_need, int* sh_count = nullptr) {
   const int lane = threadIdx.x & 31;
   // lane l owns bins 255 - 8l ... 248 - 8l (descending), so lane order == descending bin order
   int c[8];
@@ -85,7 +85,11 @@ __device__ __forceinline__ void locate_digit(const int* hist, int need, int* sh_
     int cum = before;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      if (cum < need && need <= cum + c[i]) { *sh_digit = 255 - 8 * lane - i; *sh_need = need - cum; *sh_count = c[i]; }
+      if (cum < need && need <= cum + c[i]) {
+        *sh_digit = 255 - 8 * lane - i;
+        *sh_need = need - cum;
+        if (sh_count) *sh_count = c[i];
+      }
       cum += c[i];
     }
   }
@@ -254,7 +258,7 @@ select_kernel(const StepArgs a, const float* __restrict__ scores, int32_t* __res
   HeadView hv{scores + (size_t)bh * a.cand_stride, cand, a.stored[ctx], a.t_init, a.protect_new, ctx == 0};
 
   __shared__ int hist[256];
-  __shared__ int sh_digit, sh_need, sh_count;
+  __shared__ int sh_digit, sh_need;
   __shared__ int warp_sums[33];
 
   uint32_t prefix = 0, mask = 0;
@@ -272,7 +276,7 @@ select_kernel(const StepArgs a, const float* __restrict__ scores, int32_t* __res
       if (in && lane == __ffs(peers) - 1) atomicAdd(&hist[digit], __popc(peers));
     }
     __syncthreads();
-    if (tid < 32) locate_digit(hist, need, &sh_digit, &sh_need, &sh_count);
+    if (tid < 32) locate_digit(hist, need, &sh_digit, &sh_need);
     __syncthreads();
     prefix |= (uint32_t)sh_digit << shift;
     need = sh_need;
