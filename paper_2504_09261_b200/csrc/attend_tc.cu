@@ -860,10 +860,10 @@ int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_sta
   // type that does not wait for the compression has the SMs that launch does not hold.
   const int n_tiles = (a.n_new + kBM - 1) / kBM;
   // head_dim 64: CTAs of one tile that take half an SM each.  Two of them hide each other's start and
-  // epilogue (4.5 us of a CTA), but read every K/V tile twice as often as one CTA of two tiles.  Behind a
-  // compression, 256 heads x 100 queries, 255 keys: 21.2 against 24.8 us per step, 240 heads x 324
-  // queries, 640 keys: 38.4 against 43.8, 1 024 queries, 1 045 keys: 128.0 against 128.7; without one, 256
-  // heads x 256 queries, 680 keys: 32.0 against 30.6, 128 heads x 4 096 queries, 6 401 keys: 1 138 against 1 044.
+  // epilogue, but read every K/V tile twice as often as one CTA of two tiles.  Halves and whole SMs, us a step, behind a
+  // compression: 240 heads x 324 queries, 640 keys 35.3 and 36.9, 576 queries, 964 keys 69.0 and 72.4, but 1 024 queries, 1 045
+  // keys 100.3 and 94.5, 1 600 keys 180.9 and 171.3, 2 400 keys 152.9 and 141.3; without one: 256 heads x 256 queries, 655 keys 25.6 and
+  // 23.9, 64 heads x 1 024 queries, 2 200 keys 69.6 and 61.4, 100 queries, 181 keys 10.0 and 13.3.
   const int longest = (std::max(a.kept[0], a.kept[1]) + kBN - 1) / kBN;
   const bool halves = a.head_dim == 64 && longest <= (compression_ctas > 0 ? 12 : 4);
   const int slots = sm_count() * (halves ? 2 : 1);           // CTAs that run at once

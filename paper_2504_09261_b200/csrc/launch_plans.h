@@ -18,7 +18,9 @@ constexpr size_t kSmallMoveBytes = 384 * 1024;
 // 77.9 and, in a second wave, 81.5).  At head_dim 64 two of them meet on an SM if the launch leaves too few, so there it
 // leaves one each of attention_ctas (8 heads, 196 queries, 64 CTAs 23.0, 23.0 and 21.5; 16 heads, 112 CTAs 33.3, 31.7 and 36.4, 256
 // queries, 128 CTAs 28.4, 30.5 and 30.0; 26 heads, 182 CTAs 28.4, 32.3 and 34.3), unless there are two for every SM anyway (33
-// heads, 324 queries, 363 CTAs 60.2, 56.3 and 55.5; 45 heads, 256 queries, 360 CTAs 57.7 and 55.2).
+// heads, 324 queries, 363 CTAs 60.2, 56.3 and 55.5; 45 heads, 256 queries, 360 CTAs 57.7 and 55.2) or they come in clusters, one on an
+// SM (attention_ctas 0; 12 heads, a whole loop of 680 tokens 123.8 with two and one at its last scales, 121.2 with four).  In loops of one or two layers
+// four CTAs for 16 heads are 1 % faster, in loops of four and more 1 to 2 % slower.
 template <typename Places>
 int move_ctas(int heads, int attention_ctas, int sms, Places places) {
   int cl = 1;

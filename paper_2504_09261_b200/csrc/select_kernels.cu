@@ -309,7 +309,8 @@ int launch_select_move(const StepArgs& a, int dtype, const float* scores, const 
   const int row_pieces = a.head_dim * (dtype == HACK_F32 ? 4 : 2) / 16;
   if (max_cand > 4 * kSelThreads || (size_t)max_keep * row_pieces * 32 > kSmallMoveBytes) return 0;
   const int heads = a.batch * a.n_heads;
-  const int beside = dtype == HACK_F32 && a.head_dim == 64 ? simt::simt_plan(64, a.n_new, a.kept, a.heads_of, sm_count()).ctas : 0;
+  const simt::SimtPlan plan = simt::simt_plan(a.head_dim, a.n_new, a.kept, a.heads_of, sm_count());
+  const int beside = dtype == HACK_F32 && a.head_dim == 64 && plan.cluster == 1 ? plan.ctas : 0;
   const int cl = move_ctas(heads, beside, sm_count(), [](int ctas) {
     return cluster_places(reinterpret_cast<const void*>(select_move_kernel<4>), ctas, kSelThreads, 4 * kSelThreads * sizeof(int32_t));
   });

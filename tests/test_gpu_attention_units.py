@@ -58,3 +58,26 @@ def test_last_blocks_of_both_segments(dim, heads, batch, sides):
 ])
 def test_rounds_and_units_that_change_hands(dim, heads, batch, sides, b_c, b_s):
     decode(dim, heads, batch, sides, b_c, b_s, [(0, 0), (0, 1), (batch // 2, heads - 1), (batch - 1, heads - 2)])
+
+
+@pytest.mark.parametrize("dim,sides", [(64, (2, 9, 21)), (64, (3, 20, 40)), (128, (2, 9, 21))])
+def test_an_output_tensor_that_starts_between_two_sectors(dim, sides):
+    """Outputs 16 bytes past a 32-byte boundary are written in halves: the same bits, and nothing around them."""
+    import torch
+    import paper_2504_09261_b200 as hb
+    heads, batch = 6, 2
+    caches = [hb.HackCache(1, heads, dim, batch, sides, hb.HACK_BF16, [0, 1] * (heads // 2), 100, 400) for _ in range(2)]
+    g = torch.Generator(device="cuda").manual_seed(dim)
+    for k, side in enumerate(sides):
+        q, kk, v = (torch.randn((batch, heads, side * side, dim), generator=g, device="cuda").bfloat16() for _ in range(3))
+        out = torch.empty_like(q)
+        room = torch.full((q.numel() + 16,), 7.0, dtype=torch.bfloat16, device="cuda")
+        odd = room[8:-8].view(q.shape)
+        assert out.data_ptr() % 32 == 0 and odd.data_ptr() % 32 == 16
+        caches[0].hack_scale_step(0, k, q, kk, v, out)
+        caches[1].hack_scale_step(0, k, q, kk, v, odd)
+        assert torch.equal(out.view(torch.int16), odd.view(torch.int16)), k
+        assert bool((room[:8] == 7).all()) and bool((room[-8:] == 7).all())
+    for c in caches:
+        c.hack_poll_status()
+        c.close()

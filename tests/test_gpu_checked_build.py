@@ -35,7 +35,8 @@ def test_gpu_suite_passes_in_the_checked_build():
     files = ["tests/test_gpu_checked_build.py", "tests/test_gpu_parity.py", "tests/test_gpu_edges.py",
              "tests/test_gpu_merge.py", "tests/test_gpu_variance.py", "tests/test_gpu_timeout.py",
              "tests/test_gpu_parity_stack.py", "tests/test_gpu_small_steps.py", "tests/test_gpu_compress_shapes.py",
-             "tests/test_gpu_simt_tiles.py", "tests/test_gpu_attention_units.py", "tests/test_gpu_stream_order.py", "tests/test_zz_no_alloc.py"]
+             "tests/test_gpu_simt_tiles.py", "tests/test_gpu_attention_units.py", "tests/test_gpu_stream_order.py", "tests/test_zz_no_alloc.py",
+             "tests/test_gpu_merge_lists.py", "tests/test_gpu_merge_fused.py", "tests/test_gpu_cluster_places.py"]
     res = subprocess.run([sys.executable, "-m", "pytest", "-m", "gpu", "-x", "-q", "-p", "no:cacheprovider",
                           "-k", "not config4_every_point and not config2_triples"] + files,
                          cwd=ROOT, env=env, capture_output=True, text=True, timeout=1500)

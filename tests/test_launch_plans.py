@@ -103,7 +103,7 @@ def test_query_tiles_in_shares_at_head_dim_128(plans, queries, kept_s, kept_c, s
 def test_ctas_that_move_the_rows_of_a_head(plans, dim, heads, queries, kept_s, kept_c, us):
     out = (ctypes.c_int * 3)()
     plans.attention(dim, queries, kept_s, kept_c, heads - heads // 2, heads // 2, out)
-    cl = plans.move_ctas(heads, out[2] if dim == 64 else 0)
+    cl = plans.move_ctas(heads, out[2] if dim == 64 and out[0] == 1 else 0)
     best = min(t for t in us if t is not None)
     assert us[{1: 0, 2: 1, 4: 2}[cl]] <= 1.02 * best, (cl, list(out))
 
