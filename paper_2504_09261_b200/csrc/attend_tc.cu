@@ -183,8 +183,7 @@ __device__ __forceinline__ bool wait_timed(uint64_t* bar, uint32_t parity, Bars*
   return true;
 }
 
-// kAhead: the other warps do not wait behind the producer's wait for the launch ahead.
-template <int D, int T, bool kAhead = T == 2>
+template <int D, int T>
 __global__ void __launch_bounds__(Shape<T>::kThreads, Shape<T>::kCtasPerSm)
 attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kn,
@@ -277,10 +276,11 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (kAhead && warp == kProducerWarp) {
+  if (T == 2 && warp == kProducerWarp) {
     // The barriers are ready; the producer does not wait for the others, nor they for its wait for the launch ahead:
     // with all of them behind that wait, their code came in from L2 only then (3.0 instead of 2.1 us from the end of the
-    // compression to the first logits).  On half an SM only where heads are few and short (launch_attend_tc).
+    // compression to the first logits).  Not on half an SM, whose other half may be a CTA of the launch ahead that
+    // their polling slows down (240 heads x 64, 1 045 keys: 110 against 114 us a step).
     __syncwarp();
     asm volatile("bar.arrive 1, %0;" ::"n"(Shape<T>::kThreads) : "memory");
     reg_dec<kOtherRegs>();
@@ -313,7 +313,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     pdl_launch_dependents();
   }
   tc_fence_before();
-  if (!kAhead) __syncthreads();
+  if (T == 1) __syncthreads();
   else if (warp != kProducerWarp) asm volatile("bar.sync 1, %0;" ::"n"(Shape<T>::kThreads) : "memory");
   tc_fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&bars->tmem_base);
@@ -432,7 +432,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     if (lane == 0) bulk_wait<0>();                   // every store has been performed before the CTA may leave
   } else if (warp == kProducerWarp) {
     // ------------------------------------------------------------------ TMA producer, and the CTA's next unit
-    if (!kAhead) reg_dec<kOtherRegs>();
+    if (T == 1) reg_dec<kOtherRegs>();
     if (lane == 0) {
       bool ok = true, pending = false;              // pending: an answer of cluster launch control is on its way
       uint32_t g = 0, issued_k = 1, issued_v = 1;   // K / V tiles of the units before this one; tiles on their way so far
@@ -804,13 +804,13 @@ bool make_rows_map(void* out_map, const void* base, uint64_t rows, int head_dim)
 }
 
 namespace {
-template <int D, int T, bool kAhead = T == 2>
+template <int D, int T>
 int launch_tc(int grid, cudaStream_t st, const CUtensorMap& tm_q, const CUtensorMap& tk, const CUtensorMap& tv,
               const CUtensorMap& tm_kn, const CUtensorMap& tm_vn, const TcParams& p) {
   // two tiles of head_dim 64 ask for as much as head_dim 128: one CTA per SM, it owns all of tensor memory
   const size_t smem = T == 2 ? tc_smem_bytes<128, 2>() : tc_smem_bytes<D, T>();
-  if (!allow_dynamic_smem(attend_tc_kernel<D, T, kAhead>, smem)) return -1;
-  launch_k(attend_tc_kernel<D, T, kAhead>, grid, Shape<T>::kThreads, smem, st, tm_q, tk, tv, tm_kn, tm_vn, p);
+  if (!allow_dynamic_smem(attend_tc_kernel<D, T>, smem)) return -1;
+  launch_k(attend_tc_kernel<D, T>, grid, Shape<T>::kThreads, smem, st, tm_q, tk, tv, tm_kn, tm_vn, p);
   return launched(1);
 }
 }  // namespace
@@ -859,13 +859,15 @@ int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_sta
   // One query tile per CTA while that still fits one wave (twice the CTAs, no idle SMs), else two.  A
   // type that does not wait for the compression has the SMs that launch does not hold.
   const int n_tiles = (a.n_new + kBM - 1) / kBM;
-  // head_dim 64: CTAs of one tile that take half an SM each.  Two of them hide each other's start and
-  // epilogue, but read every K/V tile twice as often as one CTA of two tiles.  Halves and whole SMs, us a step, behind a
-  // compression: 240 heads x 324 queries, 640 keys 35.3 and 36.9, 576 queries, 964 keys 69.0 and 72.4, but 1 024 queries, 1 045
-  // keys 100.3 and 94.5, 1 600 keys 180.9 and 171.3, 2 400 keys 152.9 and 141.3; without one: 256 heads x 256 queries, 655 keys 25.6 and
-  // 23.9, 64 heads x 1 024 queries, 2 200 keys 69.6 and 61.4, 100 queries, 181 keys 10.0 and 13.3.
+  // head_dim 64: CTAs of one tile that take half an SM each.  They read every K/V tile twice as often as CTAs of two
+  // tiles, but a head of an odd number of tiles leaves none of those half empty.  Halves and whole SMs behind a compression, us a
+  // step: 240 heads, 3 tiles, 5 to 9 blocks of keys 48.1 to 73.7 and 51.2 to 77.3, 5 tiles, 8 blocks 84.0 and 85.5, but 4 tiles, 8
+  // blocks 75.3 and 72.2, 8 tiles, 9 and 12 blocks 119.8 and 113.9, 150.5 and 141.8; where every tile finds an SM whole ones, whose warps
+  // run ahead of the wait, are as fast or faster (34 heads, 3 tiles, 8 blocks 29.7 and 28.1, 4 tiles, 5 blocks 24.6 and 23.6).
+  // Without one: 256 heads, 1 tile, 2 blocks 10.0 and 13.3, 2 tiles, 3 blocks 20.1 and 18.8, 64 heads, 8 tiles, 18 blocks 69.6 and 61.4.
   const int longest = (std::max(a.kept[0], a.kept[1]) + kBN - 1) / kBN;
-  const bool halves = a.head_dim == 64 && longest <= (compression_ctas > 0 ? 12 : 4);
+  const bool halves = a.head_dim == 64 && n_tiles % 2 == 1 && n_tiles * (a.heads_of[0] + a.heads_of[1]) > sm_count() &&
+                      longest <= (compression_ctas > 0 ? 12 : 4);
   const int slots = sm_count() * (halves ? 2 : 1);           // CTAs that run at once
   const bool apart = p.dep[p.first_type] == kDepNothing && p.dep[1 - p.first_type] != kDepNothing;   // one type runs after the other
   for (int t = 0; t < 2; ++t) {
@@ -903,12 +905,6 @@ int launch_attend_tc(const StepArgs& a, const void* q, void* out, float* row_sta
   p.row_stats = row_stats;
   p.status = a.status;
   if (a.head_dim == 128) return launch_tc<128, 2>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, p);
-  // Half an SM: a CTA's other warps run ahead of the wait for the compression if all CTAs run at once and heads have a
-  // few blocks (34 heads, 400 queries, 430 keys 22.4 -> 21.8 us a step, 60 heads 24.2 -> 23.6); beside a compression on the
-  // other half of their SMs their polling would slow that down (240 heads, 1 045 keys 110 -> 114; 120 heads, 576 queries, 918
-  // candidates 42.9 -> 43.5; 256 heads of 4 blocks 27.3 -> 28.2).
-  if (halves && compression_ctas > 0 && !p.steal && longest <= 5)
-    return launch_tc<64, 1, true>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, p);
   return halves ? launch_tc<64, 1>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, p)
                 : launch_tc<64, 2>(grid, st, tm_q, tk, tv, tm_kn, tm_vn, p);
 }
