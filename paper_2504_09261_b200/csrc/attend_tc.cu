@@ -4,7 +4,7 @@
 //
 // One CTA serves one (batch, head) and up to two 128-row query tiles, which take turns on the
 // tensor pipe so that the softmax of one tile overlaps the MMAs of the other (T = 2); or, at head_dim
-// 64 and short caches, one tile on half an SM (T = 1: no warps 8-11, half the tensor memory).  A unit of work
+// 64, short caches and an odd number of tiles, one tile on half an SM (T = 1: no warps 8-11, half the tensor memory).  A unit of work
 // is a head and its one or two tiles (heads whose keys are one block: several rounds of them); where there are
 // more units than CTAs run at once, a CTA that nears the end of its unit takes over one that has not
 // been launched yet (cluster launch control): its loads and first products run under the last softmax and the
@@ -31,7 +31,7 @@
 //    the issuers' loops rolled, rare code is out of the way of the loop over the blocks.
 //  * Work for padding: the last block of a segment is formed and weighted in groups of 32 keys.
 // Measured (a step with its compression, before -> with units, groups of 32 and rolled loops): 240 heads x 64,
-// 1 024 queries, 1 045 keys 115 -> 110 us; 256 heads x 64, 256 queries, 612 keys 38.9 -> 37.4; 32 heads x 128,
+// 1 024 queries, 1 045 keys 115 -> 110 us (94 on whole SMs); 256 heads x 64, 256 queries, 612 keys 38.9 -> 37.4; 32 heads x 128,
 // 4 096 queries, 4 208 and 2 104 keys 191 -> 187.
 // TMEM (512 columns): S [0,128)  P0 [128,192)  P1 [192,256)  O0 [256,256+D)  O1 [256+D,256+2D).
 // There is ONE logit buffer, which the two tiles use in turn, and a probability buffer per tile.  A

@@ -6,7 +6,8 @@ is normally about a second, so nothing ever reaches it.  Here hack_set_wait_limi
 for one scoring launch: the consumers' first wait for an accumulator (which needs a key tile from
 HBM and an MMA, a microsecond at least) gives up, hack_poll_status reports the time-out, and the
 same cache, reset and back on the default limit, then passes the ordinary parity run.  Nothing
-spins and nothing faults: the wait itself returns.
+spins and nothing faults: the wait itself returns.  The same with whole steps that evict, append or
+merge, and a limit that launches behind one another and long units of work must not run into.
 """
 from dataclasses import replace
 
