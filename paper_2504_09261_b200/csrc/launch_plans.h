@@ -242,7 +242,8 @@ inline StepTimes step_times(const StepSizes& z, const StepShape& s, int per_sm, 
 // This side has become faster since the fit where every CTA has an SM and a cluster is smaller than eight, so there it
 // is taken up to a tenth past the line, to 256 queries: 13 heads x 128, 121 queries 20.5 -> 15.7 us, 36 heads, 169 queries
 // 22.2 -> 18.4, 52 heads x 64, 196 queries 22.5 -> 19.1.  Elsewhere it keeps a margin of a tenth (81 heads x 64, 169 queries
-// 20.5 against 24.6; 18 heads, 400 queries 21.2 against 22.5).  16 heads x 64, 36 queries, 91 candidates: 5.9 against 12.6;
+// 20.5 against 24.6; 18 heads, 400 queries 21.2 against 22.5; at 289 and 324 queries, 26 and 22 heads x 64, 13.6-16.4 against
+// 16.1-19.5, either margin takes it).  16 heads x 64, 36 queries, 91 candidates: 5.9 against 12.6;
 // 256 heads: 9.3 against 18.2; 100 queries, 168 and 255 candidates: 7.3 against 12.8 (16 heads), 20.2 against
 // 19.9 (256 heads: not taken); 16 heads x 128, 36 queries, 91 candidates: 7.5 against 15.0; 256 heads: 18.6
 // against 25.2.
