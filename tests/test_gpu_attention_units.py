@@ -81,3 +81,13 @@ def test_an_output_tensor_that_starts_between_two_sectors(dim, sides):
     for c in caches:
         c.hack_poll_status()
         c.close()
+
+
+@pytest.mark.parametrize("heads,batch,sides,b_c,b_s", [
+    (16, 16, (2, 8, 20, 29), 33, 1045),          # 7 query tiles, contextual heads of one short block: several rounds of one tile
+    (30, 8, (3, 9, 18), 128, 396),               # 3 tiles, a whole block and a last block of 12 keys
+    (20, 15, (2, 10, 13, 24), 230, 700),         # 5 tiles, more units than half SMs
+    (5, 60, (9, 10, 11), 400, 400),              # one tile, nothing is evicted
+])
+def test_odd_numbers_of_query_tiles_on_half_an_sm(heads, batch, sides, b_c, b_s):
+    decode(64, heads, batch, sides, b_c, b_s, [(0, 0), (0, 1), (batch // 2, heads - 1), (batch - 1, heads - 2)])
